@@ -13,7 +13,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libturboboa.so")
 
-SOURCES = ["tb_api.cu", "tb_hessian.cu", "tb_syrk_tc.cu", "tb_syrk_tc2.cu", "tb_cross_tc.cu", "tb_gemm_tc.cu", "tb_factor.cu", "tb_factor_static.cu", "tb_quantize.cu", "tb_block.cu", "tb_pack.cu"]
+SOURCES = ["tb_api.cu", "tb_hessian.cu", "tb_syrk_tc.cu", "tb_syrk_tc2.cu", "tb_cross_tc.cu", "tb_gemm_tc.cu", "tb_factor.cu", "tb_factor_static.cu", "tb_quantize.cu", "tb_sweep.cu", "tb_block.cu", "tb_pack.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Werror=pointer-arith",   # no arithmetic on untyped pointers
               "-I", INCLUDE, "-I", CSRC]
@@ -47,6 +47,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu file and link the shared library; returns its path."""
     os.makedirs(OBJ_DIR, exist_ok=True)
     deps = _deps()
+    # a library newer than every source is current, with or without its object files (they do not travel with it)
+    if not force and not _stale(LIB, [os.path.join(CSRC, s) for s in sources()] + deps):
+        return LIB
     nvcc = _nvcc()
     jobs = []
     objs = []
