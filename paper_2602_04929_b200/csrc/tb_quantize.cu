@@ -2,7 +2,7 @@
 //
 // Per step i (a group of g = out_block rows of every head, M = n_heads * g
 // rows in all, heads being independent):
-//   grid     k_grid           Algorithm 1, grid     candidate search per (row, column group)
+//   grid     k_grid_tri       Algorithm 1, grid     candidate search per (row, column group)
 //   sweep    k_sweep_rows     Algorithm 2 / Eq. 2   one launch, 8 rows per CTA for the whole sweep
 //   residual k_residual       E = W0 - Q_B          (Proposition 3.1)
 //            GEMM             E -= W0 C             (Proposition 3.2, only with R)
@@ -20,6 +20,7 @@
 #include "tb_common.cuh"
 #include "tb_gemm.cuh"
 #include "tb_profile.cuh"
+#include "tb_rows.cuh"
 #include "tb_tma.cuh"
 
 namespace cg = cooperative_groups;
@@ -38,18 +39,6 @@ tb_status split3(const float* B, __nv_bfloat16* Bp, long long n, cudaStream_t st
 }
 
 namespace tb {
-
-// ---------------------------------------------------------------------------
-// Row bookkeeping.  Active row m of a step maps to head m / g, row i0 + m % g
-// of that head.  "Units" are sets of rows that share one H_in / U_in: the
-// whole step when H_in is shared, one head otherwise.
-// ---------------------------------------------------------------------------
-struct RowMap {
-  int g, d_head, i0;
-  __host__ __device__ long long row(int m) const {
-    return (long long)(m / g) * d_head + i0 + (m % g);
-  }
-};
 
 __global__ void k_widen(const float* __restrict__ W, double* __restrict__ Wt, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -98,165 +87,11 @@ __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restri
 // Grid search (Algorithm 1, grid step).  For every (row, column group): n_cand
 // clipped min-max grids, p_k = 1 - k/32; score e H_in[G,G] e^T with e the
 // round-to-nearest error on that grid; the lowest score wins, lowest k on ties.
-//
-// One CTA takes RT = 128 / NCP rows (NCP = n_cand rounded up to a power of
-// two) of one column group: RT * NCP = 128 "candidate rows".  The scores are
-// the row-wise dots of (E H) with E, where E [128 x seg] holds the candidate
-// errors; E H runs on the GEMM tile engine with E produced on the fly.
-// ---------------------------------------------------------------------------
-struct GridP {
-  const double* Wt;   // [d_out][d]
-  const float* Hin;   // [n_hin][d][d]
-  double* sD;         // [d_out][ng]
-  float* s_out;       // [d_out][ng]
-  int* z_out;         // [d_out][ng]
-  unsigned char* cand_out;  // or nullptr
-  RowMap rm;
-  int M, d, seg, ng, maxq, n_cand, ncp, rt;
-  int units, rows_per_unit, tiles_per_unit;
-  const double* Wloc;  // or nullptr: the step's rows as a contiguous [M][d] working copy, read instead of Wt
-  int grp0;            // column group of blockIdx.x = 0
-};
-
-__global__ void __launch_bounds__(GEMM_THREADS, 1) k_grid(GridP p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double c_s[128], c_rs[128], c_z[128], c_J[128];
-  __shared__ long long c_row[128];  // global row of a candidate row, or -1
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int grp = p.grp0 + blockIdx.x;
-  const int unit = blockIdx.y / p.tiles_per_unit;
-  const int tile = blockIdx.y % p.tiles_per_unit;
-  const int seg0 = grp * p.seg;
-  const double maxq = (double)p.maxq;
-
-  // Phase 1: min / max of every row segment, then the candidates' (s, z).
-  for (int r = warp; r < p.rt; r += GEMM_THREADS / 32) {
-    const int rloc = tile * p.rt + r;
-    const bool valid = rloc < p.rows_per_unit;
-    long long grow = -1;
-    double mn = 0.0, mx = 0.0;
-    if (valid) {
-      grow = p.rm.row(unit * p.rows_per_unit + rloc);
-      const double* w = p.Wt + grow * p.d + seg0;
-      for (int a = lane; a < p.seg; a += 32) {
-        const double v = w[a];
-        mn = fmin(mn, v);
-        mx = fmax(mx, v);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      }
-    }
-    if (lane < p.ncp) {
-      const int k = lane, cr = r * p.ncp + k;
-      double s = 1.0, z = 0.0;
-      if (valid && k < p.n_cand) {
-        const double pk = 1.0 - (double)k / 32.0;
-        const double lo = pk * mn, hi = pk * mx;
-        if (hi != lo) {
-          s = (hi - lo) / maxq;
-          z = fmin(fmax(rne(-lo / s), 0.0), maxq);
-        }
-      }
-      c_s[cr] = s;
-      c_rs[cr] = 1.0 / s;
-      c_z[cr] = z;
-      c_row[cr] = (valid && k < p.n_cand) ? grow : -1;
-    }
-  }
-  // candidate rows beyond rt * ncp do not exist when ncp divides 128 (it does)
-  __syncthreads();
-
-  const float* H = p.Hin + (long long)unit * p.d * p.d * (p.units > 1 ? 1 : 0);
-  const double* Wt = p.Wt;
-  const int d = p.d, seg = p.seg;
-
-  // round-to-nearest error of weight w on the grid of candidate row cr (0 for w = 0,
-  // which is what rows and columns outside the problem are given)
-  auto err_of = [&](int cr, double w) -> double {
-    const double s = c_s[cr], z = c_z[cr];
-    double q = rne(fma(w, c_rs[cr], z));
-    q = fmin(fmax(q, 0.0), maxq);
-    return w - s * (q - z);
-  };
-  // quantization error of candidate row cr at segment column a
-  auto err_at = [&](int cr, int a) -> double {
-    const long long grow = c_row[cr];
-    if (grow < 0 || a >= seg) return 0.0;
-    return err_of(cr, Wt[grow * d + seg0 + a]);
-  };
-
-  double jpart[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) jpart[i] = 0.0;
-
-  for (int a0 = 0; a0 < seg; a0 += GEMM_BN) {
-    GemmAcc<double> acc;
-    acc.clear();
-    // fetch the weight; the candidate's error is formed when the chunk is staged
-    auto la = [&](int mm, int k) -> double {
-      const long long grow = c_row[mm];
-      return (grow >= 0 && k < seg) ? Wt[grow * d + seg0 + k] : 0.0;
-    };
-    auto ca = [&](double w, int mm, int) -> double { return err_of(mm, w); };
-    auto lb = [&](int nn, int k) -> float {
-      const int a = a0 + nn;
-      return (a < seg && k < seg) ? H[(long long)(seg0 + k) * d + seg0 + a] : 0.0f;
-    };
-    auto cb = [](float v, int, int) -> double { return (double)v; };
-    gemm_mainloop<double, true, true>(acc, la, ca, lb, cb, 0, seg, smem_raw);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int cr = GemmAcc<double>::row(i);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        jpart[i] = fma(acc.at(i, j), err_at(cr, a0 + GemmAcc<double>::col(j)), jpart[i]);
-    }
-  }
-  // A candidate row's score is spread over the 4 lanes of a quad and the 4 warps that
-  // share its rows; quads reduce by shuffle, warps through shared memory in a fixed order.
-  double* c_Jw = reinterpret_cast<double*>(smem_raw);  // [4][128], the tile buffers are free now
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    double v = jpart[i];
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    if ((lane & 3) == 0) c_Jw[(warp & 3) * 128 + GemmAcc<double>::row(i)] = v;
-  }
-  __syncthreads();
-  if (tid < 128) c_J[tid] = ((c_Jw[tid] + c_Jw[128 + tid]) + c_Jw[256 + tid]) + c_Jw[384 + tid];
-  __syncthreads();
-
-  // Phase 3: argmin per row, strict '<' so that the lowest k wins ties.
-  if (tid < p.rt) {
-    const int r = tid;
-    const long long grow = c_row[r * p.ncp];
-    if (grow >= 0) {
-      int best = 0;
-      double bj = c_J[r * p.ncp];
-      for (int k = 1; k < p.n_cand; ++k) {
-        const double j = c_J[r * p.ncp + k];
-        if (j < bj) {
-          bj = j;
-          best = k;
-        }
-      }
-      const int cr = r * p.ncp + best;
-      const long long o = grow * p.ng + grp;
-      p.sD[o] = c_s[cr];
-      p.s_out[o] = (float)c_s[cr];
-      p.z_out[o] = (int)c_z[cr];
-      if (p.cand_out) p.cand_out[o] = (unsigned char)best;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The same search for groups of at most 128 columns, where the whole problem of a
-// CTA (128 candidate rows x one group) fits shared memory.  H_in[G,G] is symmetric,
+// Groups wider than 128 columns: tb_grid_wide.cu.  Here the search
+// for groups of at most 128 columns, where the whole problem of a CTA (128
+// candidate rows x one group) fits shared memory.  One CTA takes RT = 128 / NCP
+// rows (NCP = n_cand rounded up to a power of two) of one column group:
+// RT * NCP = 128 "candidate rows".  H_in[G,G] is symmetric,
 // so e H e^T = 2 e T e^T with T the upper triangle of H (diagonal halved): only the
 // part k <= n of the product is formed, about half of the tensor-pipe work.  The
 // scores are compared, never output, so the factor 2 is dropped.  The candidate
@@ -1788,16 +1623,14 @@ static tb_status run_grid(const Plan& p, const float* H_in, float* scales, int* 
   gp.tiles_per_unit = (gp.rows_per_unit + p.rt - 1) / p.rt;
   gp.Wloc = nullptr;
   gp.grp0 = 0;
-  static bool configured[64] = {false}, configured_tri[64] = {false};
-  TB_TRY(allow_smem(k_grid, GemmSmem<double>::bytes, configured));
+  if (p.seg > 128)  // E is free until the sweep of a step
+    return grid_wide(gp, p.E, (size_t)p.Mmax * p.d, st);
+  static bool configured_tri[64] = {false};
   TB_TRY(allow_smem(k_grid_tri, GRID_TRI_SMEM, configured_tri));
   const long long ytiles = (long long)gp.units * gp.tiles_per_unit;
   if (ytiles > 65535) return TB_ERR_UNSUPPORTED;
   dim3 grid(p.ng, (unsigned)ytiles);
-  if (p.seg <= 128)
-    k_grid_tri<<<grid, GEMM_THREADS, GRID_TRI_SMEM, st>>>(gp);
-  else
-    k_grid<<<grid, GEMM_THREADS, GemmSmem<double>::bytes, st>>>(gp);
+  k_grid_tri<<<grid, GEMM_THREADS, GRID_TRI_SMEM, st>>>(gp);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
