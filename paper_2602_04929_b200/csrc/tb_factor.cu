@@ -8,9 +8,10 @@
 // No inverse of H is formed.  Everything runs in double: with cond(H_in) ~ 1e5
 // a float factorisation would lose most of U's digits.
 //
-// The matrix is embedded in a dp x dp one (dp = 64 * 2^k >= d, identity in the
-// padding) so that every block step below is uniform.
-//   1. A = J H J                                        (k_reverse_in)
+// H is first scaled by powers of two to diagonal entries in [1/2, 2), H = D A D: exact, undone exactly in U (whose
+// columns it scales), and every entry of L is then below 1.42.  The matrix is padded to dp, the next
+// multiple of 64 (identity in the padding).
+//   1. A = J D^-1 H D^-1 J                              (k_scale_exp, k_reverse_in)
 //   2. right-looking blocked Cholesky, 64-column panels, two launches per panel:
 //        k_chol_panel  every CTA factors the 64 x 64 diagonal block (one thread
 //                      per row, the row in registers, right-looking) and then
@@ -23,38 +24,80 @@
 //      neighbouring inverted blocks A, B with coupling C = L[B rows, A cols] gets
 //      its off-diagonal block -B^{-1} C A^{-1} from two batched GEMMs.  Steps 3 and 4
 //      follow the factorisation block by block of 512 columns, so that with the
-//      look-ahead they run beside the later panels.
-//   5. U = J L^{-1} J, written as float with an explicit zero lower triangle.
+//      look-ahead they run beside the later panels.  L^{-1} takes the place of L: a block of L
+//      is dead once its pair has been formed.
+//   5. U = J L^{-1} J D^-1, written as float with an explicit zero lower triangle.
+// From 1024 columns on the rank-256 updates and the doubling steps of 512 columns and more run on the
+// integer tensor cores (tb_i8.cuh).  The digits of L (one exponent for all, see the scaling) serve the
+// updates and the first product of a pair; the digits of a pair's inverse halves and of its first product
+// take the places of the digits of L that the pair has used up.
 #include "tb_common.cuh"
 #include "tb_gemm.cuh"
 #include "tb_gemm64.cuh"
+#include "tb_i8.cuh"
 
 namespace tb {
 
 enum { FNB = 64 };
 
-// A (dp x dp) <- J H J in the leading d x d block, identity elsewhere
-__global__ void k_reverse_in(const float* __restrict__ H, double* __restrict__ A, int d, int dp) {
-  const long long n = (long long)dp * dp;
-  const float* Hb = H + (long long)blockIdx.y * d * d;
-  double* Ab = A + (long long)blockIdx.y * n;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(idx / dp), j = (int)(idx % dp);
+// exps[i] = e with H_ii 2^(-2e) in [1/2, 2) (0 where the diagonal is not positive and finite); also clears the
+// error words of the matrix.  Rows in elimination order: row r of A is row d - 1 - r of H.
+__global__ void k_scale_exp(const float* __restrict__ H, int* __restrict__ exps, int* __restrict__ bad, int* info, int d,
+                            int dp) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+  if (r == 0) info[b] = 0;
+  if (r >= dp) return;
+  int e = 0;
+  if (r < d) {
+    const int i = d - 1 - r;
+    const float h = H[((long long)b * d + i) * d + i];
+    if (h > 0.0f && h <= 3.4e38f) {
+      int x;
+      frexp((double)h, &x);  // h = f 2^x, f in [1/2, 1)
+      e = x >> 1;            // floor(x / 2): f or 2 f remains
+    }
+  }
+  exps[(long long)b * dp + r] = e;
+  bad[(long long)b * dp + r] = 0;
+}
+__device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// A (dp x dp) <- J D^-1 H D^-1 J in the leading d x d block, identity elsewhere (lower triangle and the
+// diagonal blocks only: nothing else is read).  A CTA: 8 rows x 256 columns.
+__global__ void __launch_bounds__(256) k_reverse_in(const float* __restrict__ H, const int* __restrict__ exps,
+                                                    double* __restrict__ A, int d, int dp) {
+  const int j = blockIdx.x * 256 + threadIdx.x, i0 = blockIdx.y * 8;
+  if (j >= dp || blockIdx.x * 256 > i0 + 7 + FNB) return;
+  const float* Hb = H + (long long)blockIdx.z * d * d;
+  const int* eb = exps + (long long)blockIdx.z * dp;
+  double* Ab = A + (long long)blockIdx.z * dp * dp;
+  const int ej = eb[j];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = i0 + k;
     double v = (i == j) ? 1.0 : 0.0;
-    if (i < d && j < d) v = (double)Hb[(long long)(d - 1 - i) * d + (d - 1 - j)];
-    Ab[idx] = v;
+    if (i < d && j < d) v = (double)Hb[(long long)(d - 1 - i) * d + (d - 1 - j)] * pow2i(-(eb[i] + ej));
+    Ab[(long long)i * dp + j] = v;
   }
 }
 
-__global__ void k_reverse_out(const double* __restrict__ Li, float* __restrict__ U, int d, int dp) {
-  const long long n = (long long)d * d;
-  const double* Lb = Li + (long long)blockIdx.y * dp * dp;
-  float* Ub = U + (long long)blockIdx.y * n;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(idx / d), j = (int)(idx % d);
-    Ub[idx] = (j >= i) ? (float)Lb[(long long)(d - 1 - i) * dp + (d - 1 - j)] : 0.0f;
+// U = J L^-1 J D^-1; clean: L^-1 D^-1 (columns scaled, zeros above the diagonal) also replaces L^-1
+__global__ void __launch_bounds__(256) k_reverse_out(double* __restrict__ Li, const int* __restrict__ exps,
+                                                     float* __restrict__ U, int d, int dp, int clean) {
+  const int j = blockIdx.x * 256 + threadIdx.x;
+  if (j >= d) return;
+  double* Lb = Li + (long long)blockIdx.z * dp * dp;
+  float* Ub = U + (long long)blockIdx.z * d * d;
+  const int c = d - 1 - j;
+  const double sc = pow2i(-exps[(long long)blockIdx.z * dp + c]);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = blockIdx.y * 8 + k;
+    if (i >= d) break;
+    double* l = Lb + (long long)(d - 1 - i) * dp + c;
+    const double v = (j >= i) ? *l * sc : 0.0;
+    Ub[(long long)i * d + j] = (float)v;
+    if (clean) *l = v;
   }
 }
 
@@ -89,7 +132,8 @@ __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
 
 __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict__ A, double* __restrict__ Ldiag,
                                                               long long ldiag_batch, int* __restrict__ info, int dp,
-                                                              int k0, int d_fact, int update_first) {
+                                                              int k0, int d_fact, int update_first,
+                                                              const int* __restrict__ bad) {
   extern __shared__ __align__(16) unsigned char panel_raw[];
   double* sA = reinterpret_cast<double*>(panel_raw);  // this CTA's 64 panel rows
   double* sC = sA + 64 * PLD;                         // the diagonal block, then its raw columns: sC[j * PLD + r]
@@ -98,6 +142,8 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
   double* sPd = sY + 2 * PQ * 64;                     // previous panel, rows of the diagonal block: sPd[k * PLD + row]
   double* sPr = sPd + 64 * PLD;                       // previous panel, this CTA's rows, same layout
   const int tid = threadIdx.x, r = tid & 63, q = tid >> 6, b = blockIdx.y;
+  __shared__ int sbad[FNB];  // rows whose entries left of this panel were not finite
+  if (tid < FNB) sbad[tid] = bad[(long long)b * dp + k0 + tid];
   double* Ab = A + (long long)b * dp * dp;
   double* diag = Ab + (long long)k0 * dp + k0;
   const long long row0 = (long long)k0 + FNB + (long long)FNB * blockIdx.x;
@@ -186,7 +232,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
       if (q < jb || (r | 31) < j) continue;  // warps wholly left of or above the pivot only keep the barriers
       const double* col = sC + j * PLD;
       double piv = col[j];
-      if (!(piv > 0.0)) {
+      if (!(piv > 0.0) || sbad[j]) {
         if (tid == j + 64 * jb && blockIdx.x == 0) atomicCAS(&info[b], 0, k0 + j + 1);
         piv = 1.0;
       }
@@ -264,15 +310,16 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
 
 // Inverse of every 64 x 64 diagonal block of L into the same block of Li (lower triangular):
 // forward substitution, one thread per column, the column in registers.
+// The part of the block's rows right of it, up to the end of its block of 512 columns, becomes zero: the doubling
+// products inside that block read it.
 __global__ void __launch_bounds__(64) k_inv_diag64(const double* __restrict__ Ldiag, long long ldiag_batch,
-                                                   int n_factored, double* __restrict__ Li, int dp, int blk0) {
+                                                   double* __restrict__ Li, int dp, int blk0, int col_end) {
   __shared__ double Ls[FNB][FNB + 1];
   __shared__ double rdiag[FNB];
   const int blk = blk0 + blockIdx.x, b = blockIdx.y, c = threadIdx.x;
   const long long off = (long long)b * dp * dp + (long long)blk * FNB * (dp + 1);
-  // blocks of the identity padding were never factored: their factor is the identity
   const double* src = Ldiag + (long long)b * ldiag_batch + (long long)blk * FNB * FNB;
-  for (int r = 0; r < FNB; ++r) Ls[r][c] = (blk < n_factored) ? src[r * FNB + c] : (r == c ? 1.0 : 0.0);
+  for (int r = 0; r < FNB; ++r) Ls[r][c] = src[r * FNB + c];
   __syncthreads();
   rdiag[c] = 1.0 / Ls[c][c];
   __syncthreads();
@@ -286,6 +333,9 @@ __global__ void __launch_bounds__(64) k_inv_diag64(const double* __restrict__ Ld
   }
 #pragma unroll
   for (int r = 0; r < FNB; ++r) Li[off + (long long)r * dp + c] = x[r];
+  const int right = col_end - (blk + 1) * FNB;
+  for (int r = 0; r < FNB; ++r)
+    for (int k = c; k < right; k += 64) Li[off + (long long)r * dp + FNB + k] = 0.0;
 }
 
 // strictly-upper mask of a square matrix (Algorithm 2: (R U^T) .* M_U)
@@ -301,7 +351,11 @@ __global__ void k_mask_strict_upper(const double* __restrict__ src, double* __re
 enum { INV_BLOCK = 512 };  // the inverse is completed block by block of this many columns (see factor_run)
 
 struct FactorWs {
-  double *A, *Li, *tmp;
+  double *A, *tmp;  // A: the scaled matrix, then L, then L^-1
+  int *exps, *bad;
+  unsigned long long* mx;  // largest magnitudes of the rows and columns of the doubling products' operands
+  I8Mat digits;            // of L, then of the operands of the doubling products
+  bool use_i8;
   int dp;
   size_t tmp_per;   // doubles of tmp per matrix
   size_t low_off;   // products of the doubling levels inside one block of INV_BLOCK columns (two regions in turn)
@@ -309,28 +363,38 @@ struct FactorWs {
   size_t total;
 };
 
-static int padded_dim(int d) {
-  int dp = FNB;
-  while (dp < d) dp <<= 1;
-  return dp;
-}
+// The digits pay where the contraction and the matrix are large: one factor of 2048 columns takes the same time
+// either way (1.36 ms on the FP64 pipe, 1.37), of 4096 3.44 and 2.86, 8 x 8192 114 and 62; below 1024 there
+// is no block update wide enough.
+enum { FACTOR_I8_MIN = 1024 };
 
 static FactorWs factor_ws(int n_batch, int d, void* ws) {
   FactorWs f;
   Bump b(ws);
-  f.dp = padded_dim(d);
-  const size_t n = (size_t)f.dp * f.dp;
+  f.dp = ((d + FNB - 1) / FNB) * FNB;
+  const size_t dp = (size_t)f.dp, n = dp * dp;
+  f.use_i8 = f.dp >= FACTOR_I8_MIN;
   f.A = b.take<double>((size_t)n_batch * n);
-  f.Li = b.take<double>((size_t)n_batch * n);
+  f.exps = b.take<int>((size_t)n_batch * dp);
+  f.bad = b.take<int>((size_t)n_batch * dp);
   // tmp per matrix: the factored diagonal blocks (dp x 64), then the intermediate products of the
   // doubling steps.  The inverse proceeds while later panels are still being factored, and a product
   // of a high level stays alive while lower levels run, so each gets a region of its own.
-  const size_t gdim = (f.dp < INV_BLOCK) ? (size_t)f.dp : (size_t)INV_BLOCK;
-  f.low_off = (size_t)f.dp * FNB;
+  const size_t gdim = (dp < INV_BLOCK) ? dp : (size_t)INV_BLOCK;
+  f.low_off = dp * FNB;
   f.high_off = f.low_off + 2 * (gdim * gdim / 4);  // two regions: neighbouring blocks are inverted side by side
   f.tmp_per = f.high_off;
-  for (size_t sb = gdim; sb < (size_t)f.dp; sb <<= 1) f.tmp_per += sb * sb;
+  for (size_t sb = INV_BLOCK; sb < dp; sb <<= 1) f.tmp_per += sb * sb;
   f.tmp = b.take<double>((size_t)n_batch * f.tmp_per + 64);
+  f.mx = nullptr;
+  f.digits = I8Mat{nullptr, 0, 0};
+  if (f.use_i8) {
+    f.digits.row_blocks = (long long)n_batch * (f.dp / I8_RB);
+    f.digits.k_blocks = f.dp / I8_KB;
+    f.digits.data = b.take<unsigned char>(i8_bytes(f.digits.row_blocks, f.digits.k_blocks));
+    // columns of the first product's right operand, rows and columns of the second's
+    f.mx = b.take<unsigned long long>((size_t)n_batch * 3 * dp);
+  }
   f.total = b.total();
   return f;
 }
@@ -421,17 +485,15 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   FactorWs f = factor_ws(n_batch, d, ws);
   const int dp = f.dp;
   const long long pp = (long long)dp * dp;
-  TB_CUDA_CHECK(cudaMemsetAsync(info, 0, sizeof(int) * (size_t)n_batch, st));
-  TB_CUDA_CHECK(cudaMemsetAsync(f.Li, 0, sizeof(double) * (size_t)n_batch * pp, st));
-  int eb = (int)((pp + 255) / 256);
-  if (eb > 148 * 8) eb = 148 * 8;
-  k_reverse_in<<<dim3(eb, n_batch), 256, 0, st>>>(H, f.A, d, dp);
+  if (dp > 65536) return TB_ERR_UNSUPPORTED;
+  k_scale_exp<<<dim3((dp + 255) / 256, n_batch), 256, 0, st>>>(H, f.exps, f.bad, info, d, dp);
+  TB_LAUNCH_CHECK();
+  k_reverse_in<<<dim3((dp + 255) / 256, dp / 8, n_batch), 256, 0, st>>>(H, f.exps, f.A, d, dp);
   TB_LAUNCH_CHECK();
 
   static bool panel_configured[64] = {false};
   TB_TRY(allow_smem(k_chol_panel, PANEL_SMEM, panel_configured));
-  // the padding is an identity block decoupled from the rest: factor the leading part only
-  const int d_fact = ((d + FNB - 1) / FNB) * FNB;
+  const int d_fact = dp;
   FactorSide* side = nullptr;
   if (lookahead && d_fact >= 16 * FNB) {
     side = factor_side();
@@ -448,51 +510,40 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   // on a stream of its own beside the later panels, and little of the inverse is left after the last
   // panel; without it the same launches follow the panels on the caller's stream.  Every product is
   // the same launch either way, so the result is the same bit for bit.
-  const int G = (dp < INV_BLOCK) ? dp : INV_BLOCK;
-  const int n_inv_blocks = dp / G, n_panels = d_fact / FNB;
+  const int G = INV_BLOCK;
+  const int n_inv_blocks = (dp + G - 1) / G, n_panels = dp / FNB;
+  const long long rb = dp / I8_RB;  // row blocks of digits per matrix
   cudaStream_t inv_st = side ? side->inv : st;
   cudaStream_t cs = side ? side->crit : st;  // stream of the panels
-  // first product of a pair at level sblk: T = C A^{-1}, C = L[s:2s, 0:s], A^{-1} = Li[0:s, 0:s] (lower triangular)
-  // Launched in pieces of at most 768 columns (96 tiles at 2048 rows): the tiles of the upper levels
-  // run for hundreds of microseconds, and a launch that fills every SM with them would keep the panels
-  // waiting.  The first columns meet the longest part of the triangle, so the pieces get shorter.  A
-  // piece is the same set of tiles, so nothing changes in the result.
-  auto pair_first = [&](int sblk, long long off, long long pair_stride, int batch, double* tmp, long long tmp_stride,
+  // A pair at level s: columns off .. off + s - 1 (inverse A^{-1} in place) and the m2 <= s rows below them.
+  // first product: T = C A^{-1}, C = L[off+s.., off..], m2 x s
+  auto pair_first = [&](int sblk, int m2, long long off, long long pair_stride, int batch, double* tmp, long long tmp_stride,
                         cudaStream_t stream_first) -> tb_status {
     GemmP g = gemm_params();
     g.A = f.A + off + (long long)sblk * dp;
     g.a_m = dp;
     g.a_k = 1;
     g.a_batch = pair_stride;
-    g.B = f.Li + off;
+    g.B = f.A + off;
     g.b_k = dp;
     g.b_n = 1;
     g.b_batch = pair_stride;
     g.C = tmp;
     g.ldc = sblk;
     g.c_batch = tmp_stride;
-    g.M = sblk;
+    g.M = m2;
     g.N = sblk;
     g.K = sblk;
     g.n_batch = batch;
     g.btrim = 2;
     g.flags = GEMM_HEAVY_N_FIRST;
-    const int piece = (sblk > 1024) ? 768 : sblk;
-    for (int n0 = 0; n0 < sblk; n0 += piece) {
-      GemmP gp = g;
-      gp.B = f.Li + off + n0;  // B(k, n0 + n), zero for k < n0 + n
-      gp.boff = n0;
-      gp.C = tmp + n0;
-      gp.N = (sblk - n0 < piece) ? sblk - n0 : piece;
-      TB_TRY((gemm64_launch<true>(gp, stream_first)));
-    }
-    return TB_OK;
+    return gemm64_launch<true>(g, stream_first);
   };
-  // second product: Li[s:2s, 0:s] = -B^{-1} T, B^{-1} = Li[s:2s, s:2s] (lower triangular)
-  auto pair_second = [&](int sblk, long long off, long long pair_stride, int batch, double* tmp, long long tmp_stride,
+  // second product: L^{-1}[off+s.., off..] = -B^{-1} T, B^{-1} = L^{-1}[off+s.., off+s..] (lower triangular)
+  auto pair_second = [&](int sblk, int m2, long long off, long long pair_stride, int batch, double* tmp, long long tmp_stride,
                          cudaStream_t stream_second) -> tb_status {
     GemmP h = gemm_params();
-    h.A = f.Li + off + (long long)sblk * (dp + 1);
+    h.A = f.A + off + (long long)sblk * (dp + 1);
     h.a_m = dp;
     h.a_k = 1;
     h.a_batch = pair_stride;
@@ -500,17 +551,83 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     h.b_k = sblk;
     h.b_n = 1;
     h.b_batch = tmp_stride;
-    h.C = f.Li + off + (long long)sblk * dp;
+    h.C = f.A + off + (long long)sblk * dp;
     h.ldc = dp;
     h.c_batch = pair_stride;
-    h.M = sblk;
+    h.M = m2;
     h.N = sblk;
-    h.K = sblk;
+    h.K = m2;
     h.n_batch = batch;
     h.alpha = -1.0;
     h.atrim = 1;
     h.flags = GEMM_HEAVY_M_LAST;
     return gemm64_launch<true>(h, stream_second);
+  };
+  // The same two products on the integer tensor cores, all matrices of the batch (o: first column of the pair).  The
+  // digits of A^{-1} (by columns) take the place of those of the square of L it is the inverse of, and so do the
+  // digits of B^{-1}; the digits of T (by columns) that of C's.  Every update that reads one of these parts of L
+  // belongs to columns that have been factored by then.
+  const int tile_life = side ? 2 : 0;  // beside the panels: CTAs that end soon
+  // row / column maxima, indexed by the pair's columns: pairs whose products run side by side have no column in common
+  auto level_max = [&](int which) { return f.mx + (size_t)n_batch * dp * which; };
+  auto pair_first_i8 = [&](int sblk, int m2, int o, double* tmp, cudaStream_t s1) -> tb_status {
+    unsigned long long* mx = level_max(0) + o;
+    I8Src b{f.A + (long long)o * (dp + 1), dp, pp, sblk, sblk, n_batch, false, false, 2};
+    TB_TRY(i8_row_max(b, mx, dp, s1));
+    TB_TRY(i8_slice(b, mx, dp, 0, f.digits, o / I8_RB, rb, o / I8_KB, s1));
+    I8Gemm g = i8_gemm_params();
+    g.A = g.B = f.digits;
+    g.a_rb = (o + sblk) / I8_RB;
+    g.b_rb = o / I8_RB;
+    g.a_rb_batch = g.b_rb_batch = rb;
+    g.a_kb = g.b_kb = o / I8_KB;
+    g.k_blocks = sblk / I8_KB;
+    g.a_exp = 1;
+    g.b_max = mx;
+    g.b_max_batch = dp;
+    g.C = tmp;
+    g.ldc = sblk;
+    g.c_batch = (long long)f.tmp_per;
+    g.M = m2;
+    g.N = sblk;
+    g.n_batch = n_batch;
+    g.zeros = 2;
+    g.order = 1;
+    g.tiles_per_cta = tile_life;
+    return i8_gemm(g, s1);
+  };
+  auto pair_second_i8 = [&](int sblk, int m2, int o, double* tmp, cudaStream_t s2) -> tb_status {
+    unsigned long long *ma = level_max(1) + o, *mt = level_max(2) + o;
+    const int o2 = o + sblk;
+    I8Src a{f.A + (long long)o2 * (dp + 1), dp, pp, m2, m2, n_batch, false, true, 1};
+    TB_TRY(i8_row_max(a, ma, dp, s2));
+    TB_TRY(i8_slice(a, ma, dp, 0, f.digits, o2 / I8_RB, rb, o2 / I8_KB, s2));
+    // T: sblk columns (rows of digits), m2 contraction steps
+    I8Src t{tmp, sblk, (long long)f.tmp_per, sblk, m2, n_batch, false, false, 0};
+    TB_TRY(i8_row_max(t, mt, dp, s2));
+    TB_TRY(i8_slice(t, mt, dp, 0, f.digits, o / I8_RB, rb, o2 / I8_KB, s2));
+    I8Gemm g = i8_gemm_params();
+    g.A = g.B = f.digits;
+    g.a_rb = o2 / I8_RB;
+    g.b_rb = o / I8_RB;
+    g.a_rb_batch = g.b_rb_batch = rb;
+    g.a_kb = g.b_kb = o2 / I8_KB;
+    g.k_blocks = m2 / I8_KB;
+    g.a_max = ma;
+    g.a_max_batch = dp;
+    g.b_max = mt;
+    g.b_max_batch = dp;
+    g.C = f.A + (long long)o2 * dp + o;
+    g.ldc = dp;
+    g.c_batch = pp;
+    g.M = m2;
+    g.N = sblk;
+    g.n_batch = n_batch;
+    g.alpha = -1.0;
+    g.zeros = 1;
+    g.order = 2;
+    g.tiles_per_cta = tile_life;
+    return i8_gemm(g, s2);
   };
   auto high_tmp = [&](int sblk) {  // region of the level-sblk product (first matrix of the batch)
     size_t o = f.high_off;
@@ -518,51 +635,68 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     return f.tmp + o;
   };
   auto invert_block = [&](int j) -> tb_status {
-    const long long boff = (long long)j * G * (dp + 1);
+    const int o0 = j * G, width = (dp - o0 < G) ? dp - o0 : G;  // the last block may be narrower
+    const long long boff = (long long)o0 * (dp + 1);
     // inside the block: a stream per block parity, so that a block does not wait for its neighbour's
     // upper levels; the caller has just recorded block_done
     cudaStream_t low_st = side ? side->low[j & 1] : inv_st;
-    const size_t low_region = f.low_off + (size_t)(j & 1) * ((size_t)G * G / 4);
+    const size_t low_region = f.low_off + (size_t)(j & 1) * ((f.high_off - f.low_off) / 2);
     if (side) TB_CUDA_CHECK(cudaStreamWaitEvent(low_st, side->block_done, 0));
-    k_inv_diag64<<<dim3(G / FNB, n_batch), 64, 0, low_st>>>(f.tmp, (long long)f.tmp_per, n_panels, f.Li, dp,
-                                                             j * (G / FNB));
+    k_inv_diag64<<<dim3(width / FNB, n_batch), 64, 0, low_st>>>(f.tmp, (long long)f.tmp_per, f.A, dp, j * (G / FNB),
+                                                                 o0 + width);
     TB_LAUNCH_CHECK();
-    for (int sblk = FNB; sblk < G; sblk <<= 1) {
-      const int pairs = G / (2 * sblk);
+    for (int sblk = FNB; sblk < width; sblk <<= 1) {
+      const int full = width / (2 * sblk);                  // pairs with both halves complete
+      const int rest = width - full * 2 * sblk - sblk;      // rows of a shorter second half, if positive
       // one batched launch covers all pairs of one matrix's block, or (a single pair) all matrices
-      const int outer = (pairs == 1) ? 1 : n_batch;
-      for (int mb = 0; mb < outer; ++mb) {
+      const int outer = (full <= 1) ? 1 : n_batch;
+      for (int mb = 0; full > 0 && mb < outer; ++mb) {
         const long long off = (long long)mb * pp + boff;
-        const long long pair_stride = (pairs == 1) ? pp : (long long)2 * sblk * (dp + 1);
-        const int batch = (pairs == 1) ? n_batch : pairs;
+        const long long pair_stride = (full == 1) ? pp : (long long)2 * sblk * (dp + 1);
+        const int batch = (full == 1) ? n_batch : full;
         double* tmp = f.tmp + (size_t)mb * f.tmp_per + low_region;
-        const long long tmp_stride = (pairs == 1) ? (long long)f.tmp_per : (long long)sblk * sblk;
-        TB_TRY(pair_first(sblk, off, pair_stride, batch, tmp, tmp_stride, low_st));
-        TB_TRY(pair_second(sblk, off, pair_stride, batch, tmp, tmp_stride, low_st));
+        const long long tmp_stride = (full == 1) ? (long long)f.tmp_per : (long long)sblk * sblk;
+        TB_TRY(pair_first(sblk, sblk, off, pair_stride, batch, tmp, tmp_stride, low_st));
+        TB_TRY(pair_second(sblk, sblk, off, pair_stride, batch, tmp, tmp_stride, low_st));
+      }
+      if (rest > 0) {
+        const long long off = boff + (long long)full * 2 * sblk * (dp + 1);
+        double* tmp = f.tmp + low_region;
+        TB_TRY(pair_first(sblk, rest, off, pp, n_batch, tmp, (long long)f.tmp_per, low_st));
+        TB_TRY(pair_second(sblk, rest, off, pp, n_batch, tmp, (long long)f.tmp_per, low_st));
       }
     }
     if (side) {
       TB_CUDA_CHECK(cudaEventRecord(side->low_done[j & 1], low_st));
       TB_CUDA_CHECK(cudaStreamWaitEvent(side->inv, side->low_done[j & 1], 0));
     }
+    const bool last = j == n_inv_blocks - 1;
     int level = 0;
     for (int sblk = G; sblk < dp; sblk <<= 1, ++level) {
       const int mblk = sblk / G;  // blocks per half of a pair at this level
-      if ((j + 1) % mblk) break;
-      const int halves = (j + 1) / mblk;
-      if (halves & 1) {  // block j completes the first half of its pair
+      if (!last && (j + 1) % mblk) break;
+      const int half = j / mblk;  // which half of that size this block completes (the last one may be short)
+      if (!(half & 1)) {
+        if (last) continue;  // a first half without a second one: its inverse is complete
         if (side) {
           TB_CUDA_CHECK(cudaEventRecord(side->half_done, side->inv));
           TB_CUDA_CHECK(cudaStreamWaitEvent(side->inv2[level & 7], side->half_done, 0));
         }
-        TB_TRY(pair_first(sblk, (long long)(j + 1 - mblk) * G * (dp + 1), pp, n_batch, high_tmp(sblk),
-                          (long long)f.tmp_per, side ? side->inv2[level & 7] : inv_st));
+        const int o = half * sblk, m2 = (dp - o - sblk < sblk) ? dp - o - sblk : sblk;
+        cudaStream_t s1 = side ? side->inv2[level & 7] : inv_st;
+        if (f.use_i8)
+          TB_TRY(pair_first_i8(sblk, m2, o, high_tmp(sblk), s1));
+        else
+          TB_TRY(pair_first(sblk, m2, (long long)o * (dp + 1), pp, n_batch, high_tmp(sblk), (long long)f.tmp_per, s1));
         if (side) TB_CUDA_CHECK(cudaEventRecord(side->first_done[level & 7], side->inv2[level & 7]));
         break;
       }
       if (side) TB_CUDA_CHECK(cudaStreamWaitEvent(side->inv, side->first_done[level & 7], 0));
-      TB_TRY(pair_second(sblk, (long long)(j + 1 - 2 * mblk) * G * (dp + 1), pp, n_batch, high_tmp(sblk),
-                         (long long)f.tmp_per, inv_st));
+      const int o = (half - 1) * sblk, m2 = (dp - o - sblk < sblk) ? dp - o - sblk : sblk;
+      if (f.use_i8)
+        TB_TRY(pair_second_i8(sblk, m2, o, high_tmp(sblk), inv_st));
+      else
+        TB_TRY(pair_second(sblk, m2, (long long)o * (dp + 1), pp, n_batch, high_tmp(sblk), (long long)f.tmp_per, inv_st));
     }
     return TB_OK;
   };
@@ -588,6 +722,26 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   auto rank_update = [&](int k_lo, int k_cnt, int c_lo, int c_hi, cudaStream_t stream_u) -> tb_status {
     // A[r][c] -= sum_k L[r][k_lo + k] L[c][k_lo + k] for c in [c_lo, c_hi), r >= c (tiles on or below the diagonal)
     if (c_hi <= c_lo) return TB_OK;
+    if (f.use_i8 && k_cnt > FNB) {
+      I8Gemm g = i8_gemm_params();
+      g.A = g.B = f.digits;
+      g.a_rb = g.b_rb = c_lo / I8_RB;
+      g.a_rb_batch = g.b_rb_batch = rb;
+      g.a_kb = g.b_kb = k_lo / I8_KB;
+      g.k_blocks = k_cnt / I8_KB;
+      g.a_exp = g.b_exp = 1;
+      g.C = f.A + (long long)c_lo * (dp + 1);
+      g.ldc = dp;
+      g.c_batch = pp;
+      g.M = d_fact - c_lo;
+      g.N = c_hi - c_lo;
+      g.n_batch = n_batch;
+      g.alpha = -1.0;
+      g.beta = 1.0;
+      g.zeros = 4;
+      g.tiles_per_cta = tile_life;
+      return i8_gemm(g, stream_u);
+    }
     GemmP t = gemm_params();
     t.A = f.A + (long long)c_lo * dp + k_lo;
     t.a_m = dp;
@@ -619,8 +773,12 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     auto clip = [&](int c) { return c < d_fact ? c : d_fact; };
     if (side && trail_set[pi & 1]) TB_CUDA_CHECK(cudaStreamWaitEvent(cs, side->trail[pi & 1], 0));
     k_chol_panel<<<dim3(xt, n_batch), PANEL_THREADS, PANEL_SMEM, cs>>>(f.A, f.tmp, (long long)f.tmp_per, info, dp, k0,
-                                                                       d_fact, k0 > 0 ? 1 : 0);
+                                                                       d_fact, k0 > 0 ? 1 : 0, f.bad);
     TB_LAUNCH_CHECK();
+    if (f.use_i8 && last_in_block) {  // digits of the outer block's columns, for the updates and the inverse
+      I8Src l{f.A + (long long)j0 * (dp + 1), dp, pp, d_fact - j0, j1 - j0, n_batch, false, true, 0};
+      TB_TRY(i8_slice(l, nullptr, dp, 1, f.digits, j0 / I8_RB, rb, j0 / I8_KB, cs, f.bad + j0));
+    }
     if (side) {
       // blocks whose last factored panel this was (the identity padding needs no panel)
       bool waited = false;
@@ -693,15 +851,13 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     TB_CUDA_CHECK(cudaEventRecord(side->inv_done, side->inv));
     TB_CUDA_CHECK(cudaStreamWaitEvent(st, side->inv_done, 0));
   }
-  int eo = (int)(((long long)d * d + 255) / 256);
-  if (eo > 148 * 8) eo = 148 * 8;
-  k_reverse_out<<<dim3(eo, n_batch), 256, 0, st>>>(f.Li, U, d, dp);
+  k_reverse_out<<<dim3((d + 255) / 256, (d + 7) / 8, n_batch), 256, 0, st>>>(f.A, f.exps, U, d, dp, Hinv ? 1 : 0);
   TB_LAUNCH_CHECK();
 
   if (Hinv) {
     // Hinv = U^T U with U(k, m) = Li[d-1-k][d-1-m]: negative strides from element (d-1, d-1)
     GemmP g = gemm_params();
-    const double* last = f.Li + (long long)(d - 1) * dp + (d - 1);
+    const double* last = f.A + (long long)(d - 1) * dp + (d - 1);
     g.A = last;  // A(m, k) = U[k][m]
     g.a_m = -1;
     g.a_k = -(long long)dp;
