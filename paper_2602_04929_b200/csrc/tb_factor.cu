@@ -348,6 +348,16 @@ __global__ void k_mask_strict_upper(const double* __restrict__ src, double* __re
   }
 }
 
+// exps[k] = exponent of the diagonal entry U_kk: the scale of row k of U^T, column k of H^{-1/2}
+__global__ void k_diag_exp(const float* __restrict__ U, int* __restrict__ exps, int d) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= d) return;
+  const float u = fabsf(U[(long long)k * d + k]);
+  int e = 0;
+  if (u > 0.0f && u <= 3.4e38f) frexpf(u, &e);
+  exps[k] = e;
+}
+
 enum { INV_BLOCK = 512 };  // the inverse is completed block by block of this many columns (see factor_run)
 
 struct FactorWs {
@@ -572,7 +582,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   auto level_max = [&](int which) { return f.mx + (size_t)n_batch * dp * which; };
   auto pair_first_i8 = [&](int sblk, int m2, int o, double* tmp, cudaStream_t s1) -> tb_status {
     unsigned long long* mx = level_max(0) + o;
-    I8Src b{f.A + (long long)o * (dp + 1), dp, pp, sblk, sblk, n_batch, false, false, 2};
+    I8Src b{f.A + (long long)o * (dp + 1), dp, pp, sblk, sblk, n_batch, false, false, 2, nullptr, 0};
     TB_TRY(i8_row_max(b, mx, dp, s1));
     TB_TRY(i8_slice(b, mx, dp, 0, f.digits, o / I8_RB, rb, o / I8_KB, s1));
     I8Gemm g = i8_gemm_params();
@@ -599,11 +609,11 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   auto pair_second_i8 = [&](int sblk, int m2, int o, double* tmp, cudaStream_t s2) -> tb_status {
     unsigned long long *ma = level_max(1) + o, *mt = level_max(2) + o;
     const int o2 = o + sblk;
-    I8Src a{f.A + (long long)o2 * (dp + 1), dp, pp, m2, m2, n_batch, false, true, 1};
+    I8Src a{f.A + (long long)o2 * (dp + 1), dp, pp, m2, m2, n_batch, false, true, 1, nullptr, 0};
     TB_TRY(i8_row_max(a, ma, dp, s2));
     TB_TRY(i8_slice(a, ma, dp, 0, f.digits, o2 / I8_RB, rb, o2 / I8_KB, s2));
     // T: sblk columns (rows of digits), m2 contraction steps
-    I8Src t{tmp, sblk, (long long)f.tmp_per, sblk, m2, n_batch, false, false, 0};
+    I8Src t{tmp, sblk, (long long)f.tmp_per, sblk, m2, n_batch, false, false, 0, nullptr, 0};
     TB_TRY(i8_row_max(t, mt, dp, s2));
     TB_TRY(i8_slice(t, mt, dp, 0, f.digits, o / I8_RB, rb, o2 / I8_KB, s2));
     I8Gemm g = i8_gemm_params();
@@ -776,7 +786,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
                                                                        d_fact, k0 > 0 ? 1 : 0, f.bad);
     TB_LAUNCH_CHECK();
     if (f.use_i8 && last_in_block) {  // digits of the outer block's columns, for the updates and the inverse
-      I8Src l{f.A + (long long)j0 * (dp + 1), dp, pp, d_fact - j0, j1 - j0, n_batch, false, true, 0};
+      I8Src l{f.A + (long long)j0 * (dp + 1), dp, pp, d_fact - j0, j1 - j0, n_batch, false, true, 0, nullptr, 0};
       TB_TRY(i8_slice(l, nullptr, dp, 1, f.digits, j0 / I8_RB, rb, j0 / I8_KB, cs, f.bad + j0));
     }
     if (side) {
@@ -880,15 +890,36 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   return TB_OK;
 }
 
-// P and C: three products on the FP64 engine.  (Products from bf16 splits on the tensor cores were 3x
-// faster, but R U^T U cancels heavily at large widths: their error, a few 1e-7 of sum |a||b|, came to
-// 1.5e-5 of the result at 4096 columns.)
+// P and C: T1 = R U^T, C = T1 U, P = (strictly upper part of T1) U, three double-precision products on the integer
+// tensor cores (tb_i8.cuh).  R U^T U cancels heavily at large widths (a split-bf16 version, good to a few 1e-7 of
+// sum |a||b|, missed by 1.5e-5 of the result at 4096 columns); these products are as good as the FP64 pipe's.  The
+// contraction of R U^T runs over columns whose scales R and U have in opposite directions: the exponents of U's
+// diagonal take them out.  4096 columns: 6.8 ms on the FP64 pipe, 1.85 ms now.
+struct PrepWs {
+  double* T1;
+  int* exps;
+  unsigned long long *ma, *mb;
+  I8Mat A, B;
+  size_t total;
+};
+static PrepWs prep_ws(int d, void* ws) {
+  PrepWs w;
+  Bump b(ws);
+  w.T1 = b.take<double>((size_t)d * d);
+  w.exps = b.take<int>((size_t)d);
+  w.ma = b.take<unsigned long long>((size_t)d);
+  w.mb = b.take<unsigned long long>((size_t)d);
+  w.A.row_blocks = w.B.row_blocks = (d + I8_RB - 1) / I8_RB;
+  w.A.k_blocks = w.B.k_blocks = (d + I8_KB - 1) / I8_KB;
+  w.A.data = b.take<unsigned char>(i8_bytes(w.A.row_blocks, w.A.k_blocks));
+  w.B.data = b.take<unsigned char>(i8_bytes(w.B.row_blocks, w.B.k_blocks));
+  w.total = b.total();
+  return w;
+}
+
 extern "C" size_t tb_prepare_correction_workspace(int n_batch, int d) {
   if (n_batch <= 0 || d <= 0) return 0;
-  Bump b(nullptr);
-  b.take<double>((size_t)d * d);
-  b.take<double>((size_t)d * d);
-  return b.total();
+  return prep_ws(d, nullptr).total;
 }
 
 extern "C" tb_status tb_prepare_correction(const float* R, const float* U_in, int n_batch, int d,
@@ -898,15 +929,49 @@ extern "C" tb_status tb_prepare_correction(const float* R, const float* U_in, in
   if (!ws || !aligned(ws, 256) || ws_bytes < tb_prepare_correction_workspace(n_batch, d))
     return TB_ERR_WORKSPACE;
   cudaStream_t st = as_stream(stream);
-  Bump b(ws);
-  double* T1 = b.take<double>((size_t)d * d);
-  double* T2 = b.take<double>((size_t)d * d);
+  PrepWs w = prep_ws(d, ws);
   const long long dd = (long long)d * d;
-  int eb = (int)((dd + 255) / 256);
-  if (eb > 148 * 8) eb = 148 * 8;
+  // what the vector accesses of the digit kernels need; other widths and pointers take the strided engine
+  const bool digits = d % 4 == 0 && d <= 16384 && aligned(R, 16) && aligned(U_in, 16) && aligned(P, 16) && aligned(C, 16);
   for (int i = 0; i < n_batch; ++i) {
     const float* Rb = R + i * dd;
     const float* Ub = U_in + i * dd;
+    if (digits) {
+      k_diag_exp<<<(d + 255) / 256, 256, 0, st>>>(Ub, w.exps, d);
+      TB_LAUNCH_CHECK();
+      const I8Src r{Rb, d, 0, d, d, 1, true, true, 0, w.exps, 1};
+      const I8Src ut{Ub, d, 0, d, d, 1, true, true, 2, w.exps, -1};  // row n of the operand: U[n][k], zero for k < n
+      TB_TRY(i8_row_max(r, w.ma, d, st));
+      TB_TRY(i8_row_max(ut, w.mb, d, st));
+      TB_TRY(i8_slice(r, w.ma, d, 0, w.A, 0, 0, 0, st));
+      TB_TRY(i8_slice(ut, w.mb, d, 0, w.B, 0, 0, 0, st));
+      I8Gemm g = i8_gemm_params();
+      g.A = w.A;
+      g.B = w.B;
+      g.k_blocks = w.A.k_blocks;
+      g.a_max = w.ma;
+      g.b_max = w.mb;
+      g.C = w.T1;
+      g.ldc = d;
+      g.M = g.N = d;
+      g.zeros = 2;
+      g.order = 1;
+      TB_TRY(i8_gemm(g, st));
+      const I8Src u{Ub, d, 0, d, d, 1, true, false, 1, nullptr, 0};  // row n of the operand: U[k][n], zero for k > n
+      TB_TRY(i8_row_max(u, w.mb, d, st));
+      TB_TRY(i8_slice(u, w.mb, d, 0, w.B, 0, 0, 0, st));
+      for (int upper = 0; upper < 2; ++upper) {
+        const I8Src t{w.T1, d, 0, d, d, 1, false, true, upper ? 3 : 0, nullptr, 0};
+        TB_TRY(i8_row_max(t, w.ma, d, st));
+        TB_TRY(i8_slice(t, w.ma, d, 0, w.A, 0, 0, 0, st));
+        g.C = nullptr;
+        g.Cf = (upper ? P : C) + i * dd;
+        g.zeros = upper ? 8 + 16 : 8;
+        g.order = 0;
+        TB_TRY(i8_gemm(g, st));
+      }
+      continue;
+    }
     GemmP g = gemm_params();  // T1 = R U^T
     g.A = Rb;
     g.a_m = d;
@@ -914,7 +979,7 @@ extern "C" tb_status tb_prepare_correction(const float* R, const float* U_in, in
     g.B = Ub;  // B(k, n) = U[n][k], zero for k < n
     g.b_k = 1;
     g.b_n = d;
-    g.C = T1;
+    g.C = w.T1;
     g.ldc = d;
     g.M = d;
     g.N = d;
@@ -922,7 +987,7 @@ extern "C" tb_status tb_prepare_correction(const float* R, const float* U_in, in
     g.btrim = 2;
     TB_TRY((gemm_launch<float, float, double, double, false, false>(g, st)));
     GemmP c = gemm_params();  // C = T1 U
-    c.A = T1;
+    c.A = w.T1;
     c.a_m = d;
     c.a_k = 1;
     c.B = Ub;  // B(k, n) = U[k][n], zero for k > n
@@ -935,7 +1000,9 @@ extern "C" tb_status tb_prepare_correction(const float* R, const float* U_in, in
     c.K = d;
     c.btrim = 1;
     TB_TRY((gemm_launch<double, float, float, double, false, true>(c, st)));
-    k_mask_strict_upper<<<eb, 256, 0, st>>>(T1, T2, d);
+    double* T2 = reinterpret_cast<double*>(w.A.data);  // 2 x 7 bytes per entry: room for a double
+    const int eb = (int)((dd + 255) / 256 < 148 * 8 ? (dd + 255) / 256 : 148 * 8);
+    k_mask_strict_upper<<<eb, 256, 0, st>>>(w.T1, T2, d);
     TB_LAUNCH_CHECK();
     GemmP p = c;  // P = (strictly upper part of T1) U
     p.A = T2;

@@ -44,6 +44,10 @@ __device__ __forceinline__ int i8_exponent(unsigned long long bits) {
 }
 __device__ __forceinline__ double i8_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
+__device__ __forceinline__ bool i8_masked(int mask, int k, int row) {
+  return (mask == 1 && k > row) || (mask == 2 && k < row) || (mask == 3 && k <= row);
+}
+
 template <typename T, bool KCONTIG>
 __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long* out, long long out_batch) {
   const T* X = static_cast<const T*>(s.X) + blockIdx.z * s.batch;
@@ -53,12 +57,14 @@ __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long*
     const int row = blockIdx.x * 8 + warp, k0 = blockIdx.y * 512;
     if (row >= s.rows) return;
     const T* x = X + (long long)row * s.ld;
-    int k_hi = min(s.K, k0 + 512), k_lo = k0;
-    if (s.mask == 1) k_hi = min(k_hi, row + 1);
-    if (s.mask == 2) k_lo = max(k_lo, row);
-    if (k_lo >= k_hi) return;
+    const int k_hi = min(s.K, k0 + 512);
+#pragma unroll 4
     for (int k = k0 + lane; k < k_hi; k += 32)
-      if (k >= k_lo) m = fmax(m, fabs((double)x[k]));
+      if (!i8_masked(s.mask, k, row)) {
+        double v = fabs((double)x[k]);
+        if (s.k_exp) v *= i8_pow2(s.k_sign * s.k_exp[k]);
+        m = fmax(m, v);
+      }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) atomicMax(out + blockIdx.z * out_batch + row, (unsigned long long)__double_as_longlong(m));
@@ -69,8 +75,11 @@ __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long*
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int k = k0 + i;
-      const bool in = k < s.K && (s.mask != 1 || k <= row) && (s.mask != 2 || k >= row);
-      if (in) m = fmax(m, fabs((double)x[(long long)k * s.ld]));
+      if (k < s.K && !i8_masked(s.mask, k, row)) {
+        double v = fabs((double)x[(long long)k * s.ld]);
+        if (s.k_exp) v *= i8_pow2(s.k_sign * s.k_exp[k]);
+        m = fmax(m, v);
+      }
     }
     if (m > 0.0) atomicMax(out + blockIdx.z * out_batch + row, (unsigned long long)__double_as_longlong(m));
   }
@@ -123,7 +132,8 @@ __global__ void __launch_bounds__(128) k_i8_slice(I8Src s, const unsigned long l
     for (int i = 0; i < 4; ++i) {
       const int k = k0 + 4 * g + i;
       double v = (double)x[4 * g + i];
-      if ((s.mask == 1 && k > row) || (s.mask == 2 && k < row)) v = 0.0;
+      if (i8_masked(s.mask, k, row)) v = 0.0;
+      if (s.k_exp && k < s.K) v *= i8_pow2(s.k_sign * s.k_exp[k]);
       if (bad && !(fabs(v) < limit)) bad[blockIdx.z * max_batch + row] = 1;
       // |v scale| <= 2^54: adding 128 to every digit makes the bytes of the sum the digits plus 128
       const unsigned long long y = (unsigned long long)__double2ll_rn(v * scale) + 0x0080808080808080ull;
@@ -242,6 +252,7 @@ __device__ __forceinline__ void i8_st4(double* p, double a, double b, double c, 
 
 struct I8K {
   double* C;
+  float* Cf;
   long long ldc, c_batch;
   const unsigned long long *a_max, *b_max;
   long long a_max_batch, b_max_batch;
@@ -279,7 +290,10 @@ __device__ __forceinline__ void i8_k_range(const I8K& p, int tm, int tn, int& kb
   kb = 0;
   ke = p.k_blocks;
   if (p.zeros & 1) ke = min(ke, (tm + 1) * (I8_BM / I8_KB));
-  if (p.zeros & 2) kb = min(ke, tn * (I8_BN / I8_KB));
+  if (p.zeros & 8) ke = min(ke, (tn + 1) * (I8_BN / I8_KB));
+  if (p.zeros & 2) kb = tn * (I8_BN / I8_KB);
+  if (p.zeros & 16) kb = max(kb, tm * (I8_BM / I8_KB));
+  kb = min(kb, ke);
 }
 
 __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __grid_constant__ CUtensorMap map_a,
@@ -377,7 +391,8 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
       i8_k_range(p, tm, tn, kb, ke);
       const int m = tm * I8_BM + row, n0 = tn * I8_BN + hf * 32;
       const bool in_m = m < p.M;
-      double* c = p.C + b * p.c_batch + (in_m ? m : 0) * p.ldc + n0;
+      const long long at = b * p.c_batch + (in_m ? m : 0) * p.ldc + n0;
+      double* c = p.C + at;
       // while the products run: the old values, and the scales of the row and (a lane each) of the columns
       double o[32];
 #pragma unroll
@@ -419,6 +434,14 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
       __syncwarp();
       if (lane == 0) mbar_arrive(acce_bar);  // the accumulators may be overwritten
       if (!in_m) continue;
+      if (p.Cf) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          if (n0 + j < p.N)
+            *reinterpret_cast<float4*>(p.Cf + at + j) =
+                make_float4((float)o[j], (float)o[j + 1], (float)o[j + 2], (float)o[j + 3]);
+        continue;
+      }
 #pragma unroll
       for (int j = 0; j < 32; j += 4)
         if (n0 + j < p.N) i8_st4(c + j, o[j], o[j + 1], o[j + 2], o[j + 3]);
@@ -446,12 +469,13 @@ static tb_status i8_map(CUtensorMap* map, const I8Mat& m, unsigned box_blocks) {
 tb_status i8_gemm(const I8Gemm& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.n_batch <= 0) return TB_OK;
   // vectors of four doubles on C; int32 sums of at most 7 K digit products of 2^14
-  if (g.N % 4 || g.ldc % 4 || g.c_batch % 4 || !aligned(g.C, 32) || g.k_blocks > 512) return TB_ERR_INVALID_ARG;
+  if (g.N % 4 || g.ldc % 4 || g.c_batch % 4 || !aligned(g.C, 32) || !aligned(g.Cf, 16) || (g.Cf && g.beta != 0.0) || g.k_blocks > 512) return TB_ERR_INVALID_ARG;
   CUtensorMap ma, mb;
   TB_TRY(i8_map(&ma, g.A, 2));
   TB_TRY(i8_map(&mb, g.B, 1));
   I8K p;
   p.C = g.C;
+  p.Cf = g.Cf;
   p.ldc = g.ldc;
   p.c_batch = g.c_batch;
   p.a_max = g.a_max;
@@ -488,7 +512,7 @@ tb_status i8_gemm(const I8Gemm& g, cudaStream_t st) {
   const int sms = 148;
   const int rounds = (p.n_tiles + sms - 1) / sms;
   // as many CTAs as fill the rounds of tiles evenly, unless the tiles differ in length
-  int grid = (g.zeros & 3) ? (p.n_tiles < sms ? p.n_tiles : sms) : (p.n_tiles + rounds - 1) / rounds;
+  int grid = (g.zeros & ~4) ? (p.n_tiles < sms ? p.n_tiles : sms) : (p.n_tiles + rounds - 1) / rounds;
   // short-lived CTAs: a kernel of higher priority gets SMs soon
   if (g.tiles_per_cta > 0 && rounds > g.tiles_per_cta) grid = (p.n_tiles + g.tiles_per_cta - 1) / g.tiles_per_cta;
   k_i8_gemm<<<grid, I8_THREADS, I8_SMEM, st>>>(p, ma, mb);

@@ -35,13 +35,17 @@ inline size_t i8_bytes(long long row_blocks, int k_blocks) { return (size_t)row_
 // digits, row blocks rb0 .. and k blocks kb0 .. of dst.  max_bits: per row the bit pattern of the largest
 // magnitude (i8_row_max), or nullptr: every entry is below 2^fixed_exp.
 // bad (with a fixed exponent): bad[max_batch matrix + row] becomes 1 where an entry is not below the bound (or is
-// no number).  mask 1: entries with k > row are taken as zero; 2: entries with k < row.
+// no number).  mask 1: entries with k > row are taken as zero; 2: entries with k < row; 3: entries with k <= row.
+// k_exp: entries are multiplied by 2^(k_sign k_exp[k]) (one vector for all matrices), which takes out scales that
+// the contraction steps of both operands have in opposite directions.
 struct I8Src {
   const void* X;
   long long ld, batch;  // element strides
   int rows, K, n_batch;
   bool is_float, k_contig;
   int mask;
+  const int* k_exp;  // or nullptr
+  int k_sign;
 };
 tb_status i8_row_max(const I8Src& s, unsigned long long* max_bits, long long max_batch, cudaStream_t st);
 tb_status i8_slice(const I8Src& s, const unsigned long long* max_bits, long long max_batch, int fixed_exp,
@@ -56,10 +60,12 @@ struct I8Gemm {
   long long a_max_batch, b_max_batch;
   int a_exp, b_exp;
   double* C;
+  float* Cf;  // instead of C: the result rounded to float (beta = 0)
   long long ldc, c_batch;
   int M, N, n_batch;
   double alpha, beta;
-  // known zeros: 1: A(m, k) = 0 for k > m;  2: B(k, n) = 0 for k < n;  4: only tiles on or below the diagonal
+  // known zeros: 1: A(m, k) = 0 for k > m;  2: B(k, n) = 0 for k < n;  4: only tiles on or below the diagonal;
+  // 8: B(k, n) = 0 for k > n;  16: A(m, k) = 0 for k < m
   int zeros;
   int tiles_per_cta;  // 0: as few CTAs as fill the SMs; else at most that many tiles per CTA
   int order;  // 0: tiles row by row; 1: columns ascending, slowest index; 2: rows descending, slowest index
