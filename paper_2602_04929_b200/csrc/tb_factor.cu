@@ -13,13 +13,12 @@
 // multiple of 64 (identity in the padding).
 //   1. A = J D^-1 H D^-1 J                              (k_scale_exp, k_reverse_in)
 //   2. right-looking blocked Cholesky, 64-column panels, two launches per panel:
-//        k_chol_panel  every CTA factors the 64 x 64 diagonal block (one thread
-//                      per row, the row in registers, right-looking) and then
-//                      solves its 64 rows of the panel against it
+//        k_chol_panel  every CTA factors the 64 x 64 diagonal block and inverts its factor,
+//                      then multiplies its rows of the panel by the inverse
 //                      (after applying the previous panel's update to its own columns)
 //        GEMM          trailing matrix -= panel panel^T from the panel after the next on
 //                      (tiles on/below the diagonal)
-//   3. inverses of the 64 x 64 diagonal blocks (k_inv_diag64)
+//   3. the inverses of the 64 x 64 diagonal blocks, a by-product of the panels, to their places (k_inv_diag64)
 //   4. L^{-1} by recursive doubling: for block size s = 64, 128, ... every pair of
 //      neighbouring inverted blocks A, B with coupling C = L[B rows, A cols] gets
 //      its off-diagonal block -B^{-1} C A^{-1} from two batched GEMMs.  Steps 3 and 4
@@ -102,240 +101,291 @@ __global__ void __launch_bounds__(256) k_reverse_out(double* __restrict__ Li, co
 }
 
 // One panel step of the Cholesky factorisation, columns k0 .. k0+63 of the dp x dp matrix.
-// Every CTA factors the diagonal block itself (same arithmetic everywhere, so the same
-// result); CTA x then solves rows k0+64+64x .. +63 of the panel, X L_kk^T = A_panel.
-// L_kk itself is stored in Ldiag[k0 / 64] (64 x 64, row-major), not in A.
-// A non-positive pivot is recorded in info (first one wins) and replaced by 1.
+// Every CTA factors the diagonal block itself (same arithmetic everywhere, so the same result) and inverts its factor;
+// CTA x then forms rows k0+64+64y, y = x, x + gridDim.x, .. of the panel, X = A_panel L_kk^{-T}.  L_kk^{-1} is stored in
+// Linv[k0 / 64] (64 x 64, row-major, zero upper triangle); nothing reads L_kk itself.  A non-positive pivot is recorded
+// in info (first one wins) and replaced by 1.
 //
-// 256 threads; thread (r, q) keeps columns 16q .. 16q+15 of row r in registers, a warp
-// shares q.  The loops over 16-column blocks are rolled (straight-line code executed once
-// is bound by instruction fetch), the 16 steps inside a block are unrolled.
-//
-// Factorisation, right-looking.  Step j: the owners publish their (final) entries of
-// column j, one barrier, then every thread forms the reciprocal pivot itself and applies
-// a[c] -= a[j] / piv * col_j[c] to its part of the row.  The published raw columns stay in
-// shared memory: the panel solve runs the same elimination on its rows (x_j = a_j / L_jj,
-// then a_c -= x_j / L_jj * col_j[c]), so neither L nor an inverse is stored in between.
-// Entries right of the diagonal go through the same updates and are never used.
+// The chain of 64 dependent pivots bounds a panel.  It runs in one warp, 16 columns at a time: lane (row, half) holds
+// 8 entries of its row of [remaining block | inverse so far] (what is eliminated on the left becomes the inverse of
+// the unit factor in the same registers), a step is a broadcast of the pivot row, a reciprocal (the hardware's
+// approximation and one third-order step) and one multiply-add per entry, about 100 clocks of dependent work.  Nothing
+// else runs on that warp's scheduler meanwhile (beside FP64 tensor steps a dependent multiply-add waits 137 clocks
+// instead of 9); the warps of the other three apply the previous panel's update to the panel rows.  Everything
+// between the blocks of 16 - solving the rows below, updating them - is FP64 tensor steps from shared memory, and so
+// is the joining of the 16 x 16 inverses, most of it beside the chain too.  A panel of 2048 columns: 31.6 us with 64
+// barrier-separated steps of all threads, 16.4 us now.
 //
 // update_first: the previous panel's rank-64 update of these 64 columns has not been applied yet (the
 // trailing update after a panel leaves out the next panel's columns); the kernel applies it to the
-// diagonal block and to its own rows before it starts, from the previous panel's rows staged
-// k-major.  That keeps a GEMM launch per panel off the chain of dependent launches.
-enum { PLD = 66, PQ = 16, PANEL_THREADS = 256 };  // PLD: row pitch of the staged 64 x 64 tiles (doubles)
-static constexpr size_t PANEL_SMEM = (4 * 64 * PLD + 64 + 2 * PQ * 64) * sizeof(double);
+// diagonal block and to its own rows.  That keeps a GEMM launch per panel off the chain of dependent launches.
+enum { PLD = 68, PANEL_THREADS = 256 };  // PLD: row pitch of the 64 x 64 tiles (doubles); fragment loads without conflicts
+static constexpr size_t PANEL_SMEM = (size_t)(5 * 64 + 32) * PLD * sizeof(double);
 
 __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem_dst)), "l"(gsrc)
                : "memory");
 }
+__device__ __forceinline__ void pmma(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+               : "+d"(c[0]), "+d"(c[1])
+               : "d"(a), "d"(b));
+}
+// 1 / p: the hardware's approximation (2^-20) and one third-order step, r (1 + e + e^2) with e = 1 - p r
+__device__ __forceinline__ double panel_rcp(double p) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+  const double e = fma(-p, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 
-__global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict__ A, double* __restrict__ Ldiag,
-                                                              long long ldiag_batch, int* __restrict__ info, int dp,
-                                                              int k0, int d_fact, int update_first,
+// 16 x 16 block at (o, o) of D (lower triangle) -> inverse of its lower Cholesky factor at (o, o) of I, by one warp
+__device__ __forceinline__ void panel_factor16(const double* D, double* I, int o, const int* sbad, int* info, int first,
+                                               bool report) {
+  const int lane = threadIdx.x & 31, row = lane & 15, half = lane >> 4;
+  double v[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int col = 8 * half + c, hi = max(row, col), lo = min(row, col);
+    v[c] = D[(o + hi) * PLD + o + lo];
+  }
+  constexpr unsigned all = 0xffffffffu;
+  const unsigned badmask = __ballot_sync(all, sbad[o + row] != 0);  // lanes 0-15: the block's rows
+  unsigned fail = 0;
+  double piv = 1.0;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int hj = j >> 3, cj = j & 7;
+    double pj = __shfl_sync(all, v[cj], hj * 16 + j);
+    const double fi = __shfl_sync(all, v[cj], hj * 16 + row);
+    double t[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) t[c] = fi * __shfl_sync(all, v[c], half * 16 + j);
+    const bool ok = (pj > 0.0) && !((badmask >> j) & 1u);
+    fail |= ok ? 0u : 1u << j;
+    pj = ok ? pj : 1.0;
+    const double r = panel_rcp(pj);
+    if (row == j) piv = pj;
+    if (row > j) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = fma(-t[c], r, v[c]);
+      if (half == hj) v[cj] = -fi * r;
+    }
+  }
+  if (fail && report && lane == 0) atomicCAS(info, 0, first + o + __ffs(fail));
+  const double rs = rsqrt(piv);
+#pragma unroll
+  for (int c = 0; c < 8; c += 2) {
+    const int col = 8 * half + c;
+    const double x = (col < row) ? v[c] * rs : (col == row) ? rs : 0.0;
+    const double y = (col + 1 < row) ? v[c + 1] * rs : (col + 1 == row) ? rs : 0.0;
+    *reinterpret_cast<double2*>(I + (o + row) * PLD + o + col) = make_double2(x, y);
+  }
+}
+
+__global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict__ A, double* __restrict__ Linv,
+                                                              long long linv_batch, int* __restrict__ info, int dp,
+                                                              int k0, int row_blocks, int update_first,
                                                               const int* __restrict__ bad) {
   extern __shared__ __align__(16) unsigned char panel_raw[];
-  double* sA = reinterpret_cast<double*>(panel_raw);  // this CTA's 64 panel rows
-  double* sC = sA + 64 * PLD;                         // the diagonal block, then its raw columns: sC[j * PLD + r]
-  double* rsv = sC + 64 * PLD;                        // 1 / L_jj
-  double* sY = rsv + 64;                              // multipliers of the panel solve, [2][16][64]
-  double* sPd = sY + 2 * PQ * 64;                     // previous panel, rows of the diagonal block: sPd[k * PLD + row]
-  double* sPr = sPd + 64 * PLD;                       // previous panel, this CTA's rows, same layout
-  const int tid = threadIdx.x, r = tid & 63, q = tid >> 6, b = blockIdx.y;
+  double* sD = reinterpret_cast<double*>(panel_raw);  // the diagonal block, its factor's off-diagonal 16 x 16 blocks
+  double* sI = sD + 64 * PLD;                         // inverse of the factor
+  double* sR = sI + 64 * PLD;                         // panel rows
+  double* sPd = sR + 64 * PLD;                        // previous panel, rows of the diagonal block
+  double* sPr = sPd + 64 * PLD;                       // previous panel, the panel rows
+  double* sT = sPr + 64 * PLD;                        // scratch of the joins, 32 rows
   __shared__ int sbad[FNB];  // rows whose entries left of this panel were not finite
-  if (tid < FNB) sbad[tid] = bad[(long long)b * dp + k0 + tid];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, b = blockIdx.y;
+  const int fr = lane >> 2, fk = lane & 3;
   double* Ab = A + (long long)b * dp * dp;
   double* diag = Ab + (long long)k0 * dp + k0;
-  const long long row0 = (long long)k0 + FNB + (long long)FNB * blockIdx.x;
-  const bool has_rows = row0 < d_fact;
-  double* pan = Ab + row0 * dp + k0;
-  {
-    const int ch = tid & 31, rr0 = tid >> 5;  // 16-byte piece ch of rows rr0, rr0 + 8, ...
+  if (tid < FNB) sbad[tid] = bad[(long long)b * dp + k0 + tid];
+  auto load_tile = [&](double* dst, const double* src) {
+    const int ch = tid & 31, r0 = tid >> 5;  // 16-byte piece ch of rows r0, r0 + 8, ...
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int rr = 8 * i + rr0;
-      cp_async_16(sC + rr * PLD + 2 * ch, diag + (long long)rr * dp + 2 * ch);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    if (has_rows) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int rr = 8 * i + rr0;
-        cp_async_16(sA + rr * PLD + 2 * ch, pan + (long long)rr * dp + 2 * ch);
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    if (update_first) {
-      const double* dprev = diag - FNB;
-      const double* pprev = pan - FNB;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int rr = 8 * i + rr0;
-        const double2 v = *reinterpret_cast<const double2*>(dprev + (long long)rr * dp + 2 * ch);
-        sPd[(2 * ch) * PLD + rr] = v.x;
-        sPd[(2 * ch + 1) * PLD + rr] = v.y;
-        if (has_rows) {
-          const double2 w = *reinterpret_cast<const double2*>(pprev + (long long)rr * dp + 2 * ch);
-          sPr[(2 * ch) * PLD + rr] = w.x;
-          sPr[(2 * ch + 1) * PLD + rr] = w.y;
-        }
-      }
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    }
+    for (int i = 0; i < 8; ++i) cp_async_16(dst + (8 * i + r0) * PLD + 2 * ch, src + (long long)(8 * i + r0) * dp + 2 * ch);
+  };
+  auto panel_row = [&](int y) { return diag + (long long)(y + 1) * FNB * dp; };
+  int y = blockIdx.x;
+  load_tile(sD, diag);
+  if (update_first) load_tile(sPd, diag - FNB);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  if (y < row_blocks) {
+    load_tile(sR, panel_row(y));
+    if (update_first) load_tile(sPr, panel_row(y) - FNB);
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int i = tid; i < 64 * 32; i += PANEL_THREADS)
+    *reinterpret_cast<double2*>(sI + (i >> 5) * PLD + (i & 31) * 2) = make_double2(0.0, 0.0);
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
   __syncthreads();
-  double a[PQ];
+  if (update_first) {  // D -= Pd Pd^T, the 36 fragments on and below the diagonal dealt to the warps in turn
+    int fm[5], fn[5];
+    double acc[5][2];
 #pragma unroll
-  for (int i = 0; i < PQ; i += 2) {
-    const double2 v = *reinterpret_cast<const double2*>(sC + r * PLD + q * PQ + i);
-    a[i] = v.x;
-    a[i + 1] = v.y;
-  }
-  if (update_first) {
-    // a[c] -= sum_k Pd[r][k] Pd[c][k], and the same for this CTA's rows against Pr[r][k]
-    double xr[PQ];
-#pragma unroll
-    for (int i = 0; i < PQ; i += 2) {
-      const double2 v = has_rows ? *reinterpret_cast<const double2*>(sA + r * PLD + q * PQ + i) : make_double2(0.0, 0.0);
-      xr[i] = v.x;
-      xr[i + 1] = v.y;
+    for (int i = 0; i < 5; ++i) {
+      int m = 0, n = warp + 8 * i;
+      while (n > m) n -= ++m;
+      fm[i] = m;
+      fn[i] = n;
+      acc[i][0] = acc[i][1] = 0.0;
     }
-#pragma unroll 2
-    for (int k = 0; k < FNB; ++k) {
-      const double pd = sPd[k * PLD + r];
-      const double pr = has_rows ? sPr[k * PLD + r] : 0.0;
+    const int nt = (warp < 4) ? 5 : 4;
+#pragma unroll 4
+    for (int q = 0; q < 16; ++q)
 #pragma unroll
-      for (int i = 0; i < PQ; i += 2) {
-        const double2 c = *reinterpret_cast<const double2*>(sPd + k * PLD + q * PQ + i);
-        a[i] = fma(-pd, c.x, a[i]);
-        a[i + 1] = fma(-pd, c.y, a[i + 1]);
-        xr[i] = fma(-pr, c.x, xr[i]);
-        xr[i + 1] = fma(-pr, c.y, xr[i + 1]);
+      for (int i = 0; i < 5; ++i)
+        if (i < nt) pmma(acc[i], sPd[(8 * fm[i] + fr) * PLD + 4 * q + fk], sPd[(8 * fn[i] + fr) * PLD + 4 * q + fk]);
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      if (i < nt) {
+        double2* d = reinterpret_cast<double2*>(sD + (8 * fm[i] + fr) * PLD + 8 * fn[i] + 2 * fk);
+        const double2 v = *d;
+        *d = make_double2(v.x - acc[i][0], v.y - acc[i][1]);
       }
-    }
-    if (has_rows) {
-#pragma unroll
-      for (int i = 0; i < PQ; i += 2)
-        *reinterpret_cast<double2*>(sA + r * PLD + q * PQ + i) = make_double2(xr[i], xr[i + 1]);
-    }
   }
-  __syncthreads();  // the block has been read: its storage now takes the columns
-#pragma unroll 1
-  for (int jb = 0; jb < FNB / PQ; ++jb) {
-#pragma unroll
-    for (int jl = 0; jl < PQ; ++jl) {
-      const int j = jb * PQ + jl;
-      if (q == jb) sC[j * PLD + r] = a[jl];
-      __syncthreads();
-      if (q < jb || (r | 31) < j) continue;  // warps wholly left of or above the pivot only keep the barriers
-      const double* col = sC + j * PLD;
-      double piv = col[j];
-      if (!(piv > 0.0) || sbad[j]) {
-        if (tid == j + 64 * jb && blockIdx.x == 0) atomicCAS(&info[b], 0, k0 + j + 1);
-        piv = 1.0;
-      }
-      const double mult = col[r] * __drcp_rn(piv);
-      if (q == jb) {
-#pragma unroll
-        for (int i = jl + 1; i < PQ; ++i) a[i] = fma(-mult, col[jb * PQ + i], a[i]);
-        const double rs = rsqrt(piv);
-        a[jl] = (r == j) ? piv * rs : a[jl] * rs;
-        if (r == j) rsv[j] = rs;
-      } else {
-#pragma unroll
-        for (int i = 0; i < PQ; ++i) a[i] = fma(-mult, col[q * PQ + i], a[i]);
-      }
-    }
-  }
-  if (blockIdx.x == 0) {
-    // The factored block goes to its own array, never over the input: the CTAs of this launch need
-    // not run at the same time, and one that starts late must still find the unfactored block.
-    double* dst = Ldiag + (long long)b * ldiag_batch + (long long)(k0 / FNB) * FNB * FNB + r * FNB + q * PQ;
-#pragma unroll
-    for (int i = 0; i < PQ; ++i) dst[i] = (q * PQ + i <= r) ? a[i] : 0.0;
-  }
-  if (!has_rows) return;
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();  // panel rows staged by every thread; rsv complete
-  double x[PQ];
-#pragma unroll
-  for (int i = 0; i < PQ; i += 2) {
-    const double2 v = *reinterpret_cast<const double2*>(sA + r * PLD + q * PQ + i);
-    x[i] = v.x;
-    x[i + 1] = v.y;
-  }
-#pragma unroll 1
-  for (int jb = 0; jb < FNB / PQ; ++jb) {
-    double* yb = sY + (jb & 1) * PQ * 64;
-    if (q == jb) {
-#pragma unroll
-      for (int jl = 0; jl < PQ; ++jl) {
-        const int j = jb * PQ + jl;
-        const double rs = rsv[j];
-        const double xj = x[jl] * rs;
-        x[jl] = xj;
-        const double y = xj * rs;
-        yb[jl * 64 + r] = y;
-#pragma unroll
-        for (int i = jl + 1; i < PQ; ++i) x[i] = fma(-y, sC[j * PLD + jb * PQ + i], x[i]);
+  __syncthreads();
+  // fragment (m, n) of R -= Pr Pd^T
+  auto update_rows = [&](int m, int n) {
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll 4
+    for (int q = 0; q < 16; ++q)
+      pmma(acc[q & 1], sPr[(8 * m + fr) * PLD + 4 * q + fk], sPd[(8 * n + fr) * PLD + 4 * q + fk]);
+    double2* d = reinterpret_cast<double2*>(sR + (8 * m + fr) * PLD + 8 * n + 2 * fk);
+    const double2 v = *d;
+    *d = make_double2(v.x - (acc[0][0] + acc[1][0]), v.y - (acc[0][1] + acc[1][1]));
+  };
+  // Joining two neighbouring inverses of s columns, [A 0; C B]^{-1} = [A^{-1} 0; -B^{-1} (C A^{-1}) B^{-1}], A at
+  // column o: the first product goes to scratch (sT, column tc), fragments dealt to nw warps
+  auto first_product = [&](int o, int s, int tc, int w, int nw) {
+    const int nfs = s / 8;
+    for (int i = w; i < nfs * nfs; i += nw) {
+      const int m = i / nfs, n = i % nfs;
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+      for (int q = 2 * n; q < s / 4; q += 2) {  // A^{-1}(k, n) = 0 for k < n
+        pmma(acc[0], sD[(o + s + 8 * m + fr) * PLD + o + 4 * q + fk], sI[(o + 4 * q + fk) * PLD + o + 8 * n + fr]);
+        pmma(acc[1], sD[(o + s + 8 * m + fr) * PLD + o + 4 * q + 4 + fk], sI[(o + 4 * q + 4 + fk) * PLD + o + 8 * n + fr]);
       }
+      *reinterpret_cast<double2*>(sT + (8 * m + fr) * PLD + tc + 8 * n + 2 * fk) =
+          make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+    }
+  };
+  auto second_product = [&](int o, int s, int tc, int w, int nw) {
+    const int nfs = s / 8;
+    for (int i = w; i < nfs * nfs; i += nw) {
+      const int m = nfs - 1 - i / nfs, n = i % nfs;
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+      for (int q = 0; q < 2 * (m + 1); q += 2) {  // B^{-1}(m, k) = 0 for k > m
+        pmma(acc[0], sI[(o + s + 8 * m + fr) * PLD + o + s + 4 * q + fk], sT[(4 * q + fk) * PLD + tc + 8 * n + fr]);
+        pmma(acc[1], sI[(o + s + 8 * m + fr) * PLD + o + s + 4 * q + 4 + fk], sT[(4 * q + 4 + fk) * PLD + tc + 8 * n + fr]);
+      }
+      *reinterpret_cast<double2*>(sI + (o + s + 8 * m + fr) * PLD + o + 8 * n + 2 * fk) =
+          make_double2(-(acc[0][0] + acc[1][0]), -(acc[0][1] + acc[1][1]));
+    }
+  };
+#pragma unroll 1
+  for (int jb = 0; jb < 4; ++jb) {
+    const int o = 16 * jb;
+    if (warp == 0) {
+      panel_factor16(sD, sI, o, sbad, info + b, k0, blockIdx.x == 0);
+    } else if (warp != 4) {  // warp 4 shares warp 0's scheduler
+      const int w = warp < 4 ? warp - 1 : warp - 2;
+      // what the inverse needs of finished blocks: the join of the first two, then the first products of the rest
+      if (jb == 2 && w == 0) {
+        first_product(0, 16, 0, 0, 1);
+        __syncwarp();
+        second_product(0, 16, 0, 0, 1);
+      }
+      if (jb == 3) {
+        first_product(0, 32, 0, w, 6);
+        if (w == 5) first_product(32, 16, 32, 0, 1);
+      }
+      if (update_first && y < row_blocks)
+        for (int i = w; i < 16; i += 6) update_rows(2 * jb + (i >> 3), i & 7);
     }
     __syncthreads();
-    if (q > jb) {
+    if (jb == 3) break;
+    const int nf = 2 * (3 - jb);
+    if (warp < nf) {  // rows below: L = D I^T, 8 rows a warp
+      const int r = o + 16 + 8 * warp;
+      double a[4], acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
-      for (int jl = 0; jl < PQ; ++jl) {
-        const double y = yb[jl * 64 + r];
-        const double* col = sC + (jb * PQ + jl) * PLD + q * PQ;
+      for (int q = 0; q < 4; ++q) a[q] = sD[(r + fr) * PLD + o + 4 * q + fk];
 #pragma unroll
-        for (int i = 0; i < PQ; ++i) x[i] = fma(-y, col[i], x[i]);
-      }
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int n = 0; n < 2; ++n) pmma(acc[n], a[q], sI[(o + 8 * n + fr) * PLD + o + 4 * q + fk]);
+      __syncwarp();
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+        *reinterpret_cast<double2*>(sD + (r + fr) * PLD + o + 8 * n + 2 * fk) = make_double2(acc[n][0], acc[n][1]);
     }
+    __syncthreads();
+    for (int i = warp; i < nf * (nf + 1) / 2; i += 8) {  // D -= L L^T, fragments on and below the diagonal
+      int m = 0, n = i;
+      while (n > m) n -= ++m;
+      const int r = o + 16 + 8 * m, c = o + 16 + 8 * n;
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        pmma(acc[q & 1], sD[(r + fr) * PLD + o + 4 * q + fk], sD[(c + fr) * PLD + o + 4 * q + fk]);
+      double2* d = reinterpret_cast<double2*>(sD + (r + fr) * PLD + c + 2 * fk);
+      const double2 v = *d;
+      *d = make_double2(v.x - (acc[0][0] + acc[1][0]), v.y - (acc[0][1] + acc[1][1]));
+    }
+    __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < PQ; i += 2)
-    *reinterpret_cast<double2*>(sA + r * PLD + q * PQ + i) = make_double2(x[i], x[i + 1]);
+  second_product(32, 16, 32, warp, 8);
   __syncthreads();
-  {
-    const int ch = tid & 31, rr0 = tid >> 5;
+  second_product(0, 32, 0, warp, 8);
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    // never over the input: the CTAs of this launch need not run at the same time, and one that starts late must
+    // still find the unfactored block
+    double* dst = Linv + (long long)b * linv_batch + (long long)(k0 / FNB) * FNB * FNB;
+    for (int i = tid; i < 64 * 32; i += PANEL_THREADS)
+      *reinterpret_cast<double2*>(dst + 2 * i) = *reinterpret_cast<const double2*>(sI + (i >> 5) * PLD + (i & 31) * 2);
+  }
+  for (; y < row_blocks; y += gridDim.x) {
+    if (y != (int)blockIdx.x) {  // further rows of this CTA
+      __syncthreads();
+      load_tile(sR, panel_row(y));
+      if (update_first) load_tile(sPr, panel_row(y) - FNB);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (update_first)
+        for (int n = 0; n < 8; ++n) update_rows(warp, n);
+      __syncwarp();  // a warp's rows are its own from here on
+    }
+    // X = R I^T, 8 rows a warp; I(n, k) = 0 for k > n
+    double a[16];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int rr = 8 * i + rr0;
-      *reinterpret_cast<double2*>(pan + (long long)rr * dp + 2 * ch) =
-          *reinterpret_cast<const double2*>(sA + rr * PLD + 2 * ch);
+    for (int q = 0; q < 16; ++q) a[q] = sR[(8 * warp + fr) * PLD + 4 * q + fk];
+    double* out = panel_row(y) + (long long)(8 * warp + fr) * dp + 2 * fk;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+      for (int q = 0; q < 2 * (n + 1); ++q) pmma(acc[q & 1], a[q], sI[(8 * n + fr) * PLD + 4 * q + fk]);
+      *reinterpret_cast<double2*>(out + 8 * n) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
     }
   }
 }
 
-// Inverse of every 64 x 64 diagonal block of L into the same block of Li (lower triangular):
-// forward substitution, one thread per column, the column in registers.
-// The part of the block's rows right of it, up to the end of its block of 512 columns, becomes zero: the doubling
-// products inside that block read it.
-__global__ void __launch_bounds__(64) k_inv_diag64(const double* __restrict__ Ldiag, long long ldiag_batch,
-                                                   double* __restrict__ Li, int dp, int blk0, int col_end) {
-  __shared__ double Ls[FNB][FNB + 1];
-  __shared__ double rdiag[FNB];
-  const int blk = blk0 + blockIdx.x, b = blockIdx.y, c = threadIdx.x;
-  const long long off = (long long)b * dp * dp + (long long)blk * FNB * (dp + 1);
-  const double* src = Ldiag + (long long)b * ldiag_batch + (long long)blk * FNB * FNB;
-  for (int r = 0; r < FNB; ++r) Ls[r][c] = src[r * FNB + c];
-  __syncthreads();
-  rdiag[c] = 1.0 / Ls[c][c];
-  __syncthreads();
-  double x[FNB];
-#pragma unroll
-  for (int r = 0; r < FNB; ++r) {
-    double s0 = (r == c) ? 1.0 : 0.0;
-#pragma unroll
-    for (int k = 0; k < r; ++k) s0 = fma(-Ls[r][k], x[k], s0);
-    x[r] = (r < c) ? 0.0 : s0 * rdiag[r];
+// The inverses of the 64 x 64 diagonal blocks of L to their places in L^{-1}.  The part of the block's rows right of
+// it, up to the end of its block of 512 columns, becomes zero: the doubling products inside that block read it.
+__global__ void __launch_bounds__(256) k_inv_diag64(const double* __restrict__ Linv, long long linv_batch,
+                                                    double* __restrict__ Li, int dp, int blk0, int col_end) {
+  const int blk = blk0 + blockIdx.x, b = blockIdx.y;
+  double* dst = Li + (long long)b * dp * dp + (long long)blk * FNB * (dp + 1);
+  const double2* src = reinterpret_cast<const double2*>(Linv + (long long)b * linv_batch + (long long)blk * FNB * FNB);
+  const int width = (col_end - blk * FNB) / 2;
+  for (int i = threadIdx.x; i < FNB * width; i += 256) {
+    const int r = i / width, c = i % width;
+    reinterpret_cast<double2*>(dst + (long long)r * dp)[c] = (c < FNB / 2) ? src[r * (FNB / 2) + c] : make_double2(0.0, 0.0);
   }
-#pragma unroll
-  for (int r = 0; r < FNB; ++r) Li[off + (long long)r * dp + c] = x[r];
-  const int right = col_end - (blk + 1) * FNB;
-  for (int r = 0; r < FNB; ++r)
-    for (int k = c; k < right; k += 64) Li[off + (long long)r * dp + FNB + k] = 0.0;
 }
 
 // strictly-upper mask of a square matrix (Algorithm 2: (R U^T) .* M_U)
@@ -387,7 +437,7 @@ static FactorWs factor_ws(int n_batch, int d, void* ws) {
   f.A = b.take<double>((size_t)n_batch * n);
   f.exps = b.take<int>((size_t)n_batch * dp);
   f.bad = b.take<int>((size_t)n_batch * dp);
-  // tmp per matrix: the factored diagonal blocks (dp x 64), then the intermediate products of the
+  // tmp per matrix: the inverses of the factored diagonal blocks (dp x 64), then the intermediate products of the
   // doubling steps.  The inverse proceeds while later panels are still being factored, and a product
   // of a high level stays alive while lower levels run, so each gets a region of its own.
   const size_t gdim = (dp < INV_BLOCK) ? dp : (size_t)INV_BLOCK;
@@ -577,7 +627,8 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   // digits of A^{-1} (by columns) take the place of those of the square of L it is the inverse of, and so do the
   // digits of B^{-1}; the digits of T (by columns) that of C's.  Every update that reads one of these parts of L
   // belongs to columns that have been factored by then.
-  const int tile_life = side ? 2 : 0;  // beside the panels: CTAs that end soon
+  // beside the panels: CTAs that end soon, unless the products of many matrices bound the time anyway
+  const int tile_life = side ? (n_batch >= 4 ? 8 : 2) : 0;
   // row / column maxima, indexed by the pair's columns: pairs whose products run side by side have no column in common
   auto level_max = [&](int which) { return f.mx + (size_t)n_batch * dp * which; };
   auto pair_first_i8 = [&](int sblk, int m2, int o, double* tmp, cudaStream_t s1) -> tb_status {
@@ -652,7 +703,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     cudaStream_t low_st = side ? side->low[j & 1] : inv_st;
     const size_t low_region = f.low_off + (size_t)(j & 1) * ((f.high_off - f.low_off) / 2);
     if (side) TB_CUDA_CHECK(cudaStreamWaitEvent(low_st, side->block_done, 0));
-    k_inv_diag64<<<dim3(width / FNB, n_batch), 64, 0, low_st>>>(f.tmp, (long long)f.tmp_per, f.A, dp, j * (G / FNB),
+    k_inv_diag64<<<dim3(width / FNB, n_batch), 256, 0, low_st>>>(f.tmp, (long long)f.tmp_per, f.A, dp, j * (G / FNB),
                                                                  o0 + width);
     TB_LAUNCH_CHECK();
     for (int sblk = FNB; sblk < width; sblk <<= 1) {
@@ -716,11 +767,11 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
   // update of panel k-1 to its own 64 columns itself; the rank-64 update after panel k covers the
   // columns from panel k+2 on up to ZL = 128 columns past the end of its outer block (a strip at most
   // 256 columns wide), so that the first two panels of the next block never wait for anything wide.
-  // After a block's last panel its 256 columns update everything further right in one rank-256
-  // product, in two launches: the columns up to ZL past the next block's end ("near": the next block's
-  // third panel is the first to need it), then the rest ("far").  A rank-64 update of the whole
-  // trailing matrix moves the matrix through memory once per panel and is bound by that traffic;
-  // rank-256 updates move it a quarter as often and run at the GEMM engine's large-K efficiency.
+  // After a block's last panel its 256 columns update the columns up to ZL past the next block's end ("near": the
+  // next block's third panel is the first to need it), and all columns finished so far update the OB columns
+  // behind those ("far"), which the next block's near update will meet.  So every column is read and written
+  // by one far update with a long contraction, not by one per block: rank-256 updates of the whole
+  // trailing matrix moved it through memory once per block and spent half their time on that.
   // With the look-ahead: panels on the high-priority stream, the rank-64 strips and the near updates
   // in order on the trailing stream, the far updates on a low-priority stream beside the next block's
   // panels.  The far update of block J and the near update of block J+1 overlap in their columns, so
@@ -773,6 +824,15 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     t.flags = GEMM_LOWER_TILES;
     return gemm64_launch<false>(t, stream_u);
   };
+  // all finished columns [0, done) into the columns [c_lo, c_lo + OB), a piece of the contraction at a time: a piece's
+  // tiles end soon enough for the panels of one matrix, of many matrices the products bound the time anyway
+  auto far_update = [&](int done, int c_lo, cudaStream_t stream_u) -> tb_status {
+    const int c_hi = (c_lo + OB < d_fact) ? c_lo + OB : d_fact;
+    const int piece = (n_batch >= 4) ? 4096 : 1024;
+    for (int k = 0; k < done; k += piece)
+      TB_TRY(rank_update(k, (done - k < piece) ? done - k : piece, c_lo, c_hi, stream_u));
+    return TB_OK;
+  };
   for (int k0 = 0; k0 < d_fact; k0 += FNB) {
     const int r0 = k0 + FNB, m = d_fact - r0;
     const int xt = (m > 0) ? m / FNB : 1;
@@ -782,8 +842,10 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     const bool last_in_block = (r0 >= j1);
     auto clip = [&](int c) { return c < d_fact ? c : d_fact; };
     if (side && trail_set[pi & 1]) TB_CUDA_CHECK(cudaStreamWaitEvent(cs, side->trail[pi & 1], 0));
-    k_chol_panel<<<dim3(xt, n_batch), PANEL_THREADS, PANEL_SMEM, cs>>>(f.A, f.tmp, (long long)f.tmp_per, info, dp, k0,
-                                                                       d_fact, k0 > 0 ? 1 : 0, f.bad);
+    // a CTA per 64 rows while the SMs hold them, else several row blocks per CTA: the diagonal block is every CTA's work
+    const int px = (xt * n_batch <= 148) ? xt : (148 / n_batch > 0 ? 148 / n_batch : 1);
+    k_chol_panel<<<dim3(px < xt ? px : xt, n_batch), PANEL_THREADS, PANEL_SMEM, cs>>>(
+        f.A, f.tmp, (long long)f.tmp_per, info, dp, k0, m / FNB, k0 > 0 ? 1 : 0, f.bad);
     TB_LAUNCH_CHECK();
     if (f.use_i8 && last_in_block) {  // digits of the outer block's columns, for the updates and the inverse
       I8Src l{f.A + (long long)j0 * (dp + 1), dp, pp, d_fact - j0, j1 - j0, n_batch, false, true, 0, nullptr, 0};
@@ -825,7 +887,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     const int n_lo = clip(j1 + ZL), n_hi = clip(j1 + OB + ZL);
     if (!side) {
       TB_TRY(rank_update(j0, j1 - j0, n_lo, n_hi, st));
-      TB_TRY(rank_update(j0, j1 - j0, n_hi, d_fact, st));
+      TB_TRY(far_update(j1, n_hi, st));
       continue;
     }
     if (n_hi > n_lo) {
@@ -838,7 +900,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     }
     if (n_hi < d_fact) {
       TB_CUDA_CHECK(cudaStreamWaitEvent(side->rest, side->panel, 0));
-      TB_TRY(rank_update(j0, j1 - j0, n_hi, d_fact, side->rest));
+      TB_TRY(far_update(j1, n_hi, side->rest));
       TB_CUDA_CHECK(cudaEventRecord(side->rest_done, side->rest));
       rest_set = true;
     }

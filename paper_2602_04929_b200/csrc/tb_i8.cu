@@ -22,7 +22,8 @@ enum {
   I8_B_BYTES = I8_BLOCK,
   I8_STAGE_BYTES = I8_A_BYTES + I8_B_BYTES,
   I8_SMEM = I8_STAGES * I8_STAGE_BYTES + 1024 + 128,
-  I8_THREADS = 320  // 8 epilogue warps, TMA warp, MMA warp
+  I8_EPI = 16,  // epilogue warps: 32 rows x 16 columns each
+  I8_THREADS = 32 * (I8_EPI + 2)  // and a TMA warp, an MMA warp
 };
 
 __device__ int g_i8_error = 0;
@@ -316,11 +317,11 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
       mbar_init(empty_bar(s), 1);
     }
     mbar_init(accf_bar, 1);
-    mbar_init(acce_bar, 8);
+    mbar_init(acce_bar, I8_EPI);
     *abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 8) {
+  if (warp == I8_EPI) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 8) {
+  if (warp == I8_EPI) {
     if (lane == 0) {
       uint32_t it = 0;
       for (int t = blockIdx.x; t < p.n_tiles && !*abort_flag; t += gridDim.x) {
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
         }
       }
     }
-  } else if (warp == 9) {
+  } else if (warp == I8_EPI + 1) {
     if (lane == 0) {
       uint32_t it = 0, tile_it = 0;
       for (int t = blockIdx.x; t < p.n_tiles && !*abort_flag; t += gridDim.x, ++tile_it) {
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
       }
     }
   } else {
-    // epilogue warps: TMEM lanes 32 (w % 4) .., columns 32 (w / 4) .. of every accumulator
+    // epilogue warps: TMEM lanes 32 (w % 4) .., columns 16 (w / 4) .. of every accumulator
     const int q = warp & 3, hf = warp >> 2;
     const int row = q * 32 + lane;
     uint32_t tile_it = 0;
@@ -389,28 +390,28 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
       int b, tm, tn, kb, ke;
       i8_tile(p, t, b, tm, tn);
       i8_k_range(p, tm, tn, kb, ke);
-      const int m = tm * I8_BM + row, n0 = tn * I8_BN + hf * 32;
+      const int m = tm * I8_BM + row, n0 = tn * I8_BN + hf * 16;
       const bool in_m = m < p.M;
       const long long at = b * p.c_batch + (in_m ? m : 0) * p.ldc + n0;
       double* c = p.C + at;
       // while the products run: the old values, and the scales of the row and (a lane each) of the columns
-      double o[32];
+      double o[16];
 #pragma unroll
-      for (int j = 0; j < 32; j += 4) {  // N is a multiple of 4
+      for (int j = 0; j < 16; j += 4) {  // N is a multiple of 4
         o[j] = o[j + 1] = o[j + 2] = o[j + 3] = 0.0;
         if (p.add && in_m && n0 + j < p.N) i8_ld4(c + j, o[j], o[j + 1], o[j + 2], o[j + 3]);
       }
       const int ea = (p.a_max && in_m) ? i8_exponent(p.a_max[b * p.a_max_batch + m]) : p.a_exp;
-      const int eb = (p.b_max && n0 + lane < p.N) ? i8_exponent(p.b_max[b * p.b_max_batch + n0 + lane]) : p.b_exp;
+      const int eb = (p.b_max && lane < 16 && n0 + lane < p.N) ? i8_exponent(p.b_max[b * p.b_max_batch + n0 + lane]) : p.b_exp;
       double sa = i8_pow2(ea - 54 + 24);
       if (p.negate) sa = -sa;
       if (!mbar_wait(accf_bar, tile_it & 1u, abort_flag, &g_i8_error)) break;
       __syncwarp();
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (ke > kb) {  // otherwise the accumulators were not written
-        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * 32);
+        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * 16);
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
+        for (int g = 0; g < 2; ++g) {
           uint32_t r[I8_DIGITS][8];
 #pragma unroll
           for (int s = 0; s < I8_DIGITS; ++s) i8_tmem_ld8(ta + I8_BN * s + 8 * g, r[s]);
@@ -436,20 +437,20 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
       if (!in_m) continue;
       if (p.Cf) {
 #pragma unroll
-        for (int j = 0; j < 32; j += 4)
+        for (int j = 0; j < 16; j += 4)
           if (n0 + j < p.N)
             *reinterpret_cast<float4*>(p.Cf + at + j) =
                 make_float4((float)o[j], (float)o[j + 1], (float)o[j + 2], (float)o[j + 3]);
         continue;
       }
 #pragma unroll
-      for (int j = 0; j < 32; j += 4)
+      for (int j = 0; j < 16; j += 4)
         if (n0 + j < p.N) i8_st4(c + j, o[j], o[j + 1], o[j + 2], o[j + 3]);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  if (warp == I8_EPI) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
 static tb_status i8_map(CUtensorMap* map, const I8Mat& m, unsigned box_blocks) {
