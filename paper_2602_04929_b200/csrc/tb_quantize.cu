@@ -3,7 +3,7 @@
 // Per step i (a group of g = out_block rows of every head, M = n_heads * g
 // rows in all, heads being independent):
 //   grid     k_grid_tri       Algorithm 1, grid     candidate search per (row, column group)
-//   sweep    k_sweep_rows     Algorithm 2 / Eq. 2   one launch, 8 rows per CTA for the whole sweep
+//   sweep    k_sweep_rows     Algorithm 2 / Eq. 2   one launch, 8 to 32 rows per CTA for the whole sweep (tb_sweep.cu)
 //   residual k_residual       E = W0 - Q_B          (Proposition 3.1)
 //            GEMM             E -= W0 C             (Proposition 3.2, only with R)
 //   update   GEMM             W~[rem] -= T_i E      (Algorithm 1, update)
@@ -22,7 +22,6 @@
 #include "tb_i8.cuh"
 #include "tb_profile.cuh"
 #include "tb_rows.cuh"
-#include "tb_tma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -289,488 +288,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_grid_tri(GridP p) {
       if (p.cand_out) p.cand_out[o] = (unsigned char)best;
     }
   }
-}
-
-// ---------------------------------------------------------------------------
-// Column sweep (Algorithm 2; Eq. 2), one launch per step.  Rows never interact
-// inside the sweep, so a CTA keeps 8 active rows for the whole sweep and no CTA
-// ever waits for another.
-//
-// Left-looking form: the values of block b on arrival are
-//   w[:, b] = W0[:, b] - Err[:, 0 : 128 b] U[0 : 128 b, b]  (- Arr[:, 0 : 128 b] P[0 : 128 b, b]),
-// where Err holds the normalised errors and Arr the arrival values of the
-// columns already quantized (the second product only with the propagated-error
-// term, WITH_P).  16 warps: warps 0-7 are the panel warps (one row each, one
-// lane per column, the 128 columns of a block strictly in order); warps 8-15
-// are the update warps (two 8-column fragments each, on the FP64 tensor pipe,
-// four accumulators per fragment in turn so that enough independent tensor
-// instructions are in flight).
-// While the panel warps walk block b, the update warps form the part of block
-// b+1's sum that needs only blocks < b: 64-row chunks of U (and P) and of the
-// histories arrive by TMA (one box each, 8 spare columns per row so that
-// fragment loads are free of bank conflicts) in a ring guarded by full / empty
-// mbarriers; when the panel is done they add the last 128 terms (block b's
-// errors and arrival values straight from shared memory) and hand block b+1
-// over.  The two warp groups meet at hardware barriers with fixed participant
-// counts; every trip count depends on the block index alone.  mbarrier waits
-// are bounded: when a bound runs out the kernel raises a device error word and
-// stops computing, but still passes every barrier, so it always terminates.
-// ---------------------------------------------------------------------------
-enum { RS_CCHUNK = 128, RS_CLDE = 132 };  // cluster form: contraction rows per chunk, row pitch of its history box
-enum { RS_THREADS = 512, RS_LDB = 136, RS_LDE = 68, RS_CHUNK = 64, RS_LDW = 132, RS_TRI = 10240 };
-struct RowSweepP {
-  const double* Wt;      // [d_out][d] current W~ (rows of the step are read, never written)
-  const float* U;        // [n_hin][d][d]
-  const float* P;        // [n_hin][d][d] (WITH_P)
-  double* ErrG;          // [M][d] normalised errors of the step's rows
-  double* ArrG;          // [M][d] arrival values of the step's rows (WITH_P)
-  unsigned char* codes;  // [d_out][d]
-  const double* sD;      // [d_out][ng]
-  const int* z;          // [d_out][ng]
-  tb_stats* stats;       // or nullptr
-  RowMap rm;
-  int M, d, seg, ng, maxq, nblk;
-  int units, rows_per_unit, ctas_per_unit;
-  int cs;                // CTAs that share a group of 8 rows (1, or a cluster of 2 or 4 when rows are few)
-};
-struct RowSweepStage {
-  float Ub[RS_CHUNK][RS_LDB];   // 64 rows of U or P: 128 columns of the target block + 8 spare
-  double Eb[8][RS_LDE];         // the same 64 columns of a history (+ 4 spare), 8 rows
-};
-// The panel only touches the upper triangle of a diagonal block: rows of sub-block sb
-// (32 rows) are stored from column 32 sb on, 128 - 32 sb wide.
-__host__ __device__ constexpr int tri_base(int sb) { return sb * 4096 - 512 * sb * (sb - 1); }
-template <bool WITH_P>
-struct RowSweepSmem {
-  static constexpr int STAGES = WITH_P ? 3 : 4;
-  float sU[RS_TRI];             // diagonal block of U, upper part
-  float sP[WITH_P ? RS_TRI : 4];
-  alignas(128) RowSweepStage ring[STAGES];  // TMA destinations
-  double wblk[8][128];          // arrival values of the current block before its own feedback
-  double Es[8][RS_LDW];         // normalised errors of the current block
-  double As[WITH_P ? 8 : 1][RS_LDW];  // arrival values of the current block
-  unsigned long long full_bar[STAGES], empty_bar[STAGES];
-  unsigned long long cfull_bar[8], cempty_bar[8];  // ring of the cluster form (more, smaller stages)
-  int abort_flag;
-};
-__device__ int g_sweep_error = 0;
-
-__device__ __forceinline__ void mma_f64(double (&c)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-               : "+d"(c[0]), "+d"(c[1])
-               : "d"(a), "d"(b));
-}
-__device__ __forceinline__ void bar_all() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
-
-
-template <bool WITH_P>
-__global__ void __launch_bounds__(RS_THREADS, 1)
-    k_sweep_rows(RowSweepP p, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_e,
-                 const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_a) {
-  extern __shared__ __align__(128) unsigned char rs_raw[];
-  using Smem = RowSweepSmem<WITH_P>;
-  constexpr int STAGES = Smem::STAGES;
-  constexpr int NOP = WITH_P ? 2 : 1;  // operand pairs per 64-row chunk: (Err, U) and (Arr, P)
-  Smem& sm = *reinterpret_cast<Smem*>(rs_raw);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // With few rows per launch a cluster of cs CTAs shares a group of 8 rows: each prepares 128 / cs
-  // columns of the next block (its share of the contraction work) and writes them into the shared
-  // memory of all; the panel runs in every CTA on the same values, so all of them hold the block's
-  // errors and write identical results.
-  cg::cluster_group cluster = cg::this_cluster();
-  const int cs = p.cs;
-  const int crank = (cs > 1) ? (int)cluster.block_rank() : 0;
-  const int grp = blockIdx.x / cs;
-  const int unit = grp / p.ctas_per_unit;
-  const int r_first = (grp % p.ctas_per_unit) * 8;  // first row of this group inside its unit
-  // arrival values of the blocks: with a cluster the buffers alternate (a fast CTA may write block b + 1
-  // while a slow one still reads block b); the second one sits in the part of ring stage 0 that the
-  // narrower boxes of a cluster leave free
-  // The cluster form cuts the ring's memory into more, smaller stages (its boxes of U are 128 / cs + 8
-  // floats wide), as many as fit beside the second arrival buffer, at most 8: with short chunks only
-  // the number of loads in flight hides their latency.
-  const int c_ldb = 128 / cs + 8;
-  const int c_stage_bytes = RS_CCHUNK * c_ldb * (int)sizeof(float) + 8 * RS_CLDE * (int)sizeof(double);
-  const int c_nst = min(8, (int)((sizeof(sm.ring) - sizeof(sm.wblk)) / c_stage_bytes));
-  unsigned char* ring_base = reinterpret_cast<unsigned char*>(&sm.ring[0]);
-  double* wbuf0 = &sm.wblk[0][0];
-  double* wbuf1 = (cs > 1) ? reinterpret_cast<double*>(ring_base + (size_t)c_nst * c_stage_bytes) : wbuf0;
-  const int d = p.d;
-  const long long uoff = (long long)unit * d * d * (p.units > 1 ? 1 : 0);
-  const float* U = p.U + uoff;
-  const float* Pm = WITH_P ? p.P + uoff : nullptr;
-  const double maxq = (double)p.maxq;
-  const int m_base = unit * p.rows_per_unit + r_first;
-  const int rows_here = min(8, p.rows_per_unit - r_first);
-
-  // block 0 arrives unchanged
-  for (int idx = tid; idx < 8 * 128; idx += RS_THREADS) {
-    const int r = idx >> 7, c = idx & 127;
-    sm.wblk[r][c] = (r < rows_here) ? p.Wt[p.rm.row(m_base + r) * d + c] : 0.0;
-  }
-  if (tid == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(smem_u32(&sm.full_bar[s]), 1);
-      mbar_init(smem_u32(&sm.empty_bar[s]), 8);  // one arrival per update warp
-    }
-    for (int s = 0; s < 8; ++s) {
-      mbar_init(smem_u32(&sm.cfull_bar[s]), 1);
-      mbar_init(smem_u32(&sm.cempty_bar[s]), (cs > 1) ? 16 / cs : 8);  // one arrival per working update warp
-    }
-    sm.abort_flag = 0;
-    mbar_fence_init();
-  }
-  bar_all();
-
-  if (warp < 8) {
-    // =========================== panel warps: row `warp` ===========================
-    const bool valid = warp < rows_here;
-    const long long grow = valid ? p.rm.row(m_base + warp) : 0;
-    const double magic = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer, ties to even
-    unsigned int n_near = 0, n_clamp = 0;
-    for (int b = 0; b < p.nblk; ++b) {
-      const int c0 = b * 128;
-      // grids of this lane's four columns (fetched while the diagonal block is staged)
-      double s4[4], z4[4];
-#pragma unroll
-      for (int sb = 0; sb < 4; ++sb) {
-        const long long so = grow * p.ng + (c0 + sb * 32 + lane) / p.seg;
-        s4[sb] = valid ? p.sD[so] : 1.0;
-        z4[sb] = valid ? (double)p.z[so] : 0.0;
-      }
-      // upper part of the diagonal block(s): row r of sub-block sb from column 32 sb on
-      for (int idx = tid; idx < 128 * 32; idx += 256) {
-        const int r = idx >> 5, c4 = (idx & 31) * 4, sb = r >> 5;
-        if (c4 >= 32 * sb) {
-          const int o = tri_base(sb) + (r - 32 * sb) * (128 - 32 * sb) + (c4 - 32 * sb);
-          *reinterpret_cast<float4*>(sm.sU + o) =
-              *reinterpret_cast<const float4*>(U + (long long)(c0 + r) * d + c0 + c4);
-          if (WITH_P)
-            *reinterpret_cast<float4*>(sm.sP + o) =
-                *reinterpret_cast<const float4*>(Pm + (long long)(c0 + r) * d + c0 + c4);
-        }
-      }
-      asm volatile("bar.sync 2, 256;" ::: "memory");
-      double w[4], rs4[4], rd4[4];
-#pragma unroll
-      for (int sb = 0; sb < 4; ++sb) {
-        w[sb] = ((b & 1) ? wbuf1 : wbuf0)[warp * 128 + sb * 32 + lane];
-        rs4[sb] = 1.0 / s4[sb];
-        rd4[sb] = 1.0 / (double)sm.sU[tri_base(sb) + lane * (128 - 32 * sb) + lane];
-      }
-#pragma unroll 1
-      for (int sb = 0; sb < 4; ++sb) {
-        const int cl = sb * 32 + lane, col = c0 + cl;
-        const int wd = 128 - 32 * sb;                 // width of this sub-block's stored rows
-        const float* ub = sm.sU + tri_base(sb) + lane;  // element (32 sb + j, 32 sb + lane + 32 t) at ub[j * wd + 32 t]
-        const float* pb = sm.sP + (WITH_P ? tri_base(sb) + lane : 0);
-        const double s_l = (sb == 0) ? s4[0] : (sb == 1) ? s4[1] : (sb == 2) ? s4[2] : s4[3];
-        const double z_l = (sb == 0) ? z4[0] : (sb == 1) ? z4[1] : (sb == 2) ? z4[2] : z4[3];
-        const double rs_l = (sb == 0) ? rs4[0] : (sb == 1) ? rs4[1] : (sb == 2) ? rs4[2] : rs4[3];
-        const double rd_l = (sb == 0) ? rd4[0] : (sb == 1) ? rd4[1] : (sb == 2) ? rd4[2] : rd4[3];
-        const double srd_l = s_l * rd_l;
-        const double szrd_l = s_l * z_l * rd_l;
-        const double zm_l = z_l + magic;
-        float u[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) u[j] = ub[j * wd];
-        double v = (sb == 0) ? w[0] : (sb == 1) ? w[1] : (sb == 2) ? w[2] : w[3];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          // e = (v - s (q - z)) / U_jj = (v / U_jj + s z / U_jj) - (s / U_jj) q, with q = clamp(rne(v / s + z)).
-          // The fused multiply-add into z + 1.5 * 2^52 performs the rounding itself and leaves the
-          // integer in the low word of the result, where the clamp is two integer instructions
-          // instead of two slow double-precision min / max.  The low word alone is the integer only
-          // for |v / s + z| < 2^31; the high word tells (it is the constant's, or one less for a
-          // negative integer, exactly when the low word's sign says the same), and beyond that
-          // range, infinities included, the code saturates like the clamp of the full value.
-          const double ard = fma(v, rd_l, szrd_l);
-          const double xm = fma(v, rs_l, zm_l);
-          const int lo = __double2loint(xm), hw = __double2hiint(xm) - 0x43380000;
-          int n = min(max(lo, 0), p.maxq);
-          n = (hw == (lo >> 31)) ? n : ((hw >= 0) ? p.maxq : 0);
-          const double q = __hiloint2double(0x43380000, n) - magic;
-          const double e = fma(-srd_l, q, ard);
-          const double ej = shfl_d(e, j);
-          if (WITH_P) {
-            const double vj = shfl_d(v, j);  // value of column j on arrival
-            if (lane > j) v = fma(-vj, (double)pb[j * wd], fma(-ej, (double)u[j], v));
-          } else {
-            if (lane > j) v = fma(-ej, (double)u[j], v);
-          }
-        }
-        const double x = fma(v, rs_l, z_l);
-        const double xr = fma(v, rs_l, zm_l) - magic;
-        const double q = fmin(fmax(xr, 0.0), maxq);
-        const double e_mine = fma(-srd_l, q, fma(v, rd_l, szrd_l));  // the value broadcast at step `lane`
-        sm.Es[warp][cl] = valid ? e_mine : 0.0;
-        if (WITH_P) sm.As[warp][cl] = valid ? v : 0.0;
-        if (valid) {
-          p.codes[grow * d + col] = (unsigned char)(int)q;
-          p.ErrG[(long long)(m_base + warp) * d + col] = e_mine;
-          if (WITH_P) p.ArrG[(long long)(m_base + warp) * d + col] = v;
-          const double fl = floor(x);
-          const double a0 = fmin(fmax(fl, 0.0), maxq), a1 = fmin(fmax(fl + 1.0, 0.0), maxq);
-          if (fabs(x - (fl + 0.5)) < 1e-6 && a0 != a1) ++n_near;
-          if (xr != q) ++n_clamp;
-        }
-        // the sub-block's errors (and arrival values) update the later sub-blocks of this block:
-        // one branch-free loop per case, so that shuffles, loads and multiply-adds of different j overlap
-        if (sb == 0) {
-#pragma unroll 8
-          for (int j = 0; j < 32; ++j) {
-            const double ej = shfl_d(e_mine, j);
-            w[1] = fma(-ej, (double)ub[j * 128 + 32], w[1]);
-            w[2] = fma(-ej, (double)ub[j * 128 + 64], w[2]);
-            w[3] = fma(-ej, (double)ub[j * 128 + 96], w[3]);
-            if (WITH_P) {
-              const double vj = shfl_d(v, j);
-              w[1] = fma(-vj, (double)pb[j * 128 + 32], w[1]);
-              w[2] = fma(-vj, (double)pb[j * 128 + 64], w[2]);
-              w[3] = fma(-vj, (double)pb[j * 128 + 96], w[3]);
-            }
-          }
-        } else if (sb == 1) {
-#pragma unroll 8
-          for (int j = 0; j < 32; ++j) {
-            const double ej = shfl_d(e_mine, j);
-            w[2] = fma(-ej, (double)ub[j * 96 + 32], w[2]);
-            w[3] = fma(-ej, (double)ub[j * 96 + 64], w[3]);
-            if (WITH_P) {
-              const double vj = shfl_d(v, j);
-              w[2] = fma(-vj, (double)pb[j * 96 + 32], w[2]);
-              w[3] = fma(-vj, (double)pb[j * 96 + 64], w[3]);
-            }
-          }
-        } else if (sb == 2) {
-#pragma unroll 8
-          for (int j = 0; j < 32; ++j) {
-            const double ej = shfl_d(e_mine, j);
-            w[3] = fma(-ej, (double)ub[j * 64 + 32], w[3]);
-            if (WITH_P) {
-              const double vj = shfl_d(v, j);
-              w[3] = fma(-vj, (double)pb[j * 64 + 32], w[3]);
-            }
-          }
-        }
-      }
-      // the histories are read back by TMA (async proxy): order these stores before it
-      asm volatile("fence.proxy.async;" ::: "memory");
-      bar_all();  // block b is quantized: its errors are in Es and in the history
-      if (cs > 1)
-        cluster.sync();  // block b+1 has been handed over by all CTAs of the cluster
-      else
-        bar_all();       // block b+1 has been handed over in wblk
-    }
-    if (p.stats && crank == 0) {
-      n_near = __reduce_add_sync(0xffffffffu, n_near);
-      n_clamp = __reduce_add_sync(0xffffffffu, n_clamp);
-      if (lane == 0) {
-        if (n_near) atomicAdd(&p.stats->near_tie_codes, (unsigned long long)n_near);
-        if (n_clamp) atomicAdd(&p.stats->clamped_codes, (unsigned long long)n_clamp);
-        if (grp == 0 && warp == 0) atomicAdd(&p.stats->column_steps, (unsigned long long)d);
-      }
-    }
-    return;
-  }
-
-  // =========================== update warps ===========================
-  const int uw = warp - 8;
-  const int fr = lane >> 2, fk = lane & 3;   // fragment row / k (and column) index of this lane
-  const bool fr_valid = fr < rows_here;
-  const long long fr_grow = fr_valid ? p.rm.row(m_base + fr) : 0;
-  // This warp owns columns n_lo .. n_lo+15 of the target block: fragment 0 the even ones,
-  // fragment 1 the odd ones, so that one 8-byte load feeds both.
-  const int n_lo = uw * 16;
-  volatile int* abort_flag = &sm.abort_flag;
-  // Loading a chunk costs its issuer a few hundred cycles, and a ring slot is only free once all eight
-  // warps have released it, so a fixed issuer would hold everybody back: the duty rotates, chunk c of a
-  // block is loaded by lane 0 of update warp c mod 8.  Every warp keeps the ring position of the
-  // producer side itself (it is a function of the chunk count alone).
-  const bool lane0 = (lane == 0);
-  const int u_row0 = unit * d * (p.units > 1 ? 1 : 0);
-  // ring positions: `c_*` of the consumers (all update warps), `p_*` of the producer thread
-  int c_slot = 0, p_slot = 0;
-  uint32_t c_phase = 0, p_phase = 0;
-  if (cs > 1) {
-    // ---- cluster form: this CTA prepares columns crank * wc .. + wc - 1 of the next block, one 8-column
-    // fragment per working warp; the boxes of U are wc + 8 floats wide ----
-    const int wc = 128 / cs, ldb = c_ldb, frags = 16 / cs;
-    const int ub_bytes = RS_CCHUNK * ldb * (int)sizeof(float);
-    const int eb_bytes = 8 * RS_CLDE * (int)sizeof(double);
-    // chunks of 128 contraction rows (a whole block): with one fragment per warp a 64-row chunk is too
-    // little work beside the fixed cost of a ring step
-    const bool working = uw < frags;
-    const int n_blk = crank * wc + uw * 8;   // first column of this warp's fragment inside the block
-    for (int b = 0; b < p.nblk; ++b) {
-      if (b + 1 >= p.nblk) {
-        bar_all();
-        cluster.sync();
-        break;
-      }
-      const int cn = (b + 1) * 128;
-      const int n_hist = b * NOP, n_all = n_hist + NOP;
-      double* wnext = ((b + 1) & 1) ? wbuf1 : wbuf0;
-      if (working) {
-        double acc[8][2];  // eight accumulators in turn: one fragment per warp has to cover the latency alone
-#pragma unroll
-        for (int i = 0; i < 16; ++i) (&acc[0][0])[i] = 0.0;
-        double w0[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) w0[e] = fr_valid ? p.Wt[fr_grow * d + cn + n_blk + 2 * fk + e] : 0.0;
-        auto produce = [&](int c) {
-          if (c < n_all) {
-            if ((c % frags) == uw) {
-              unsigned char* stg = ring_base + (size_t)p_slot * c_stage_bytes;
-              const uint32_t fb = smem_u32(&sm.cfull_bar[p_slot]);
-              if (mbar_wait(smem_u32(&sm.cempty_bar[p_slot]), p_phase ^ 1u, abort_flag, &g_sweep_error)) {
-                const bool hist = c < n_hist;
-                const bool second = WITH_P && (c & 1);
-                const int kc = c / NOP;
-                mbar_expect_tx(fb, (uint32_t)(ub_bytes + (hist ? eb_bytes : 0)));
-                tma_load_2d(smem_u32(stg), second ? &map_p : &map_u, cn + crank * wc, u_row0 + kc * RS_CCHUNK, fb);
-                if (hist) tma_load_2d(smem_u32(stg + ub_bytes), second ? &map_a : &map_e, kc * RS_CCHUNK, m_base, fb);
-              }
-            }
-            if (++p_slot == c_nst) {
-              p_slot = 0;
-              p_phase ^= 1u;
-            }
-          }
-        };
-        if (lane0)
-          for (int c = 0; c < c_nst - 1; ++c) produce(c);
-        for (int c = 0; c < n_all; ++c) {
-          if (c == n_hist) bar_all();
-          const unsigned char* stg = ring_base + (size_t)c_slot * c_stage_bytes;
-          const double* eb = reinterpret_cast<const double*>(stg + ub_bytes);  // [8][RS_CLDE]
-          const bool ok = mbar_wait(smem_u32(&sm.cfull_bar[c_slot]), c_phase, abort_flag, &g_sweep_error);
-          if (ok) {
-            const double* ap;
-            if (c < n_hist)
-              ap = eb + fr * RS_CLDE + fk;
-            else if (WITH_P && (c & 1))
-              ap = &sm.As[fr][fk];
-            else
-              ap = &sm.Es[fr][fk];
-            const float* bp = reinterpret_cast<const float*>(stg) + fk * ldb + uw * 8 + fr;
-#pragma unroll
-            for (int q = 0; q < RS_CCHUNK / 4; ++q) mma_f64(acc[q & 7], ap[4 * q], (double)bp[4 * q * ldb]);
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&sm.cempty_bar[c_slot]));
-          if (++c_slot == c_nst) {
-            c_slot = 0;
-            c_phase ^= 1u;
-          }
-          if (lane0) produce(c + c_nst - 1);
-        }
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const double v = w0[e] - (((acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e])) +
-                                    ((acc[4][e] + acc[5][e]) + (acc[6][e] + acc[7][e])));
-          for (int r = 0; r < cs; ++r) cluster.map_shared_rank(wnext, r)[fr * 128 + n_blk + 2 * fk + e] = v;
-        }
-      } else {
-        bar_all();  // the barrier the working warps pass once the panel has finished block b
-      }
-      cluster.sync();  // block b+1 handed over
-    }
-    return;
-  }
-  for (int b = 0; b < p.nblk; ++b) {
-    if (b + 1 >= p.nblk) {  // nothing left to prepare
-      bar_all();
-      bar_all();
-      break;
-    }
-    const int cn = (b + 1) * 128;            // first column of the target block
-    const int n_hist = 2 * b * NOP;          // steps whose left operand comes from a history (blocks < b)
-    const int n_all = n_hist + 2 * NOP;      // plus the two chunks of block b itself
-    // four accumulators per fragment, used in turn: with two there are not enough independent
-    // tensor instructions in flight to cover their latency
-    double acc[2][4][2];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) (&acc[0][0][0])[i] = 0.0;
-    // the block's own weights, needed at the end: tile-column ci = 2 fk + e is column n_lo + 2 ci + t
-    double w0[2][2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        w0[t][e] = fr_valid ? p.Wt[fr_grow * d + cn + n_lo + 2 * (2 * fk + e) + t] : 0.0;
-
-    // step c: 64-row chunk c / NOP of the contraction, operand pair c % NOP
-    auto produce = [&](int c) {   // every lane 0 keeps count; the warp whose turn it is loads
-      if (c < n_all) {
-        if ((c & 7) == uw) {
-        RowSweepStage& st = sm.ring[p_slot];
-        const uint32_t fb = smem_u32(&sm.full_bar[p_slot]);
-        if (mbar_wait(smem_u32(&sm.empty_bar[p_slot]), p_phase ^ 1u, abort_flag, &g_sweep_error)) {
-          const bool hist = c < n_hist;
-          const bool second = WITH_P && (c & 1);
-          const int kc = c / NOP;
-          mbar_expect_tx(fb, (uint32_t)(sizeof(st.Ub) + (hist ? sizeof(st.Eb) : 0)));
-          tma_load_2d(smem_u32(&st.Ub[0][0]), second ? &map_p : &map_u, cn, u_row0 + kc * RS_CHUNK, fb);
-          if (hist) tma_load_2d(smem_u32(&st.Eb[0][0]), second ? &map_a : &map_e, kc * RS_CHUNK, m_base, fb);
-        }
-        }
-        if (++p_slot == STAGES) {
-          p_slot = 0;
-          p_phase ^= 1u;
-        }
-      }
-    };
-    if (lane0)
-      for (int c = 0; c < STAGES - 1; ++c) produce(c);
-    for (int c = 0; c < n_all; ++c) {
-      if (c == n_hist) bar_all();  // the panel warps have finished block b: Es (and As) are complete
-      const RowSweepStage& st = sm.ring[c_slot];
-      const bool ok = mbar_wait(smem_u32(&sm.full_bar[c_slot]), c_phase, abort_flag, &g_sweep_error);
-      if (ok) {
-        const int own = (c - n_hist) / NOP;  // which of block b's two chunks (when c >= n_hist)
-        const double* ap;
-        if (c < n_hist)
-          ap = &st.Eb[fr][fk];
-        else if (WITH_P && (c & 1))
-          ap = &sm.As[fr][own * RS_CHUNK + fk];
-        else
-          ap = &sm.Es[fr][own * RS_CHUNK + fk];
-        const float* bp = &st.Ub[fk][n_lo + 2 * fr];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const double a = ap[4 * q];
-          const float2 bb = *reinterpret_cast<const float2*>(bp + 4 * q * RS_LDB);
-          mma_f64(acc[0][q & 3], a, (double)bb.x);
-          mma_f64(acc[1][q & 3], a, (double)bb.y);
-        }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&sm.empty_bar[c_slot]));  // this warp is done with the stage
-      if (++c_slot == STAGES) {
-        c_slot = 0;
-        c_phase ^= 1u;
-      }
-      if (lane0) produce(c + STAGES - 1);
-    }
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        sm.wblk[fr][n_lo + 2 * (2 * fk + e) + t] =
-            w0[t][e] - ((acc[t][0][e] + acc[t][1][e]) + (acc[t][2][e] + acc[t][3][e]));
-    bar_all();  // block b+1 handed over
-  }
-}
-
-int sweep_error_read_clear() {
-  int v = 0;
-  if (cudaMemcpyFromSymbol(&v, g_sweep_error, sizeof(int)) != cudaSuccess) return -1;
-  if (v) {
-    int z = 0;
-    cudaMemcpyToSymbol(g_sweep_error, &z, sizeof(int));
-  }
-  return v;
 }
 
 // ---------------------------------------------------------------------------
@@ -1474,6 +991,7 @@ struct Plan {
   long long cd_rows;  // rows per coordinate-descent batch
   // workspace
   double *Wt, *Wk, *W0c, *E, *sD, *T, *Dq, *Dm, *Yw, *n0, *Amat, *G2;
+  SweepScratch sweep;
   I8Mat Cdig, Wdig;                // digits of C (all steps) and of the step's W0 (propagated error, one shared H_in)
   unsigned long long *c_max, *w_max;
   float* Wb;
@@ -1538,6 +1056,12 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
   p.Wk = b.take<double>((size_t)p.Mmax * dd);
   p.E = b.take<double>((size_t)p.Mmax * dd);
   p.W0c = with_r ? b.take<double>((size_t)p.Mmax * dd) : nullptr;
+  p.sweep = SweepScratch{};
+  if (!p.dynamic) {
+    const int units = (p.n_hin == 1) ? 1 : p.H;
+    sweep_scratch(b, p.Mmax, p.d, units, with_r, sweep_wants_i8(p.d, p.Mmax / units) && units == 1, &p.sweep);
+    p.sweep.work = p.Wk;
+  }
   p.Cdig = p.Wdig = I8Mat{nullptr, 0, 0};
   p.c_max = p.w_max = nullptr;
   if (with_r && has_hout && p.S > 1 && p.n_hin == 1 && p.d <= 16384) {
@@ -1649,76 +1173,29 @@ static tb_status run_grid(const Plan& p, const float* H_in, float* scales, int* 
   return TB_OK;
 }
 
-template <bool WITH_P>
-static tb_status launch_sweep_rows(const RowSweepP& sp, const CUtensorMap& mu, const CUtensorMap& me,
-                                   const CUtensorMap& mp, const CUtensorMap& ma, cudaStream_t st) {
-  auto kern = k_sweep_rows<WITH_P>;
-  static bool configured[64] = {false};
-  TB_TRY(allow_smem(kern, sizeof(RowSweepSmem<WITH_P>), configured));
-  const long long ctas = (long long)sp.ctas_per_unit * sp.units * sp.cs;
-  if (sp.cs == 1) {
-    kern<<<(unsigned)ctas, RS_THREADS, sizeof(RowSweepSmem<WITH_P>), st>>>(sp, mu, me, mp, ma);
-    TB_LAUNCH_CHECK();
-    return TB_OK;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)ctas);
-  cfg.blockDim = dim3(RS_THREADS);
-  cfg.dynamicSmemBytes = sizeof(RowSweepSmem<WITH_P>);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)sp.cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  TB_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, sp, mu, me, mp, ma));
-  TB_LAUNCH_CHECK();
-  return TB_OK;
-}
-
 static tb_status run_sweep_rows(const Plan& p, const float* U_in, const float* P, unsigned char* codes,
                                 const int* zeros, tb_stats* stats, RowMap rm, int M, cudaStream_t st) {
-  RowSweepP sp;
-  sp.Wt = p.Wt;
-  sp.U = U_in;
-  sp.P = P;
-  sp.ErrG = p.Wk;  // error history of the step's rows
-  sp.ArrG = p.E;   // arrival values; E itself is formed after the sweep
-  sp.codes = codes;
-  sp.sD = p.sD;
-  sp.z = zeros;
-  sp.stats = stats;
-  sp.rm = rm;
-  sp.M = M;
-  sp.d = p.d;
-  sp.seg = p.seg;
-  sp.ng = p.ng;
-  sp.maxq = p.maxq;
-  sp.nblk = p.d / 128;
-  sp.units = (p.n_hin == 1) ? 1 : p.H;
-  sp.rows_per_unit = M / sp.units;
-  sp.ctas_per_unit = (sp.rows_per_unit + 7) / 8;
-  // few rows: a cluster of 2 or 4 CTAs per group of 8 rows shares the contraction work of the updates
-  const long long groups = (long long)sp.ctas_per_unit * sp.units;
-  sp.cs = (p.d >= 256 && groups * 4 <= 148) ? 4 : (p.d >= 256 && groups * 2 <= 148) ? 2 : 1;
-  CUtensorMap map_u, map_e, map_p, map_a;
-  const unsigned box_full = (unsigned)((p.d >= RS_LDB) ? RS_LDB : p.d);
-  const unsigned box_u = (sp.cs > 1) ? (unsigned)(128 / sp.cs + 8) : box_full;
-  const unsigned box_e = (sp.cs > 1) ? (unsigned)RS_CLDE : (unsigned)((p.d >= RS_LDE) ? RS_LDE : p.d);
-  const unsigned box_k = (sp.cs > 1) ? (unsigned)RS_CCHUNK : (unsigned)RS_CHUNK;
-  const unsigned long long mat_rows = (unsigned long long)p.d * sp.units;
-  TB_TRY(make_map_2d(&map_u, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), U_in, (unsigned long long)p.d, mat_rows,
-                     box_u, box_k, CU_TENSOR_MAP_SWIZZLE_NONE));
-  TB_TRY(make_map_2d(&map_e, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, sizeof(double), sp.ErrG, (unsigned long long)p.d,
-                     (unsigned long long)M, box_e, 8, CU_TENSOR_MAP_SWIZZLE_NONE));
-  if (!P) return launch_sweep_rows<false>(sp, map_u, map_e, map_u, map_e, st);
-  TB_TRY(make_map_2d(&map_p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), P, (unsigned long long)p.d, mat_rows,
-                     box_u, box_k, CU_TENSOR_MAP_SWIZZLE_NONE));
-  TB_TRY(make_map_2d(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, sizeof(double), sp.ArrG, (unsigned long long)p.d,
-                     (unsigned long long)M, box_e, 8, CU_TENSOR_MAP_SWIZZLE_NONE));
-  return launch_sweep_rows<true>(sp, map_u, map_e, map_p, map_a, st);
+  SweepArgs a;
+  a.src = p.Wt;
+  a.src_mapped = true;
+  a.U = U_in;
+  a.P = P;
+  a.Err = p.Wk;  // error history of the step's rows (up to SWEEP_OUTER columns)
+  a.Arr = p.E;   // arrival values; E itself is formed after the sweep
+  a.err_ld = a.err_col0 = 0;
+  a.codes = codes;
+  a.sD = p.sD;
+  a.z = zeros;
+  a.stats = stats;
+  a.rm = rm;
+  a.M = M;
+  a.d = p.d;
+  a.seg = p.seg;
+  a.ng = p.ng;
+  a.maxq = p.maxq;
+  a.units = (p.n_hin == 1) ? 1 : p.H;
+  a.blk0 = a.blk1 = 0;
+  return sweep_step(a, p.sweep, st);
 }
 
 // Dynamic-grid variant: group by group on the working copy Wk of the step's rows.
@@ -1890,6 +1367,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
       TB_TRY(i8_row_max(c, p.c_max, d, st));
       TB_TRY(i8_slice(c, p.c_max, d, 0, p.Cdig, 0, 0, 0, st));
     }
+  }
+  if (!p.dynamic) {
+    PhaseScope ph(PH_SWEEP, st);
+    TB_TRY(sweep_prepare(U_in, P, d, (p.n_hin == 1) ? 1 : p.H, p.sweep, st));
   }
   if (!p.adaptive && !p.dynamic) {
     // fixed grid: every row, once, from the original weights

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "tb_common.cuh"
+#include "tb_i8.cuh"
 
 namespace tb {
 
@@ -28,6 +29,44 @@ struct GridP {
   const double* Wloc;  // or nullptr: the step's rows as a contiguous [M][d] working copy, read instead of Wt
   int grp0;            // column group of blockIdx.x = 0
 };
+
+// Column sweep (Algorithm 2; Eq. 2) of one step's rows over the blocks of 128 columns [blk0, blk1) (tb_sweep.cu).
+struct SweepArgs {
+  const double* src;     // values before the sweep, row m of the step at src + src_row(m) d
+  bool src_mapped;       // src_row(m) = rm.row(m) (the weights), else m (a working copy of the step's rows)
+  const float* U;        // [n_hin][d][d]
+  const float* P;        // [n_hin][d][d] or nullptr
+  double* Err;           // [M][err_ld] out: normalised errors, column c at c - err_col0
+  double* Arr;           // the same for arrival values (with P)
+  int err_ld, err_col0;
+  unsigned char* codes;  // [d_out][d]
+  const double* sD;      // [d_out][ng]
+  const int* z;          // [d_out][ng]
+  tb_stats* stats;       // or nullptr
+  RowMap rm;
+  int M, d, seg, ng, maxq;
+  int units;             // 1, or the number of heads when every head has its own U
+  int blk0, blk1;
+};
+tb_status sweep_columns(const SweepArgs& a, cudaStream_t st);
+
+// The sweep over all columns of a step.  Up to SWEEP_OUTER columns go through in one launch; more are taken that many at
+// a time, each followed by one update of everything further right in a working copy of the step's rows.
+enum { SWEEP_OUTER = 512, SWEEP_I8_ROWS = 192 };
+struct SweepScratch {
+  double *work;          // [M][d]
+  double *err, *arr;     // [M][SWEEP_OUTER], arr with P only
+  bool use_i8;           // the updates on the integer tensor cores (rows of a unit: SWEEP_I8_ROWS or more); then:
+  I8Mat Udig, Pdig;      // digits of U and P by columns (prepared by sweep_prepare, one set for all steps)
+  I8Mat Edig, Adig;      // digits of a block's errors and arrival values
+  unsigned long long *u_max, *p_max, *e_max, *a_max;
+  int* u_exp;            // exponents of U's diagonal
+};
+bool sweep_wants_i8(int d, int rows_per_unit);
+void sweep_scratch(Bump& b, int M, int d, int units, bool with_p, bool use_i8, SweepScratch* s);  // err .. u_exp
+tb_status sweep_prepare(const float* U, const float* P, int d, int units, const SweepScratch& s, cudaStream_t st);
+// a.src: the weights (mapped); a.Err, a.Arr, blk0, blk1 and the like are set here
+tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st);
 
 // The search for column groups wider than 128 columns (tb_grid_wide.cu).  scratch: grid_wide_doubles() doubles
 // for a chunk of rows; with less, the rows go through in several chunks.

@@ -1,0 +1,990 @@
+// Column sweep (Algorithm 2; Eq. 2): rows against the upper factor U (and P of the propagated-error term).
+//
+// Rows never interact inside the sweep; a CTA keeps R = 8, 16 or 32 of them.  Left-looking over blocks of 128 columns:
+//   w[:, b] = W0[:, b] - Err[:, < b] U[< b, b]  (- Arr[:, < b] P[< b, b]),
+// Err the normalised errors and Arr the arrival values of the columns already quantized.
+//
+// A row is a chain of dependent roundings, column after column; the chain bounds a launch of few rows, the FP64 pipe
+// one of many.  One warp walks it, ONE THREAD PER ROW, 16 columns in registers, in units of the row's scale:
+//   x = v + z;  q = clamp(round(x));  v' = v_next - x U' + q U',   U' = U[j][j+1] / U[j][j],
+// so that only add (rounds), integer clamp, add (back to double) and multiply-add lie between two columns: 33 clocks
+// measured, 55 with the other multiply-adds of a 16-column piece (a warp per row with the column's error broadcast
+// by shuffles, as it was, takes 88 and 150).  Whether a value lies outside the 31 bits that the integer clamp
+// sees is only looked at after a piece; such a piece is walked again with the test in the chain.
+// That warp has its scheduler for itself: beside FP64 tensor steps of the same scheduler a dependent multiply-add
+// takes 137 clocks instead of 9.  The other three schedulers run, at the same time,
+//   spread   (4 warps) after each piece: its errors onto the block's later columns, the next piece first; codes,
+//            histories and counters
+//   history  (8 warps) the next block's contraction over the earlier columns: chunks of U (and P) and of the histories
+//            arrive by TMA in a ring guarded by full / empty mbarriers and feed mma.sync m8n8k4 f64 (the cluster form,
+//            whose share of a chunk is small, reads them straight into registers); the block being walked
+//            comes last, piece by piece; before that the next block's grids and 16 x 16 triangles of U'
+// and a warp beside the chain issues the TMA loads.
+// The groups meet at hardware barriers with fixed counts; every trip count depends on the block index alone.  mbarrier
+// waits are bounded: when a bound runs out the kernel raises a device error word and stops computing, but still
+// passes every barrier, so it terminates.
+//
+// Cluster form (CLUSTER), for few rows: cs CTAs share a group of 8 rows.  Each contracts the history for 128 / cs
+// columns of the next block and writes them into the buffers of all (distributed shared memory, two buffers in
+// turn); after one cluster barrier the chain of the block runs in every CTA on identical values, so no result has
+// to travel back and all of them write the same outputs.
+#include <cooperative_groups.h>
+
+#include "tb_gemm.cuh"
+#include "tb_rows.cuh"
+#include "tb_tma.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace tb {
+
+enum { SW_THREADS = 512, SW_LDB = 136, SW_LDW = 132, SW_HIST = 8, SW_SPREAD = 4 };
+
+struct SweepP {
+  SweepArgs a;
+  int rows_per_unit, ctas_per_unit;
+  int cs;  // CTAs per cluster (CLUSTER)
+};
+
+template <bool WITH_P, int R>
+struct SweepSmem {
+  static constexpr int CHUNK = (R == 32 || (R == 16 && WITH_P)) ? 32 : 64;
+  static constexpr int STAGES = (R == 8) ? (WITH_P ? 2 : 4) : 3;
+  struct Stage {
+    float Ub[CHUNK][SW_LDB];       // rows of U or P: 128 columns of the target block + 8 spare
+    double Eb[R][CHUNK + 4];       // the same contraction columns of a history (+ 4 spare)
+  };
+  alignas(128) Stage ring[STAGES];  // TMA destinations (not in the cluster form)
+  alignas(16) double w[2][R][SW_LDW];   // values of a block; walked columns hold arrival value / scale
+  alignas(16) double Es[R][SW_LDW];     // normalised errors of the block
+  alignas(16) double As[WITH_P ? R : 1][SW_LDW];  // arrival values of the block
+  alignas(16) double cU[2][8][16][16];  // U[j][c] / U[j][j] of the 16-column pieces, zero for c <= j
+  alignas(16) double cP[WITH_P ? 2 : 1][WITH_P ? 8 : 1][16][16];
+  alignas(16) double part[R == 8 ? 512 : 2];  // partial sums of the contraction's split (cluster form)
+  alignas(16) double rd[2][128];        // 1 / U[j][j]
+  double gs[2][R][4][3];                // scale, its reciprocal and zero-point per row and 32 columns
+  unsigned long long full_bar[8], empty_bar[8];
+  int abort_flag;
+};
+
+__device__ int g_sweep_error = 0;
+
+__device__ __forceinline__ void sw_mma(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+               : "+d"(c[0]), "+d"(c[1])
+               : "d"(a), "d"(b));
+}
+template <int N>
+__device__ __forceinline__ void sw_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void sw_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
+enum { SW_PUB = 1, SW_READY = 3, SW_JOIN = 5, SW_PIECE = 8 };  // two, two, one, eight hardware barriers
+
+// Quantized integer, as a double, of xm = v + z + 1.5 * 2^52: that sum was rounded to nearest-even and holds the
+// integer in its low word, where the clamp is one integer instruction.  The low word alone is the integer only below
+// 2^31 in magnitude; the high word tells (it is the constant's, or one less for a negative integer, exactly when the
+// low word's sign says the same).  CHECKED: beyond that range, infinities included, the code saturates like the clamp
+// of the full value; otherwise `off` becomes nonzero there.
+template <bool CHECKED>
+__device__ __forceinline__ double sw_quant(double xm, int maxq, int& off) {
+  const int lo = __double2loint(xm), hw = __double2hiint(xm) - 0x43380000;
+  int n = __vimin_s32_relu(lo, maxq);
+  if (CHECKED)
+    n = (hw == (lo >> 31)) ? n : ((hw >= 0) ? maxq : 0);
+  else
+    off |= hw ^ (lo >> 31);
+  return __hiloint2double(0x43380000, n) - 6755399441055744.0;
+}
+
+// Shared-memory accesses that the compiler leaves in their order: by itself it moves all of a piece's factor loads to
+// its beginning and spills them (78 clocks a column instead of 57).
+__device__ __forceinline__ double2 sw_ld2(const double* p) {
+  double2 v;
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ double sw_ld1(const double* p) {
+  double v;
+  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sw_st2(double* p, double x, double y) {
+  asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(smem_u32(p)), "d"(x), "d"(y) : "memory");
+}
+
+// 16 columns of one row in registers, in units of its scale s.  v: values, on return on arrival.  The normalised errors
+// e s / U_jj go to er two at a time (kept for the end they would cost the registers that the walk needs).
+template <bool WITH_P, bool CHECKED>
+__device__ __forceinline__ int sw_walk(double (&v)[16], double* er, double s, double z, int maxq, const double* rd,
+                                       const double (*cu)[16], const double (*cp)[16]) {
+  const double zm = z + 6755399441055744.0;
+  int off = 0;
+  double x = v[0] + z, xm = v[0] + zm, e_even = 0.0;
+  double2 cur[8], nxt[8];  // factors of the column and of the next one, loaded a column ahead
+#pragma unroll
+  for (int c = 0; c < 8; ++c) cur[c] = sw_ld2(&cu[0][2 * c]);
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    auto u = [&](int c) { return (c & 1) ? cur[c >> 1].y : cur[c >> 1].x; };
+    double q, xn = 0.0, xmn = 0.0;
+    if (j < 15) {
+#pragma unroll
+      for (int c = (j + 2) >> 1; c < 8; ++c) nxt[c] = sw_ld2(&cu[j + 1][2 * c]);
+      double t = fma(-x, u(j + 1), v[j + 1]);
+      if (WITH_P) t = fma(-v[j], sw_ld1(&cp[j][j + 1]), t);
+      q = sw_quant<CHECKED>(xm, maxq, off);
+      v[j + 1] = fma(q, u(j + 1), t);
+      xn = v[j + 1] + z;
+      xmn = v[j + 1] + zm;
+    } else {
+      q = sw_quant<CHECKED>(xm, maxq, off);
+    }
+    const double e = x - q;
+#pragma unroll
+    for (int c = j + 2; c < 16; ++c) v[c] = fma(-e, u(c), v[c]);
+    if (WITH_P) {
+      if ((j & 1) && j + 2 < 16) v[j + 2] = fma(-v[j], sw_ld1(&cp[j][j + 2]), v[j + 2]);
+#pragma unroll
+      for (int c = (j + 3) & ~1; c < 16; c += 2) {
+        const double2 pc = sw_ld2(&cp[j][c]);
+        v[c] = fma(-v[j], pc.x, v[c]);
+        v[c + 1] = fma(-v[j], pc.y, v[c + 1]);
+      }
+    }
+    if (j & 1) {
+      const double2 r = sw_ld2(rd + j - 1);
+      sw_st2(er + j - 1, e_even * (s * r.x), e * (s * r.y));
+    }
+    e_even = e;
+    x = xn;
+    xm = xmn;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) cur[c] = nxt[c];
+  }
+  return off;
+}
+
+template <bool WITH_P, int R, bool CLUSTER>
+__global__ void __launch_bounds__(SW_THREADS, 1)
+    k_sweep_rows(SweepP p, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_e,
+                 const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_a) {
+  static_assert(!CLUSTER || R == 8, "a cluster shares 8 rows");
+  extern __shared__ __align__(128) unsigned char sw_raw[];
+  using Smem = SweepSmem<WITH_P, R>;
+  constexpr int NOP = WITH_P ? 2 : 1;  // operand pairs per chunk: (Err, U) and (Arr, P)
+  constexpr int MF = R / 8;
+  Smem& sm = *reinterpret_cast<Smem*>(sw_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int fr = lane >> 2, fk = lane & 3;  // fragment row (or column) and k index of this lane
+  const SweepArgs& a = p.a;
+  const int d = a.d;
+  const int cs = CLUSTER ? p.cs : 1;
+  const int crank = CLUSTER ? (int)cg::this_cluster().block_rank() : 0;
+  const int grp = blockIdx.x / cs;
+  const int unit = grp / p.ctas_per_unit, r_first = (grp % p.ctas_per_unit) * R;
+  const int rows_here = min(R, p.rows_per_unit - r_first);
+  const int m_base = unit * p.rows_per_unit + r_first;
+  const long long uoff = (a.units > 1) ? (long long)unit * d * d : 0;
+  const float* U = a.U + uoff;
+  const float* Pm = WITH_P ? a.P + uoff : nullptr;
+  auto src_row = [&](int r) { return (a.src_mapped ? a.rm.row(m_base + r) : (long long)(m_base + r)) * d; };
+
+  // ring of history chunks
+  constexpr int ch = Smem::CHUNK, ldb = SW_LDB, lde = ch + 4;  // the cluster form has none
+  constexpr int ub_bytes = ch * ldb * (int)sizeof(float), eb_bytes = R * lde * (int)sizeof(double);
+  constexpr int stage_bytes = ub_bytes + eb_bytes, stages = Smem::STAGES;
+  constexpr int per_blk = (128 / ch) * NOP;  // chunks per 128 contraction rows
+  unsigned char* ring = reinterpret_cast<unsigned char*>(&sm.ring[0]);
+  volatile int* abort_flag = &sm.abort_flag;
+
+  // What a block needs besides its values, by threads t of nt, in two parts with a barrier between: grids and 1 / U_jj,
+  // then the scaled triangles (consecutive threads on consecutive columns: a thread per row would meet 32-way bank
+  // conflicts, and the chain's own loads with them)
+  auto prepare_scales = [&](int b, int t, int nt) {
+    const int pb = b & 1, c0 = b * 128;
+    for (int j = t; j < 128; j += nt) sm.rd[pb][j] = 1.0 / (double)U[(long long)(c0 + j) * (d + 1)];
+    for (int i = t; i < R * 4; i += nt) {
+      const int r = i >> 2, sb = i & 3;
+      double s = 1.0, z = 0.0;
+      if (r < rows_here) {  // 32 columns lie in one group: groups are multiples of 32 columns
+        const long long so = a.rm.row(m_base + r) * a.ng + (c0 + 32 * sb) / a.seg;
+        s = a.sD[so];
+        z = (double)a.z[so];
+      }
+      sm.gs[pb][r][sb][0] = s;
+      sm.gs[pb][r][sb][1] = 1.0 / s;
+      sm.gs[pb][r][sb][2] = z;
+    }
+  };
+  auto prepare_triangles = [&](int b, int t, int nt) {
+    const int pb = b & 1, c0 = b * 128;
+#pragma unroll 4
+    for (int i = t; i < 128 * 16; i += nt) {
+      const int j = i >> 4, c = i & 15, jl = j & 15;
+      const long long o = (long long)(c0 + j) * d + c0 + (j & ~15) + c;
+      sm.cU[pb][j >> 4][jl][c] = (c > jl) ? (double)U[o] * sm.rd[pb][j] : 0.0;
+      if (WITH_P) sm.cP[pb][j >> 4][WITH_P ? jl : 0][c] = (c > jl) ? (double)Pm[o] : 0.0;
+    }
+  };
+
+  if (tid == 0) {
+    for (int s = 0; s < 8; ++s) {
+      mbar_init(smem_u32(&sm.full_bar[s]), 1);
+      mbar_init(smem_u32(&sm.empty_bar[s]), SW_HIST);
+    }
+    sm.abort_flag = 0;
+    mbar_fence_init();
+  }
+  for (int i = tid; i < R * 128; i += SW_THREADS) {  // the first block arrives unchanged
+    const int r = i >> 7, c = i & 127;
+    sm.w[a.blk0 & 1][r][c] = (r < rows_here) ? a.src[src_row(r) + a.blk0 * 128 + c] : 0.0;
+  }
+  prepare_scales(a.blk0, tid, SW_THREADS);
+  __syncthreads();
+  prepare_triangles(a.blk0, tid, SW_THREADS);
+  __syncthreads();
+  if (CLUSTER) cg::this_cluster().sync();  // every CTA of the cluster runs before anybody writes into it
+  auto next_block = [&]() {  // block b + 1 has been handed over (by all CTAs of the cluster)
+    if (CLUSTER)
+      cg::this_cluster().sync();
+    else
+      __syncthreads();
+  };
+
+  if (warp == 0) {
+    // =========================== the chain: lane = row ===========================
+    const int r = lane & (R - 1);  // with fewer than 32 rows several lanes do the same
+#pragma unroll 1
+    for (int b = a.blk0; b < a.blk1; ++b) {
+      const int pb = b & 1;
+      const bool more = b + 1 < a.blk1;
+#pragma unroll 1
+      for (int sb = 0; sb < 8; ++sb) {
+        const double* g = sm.gs[pb][r][sb >> 1];
+        const double s = g[0], rs = g[1], z = g[2];
+        double* wr = &sm.w[pb][r][16 * sb];
+        double* er = &sm.Es[r][16 * sb];
+        double v[16];
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+          const double2 t = *reinterpret_cast<const double2*>(wr + j);
+          v[j] = t.x * rs;
+          v[j + 1] = t.y * rs;
+        }
+        const int off = sw_walk<WITH_P, false>(v, er, s, z, a.maxq, &sm.rd[pb][16 * sb], sm.cU[pb][sb],
+                                               sm.cP[WITH_P ? pb : 0][WITH_P ? sb : 0]);
+        if (__any_sync(0xffffffffu, off != 0)) {  // again, with the range test in the chain
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            const double2 t = *reinterpret_cast<const double2*>(wr + j);
+            v[j] = t.x * rs;
+            v[j + 1] = t.y * rs;
+          }
+          sw_walk<WITH_P, true>(v, er, s, z, a.maxq, &sm.rd[pb][16 * sb], sm.cU[pb][sb],
+                                sm.cP[WITH_P ? pb : 0][WITH_P ? sb : 0]);
+        }
+        __syncwarp();  // (lanes of one row read its values before one of them overwrites them)
+        if (WITH_P) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) sw_st2(&sm.As[r][16 * sb + j], v[j] * s, v[j + 1] * s);
+        }
+        if (sb == 7) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) sw_st2(wr + j, v[j], v[j + 1]);
+        }
+        sw_arrive<32 + 32 * SW_SPREAD>(SW_PUB + (sb & 1));
+        if (more) sw_arrive<32 + 32 * SW_HIST>(SW_PIECE + sb);
+        if (sb < 7) {  // the arrival values are looked at a piece later
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) sw_st2(wr + j, v[j], v[j + 1]);
+        }
+        if (sb < 7) sw_sync<32 + 32 * SW_SPREAD>(SW_READY + (sb & 1));
+      }
+      next_block();
+    }
+    return;
+  }
+
+  if (warp == 11 || warp >= 13) {
+    // =========================== spread ===========================
+    const int sw = (warp == 11) ? 0 : warp - 12, st_tid = sw * 32 + lane;
+    unsigned int n_near = 0, n_clamp = 0;
+    // fragment (m, n) of the block belongs to warp (n + 2 (m & 1)) & 3: the next piece's fragments to all of them.
+    // This warp's columns are n = NS i + n_lo; of each it has all row fragments (8 rows), or those of one parity.
+    constexpr int NS = (MF == 1) ? 4 : 2, NI = 16 / NS, MS = (MF == 1) ? 1 : 2;
+    const int n_lo = (MF == 1) ? sw : (sw & 1);
+    // factor rows of a piece, right of it: fetched a piece ahead
+    float u[NI][4], pp[WITH_P ? NI : 1][4], uf[NI][4], pf[WITH_P ? NI : 1][4];
+    auto fetch = [&](int b, int sb) {
+      const long long o0 = (long long)(b * 128 + 16 * sb + fk) * d + b * 128 + fr;
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const int n = NS * i + n_lo;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (n >= 2 * (sb + 1)) {
+            uf[i][q] = U[o0 + (long long)(4 * q) * d + 8 * n];
+            if (WITH_P) pf[i][q] = Pm[o0 + (long long)(4 * q) * d + 8 * n];
+          }
+      }
+    };
+    // codes, histories and counters of a piece
+    auto outputs = [&](int b, int sb) {
+#pragma unroll
+      for (int i = 0; i < R * 16 / 128; ++i) {
+        const int idx = st_tid + 128 * i, r = idx >> 4, cl = 16 * sb + (idx & 15), col = b * 128 + cl;
+        if (r < rows_here) {
+          const double v = sm.w[b & 1][r][cl], z = sm.gs[b & 1][r][sb >> 1][2], maxq = (double)a.maxq;
+          const double x = v + z, xm = v + (z + 6755399441055744.0);  // the chain's own operations
+          const double xr = xm - 6755399441055744.0;
+          int unused = 0;
+          const double q = sw_quant<true>(xm, a.maxq, unused);
+          a.codes[a.rm.row(m_base + r) * d + col] = (unsigned char)(int)q;
+          const long long ho = (long long)(m_base + r) * a.err_ld + col - a.err_col0;
+          a.Err[ho] = sm.Es[r][cl];
+          if (WITH_P) a.Arr[ho] = sm.As[WITH_P ? r : 0][cl];
+          const double fl = floor(x);
+          const double a0 = fmin(fmax(fl, 0.0), maxq), a1 = fmin(fmax(fl + 1.0, 0.0), maxq);
+          if (fabs(x - (fl + 0.5)) < 1e-6 && a0 != a1) ++n_near;
+          if (xr != q) ++n_clamp;
+        }
+      }
+    };
+    fetch(a.blk0, 0);
+#pragma unroll 1
+    for (int b = a.blk0; b < a.blk1; ++b) {
+      const int pb = b & 1;
+#pragma unroll 1
+      for (int sb = 0; sb < 8; ++sb) {
+        const int n1 = 2 * (sb + 1);  // first fragment right of the piece
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            u[i][q] = uf[i][q];
+            if (WITH_P) pp[WITH_P ? i : 0][q] = pf[WITH_P ? i : 0][q];
+          }
+        if (sb < 6)
+          fetch(b, sb + 1);
+        else if (sb == 7 && b + 1 < a.blk1)
+          fetch(b + 1, 0);
+        // while the piece is being walked: the factor rows that the next piece waits for, negated and as double, and the
+        // next piece's values so far
+        // this warp's fragment column of the next piece, if any
+        const int nn = (MF == 1) ? n1 + ((sw - n1) & 3) : n1 + ((sw ^ n1) & 1);
+        const bool first = sb < 7 && (MF > 1 || nn < n1 + 2);
+        const int fm0 = (MF == 1) ? 0 : ((sw - nn) & 3) >> 1;
+        double nu[4], np[WITH_P ? 4 : 1];
+        double2 old[MF / MS];
+        if (first) {
+#pragma unroll
+          for (int i = 0; i < NI; ++i)
+            if (NS * i + n_lo == nn)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                nu[q] = -(double)u[i][q];
+                if (WITH_P) np[q] = -(double)pp[WITH_P ? i : 0][q];
+              }
+#pragma unroll
+          for (int mm = 0; mm < MF / MS; ++mm)
+            old[mm] = *reinterpret_cast<const double2*>(&sm.w[pb][8 * (fm0 + MS * mm) + fr][8 * nn + 2 * fk]);
+        }
+        sw_sync<32 + 32 * SW_SPREAD>(SW_PUB + (sb & 1));
+        if (sb < 7) {
+          if (first) {
+#pragma unroll
+            for (int mm = 0; mm < MF / MS; ++mm) {
+              const int m = fm0 + MS * mm;
+              double acc[2][2] = {{old[mm].x, old[mm].y}, {0.0, 0.0}};
+#pragma unroll
+              for (int q = 0; q < 4; ++q) sw_mma(acc[q & 1], sm.Es[8 * m + fr][16 * sb + 4 * q + fk], nu[q]);
+              if (WITH_P)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                  sw_mma(acc[q & 1], sm.As[WITH_P ? 8 * m + fr : 0][16 * sb + 4 * q + fk], np[WITH_P ? q : 0]);
+              *reinterpret_cast<double2*>(&sm.w[pb][8 * m + fr][8 * nn + 2 * fk]) =
+                  make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+            }
+          }
+          sw_arrive<32 + 32 * SW_SPREAD>(SW_READY + (sb & 1));
+#pragma unroll
+          for (int i = 0; i < NI; ++i) {
+            const int n = NS * i + n_lo;
+            if ((n >> 1) > sb + 1) {
+              const int m0 = (MF == 1) ? 0 : ((sw - n) & 3) >> 1;
+#pragma unroll
+              for (int mm = 0; mm < MF / MS; ++mm) {
+                const int m = m0 + MS * mm;
+                double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                  sw_mma(acc[q & 1], sm.Es[8 * m + fr][16 * sb + 4 * q + fk], (double)u[i][q]);
+                if (WITH_P)
+#pragma unroll
+                  for (int q = 0; q < 4; ++q)
+                    sw_mma(acc[q & 1], sm.As[WITH_P ? 8 * m + fr : 0][16 * sb + 4 * q + fk], (double)pp[WITH_P ? i : 0][q]);
+                double2* wp = reinterpret_cast<double2*>(&sm.w[pb][8 * m + fr][8 * n + 2 * fk]);
+                const double2 v = *wp;
+                *wp = make_double2(v.x - (acc[0][0] + acc[1][0]), v.y - (acc[0][1] + acc[1][1]));
+              }
+            }
+          }
+        }
+        if (sb > 0) outputs(b, sb - 1);
+        if (sb == 7) outputs(b, 7);
+      }
+      // the histories are read back by TMA (async proxy): order these stores before it
+      asm volatile("fence.proxy.async;" ::: "memory");
+      next_block();
+    }
+    if (a.stats && crank == 0) {
+      n_near = __reduce_add_sync(0xffffffffu, n_near);
+      n_clamp = __reduce_add_sync(0xffffffffu, n_clamp);
+      if (lane == 0) {
+        if (n_near) atomicAdd(&a.stats->near_tie_codes, (unsigned long long)n_near);
+        if (n_clamp) atomicAdd(&a.stats->clamped_codes, (unsigned long long)n_clamp);
+        if (grp == 0 && sw == 0) atomicAdd(&a.stats->column_steps, (unsigned long long)(a.blk1 - a.blk0) * 128);
+      }
+    }
+    return;
+  }
+
+  if (warp == 4) {
+    // =========================== TMA loads ===========================
+    const int u_row0 = (a.units > 1) ? unit * d : 0;
+    int slot = 0;
+    uint32_t phase = 0;
+#pragma unroll 1
+    for (int b = a.blk0; b < a.blk1; ++b) {
+      if (!CLUSTER && lane == 0 && b + 1 < a.blk1) {
+        const int n_hist = (b - a.blk0) * per_blk, n_all = n_hist + per_blk;
+        for (int c = 0; c < n_all; ++c) {
+          unsigned char* stg = ring + (size_t)slot * stage_bytes;
+          const uint32_t fb = smem_u32(&sm.full_bar[slot]);
+          if (mbar_wait(smem_u32(&sm.empty_bar[slot]), phase ^ 1u, abort_flag, &g_sweep_error)) {
+            const bool hist = c < n_hist;  // else the block being walked: its errors are in shared memory
+            const bool second = WITH_P && (c & 1);
+            const int k0 = a.blk0 * 128 + (c / NOP) * ch;
+            mbar_expect_tx(fb, (uint32_t)(ub_bytes + (hist ? eb_bytes : 0)));
+            tma_load_2d(smem_u32(stg), second ? &map_p : &map_u, (b + 1) * 128, u_row0 + k0, fb);
+            if (hist) tma_load_2d(smem_u32(stg + ub_bytes), second ? &map_a : &map_e, k0 - a.err_col0, m_base, fb);
+          }
+          if (++slot == stages) {
+            slot = 0;
+            phase ^= 1u;
+          }
+        }
+      }
+      __syncwarp();
+      next_block();
+    }
+    return;
+  }
+
+  if (warp == 8 || warp == 12) {  // nothing beside the chain
+#pragma unroll 1
+    for (int b = a.blk0; b < a.blk1; ++b) next_block();
+    return;
+  }
+
+  // =========================== history ===========================
+  const int hw = (warp < 4) ? warp - 1 : (warp < 8) ? warp - 2 : warp - 3;  // warps 1-3, 5-7, 9, 10
+  // columns and share of the contraction of this warp
+  const int frags = 16 / cs;                                 // 8-column fragments of this CTA
+  const int kgroups = CLUSTER ? max(1, SW_HIST / frags) : 1;  // cluster of 2 and more: one fragment per warp
+  const int kg = CLUSTER ? hw / frags : 0;
+  const int n_loc = CLUSTER ? (hw % frags) * 8 : hw * 16;
+  constexpr int FW = CLUSTER ? 1 : 2;  // fragments per warp
+  constexpr int NA = (MF == 1) ? 4 : (MF == 2 ? 2 : 1);  // accumulators per fragment, in turn
+  // column of accumulator (fragment t, element e): one 8-byte load feeds both fragments of a warp, so
+  // fragment 0 takes the even columns and fragment 1 the odd ones
+  auto col_of = [&](int t, int e) { return CLUSTER ? 2 * fk + e : 2 * (2 * fk + e) + t; };
+  int slot = 0;
+  uint32_t phase = 0;
+#pragma unroll 1
+  for (int b = a.blk0; b < a.blk1; ++b) {
+    if (b + 1 >= a.blk1) {
+      next_block();
+      break;
+    }
+    prepare_scales(b + 1, hw * 32 + lane, 32 * SW_HIST);
+    sw_sync<32 * SW_HIST>(SW_JOIN);
+    prepare_triangles(b + 1, hw * 32 + lane, 32 * SW_HIST);
+    double(*wn)[SW_LDW] = sm.w[(b + 1) & 1];
+    const int cn = (b + 1) * 128 + crank * (128 / cs) + n_loc;  // first column of this warp
+    double w0[MF][FW][2];
+    if (kg == 0) {
+#pragma unroll
+      for (int m = 0; m < MF; ++m) {
+        const bool ok = 8 * m + fr < rows_here;
+        const double* src = a.src + (ok ? src_row(8 * m + fr) : 0) + cn;
+#pragma unroll
+        for (int t = 0; t < FW; ++t)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) w0[m][t][e] = ok ? src[col_of(t, e)] : 0.0;
+      }
+    }
+    double acc[MF][FW][NA][2];
+#pragma unroll
+    for (int i = 0; i < MF * FW * NA * 2; ++i) (&acc[0][0][0][0])[i] = 0.0;
+    const int n_hist = (b - a.blk0) * per_blk, n_all = n_hist + per_blk;
+    if constexpr (CLUSTER) {
+      // straight from global memory: a warp has one fragment and every kgroups-th step of four rows; the next batch of
+      // eight steps is fetched while one is multiplied
+      const int n_steps = (b - a.blk0) * (32 / kgroups);  // a multiple of eight
+      const long long urow = (long long)(a.blk0 * 128 + 4 * kg + fk) * d + cn + fr;
+      const double* ep = a.Err + (long long)(m_base + min(fr, rows_here - 1)) * a.err_ld + a.blk0 * 128 - a.err_col0 + 4 * kg + fk;
+      const double* rp = WITH_P ? a.Arr + (ep - a.Err) : nullptr;
+      const long long us = (long long)4 * kgroups * d;
+      double av[8], rv[WITH_P ? 8 : 1];
+      float uv[8], pv[WITH_P ? 8 : 1];
+      auto fetch = [&](int q0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          av[i] = __ldcg(ep + (long long)(q0 + i) * 4 * kgroups);
+          uv[i] = __ldg(U + urow + (q0 + i) * us);
+          if (WITH_P) {
+            rv[i] = __ldcg(rp + (long long)(q0 + i) * 4 * kgroups);
+            pv[i] = __ldg(Pm + urow + (q0 + i) * us);
+          }
+        }
+      };
+      if (n_steps > 0) fetch(0);
+      for (int q0 = 0; q0 < n_steps; q0 += 8) {
+        double an[8], bn[8], rn[WITH_P ? 8 : 1], pn[WITH_P ? 8 : 1];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          an[i] = av[i];
+          bn[i] = (double)uv[i];
+          if (WITH_P) {
+            rn[i] = rv[i];
+            pn[i] = (double)pv[i];
+          }
+        }
+        if (q0 + 8 < n_steps) fetch(q0 + 8);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          sw_mma(acc[0][0][i & 3], an[i], bn[i]);
+          if (WITH_P) sw_mma(acc[0][0][(i + 2) & 3], rn[i], pn[i]);
+        }
+      }
+      // the block being walked, piece by piece: 4 / kgroups steps of this warp each
+      const float* uo = U + (long long)(b * 128 + 4 * kg + fk) * d + cn + fr;
+      const float* po = WITH_P ? Pm + (long long)(b * 128 + 4 * kg + fk) * d + cn + fr : nullptr;
+      const int own = 4 / kgroups;
+      float uc[4], pc[4], uf[4], pf[4];
+      auto fetch_own = [&](int sb) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < own) {
+            uf[i] = __ldg(uo + (long long)(16 * sb) * d + i * us);
+            if (WITH_P) pf[i] = __ldg(po + (long long)(16 * sb) * d + i * us);
+          }
+      };
+      fetch_own(0);
+#pragma unroll 1
+      for (int sb = 0; sb < 8; ++sb) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          uc[i] = uf[i];
+          pc[i] = pf[i];
+        }
+        if (sb < 7) fetch_own(sb + 1);
+        sw_sync<32 + 32 * SW_HIST>(SW_PIECE + sb);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < own) {
+            const int k = 16 * sb + 4 * (kg + kgroups * i) + fk;
+            sw_mma(acc[0][0][i], sm.Es[fr][k], (double)uc[i]);
+            if (WITH_P) sw_mma(acc[0][0][(i + 2) & 3], sm.As[WITH_P ? fr : 0][k], (double)pc[i]);
+          }
+      }
+    } else {
+      int met = 0;  // pieces of the block being walked that are known to be finished
+      for (int c = 0; c < n_all; ++c) {
+        const unsigned char* stg = ring + (size_t)slot * stage_bytes;
+        const bool ok = mbar_wait(smem_u32(&sm.full_bar[slot]), phase, abort_flag, &g_sweep_error);
+        __syncwarp();
+        const bool second = WITH_P && (c & 1);
+        const bool hist = c < n_hist;
+        const int own0 = ((c - n_hist) / NOP) * ch;  // first contraction column of an own chunk inside the block
+        const double* ap = hist ? reinterpret_cast<const double*>(stg + ub_bytes) + fr * lde
+                                : (second ? &sm.As[WITH_P ? fr : 0][0] : &sm.Es[fr][0]) + own0;
+        const int a_ld = hist ? lde : (int)SW_LDW;
+        ap += fk;
+        const float* bp = reinterpret_cast<const float*>(stg) + fk * ldb + n_loc + 2 * fr;
+        for (int qq = 0; qq < ch / 4; qq += 4) {
+          if (!hist) {
+            const int piece = (own0 >> 4) + (qq >> 2);
+            while (met <= piece) {
+              sw_sync<32 + 32 * SW_HIST>(SW_PIECE + met);
+              ++met;
+            }
+          }
+          if (ok) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int q = qq + i;
+              const float2 bb = *reinterpret_cast<const float2*>(bp + 4 * q * SW_LDB);
+              const double b0 = (double)bb.x, b1 = (double)bb.y;
+#pragma unroll
+              for (int m = 0; m < MF; ++m) {
+                const double av = ap[8 * m * a_ld + 4 * q];
+                sw_mma(acc[m][0][i % NA], av, b0);
+                sw_mma(acc[m][FW - 1][i % NA], av, b1);
+              }
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sm.empty_bar[slot]));  // this warp is done with the stage
+        if (++slot == stages) {
+          slot = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < MF; ++m)
+#pragma unroll
+      for (int t = 0; t < FW; ++t)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          double v = acc[m][t][0][e];
+          if (NA == 2) v += acc[m][t][NA - 1][e];
+          if (NA == 4) v = (v + acc[m][t][1 % NA][e]) + (acc[m][t][2 % NA][e] + acc[m][t][3 % NA][e]);
+          acc[m][t][0][e] = v;
+        }
+    if (CLUSTER) {
+      const int wc = 128 / cs;
+      double2 v = make_double2(acc[0][0][0][0], acc[0][0][0][1]);
+      double* mine = &sm.part[fr * wc + n_loc + 2 * fk];
+      if (kg > 0) sw_st2(mine + (kg - 1) * 8 * wc, v.x, v.y);
+      sw_sync<32 * SW_HIST>(SW_JOIN);
+      if (kg == 0) {
+        for (int k = 1; k < kgroups; ++k) {
+          const double2 o = sw_ld2(mine + (k - 1) * 8 * wc);
+          v.x += o.x;
+          v.y += o.y;
+        }
+        v = make_double2(w0[0][0][0] - v.x, w0[0][0][1] - v.y);
+        double* dst = &wn[fr][crank * wc + n_loc + 2 * fk];
+        for (int r = 0; r < cs; ++r) *reinterpret_cast<double2*>(cg::this_cluster().map_shared_rank(dst, r)) = v;
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < MF; ++m)
+#pragma unroll
+        for (int t = 0; t < FW; ++t)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) wn[8 * m + fr][n_loc + col_of(t, e)] = w0[m][t][e] - acc[m][t][0][e];
+    }
+    next_block();
+  }
+}
+
+int sweep_error_read_clear() {
+  int v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_sweep_error, sizeof(int)) != cudaSuccess) return -1;
+  if (v) {
+    int z = 0;
+    cudaMemcpyToSymbol(g_sweep_error, &z, sizeof(int));
+  }
+  return v;
+}
+
+template <bool WITH_P, int R, bool CLUSTER>
+static tb_status sweep_launch(SweepP p, cudaStream_t st) {
+  const SweepArgs& a = p.a;
+  p.ctas_per_unit = (p.rows_per_unit + R - 1) / R;
+  CUtensorMap map_u, map_e, map_p, map_a;
+  constexpr int ch = SweepSmem<WITH_P, R>::CHUNK;
+  const unsigned box_u = (unsigned)(a.d >= SW_LDB ? SW_LDB : a.d);
+  const unsigned box_e = (unsigned)(a.err_ld >= ch + 4 ? ch + 4 : a.err_ld);
+  const unsigned long long cols = (unsigned long long)a.d, mat_rows = cols * a.units;
+  TB_TRY(make_map_2d(&map_u, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), a.U, cols, mat_rows, box_u, ch,
+                     CU_TENSOR_MAP_SWIZZLE_NONE));
+  TB_TRY(make_map_2d(&map_e, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, sizeof(double), a.Err, (unsigned long long)a.err_ld,
+                     (unsigned long long)a.M, box_e, R, CU_TENSOR_MAP_SWIZZLE_NONE));
+  map_p = map_u;
+  map_a = map_e;
+  if (WITH_P) {
+    TB_TRY(make_map_2d(&map_p, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), a.P, cols, mat_rows, box_u, ch,
+                       CU_TENSOR_MAP_SWIZZLE_NONE));
+    TB_TRY(make_map_2d(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, sizeof(double), a.Arr, (unsigned long long)a.err_ld,
+                       (unsigned long long)a.M, box_e, R, CU_TENSOR_MAP_SWIZZLE_NONE));
+  }
+  auto kern = k_sweep_rows<WITH_P, R, CLUSTER>;
+  constexpr size_t smem = sizeof(SweepSmem<WITH_P, R>);
+  static_assert(smem <= 227 * 1024, "shared memory of an SM");
+  static bool configured[64] = {false};
+  TB_TRY(allow_smem(kern, smem, configured));
+  const unsigned ctas = (unsigned)((long long)p.ctas_per_unit * a.units * (CLUSTER ? p.cs : 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(SW_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)(CLUSTER ? p.cs : 1);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CLUSTER ? 1 : 0;
+  TB_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, p, map_u, map_e, map_p, map_a));
+  TB_LAUNCH_CHECK();
+  return TB_OK;
+}
+
+tb_status sweep_columns(const SweepArgs& a, cudaStream_t st) {
+  const long long sms = 148;
+  SweepP p;
+  p.a = a;
+  p.rows_per_unit = a.M / a.units;
+  p.ctas_per_unit = 0;
+  p.cs = 1;
+  const long long groups = (long long)((p.rows_per_unit + 7) / 8) * a.units;  // of 8 rows
+  const int nblk = a.blk1 - a.blk0;
+  // few rows: a cluster per group of 8 rows shares the contraction
+  if (nblk > 1 && groups * 2 <= sms) {
+    p.cs = (groups * 8 <= sms) ? 8 : (groups * 4 <= sms) ? 4 : 2;
+    return a.P ? sweep_launch<true, 8, true>(p, st) : sweep_launch<false, 8, true>(p, st);
+  }
+  // more rows per CTA as soon as 8 would take another round of CTAs: the chain's time does not depend on them
+  const long long g16 = (long long)((p.rows_per_unit + 15) / 16) * a.units;
+  if (a.P) return sweep_launch<true, 8, false>(p, st);  // the registers of 16 rows with both factors spill
+  if (groups <= sms) return sweep_launch<false, 8, false>(p, st);
+  return g16 <= sms ? sweep_launch<false, 16, false>(p, st) : sweep_launch<false, 32, false>(p, st);
+}
+
+
+// ---------------------------------------------------------------------------
+// work[m][c] = src[m][c] - sum_k Err[m][k] U[k0 + k][c] (- Arr P) for the columns c >= c1 of few rows, K = c1 - k0 <= 512.
+// The eight warps of a CTA take an eighth of the contraction each, for 8 MF rows x 8 NF columns, straight from global
+// memory (every entry of U is read once per row tile, in full sectors), and add up through shared memory in order.
+// Bound: reading U (HBM / L2) for 8 rows, the FP64 pipe from about 64 on.
+// ---------------------------------------------------------------------------
+template <bool WITH_P, int MF>
+__global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restrict__ work, int rows_per_unit, int k0, int c1,
+                                                   const double* __restrict__ err, const double* __restrict__ arr) {
+  constexpr int NF = (MF == 4) ? 4 : 8, RT = 8 * MF, CT = 8 * NF;
+  extern __shared__ double rr_part[];  // [8][RT][CT]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, fr = lane >> 2, fk = lane & 3;
+  const int unit = blockIdx.z, r0 = blockIdx.y * RT, c0 = c1 + blockIdx.x * CT;
+  const int d = a.d, K = c1 - k0;
+  const long long uoff = (a.units > 1) ? (long long)unit * d * d : 0;
+  const int m0 = unit * rows_per_unit + r0, rows = min(RT, rows_per_unit - r0);
+  const int steps = K / 32, kw = warp * (K / 8);  // steps of four contraction rows per warp (a multiple of four)
+  double acc[MF][NF][2];
+#pragma unroll
+  for (int i = 0; i < MF * NF * 2; ++i) (&acc[0][0][0])[i] = 0.0;
+  auto product = [&](const float* __restrict__ F, const double* __restrict__ E) {
+    const float* f = F + uoff + (long long)(k0 + kw + fk) * d + c0 + fr;
+    const double* e[MF];
+#pragma unroll
+    for (int m = 0; m < MF; ++m) e[m] = E + (long long)(m0 + min(8 * m + fr, rows - 1)) * a.err_ld + kw + fk;
+#pragma unroll 2
+    for (int q = 0; q < steps; ++q) {
+      float b[NF];
+      double av[MF];
+#pragma unroll
+      for (int n = 0; n < NF; ++n) b[n] = (c0 + 8 * n < d) ? __ldg(f + (long long)(4 * q) * d + 8 * n) : 0.0f;
+#pragma unroll
+      for (int m = 0; m < MF; ++m) av[m] = e[m][4 * q];
+#pragma unroll
+      for (int n = 0; n < NF; ++n) {
+        const double bd = (double)b[n];
+#pragma unroll
+        for (int m = 0; m < MF; ++m) sw_mma(acc[m][n], av[m], bd);
+      }
+    }
+  };
+  product(a.U, err);
+  if (WITH_P) product(a.P, arr);
+#pragma unroll
+  for (int m = 0; m < MF; ++m)
+#pragma unroll
+    for (int n = 0; n < NF; ++n)
+      *reinterpret_cast<double2*>(rr_part + (warp * RT + 8 * m + fr) * CT + 8 * n + 2 * fk) = make_double2(acc[m][n][0], acc[m][n][1]);
+  __syncthreads();
+  for (int i = threadIdx.x; i < RT * CT; i += 256) {
+    const int r = i / CT, c = i % CT;
+    if (r >= rows || c0 + c >= d) continue;
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += rr_part[w * RT * CT + i];
+    const long long src = (a.src_mapped ? a.rm.row(m0 + r) : (long long)(m0 + r)) * d + c0 + c;
+    work[(long long)(m0 + r) * d + c0 + c] = a.src[src] - v;
+  }
+}
+
+__global__ void k_sweep_gather(SweepArgs a, double* __restrict__ work, int c1) {
+  const int m = blockIdx.y;
+  const double2* src = reinterpret_cast<const double2*>(a.src + a.rm.row(m) * a.d);
+  double2* dst = reinterpret_cast<double2*>(work + (long long)m * a.d);
+  for (int c = c1 / 2 + blockIdx.x * blockDim.x + threadIdx.x; c < a.d / 2; c += gridDim.x * blockDim.x) dst[c] = src[c];
+}
+
+// exps[k] = exponent of the diagonal entry U_kk
+__global__ void k_sweep_exp(const float* __restrict__ U, int* __restrict__ exps, int d) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= d) return;
+  const float u = fabsf(U[(long long)blockIdx.y * d * d + (long long)k * (d + 1)]);
+  int e = 0;
+  if (u > 0.0f && u <= 3.4e38f) frexpf(u, &e);
+  exps[blockIdx.y * d + k] = e;
+}
+
+bool sweep_wants_i8(int d, int rows_per_unit) {
+  return d > SWEEP_OUTER && d <= 16384 && rows_per_unit >= SWEEP_I8_ROWS;
+}
+
+void sweep_scratch(Bump& b, int M, int d, int units, bool with_p, bool use_i8, SweepScratch* s) {
+  *s = SweepScratch{};
+  s->use_i8 = use_i8;
+  if (d <= SWEEP_OUTER) return;
+  s->err = b.take<double>((size_t)M * SWEEP_OUTER);
+  if (with_p) s->arr = b.take<double>((size_t)M * SWEEP_OUTER);
+  if (!use_i8) return;
+  auto mat = [&](long long row_blocks, int k_blocks) {
+    I8Mat m;
+    m.row_blocks = row_blocks;
+    m.k_blocks = k_blocks;
+    m.data = b.take<unsigned char>(i8_bytes(row_blocks, k_blocks));
+    return m;
+  };
+  const long long rb_unit = (M / units + I8_RB - 1) / I8_RB;
+  s->Udig = mat((long long)units * (d / I8_RB), d / I8_KB);
+  s->Edig = mat(units * rb_unit, SWEEP_OUTER / I8_KB);
+  s->u_max = b.take<unsigned long long>((size_t)units * d);
+  s->e_max = b.take<unsigned long long>((size_t)M);
+  s->u_exp = b.take<int>((size_t)units * d);
+  if (with_p) {
+    s->Pdig = mat((long long)units * (d / I8_RB), d / I8_KB);
+    s->Adig = mat(units * rb_unit, SWEEP_OUTER / I8_KB);
+    s->p_max = b.take<unsigned long long>((size_t)units * d);
+    s->a_max = b.take<unsigned long long>((size_t)M);
+  }
+}
+
+// Rows of U scale as 1 / U_kk scales the errors: the exponents of the diagonal take that out of both operands.
+tb_status sweep_prepare(const float* U, const float* P, int d, int units, const SweepScratch& s, cudaStream_t st) {
+  if (!s.use_i8) return TB_OK;
+  const long long dd = (long long)d * d;
+  k_sweep_exp<<<dim3((d + 255) / 256, units), 256, 0, st>>>(U, s.u_exp, d);
+  TB_LAUNCH_CHECK();
+  for (int u = 0; u < units; ++u) {  // (one exponent vector per matrix)
+    const I8Src us{U + u * dd, d, 0, d, d, 1, true, false, 1, s.u_exp + (long long)u * d, -1};
+    TB_TRY(i8_row_max(us, s.u_max + (long long)u * d, d, st));
+    TB_TRY(i8_slice(us, s.u_max + (long long)u * d, d, 0, s.Udig, (long long)u * (d / I8_RB), 0, 0, st));
+  }
+  if (P) {
+    const I8Src ps{P, d, dd, d, d, units, true, false, 1, nullptr, 0};
+    TB_TRY(i8_row_max(ps, s.p_max, d, st));
+    TB_TRY(i8_slice(ps, s.p_max, d, 0, s.Pdig, 0, d / I8_RB, 0, st));
+  }
+  return TB_OK;
+}
+
+template <bool WITH_P, int MF>
+static tb_status rank_launch(const SweepArgs& a, double* work, int rows_per_unit, int k0, int c1, const double* err,
+                             const double* arr, cudaStream_t st) {
+  constexpr int NF = (MF == 4) ? 4 : 8, CT = 8 * NF;
+  constexpr size_t smem = (size_t)8 * 8 * MF * CT * sizeof(double);
+  static bool configured[64] = {false};
+  auto kern = k_rank_rows<WITH_P, MF>;
+  TB_TRY(allow_smem(kern, smem, configured));
+  const dim3 grid((a.d - c1 + CT - 1) / CT, (rows_per_unit + 8 * MF - 1) / (8 * MF), a.units);
+  kern<<<grid, 256, smem, st>>>(a, work, rows_per_unit, k0, c1, err, arr);
+  TB_LAUNCH_CHECK();
+  return TB_OK;
+}
+
+tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st) {
+  const int d = a.d, rows_per_unit = a.M / a.units, nblk = d / 128;
+  constexpr int OB = SWEEP_OUTER / 128;
+  if (nblk <= OB) {  // one launch; the histories take the working copies' places
+    a.blk0 = 0;
+    a.blk1 = nblk;
+    a.err_ld = d;
+    a.err_col0 = 0;
+    return sweep_columns(a, st);
+  }
+  double* E = s.err;
+  double* A = s.arr;
+  a.Err = E;
+  a.Arr = A;
+  a.err_ld = SWEEP_OUTER;
+  if (s.use_i8) {
+    k_sweep_gather<<<dim3((d / 2 + 255) / 256, a.M), 256, 0, st>>>(a, s.work, SWEEP_OUTER);
+    TB_LAUNCH_CHECK();
+  }
+  for (int b0 = 0; b0 < nblk; b0 += OB) {
+    const int b1 = (b0 + OB < nblk) ? b0 + OB : nblk, k0 = b0 * 128, c1 = b1 * 128;
+    a.blk0 = b0;
+    a.blk1 = b1;
+    a.err_col0 = k0;
+    TB_TRY(sweep_columns(a, st));
+    if (c1 >= d) break;
+    if (s.use_i8) {
+      const long long rb_unit = (rows_per_unit + I8_RB - 1) / I8_RB, batch = (long long)rows_per_unit * SWEEP_OUTER;
+      // one exponent vector per launch: with several units the scales of all but the first stay in their digits
+      const I8Src es{E, SWEEP_OUTER, batch, rows_per_unit, c1 - k0, a.units, false, true, 0, a.units == 1 ? s.u_exp + k0 : nullptr, 1};
+      TB_TRY(i8_row_max(es, s.e_max, rows_per_unit, st));
+      TB_TRY(i8_slice(es, s.e_max, rows_per_unit, 0, s.Edig, 0, rb_unit, 0, st));
+      I8Gemm g = i8_gemm_params();
+      g.A = s.Edig;
+      g.B = s.Udig;
+      g.a_rb_batch = rb_unit;
+      g.b_rb = c1 / I8_RB;
+      g.b_rb_batch = d / I8_RB;
+      g.b_kb = k0 / I8_KB;
+      g.k_blocks = (c1 - k0) / I8_KB;
+      g.a_max = s.e_max;
+      g.a_max_batch = rows_per_unit;
+      g.b_max = s.u_max + c1;
+      g.b_max_batch = d;
+      g.C = s.work + c1;
+      g.ldc = d;
+      g.c_batch = (long long)rows_per_unit * d;
+      g.M = rows_per_unit;
+      g.N = d - c1;
+      g.n_batch = a.units;
+      g.alpha = -1.0;
+      g.beta = 1.0;
+      TB_TRY(i8_gemm(g, st));
+      if (a.P) {
+        const I8Src as{A, SWEEP_OUTER, batch, rows_per_unit, c1 - k0, a.units, false, true, 0, nullptr, 0};
+        TB_TRY(i8_row_max(as, s.a_max, rows_per_unit, st));
+        TB_TRY(i8_slice(as, s.a_max, rows_per_unit, 0, s.Adig, 0, rb_unit, 0, st));
+        g.A = s.Adig;
+        g.B = s.Pdig;
+        g.a_max = s.a_max;
+        g.b_max = s.p_max + c1;
+        TB_TRY(i8_gemm(g, st));
+      }
+    } else {
+      // rows per tile: 8, 16 or 32, as few tiles as cover the unit's rows
+      const int mf = rows_per_unit <= 8 ? 1 : rows_per_unit <= 16 ? 2 : 4;
+      if (a.P) {
+        if (mf == 1) TB_TRY((rank_launch<true, 1>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+        if (mf == 2) TB_TRY((rank_launch<true, 2>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+        if (mf == 4) TB_TRY((rank_launch<true, 4>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+      } else {
+        if (mf == 1) TB_TRY((rank_launch<false, 1>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+        if (mf == 2) TB_TRY((rank_launch<false, 2>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+        if (mf == 4) TB_TRY((rank_launch<false, 4>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+      }
+    }
+    a.src = s.work;
+    a.src_mapped = false;
+  }
+  return TB_OK;
+}
+
+}  // namespace tb

@@ -249,7 +249,7 @@ tb_status syrk_bf16_tensor(float* H, const __nv_bfloat16* X, long long n_tok, in
 // 0, or 1 once a bounded wait inside a tensor-core kernel has run out (sticky until read).
 namespace tb {
 int i8_error_read_clear();     // the products on the integer tensor cores (tb_i8.cu)
-int sweep_error_read_clear();  // the same word of the column-sweep kernel (tb_quantize.cu)
+int sweep_error_read_clear();  // the same word of the column-sweep kernel (tb_sweep.cu)
 int yw_error_read_clear();     // and of the tensor-core product of the scale refinement (tb_gemm_tc.cu)
 int cross_error_read_clear();  // and of the deviation correlation (tb_cross_tc.cu)
 int pair_error_read_clear();   // and of the CTA-pair form of the Hessian kernel (tb_syrk_tc2.cu)
