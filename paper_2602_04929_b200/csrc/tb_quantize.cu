@@ -66,19 +66,35 @@ __global__ void k_gather(const double* __restrict__ Wt, double* __restrict__ Wk,
 // With A = U_out^T lower triangular, T A_BB = A_remB is solved row by row,
 // last column first.  T is stored [head][step][d_head][g] (first rem rows used).
 // ---------------------------------------------------------------------------
+// The g factor rows of the step are staged in shared memory ([c][column from i0 on], when they fit), the solve of a
+// row keeps its T in the row's own storage.
 __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restrict__ T, int dh,
-                                int g, int n_steps) {
+                                int g, int n_steps, int staged) {
+  extern __shared__ float cm_u[];
   const int step = blockIdx.x, head = blockIdx.y;
   const int i0 = step * g, r0 = i0 + g, nrem = dh - r0;
+  if (nrem <= 0) return;
   const float* Uo = Uout + (long long)head * dh * dh;
   double* Th = T + ((long long)head * n_steps + step) * dh * g;
+  const int w = dh - i0;
+  if (staged) {
+    for (int i = threadIdx.x; i < g * w; i += blockDim.x) cm_u[i] = Uo[(long long)(i0 + i / w) * dh + i0 + i % w];
+    __syncthreads();
+  }
   for (int r = threadIdx.x; r < nrem; r += blockDim.x) {
     double* Tr = Th + (long long)r * g;
     for (int c = g - 1; c >= 0; --c) {
-      const float* urow = Uo + (long long)(i0 + c) * dh;
-      double v = (double)urow[r0 + r];
-      for (int c2 = c + 1; c2 < g; ++c2) v -= Tr[c2] * (double)urow[i0 + c2];
-      Tr[c] = v / (double)urow[i0 + c];
+      const float* urow = staged ? cm_u + c * w - i0 : Uo + (long long)(i0 + c) * dh;
+      double v0 = (double)urow[r0 + r], v1 = 0.0, v2 = 0.0, v3 = 0.0;
+      int c2 = c + 1;
+      for (; c2 + 3 < g; c2 += 4) {
+        v0 = fma(-Tr[c2], (double)urow[i0 + c2], v0);
+        v1 = fma(-Tr[c2 + 1], (double)urow[i0 + c2 + 1], v1);
+        v2 = fma(-Tr[c2 + 2], (double)urow[i0 + c2 + 2], v2);
+        v3 = fma(-Tr[c2 + 3], (double)urow[i0 + c2 + 3], v3);
+      }
+      for (; c2 < g; ++c2) v0 = fma(-Tr[c2], (double)urow[i0 + c2], v0);
+      Tr[c] = ((v0 + v1) + (v2 + v3)) / (double)urow[i0 + c];
     }
   }
 }
@@ -1100,24 +1116,21 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
     p.cd_rows = rows;
     p.Yw = b.take<double>((size_t)rows * p.ng * dd);
     // blockwise product on the tensor cores (float result): one shared H_in, groups that are whole TMA boxes
-    // With one H_in per head the heads of a batch go through the same launches, each against its own
-    // pieces of H_in; that needs heads of whole 128-row tiles and groups of at most 128 columns.
-    const bool per_head_ok = (p.n_hin > 1) && (p.dh % 128 == 0) && (p.seg <= 128) && (rows % p.dh == 0);
-    p.yw_tensor = (p.n_hin == 1 || per_head_ok) && (p.seg % 64 == 0) && (rows % 8 == 0) && (p.d_out % 8 == 0) &&
-                  (p.dh % 8 == 0 || rows == p.d_out);
-    if (p.yw_tensor) {
-      p.WbT = b.take<__nv_bfloat16>((size_t)rows * dd);
+    // With one H_in per head the heads of a batch go through the same launches, each against its own pieces of H_in.
+    const bool tiles_ok = (p.n_hin == 1 || (p.dh % 8 == 0 && rows % p.dh == 0)) && rows % 8 == 0 && p.d_out % 8 == 0 &&
+                          (p.dh % 8 == 0 || rows == p.d_out);
+    p.yw_tensor = tiles_ok && p.seg % 64 == 0;
+    p.dm_tensor = tiles_ok && p.d % 32 == 0;
+    if (p.yw_tensor) p.WbT = b.take<__nv_bfloat16>((size_t)rows * dd);
+    if (p.yw_tensor || p.dm_tensor)
       p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (p.n_hin > 1 ? (size_t)(rows / p.dh) : 1));
-      p.dm_tensor = (p.d % 32 == 0);
-    }
     const long long lines = rows;  // one set of statistics per row (the column-parallel pass keeps them all)
     p.n0 = b.take<double>((size_t)lines * p.ng);
     p.Amat = b.take<double>((size_t)lines * p.ng * p.ng);
   }
   // without the scale refinement the loss forms dW H_in itself: the same split-bf16 product
-  // (with one H_in per head the heads of a batch share the launch, each against its own pieces: that
-  // needs heads of whole 128-row tiles)
-  p.loss_tensor = with_loss && !p.cd && (p.n_hin == 1 || p.dh % 128 == 0) && (p.d % 32 == 0) && (p.d_out % 8 == 0);
+  // (with one H_in per head the heads of a batch share the launch, each against its own pieces)
+  p.loss_tensor = with_loss && !p.cd && (p.n_hin == 1 || p.dh % 8 == 0) && (p.d % 32 == 0) && (p.d_out % 8 == 0);
   p.loss_heads = 1;
   if (p.loss_tensor && p.n_hin > 1) {
     const size_t per_head = (size_t)3 * dd * dd * sizeof(__nv_bfloat16);
@@ -1359,7 +1372,11 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     k_widen<<<ew_blocks(n_all), 256, 0, st>>>(W, p.Wt, n_all);
     TB_LAUNCH_CHECK();
     if (p.T) {
-      k_comp_matrices<<<dim3(p.S, p.H), 128, 0, st>>>(U_out, p.T, p.dh, p.g, p.S);
+      const size_t cm_smem = (size_t)p.g * p.dh * sizeof(float);
+      const bool staged = cm_smem <= 96 * 1024;
+      static bool conf_cm[64] = {false};
+      TB_TRY(allow_smem(k_comp_matrices, 96 * 1024, conf_cm));
+      k_comp_matrices<<<dim3(p.S, p.H), 128, staged ? cm_smem : 0, st>>>(U_out, p.T, p.dh, p.g, p.S, staged ? 1 : 0);
       TB_LAUNCH_CHECK();
     }
     if (p.c_max) {  // C by columns, once for all steps
@@ -1484,51 +1501,54 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     TB_LAUNCH_CHECK();
     for (long long r0 = 0; r0 < p.d_out; r0 += p.cd_rows) {
       const long long rows = (p.d_out - r0 < p.cd_rows) ? (p.d_out - r0) : p.cd_rows;
-      // Dm = (Q - W) H_in (+ W R); Yw = blockwise Wbar H_in.  With one H_in per head the
-      // batch is whole heads and the products run head by head.
-      const bool heads_together = p.yw_tensor && units > 1;   // per-head H_in on the tensor-core path
-      const int hunits = heads_together ? (int)(rows / p.dh) : 1;
-      const long long rows_per_prod = (units > 1 && !heads_together) ? p.dh : rows;
-      for (long long q0 = 0; q0 < rows; q0 += rows_per_prod) {
+      // Dm = (Q - W) H_in (+ W R); Yw = blockwise Wbar H_in.  With one H_in per head the batch is whole heads: one launch
+      // for all of them on the tensor cores, head by head on the FP64 engine.
+      const int hunits = (units > 1) ? (int)(rows / p.dh) : 1;
+      const long long rows_per_prod = (units > 1) ? p.dh : rows;
+      const float* Hb = H_in + ((units > 1) ? (r0 / p.dh) * dd : 0);
+      const bool split_h = r0 == 0 || with_r || units > 1;  // with R the pieces of R replace H_in's below
+      if (p.yw_tensor)  // also splits H_in into its bf16 pieces
+        TB_TRY(yw_tensor(reinterpret_cast<float*>(p.Yw), codes + r0 * d, zeros + r0 * p.ng, Hb, p.WbT, p.Hp, split_h, rows, d,
+                         p.seg, p.ng, hunits, st));
+      else if (p.dm_tensor && split_h)
+        TB_TRY(split3(Hb, p.Hp, dd * hunits, st));
+      if (p.dm_tensor) {
+        // the pieces of (Q - W), transposed, live in this batch's rows of the W~ buffer (free by now,
+        // and overwritten by G = H_out Dm only after the product)
+        __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + r0 * d);
+        TB_TRY(split3_transpose(p.Dq + r0 * d, DqT, rows, d, st));
+        TB_TRY(gemm_split_presplit(p.Dm + r0 * d, d, DqT, p.Hp, rows, d, d, false, st, hunits));
+        if (with_r) {
+          // Dm += W R through the same split-bf16 product; the pieces of R take the place of H_in's
+          TB_TRY(split3_transpose(W + r0 * d, DqT, rows, d, st));
+          TB_TRY(split3(R + ((units > 1) ? (r0 / p.dh) * dd : 0), p.Hp, dd * hunits, st));
+          TB_TRY(gemm_split_presplit(p.Dm + r0 * d, d, DqT, p.Hp, rows, d, d, true, st, hunits));
+        }
+      }
+      for (long long q0 = 0; q0 < rows && !(p.yw_tensor && p.dm_tensor); q0 += rows_per_prod) {
         const long long rr = r0 + q0;
         const float* Hh = H_in + ((units > 1) ? (rr / p.dh) * dd : 0);
-        if (p.yw_tensor)  // also splits H_in into its bf16 pieces on the first batch
-          TB_TRY(yw_tensor(reinterpret_cast<float*>(p.Yw), codes + rr * d, zeros + rr * p.ng, Hh, p.WbT, p.Hp,
-                           r0 == 0 || with_r || units > 1, rows, d, p.seg, p.ng, hunits,
-                           st));  // with R the pieces of R replace H_in's below
-        GemmP g = gemm_params();
-        g.A = p.Dq + rr * d;
-        g.a_m = d;
-        g.a_k = 1;
-        g.B = Hh;
-        g.b_k = d;
-        g.b_n = 1;
-        g.C = p.Dm + rr * d;
-        g.ldc = d;
-        g.M = (int)rows_per_prod;
-        g.N = d;
-        g.K = d;
-        if (p.dm_tensor) {
-          // the pieces of (Q - W), transposed, live in this batch's rows of the W~ buffer (free by now,
-          // and overwritten by G = H_out Dm only after the product)
-          __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + rr * d);
-          TB_TRY(split3_transpose(p.Dq + rr * d, DqT, rows, d, st));
-          TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rows, d, d, false, st, hunits));
-        } else {
+        if (!p.dm_tensor) {
+          GemmP g = gemm_params();
+          g.A = p.Dq + rr * d;
+          g.a_m = d;
+          g.a_k = 1;
+          g.B = Hh;
+          g.b_k = d;
+          g.b_n = 1;
+          g.C = p.Dm + rr * d;
+          g.ldc = d;
+          g.M = (int)rows_per_prod;
+          g.N = d;
+          g.K = d;
           TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
-        }
-        if (with_r && p.dm_tensor) {
-          // Dm += W R through the same split-bf16 product; the pieces of R take the place of H_in's
-          __nv_bfloat16* WT = reinterpret_cast<__nv_bfloat16*>(p.Wt + rr * d);
-          TB_TRY(split3_transpose(W + rr * d, WT, rows, d, st));
-          TB_TRY(split3(R + ((units > 1) ? (rr / p.dh) * dd : 0), p.Hp, dd * hunits, st));
-          TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, WT, p.Hp, rows, d, d, true, st, hunits));
-        } else if (with_r) {
-          GemmP h = g;
-          h.A = W + rr * d;
-          h.B = R + ((units > 1) ? (rr / p.dh) * dd : 0);
-          h.beta = 1.0;
-          TB_TRY((gemm_launch<float, float, double, double, false, true>(h, st)));
+          if (with_r) {
+            GemmP h = g;
+            h.A = W + rr * d;
+            h.B = R + ((units > 1) ? (rr / p.dh) * dd : 0);
+            h.beta = 1.0;
+            TB_TRY((gemm_launch<float, float, double, double, false, true>(h, st)));
+          }
         }
         if (!p.yw_tensor) {
           GemmP y = gemm_params();

@@ -52,11 +52,11 @@ tb_status sweep_columns(const SweepArgs& a, cudaStream_t st);
 
 // The sweep over all columns of a step.  Up to SWEEP_OUTER columns go through in one launch; more are taken that many at
 // a time, each followed by one update of everything further right in a working copy of the step's rows.
-enum { SWEEP_OUTER = 512, SWEEP_I8_ROWS = 192 };
+enum { SWEEP_OUTER = 512, SWEEP_I8_WORK = 1200000 };
 struct SweepScratch {
   double *work;          // [M][d]
   double *err, *arr;     // [M][SWEEP_OUTER], arr with P only
-  bool use_i8;           // the updates on the integer tensor cores (rows of a unit: SWEEP_I8_ROWS or more); then:
+  bool use_i8;           // the updates on the integer tensor cores (sweep_wants_i8); then:
   I8Mat Udig, Pdig;      // digits of U and P by columns (prepared by sweep_prepare, one set for all steps)
   I8Mat Edig, Adig;      // digits of a block's errors and arrival values
   unsigned long long *u_max, *p_max, *e_max, *a_max;

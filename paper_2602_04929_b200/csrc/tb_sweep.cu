@@ -840,8 +840,10 @@ __global__ void k_sweep_exp(const float* __restrict__ U, int* __restrict__ exps,
   exps[blockIdx.y * d + k] = e;
 }
 
+// An update on digits costs three launches whatever its size, k_rank_rows the FP64 pipe's time for rows x width: about
+// equal at 300 rows of 4096 columns.  208 rows of 1664 with P: 11.0 ms of sweep with digits, 7.2 ms without.
 bool sweep_wants_i8(int d, int rows_per_unit) {
-  return d > SWEEP_OUTER && d <= 16384 && rows_per_unit >= SWEEP_I8_ROWS;
+  return d > SWEEP_OUTER && d <= 16384 && (long long)rows_per_unit * d >= SWEEP_I8_WORK;
 }
 
 void sweep_scratch(Bump& b, int M, int d, int units, bool with_p, bool use_i8, SweepScratch* s) {

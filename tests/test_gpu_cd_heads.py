@@ -1,0 +1,21 @@
+"""Scale refinement and loss with one H_in per head through the tensor-core products: heads that are no whole tiles of
+128 rows, wide groups, groups of 32 columns (no tensor-core Yw), with and without the propagated-error term."""
+import pytest
+
+from parity_util import compare, make_problem, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+CD, ADAPT = 2, 1
+
+
+@pytest.mark.parametrize("dh,gq,with_r,flags", [(64, 256, False, CD | ADAPT), (64, 128, True, CD | ADAPT), (40, 64, False, CD),
+                                                (136, 0, False, CD), (64, 32, True, CD | ADAPT), (72, 128, True, 0)])
+def test_heads_of_any_size(dh, gq, with_r, flags):
+    prob = make_problem(70, 512, 3, dh, 1024, n_hin=3, with_r=with_r, hout="spd")
+    compare(prob, run_gpu(prob, 4, gq, 8, flags), 4, gq, 8, flags, label=f"heads{dh}")
+
+
+def test_groups_of_32_columns_shared_hessian():
+    prob = make_problem(71, 512, 3, 64, 1024, with_r=True)
+    compare(prob, run_gpu(prob, 3, 32, 16, CD | ADAPT), 3, 32, 16, CD | ADAPT, label="gq32")
