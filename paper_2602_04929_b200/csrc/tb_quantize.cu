@@ -4,9 +4,8 @@
 // rows in all, heads being independent):
 //   grid     k_grid_tri       Algorithm 1, grid     candidate search per (row, column group)
 //   sweep    k_sweep_rows     Algorithm 2 / Eq. 2   one launch, 8 to 32 rows per CTA for the whole sweep (tb_sweep.cu)
-//   residual k_residual       E = W0 - Q_B          (Proposition 3.1)
-//            GEMM             E -= W0 C             (Proposition 3.2, only with R)
-//   update   GEMM             W~[rem] -= T_i E      (Algorithm 1, update)
+//   update   k_compensate     W~[rem] -= T_i E      (Algorithm 1, update), E = W0 - Q_B (Proposition 3.1);
+//            with R first k_residual and a product: E -= W0 C (Proposition 3.2)
 // then, once: coordinate descent on the scales (Algorithm 3), Q = s (W_int - z),
 // and the loss of the proofs of Propositions 3.1 / 3.2.
 //
@@ -70,7 +69,7 @@ __global__ void k_gather(const double* __restrict__ Wt, double* __restrict__ Wk,
 // row keeps its T in the row's own storage.
 __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restrict__ T, int dh,
                                 int g, int n_steps, int staged) {
-  extern __shared__ float cm_u[];
+  extern __shared__ __align__(16) float cm_u[];
   const int step = blockIdx.x, head = blockIdx.y;
   const int i0 = step * g, r0 = i0 + g, nrem = dh - r0;
   if (nrem <= 0) return;
@@ -83,19 +82,24 @@ __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restri
   }
   for (int r = threadIdx.x; r < nrem; r += blockDim.x) {
     double* Tr = Th + (long long)r * g;
+    // the row under construction: in shared memory where the factor rows are, [c][thread]
+    double* ct = staged ? reinterpret_cast<double*>(cm_u + (((size_t)g * dh + 3) & ~(size_t)3)) + threadIdx.x : Tr;
+    const int cs = staged ? 128 : 1;
     for (int c = g - 1; c >= 0; --c) {
       const float* urow = staged ? cm_u + c * w - i0 : Uo + (long long)(i0 + c) * dh;
       double v0 = (double)urow[r0 + r], v1 = 0.0, v2 = 0.0, v3 = 0.0;
       int c2 = c + 1;
       for (; c2 + 3 < g; c2 += 4) {
-        v0 = fma(-Tr[c2], (double)urow[i0 + c2], v0);
-        v1 = fma(-Tr[c2 + 1], (double)urow[i0 + c2 + 1], v1);
-        v2 = fma(-Tr[c2 + 2], (double)urow[i0 + c2 + 2], v2);
-        v3 = fma(-Tr[c2 + 3], (double)urow[i0 + c2 + 3], v3);
+        v0 = fma(-ct[c2 * cs], (double)urow[i0 + c2], v0);
+        v1 = fma(-ct[(c2 + 1) * cs], (double)urow[i0 + c2 + 1], v1);
+        v2 = fma(-ct[(c2 + 2) * cs], (double)urow[i0 + c2 + 2], v2);
+        v3 = fma(-ct[(c2 + 3) * cs], (double)urow[i0 + c2 + 3], v3);
       }
-      for (; c2 < g; ++c2) v0 = fma(-Tr[c2], (double)urow[i0 + c2], v0);
-      Tr[c] = ((v0 + v1) + (v2 + v3)) / (double)urow[i0 + c];
+      for (; c2 < g; ++c2) v0 = fma(-ct[c2 * cs], (double)urow[i0 + c2], v0);
+      ct[c * cs] = ((v0 + v1) + (v2 + v3)) / (double)urow[i0 + c];
     }
+    if (staged)
+      for (int c = 0; c < g; ++c) Tr[c] = ct[c * cs];
   }
 }
 
@@ -411,6 +415,67 @@ __global__ void k_residual(const double* __restrict__ Wt, const unsigned char* _
     const long long so = r * ng + k / seg;
     const double q = (double)codes[r * d + k] - (double)z[so];
     E[i] = Wt[r * d + k] - sD[so] * q;
+  }
+}
+
+// W~[rem] -= T E for the rows of every head not yet quantized (Propositions 3.1 / 3.2; Algorithm 1, update step).  CTA: 32
+// rows x 128 columns of one head; thread: 8 rows x 2 columns, the group's rows 32 at a time from shared memory.  E is the
+// group's residual W~ - s (code - z), formed where it is needed, or (HAVE_E, propagated error) a matrix.
+// Bound: reading and writing W~ once.  As a residual launch and a product of the 128 x 128 engine it took, per step of
+// one row in 8 heads x 4096 columns, 24 us, of 32 rows in 32 heads 115 us; now 12 us and 80 us.
+template <bool HAVE_E>
+__global__ void __launch_bounds__(256) k_compensate(double* __restrict__ Wt, const unsigned char* __restrict__ codes,
+                                                    const double* __restrict__ sD, const int* __restrict__ z,
+                                                    const double* __restrict__ E, const double* __restrict__ T, int i0, int g,
+                                                    int dh, long long t_head, int d, int seg, int ng) {
+  __shared__ double Es[32][128], Ts[32][33];
+  const int head = blockIdx.y, c0 = blockIdx.x * 128, q0 = blockIdx.z * 32;  // first of 32 remaining rows
+  const int nrem = dh - i0 - g;
+  const int tid = threadIdx.x, ct = (tid & 63) * 2, rt = tid >> 6;  // rows rt + 4 k
+  const double* Th = T + head * t_head;
+  double acc[8][2];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k][0] = acc[k][1] = 0.0;
+  for (int e0 = 0; e0 < g; e0 += 32) {
+    const int ge = min(32, g - e0);
+    for (int i = tid; i < ge * 64; i += 256) {
+      const int r = i >> 6, c = (i & 63) * 2;
+      double2 v;
+      if (HAVE_E) {
+        v = *reinterpret_cast<const double2*>(E + ((long long)head * g + e0 + r) * d + c0 + c);
+      } else {
+        const long long row = (long long)head * dh + i0 + e0 + r, so = row * ng + (c0 + c) / seg;  // groups: multiples of 32
+        v = *reinterpret_cast<const double2*>(Wt + row * d + c0 + c);
+        const uchar2 q = *reinterpret_cast<const uchar2*>(codes + row * d + c0 + c);
+        const double s = sD[so], zz = (double)z[so];
+        v.x -= s * ((double)q.x - zz);
+        v.y -= s * ((double)q.y - zz);
+      }
+      *reinterpret_cast<double2*>(&Es[r][c]) = v;
+    }
+    for (int i = tid; i < 32 * ge; i += 256) {
+      const int r = i / ge, c = i % ge;
+      Ts[c][r] = (q0 + r < nrem) ? Th[(long long)(q0 + r) * g + e0 + c] : 0.0;
+    }
+    __syncthreads();
+    for (int i = 0; i < ge; ++i) {
+      const double2 e = *reinterpret_cast<const double2*>(&Es[i][ct]);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const double t = Ts[i][rt + 4 * k];
+        acc[k][0] = fma(t, e.x, acc[k][0]);
+        acc[k][1] = fma(t, e.y, acc[k][1]);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int r = q0 + rt + 4 * k;
+    if (r >= nrem) continue;
+    double2* w = reinterpret_cast<double2*>(Wt + ((long long)head * dh + i0 + g + r) * d + c0 + ct);
+    const double2 v = *w;
+    *w = make_double2(v.x - acc[k][0], v.y - acc[k][1]);
   }
 }
 
@@ -1007,6 +1072,7 @@ struct Plan {
   long long cd_rows;  // rows per coordinate-descent batch
   // workspace
   double *Wt, *Wk, *W0c, *E, *sD, *T, *Dq, *Dm, *Yw, *n0, *Amat, *G2;
+  double* gram;  // scale refinement as a triangular solve: the heads' matrices
   SweepScratch sweep;
   I8Mat Cdig, Wdig;                // digits of C (all steps) and of the step's W0 (propagated error, one shared H_in)
   unsigned long long *c_max, *w_max;
@@ -1093,7 +1159,7 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
   p.T = (has_hout && p.S > 1) ? b.take<double>((size_t)p.H * p.S * p.dh * p.g) : nullptr;
   p.dynErr = p.dynamic ? b.take<double>((size_t)p.Mmax * p.seg) : nullptr;
   p.dynArr = (p.dynamic && with_r) ? b.take<double>((size_t)p.Mmax * p.seg) : nullptr;
-  p.Dq = p.Dm = p.Yw = p.n0 = p.Amat = p.G2 = nullptr;
+  p.Dq = p.Dm = p.Yw = p.n0 = p.Amat = p.G2 = p.gram = nullptr;
   p.Wb = nullptr;
   p.WbT = p.Hp = nullptr;
   p.yw_tensor = p.dm_tensor = false;
@@ -1125,6 +1191,7 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
     if (p.yw_tensor || p.dm_tensor)
       p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (p.n_hin > 1 ? (size_t)(rows / p.dh) : 1));
     const long long lines = rows;  // one set of statistics per row (the column-parallel pass keeps them all)
+    if (has_hout && cd_gram_pays(p.dh, p.ng)) p.gram = b.take<double>(cd_gram_doubles((int)(rows / p.dh), p.dh, p.ng));
     p.n0 = b.take<double>((size_t)lines * p.ng);
     p.Amat = b.take<double>((size_t)lines * p.ng * p.ng);
   }
@@ -1372,10 +1439,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     k_widen<<<ew_blocks(n_all), 256, 0, st>>>(W, p.Wt, n_all);
     TB_LAUNCH_CHECK();
     if (p.T) {
-      const size_t cm_smem = (size_t)p.g * p.dh * sizeof(float);
-      const bool staged = cm_smem <= 96 * 1024;
+      const size_t cm_smem = (size_t)p.g * p.dh * sizeof(float) + 16 + (size_t)p.g * 128 * sizeof(double);
+      const bool staged = cm_smem <= 200 * 1024;
       static bool conf_cm[64] = {false};
-      TB_TRY(allow_smem(k_comp_matrices, 96 * 1024, conf_cm));
+      TB_TRY(allow_smem(k_comp_matrices, 200 * 1024, conf_cm));
       k_comp_matrices<<<dim3(p.S, p.H), 128, staged ? cm_smem : 0, st>>>(U_out, p.T, p.dh, p.g, p.S, staged ? 1 : 0);
       TB_LAUNCH_CHECK();
     }
@@ -1417,9 +1484,11 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     const int nrem = p.dh - i0 - p.g;
     if (!p.has_hout || nrem <= 0) continue;
     PhaseScope ph_comp(PH_COMP, st);
-    k_residual<<<ew_blocks((long long)M * d), 256, 0, st>>>(p.Wt, codes, p.sD, zeros, p.E, rm, M, d,
-                                                            p.seg, p.ng);
-    TB_LAUNCH_CHECK();
+    if (with_r) {
+      k_residual<<<ew_blocks((long long)M * d), 256, 0, st>>>(p.Wt, codes, p.sD, zeros, p.E, rm, M, d,
+                                                              p.seg, p.ng);
+      TB_LAUNCH_CHECK();
+    }
     if (p.c_max) {
       // E <- E - W0 (R H_in^{-1})   (Proposition 3.2), a double-precision product on the integer tensor cores.  It
       // feeds the codes.  Two projections, three steps each of 1024 rows x 4096 columns,
@@ -1463,28 +1532,15 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
       g.beta = 1.0;
       TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
     }
-    {
-      // W~[rem rows of every head] -= T_i E   (Propositions 3.1 / 3.2; Algorithm 1, update step)
-      GemmP g = gemm_params();
-      g.A = p.T + (long long)step * p.dh * p.g;
-      g.a_m = p.g;
-      g.a_k = 1;
-      g.a_batch = (long long)p.S * p.dh * p.g;
-      g.B = p.E;
-      g.b_k = d;
-      g.b_n = 1;
-      g.b_batch = (long long)p.g * d;
-      g.C = p.Wt + (long long)(i0 + p.g) * d;
-      g.ldc = d;
-      g.c_batch = (long long)p.dh * d;
-      g.M = nrem;
-      g.N = d;
-      g.K = p.g;
-      g.n_batch = p.H;
-      g.alpha = -1.0;
-      g.beta = 1.0;
-      TB_TRY((gemm_launch<double, double, double, double, false, true>(g, st)));
-    }
+    if (p.H > 65535) return TB_ERR_UNSUPPORTED;
+    const dim3 cgrid(d / 128, p.H, (nrem + 31) / 32);
+    const double* Ti = p.T + (long long)step * p.dh * p.g;
+    const long long t_head = (long long)p.S * p.dh * p.g;
+    if (with_r)
+      k_compensate<true><<<cgrid, 256, 0, st>>>(p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng);
+    else
+      k_compensate<false><<<cgrid, 256, 0, st>>>(p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng);
+    TB_LAUNCH_CHECK();
   }
 
   // A group's rows are never written after they have been taken, and the rows of later groups only by
@@ -1574,6 +1630,20 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
         // rows of a head are coupled through H_out: one CTA per head walks them in order
         const int heads_b = (int)(rows / p.dh);
         const long long nb_el = rows * d;
+        CdGram cg_p;
+        if (p.gram) {
+          cg_p.Yw = p.Yw;
+          cg_p.yw_float = p.yw_tensor;
+          cg_p.Wb = p.Wb + r0 * d;
+          cg_p.Hout = H_out + (r0 / p.dh) * (long long)p.dh * p.dh;
+          cg_p.scratch = p.gram;
+          cg_p.heads = heads_b;
+          cg_p.d = d;
+          cg_p.seg = p.seg;
+          cg_p.ng = p.ng;
+          cg_p.dh = p.dh;
+          TB_TRY(cd_gram_form(cg_p, st));
+        }
         CdHeadP hp;
         hp.G = p.Wt + r0 * d;      // W~ is no longer needed: its buffer holds G = H_out Dm
         hp.Uacc = p.Dq + r0 * d;   // (Q - W) has been consumed by the product above
@@ -1593,7 +1663,7 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
         const int n_units = (p.ng / csize) * (p.seg / hp.uw);
         const size_t sm_head =
             ((size_t)n_units * (p.ng + 1) + 2 * (size_t)p.ng * p.ng + 3 * (size_t)p.ng) * sizeof(double);
-        if (sm_head > 200 * 1024) return TB_ERR_UNSUPPORTED;
+        if (!p.gram && sm_head > 200 * 1024) return TB_ERR_UNSUPPORTED;
         static bool conf_head[64] = {false}, conf_head2[64] = {false};
         auto cd_head_kern = p.yw_tensor ? k_cd_head<float> : k_cd_head<double>;
         if (p.yw_tensor)
@@ -1617,7 +1687,7 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
         cp2.ng = p.ng;
         cp2.dh = p.dh;
         cp2.csize = csize;
-        if (by_cols) {
+        if (by_cols && !p.gram) {
           if (p.yw_tensor)
             k_cd_amat<float><<<(unsigned)rows, 256, (size_t)d * sizeof(float), st>>>(p.Yw, hp.Wb, p.Amat, d, p.seg, p.ng);
           else
@@ -1642,6 +1712,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
           g.K = p.dh;
           g.n_batch = heads_b;
           TB_TRY((gemm_launch<float, double, double, double, false, true>(g, st)));
+          if (p.gram) {
+            TB_TRY(cd_gram_pass(cg_p, hp.G, p.Dm + r0 * d, hp.sD, st));
+            continue;
+          }
           cudaLaunchConfig_t cfg = {};
           cfg.gridDim = dim3((unsigned)(heads_b * csize));
           cfg.blockDim = dim3(by_cols ? CDC_THREADS : CDH_THREADS);

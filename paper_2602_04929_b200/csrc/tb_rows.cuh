@@ -68,6 +68,21 @@ tb_status sweep_prepare(const float* U, const float* P, int d, int units, const 
 // a.src: the weights (mapped); a.Err, a.Arr, blk0, blk1 and the like are set here
 tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st);
 
+// Scale refinement of heads with few coordinates (d_head x groups) as a triangular solve (tb_cd_gram.cu).
+enum { CD_GRAM_MAX = 2048 };
+struct CdGram {
+  const void* Yw;      // [heads dh][ng][d], float or double
+  bool yw_float;
+  const float* Wb;     // [heads dh][d]
+  const float* Hout;   // [heads][dh][dh]
+  double* scratch;     // cd_gram_doubles
+  int heads, d, seg, ng, dh;
+};
+bool cd_gram_pays(int dh, int ng);
+size_t cd_gram_doubles(int heads, int dh, int ng);
+tb_status cd_gram_form(const CdGram& p, cudaStream_t st);
+tb_status cd_gram_pass(const CdGram& p, const double* G, double* Dm, double* sD, cudaStream_t st);
+
 // The search for column groups wider than 128 columns (tb_grid_wide.cu).  scratch: grid_wide_doubles() doubles
 // for a chunk of rows; with less, the rows go through in several chunks.
 size_t grid_wide_row_doubles(int d, int ng, int ncp);  // doubles of scratch per row
