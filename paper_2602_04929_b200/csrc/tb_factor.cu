@@ -524,7 +524,11 @@ using namespace tb;
 
 extern "C" size_t tb_factor_workspace(int n_batch, int d) {
   if (n_batch <= 0 || d <= 0) return 0;
-  return factor_ws(n_batch, d, nullptr).total;
+  // never less than two matrices in double, the bound that callers' arenas go by (one place fewer is in use since
+  // L^-1 takes the place of L)
+  const size_t two = ((size_t)2 * n_batch * d * d * sizeof(double) / 256 + 1) * 256;
+  const size_t total = factor_ws(n_batch, d, nullptr).total;
+  return total > two ? total : two;
 }
 
 extern "C" tb_status tb_factor(const float* H, int n_batch, int d, float* U, float* Hinv, int* info,
