@@ -133,11 +133,17 @@ def _ptr(t, dtype=None, allow_none=False):
         raise ValueError("tensors must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise ValueError(f"expected {dtype}, got {t.dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()   # a plain integer: the argument types declared above make it a pointer
+
+
+_current_device, _raw_stream = torch.cuda.current_device, getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream's handle (without building a torch Stream object around it, where torch allows)."""
+    if _raw_stream is not None:
+        return _raw_stream(_current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _workspace(nbytes: int, device) -> torch.Tensor:
@@ -357,7 +363,7 @@ def projection_job(desc: LayerDesc, W, H_in, U_in, H_out, U_out, R, P, C, out: "
 
     def v(t, dt=None):
         q = _ptr(t, dt, True)
-        return None if q is None else q.value
+        return q
 
     return ProjectionJob(desc, v(W, f32), v(H_in, f32), v(U_in, f32), v(H_out, f32), v(U_out, f32), v(R, f32), v(P, f32),
                          v(C, f32), v(out.codes), v(out.scales), v(out.zeros), v(out.cand), v(out.w_hat),
@@ -447,10 +453,9 @@ PHASES = ("setup", "grid", "sweep", "compensation", "cd", "output", "loss",
 def tb_pack_codes(codes, bits: int):
     """codes [d_out, d_in] uint8 -> packed int32 [d_out, d_in * bits / 32] (bit stream per row)."""
     d_out, d_in = codes.shape
-    nbytes = int(load().tb_packed_bytes(d_out, d_in, bits))
-    if nbytes == 0:
+    if d_out <= 0 or d_in <= 0 or d_in % 32 or not 2 <= bits <= 8:   # where tb_packed_bytes is 0
         raise ValueError("unsupported shape or bit width for packing")
-    packed = torch.empty((d_out, nbytes // (4 * d_out)), dtype=torch.int32, device=codes.device)
+    packed = torch.empty((d_out, d_in // 32 * bits), dtype=torch.int32, device=codes.device)
     _check(load().tb_pack_codes(_ptr(codes, torch.uint8), d_out, d_in, bits, _ptr(packed), _stream()), "tb_pack_codes")
     return packed
 
