@@ -1,4 +1,5 @@
-// Grid search for column groups wider than 128 columns (one scale per row, or groups of 256 and more).
+// Grid search for column groups wider than 128 columns (one scale per row, or groups of 256 and more), few rows (with
+// many rows: tb_grid_digits.cu).
 //
 // For every (row, group): n_cand clipped min-max grids, p_k = 1 - k/32, score e H_in[G,G] e^T with e the
 // round-to-nearest error on that grid, lowest score wins, lowest k on ties.  H_in[G,G] is symmetric, so
@@ -15,6 +16,7 @@
 // a 1664-wide layer with one scale per row (6656 rows) 99.9 ms before, 16.2 ms now (0.49 of the FP64
 // rate); 32 searches of 8 rows x 256 columns 3.44 ms before, 0.67 ms now.
 #include "tb_gemm.cuh"
+#include "tb_grid.cuh"
 #include "tb_rows.cuh"
 
 namespace tb {
@@ -30,15 +32,6 @@ struct GwSmem {  // CR candidate rows x CR columns
   double part[8][CR];
   long long src[CR];  // element offset of the candidate's row in W~, or -1
 };
-
-__device__ __forceinline__ double gw_error(double w, double s, double rs, double z, int maxq) {
-  // the fused multiply-add into z + 1.5 * 2^52 rounds to nearest-even and leaves the integer in the low
-  // word (|w / s + z| < 2^31), where the clamp is two integer instructions
-  const double magic = 6755399441055744.0;
-  int n = __double2loint(fma(w, rs, z + magic));
-  n = min(max(n, 0), maxq);
-  return w - s * ((__hiloint2double(0x43380000, n) - magic) - z);
-}
 
 __global__ void __launch_bounds__(256) k_row_range(GridP p, int m0, double2* range) {
   __shared__ double smn[8], smx[8];
@@ -67,18 +60,6 @@ __global__ void __launch_bounds__(256) k_row_range(GridP p, int m0, double2* ran
     }
     range[(long long)blockIdx.y * p.ng + grp] = make_double2(mn, mx);
   }
-}
-
-__device__ __forceinline__ void gw_candidate(double2 mnmx, int k, int maxq, double* s_out, double* z_out) {
-  const double pk = 1.0 - (double)k / 32.0;
-  const double lo = pk * mnmx.x, hi = pk * mnmx.y;
-  double s = 1.0, z = 0.0;
-  if (hi != lo) {
-    s = (hi - lo) / (double)maxq;
-    z = fmin(fmax(rne(-lo / s), 0.0), (double)maxq);
-  }
-  *s_out = s;
-  *z_out = z;
 }
 
 // Candidate rows: row m of the chunk and candidate k at m * ncp + k; tiles never cross units (rows of one H_in).

@@ -107,7 +107,7 @@ __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restri
 // Grid search (Algorithm 1, grid step).  For every (row, column group): n_cand
 // clipped min-max grids, p_k = 1 - k/32; score e H_in[G,G] e^T with e the
 // round-to-nearest error on that grid; the lowest score wins, lowest k on ties.
-// Groups wider than 128 columns: tb_grid_wide.cu.  Here the search
+// Groups wider than 128 columns: tb_grid_wide.cu; many rows: tb_grid_digits.cu.  Here the search
 // for groups of at most 128 columns, where the whole problem of a CTA (128
 // candidate rows x one group) fits shared memory.  One CTA takes RT = 128 / NCP
 // rows (NCP = n_cand rounded up to a power of two) of one column group:
@@ -1074,6 +1074,8 @@ struct Plan {
   double *Wt, *Wk, *W0c, *E, *sD, *T, *Dq, *Dm, *Yw, *n0, *Amat, *G2;
   double* gram;  // scale refinement as a triangular solve: the heads' matrices
   SweepScratch sweep;
+  bool grid_digits;  // the search on the integer tensor cores, with
+  GridDigits gd;
   I8Mat Cdig, Wdig;                // digits of C (all steps) and of the step's W0 (propagated error, one shared H_in)
   unsigned long long *c_max, *w_max;
   float* Wb;
@@ -1154,6 +1156,11 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
     p.Wdig.data = b.take<unsigned char>(i8_bytes(p.Wdig.row_blocks, p.Wdig.k_blocks));
     p.c_max = b.take<unsigned long long>(dd);
     p.w_max = b.take<unsigned long long>((size_t)p.Mmax);
+  }
+  {  // the search of a fixed grid takes all rows at once, the adaptive one a step's
+    const int units = (p.n_hin == 1) ? 1 : p.H, rows = p.adaptive ? p.Mmax : p.d_out;
+    p.grid_digits = !p.dynamic && grid_wants_digits(rows, units, p.d, p.seg, p.ncp);
+    if (p.grid_digits) grid_digits_scratch(b, rows, units, p.d, p.seg, p.ncp, p.bits, &p.gd);
   }
   p.sD = b.take<double>((size_t)p.d_out * p.ng);
   p.T = (has_hout && p.S > 1) ? b.take<double>((size_t)p.H * p.S * p.dh * p.g) : nullptr;
@@ -1241,6 +1248,7 @@ static tb_status run_grid(const Plan& p, const float* H_in, float* scales, int* 
   gp.tiles_per_unit = (gp.rows_per_unit + p.rt - 1) / p.rt;
   gp.Wloc = nullptr;
   gp.grp0 = 0;
+  if (p.grid_digits) return grid_digits(gp, p.gd, st);
   if (p.seg > 128)  // E is free until the sweep of a step
     return grid_wide(gp, p.E, (size_t)p.Mmax * p.d, st);
   static bool configured_tri[64] = {false};
@@ -1455,6 +1463,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
   if (!p.dynamic) {
     PhaseScope ph(PH_SWEEP, st);
     TB_TRY(sweep_prepare(U_in, P, d, (p.n_hin == 1) ? 1 : p.H, p.sweep, st));
+  }
+  if (p.grid_digits) {
+    PhaseScope ph(PH_GRID, st);
+    TB_TRY(grid_digits_prepare(H_in, (p.n_hin == 1) ? 1 : p.H, d, p.seg, p.gd, st));
   }
   if (!p.adaptive && !p.dynamic) {
     // fixed grid: every row, once, from the original weights

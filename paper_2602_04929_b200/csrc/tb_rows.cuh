@@ -88,4 +88,17 @@ tb_status cd_gram_pass(const CdGram& p, const double* G, double* Dm, double* sD,
 size_t grid_wide_row_doubles(int d, int ng, int ncp);  // doubles of scratch per row
 tb_status grid_wide(const GridP& p, double* scratch, size_t scratch_doubles, cudaStream_t st);
 
+// The search with many rows, any group width, on the integer tensor cores (tb_grid_digits.cu).
+struct GridDigits {
+  int rows;              // rows per chunk
+  unsigned char *A, *B;  // integers of the candidates, digits of H_in (one set for all steps)
+  double *h, *r, *range, *lin, *part;
+  unsigned int* hmax;
+  int* list;
+};
+bool grid_wants_digits(int M, int units, int d, int seg, int ncp);
+void grid_digits_scratch(Bump& b, int M, int units, int d, int seg, int ncp, int bits, GridDigits* s);
+tb_status grid_digits_prepare(const float* H, int units, int d, int seg, const GridDigits& s, cudaStream_t st);
+tb_status grid_digits(const GridP& p, const GridDigits& s, cudaStream_t st);
+
 }  // namespace tb
