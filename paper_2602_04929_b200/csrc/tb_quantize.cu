@@ -310,98 +310,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_grid_tri(GridP p) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Dynamic-grid variant of the sweep (the grid of a column group is searched when
-// the sweep arrives at the group, from the group's current values).  Right-looking,
-// one column group at a time on a contiguous working copy Wk [M][d] of the step's
-// rows: k_grid_tri on the group's current values, this kernel for the group's
-// columns (Algorithm 2's column loop restricted to the group: one warp per row, a
-// lane per column of each 32-column sub-block, values in registers), then one GEMM
-// that applies the group's errors (and, with R, its arrival values) to all later
-// columns.  The group's errors only live until that GEMM has run.
-// ---------------------------------------------------------------------------
-struct GroupPanelP {
-  double* Wk;            // [M][d] working values of the step's rows
-  const float* U;        // [n_hin][d][d]
-  const float* P;        // or nullptr
-  double* Err;           // [M][seg] normalised errors of this group
-  double* Arr;           // [M][seg] arrival values of this group (with P)
-  unsigned char* codes;  // [d_out][d]
-  const double* sD;      // [d_out][ng]
-  const int* z;          // [d_out][ng]
-  tb_stats* stats;
-  RowMap rm;
-  int M, d, seg, ng, maxq, grp;
-  int units, rows_per_unit, ctas_per_unit;
-};
-
-__global__ void __launch_bounds__(256) k_group_panel(GroupPanelP p) {
-  extern __shared__ float gp_sm[];   // U[c0 + j][c0 + c] at gp_sm[j * seg + c], then P likewise
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int seg = p.seg, d = p.d, c0 = p.grp * seg, nsb = seg / 32;
-  // a CTA takes 8 rows of one unit (rows that share an H_in / U_in); the last CTA of a unit may hold fewer
-  const int unit = blockIdx.x / p.ctas_per_unit;
-  const int m0 = unit * p.rows_per_unit + (blockIdx.x % p.ctas_per_unit) * 8;
-  const long long uoff = (p.units > 1) ? (long long)unit * d * d : 0;
-  const float* U = p.U + uoff;
-  const float* Pm = p.P ? p.P + uoff : nullptr;
-  float* sU = gp_sm;
-  float* sP = gp_sm + seg * seg;
-  for (int i = tid; i < seg * seg; i += blockDim.x) {
-    const int j = i / seg, c = i % seg;
-    sU[i] = (c >= j) ? U[(long long)(c0 + j) * d + c0 + c] : 0.0f;
-    if (Pm) sP[i] = (c > j) ? Pm[(long long)(c0 + j) * d + c0 + c] : 0.0f;
-  }
-  __syncthreads();
-  const int m = m0 + warp;
-  if (m >= (unit + 1) * p.rows_per_unit) return;
-  const long long grow = p.rm.row(m);
-  const double s = p.sD[grow * p.ng + p.grp];
-  const double zz = (double)p.z[grow * p.ng + p.grp];
-  const double maxq = (double)p.maxq;
-  double* wrow = p.Wk + (long long)m * d + c0;
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-  for (int t = 0; t < 4; ++t)
-    if (t < nsb) v[t] = wrow[t * 32 + lane];
-  unsigned int n_near = 0, n_clamp = 0;
-  for (int j = 0; j < seg; ++j) {
-    const int tj = j >> 5, lj = j & 31;
-    const double mine = (tj == 0) ? v[0] : (tj == 1) ? v[1] : (tj == 2) ? v[2] : v[3];
-    const double wj = shfl_d(mine, lj);   // value of column j on arrival
-    const double x = wj / s + zz;
-    const double q = fmin(fmax(rne(x), 0.0), maxq);
-    const double ej = (wj - s * (q - zz)) / (double)sU[j * seg + j];
-    if (lane == lj) {
-      p.codes[grow * d + c0 + j] = (unsigned char)(int)q;
-      p.Err[(long long)m * seg + j] = ej;
-      if (Pm) p.Arr[(long long)m * seg + j] = wj;
-      const double fl = floor(x);
-      const double a0 = fmin(fmax(fl, 0.0), maxq), a1 = fmin(fmax(fl + 1.0, 0.0), maxq);
-      if (fabs(x - (fl + 0.5)) < 1e-6 && a0 != a1) ++n_near;
-      if (rne(x) != q) ++n_clamp;
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int c = t * 32 + lane;
-      if (t < nsb && c > j) {
-        double nv = fma(-ej, (double)sU[j * seg + c], v[t]);
-        if (Pm) nv = fma(-wj, (double)sP[j * seg + c], nv);
-        v[t] = nv;
-      }
-    }
-  }
-  if (p.stats) {
-    n_near = __reduce_add_sync(0xffffffffu, n_near);
-    n_clamp = __reduce_add_sync(0xffffffffu, n_clamp);
-    if (lane == 0) {
-      if (n_near) atomicAdd(&p.stats->near_tie_codes, (unsigned long long)n_near);
-      if (n_clamp) atomicAdd(&p.stats->clamped_codes, (unsigned long long)n_clamp);
-      if (m == 0) atomicAdd(&p.stats->column_steps, (unsigned long long)seg);
-    }
-  }
-}
-
 // E[m][k] = W~[row(m)][k] - s (code - z): the quantization error of the group on
 // the weights it saw (Proposition 3.1's W_B - Q_B).
 __global__ void k_residual(const double* __restrict__ Wt, const unsigned char* __restrict__ codes,
@@ -1292,7 +1200,6 @@ static tb_status run_sweep_dynamic(const Plan& p, const float* H_in, const float
                                    tb_stats* stats, RowMap rm, int M, cudaStream_t st) {
   const int d = p.d, seg = p.seg;
   const int units = (p.n_hin == 1) ? 1 : p.H;
-  const long long dd = (long long)d * d;
   k_gather<<<ew_blocks((long long)M * d), 256, 0, st>>>(p.Wt, p.Wk, nullptr, rm, M, d);
   TB_LAUNCH_CHECK();
   GridP gp;
@@ -1317,10 +1224,8 @@ static tb_status run_sweep_dynamic(const Plan& p, const float* H_in, const float
   gp.Wloc = p.Wk;
   const long long ytiles = (long long)gp.units * gp.tiles_per_unit;
   if (ytiles > 65535) return TB_ERR_UNSUPPORTED;
-  static bool configured_tri[64] = {false}, configured_panel[64] = {false};
+  static bool configured_tri[64] = {false};
   TB_TRY(allow_smem(k_grid_tri, GRID_TRI_SMEM, configured_tri));
-  const size_t panel_smem = (size_t)seg * seg * sizeof(float) * (P ? 2 : 1);
-  TB_TRY(allow_smem(k_group_panel, 2 * 128 * 128 * sizeof(float), configured_panel));
   GroupPanelP pp;
   pp.Wk = p.Wk;
   pp.U = U_in;
@@ -1339,41 +1244,12 @@ static tb_status run_sweep_dynamic(const Plan& p, const float* H_in, const float
   pp.maxq = p.maxq;
   pp.units = units;
   pp.rows_per_unit = M / units;
-  pp.ctas_per_unit = (pp.rows_per_unit + 7) / 8;
   for (int grp = 0; grp < p.ng; ++grp) {
-    const int c0 = grp * seg, c1 = c0 + seg;
     gp.grp0 = grp;
     k_grid_tri<<<dim3(1, (unsigned)ytiles), GEMM_THREADS, GRID_TRI_SMEM, st>>>(gp);
     TB_LAUNCH_CHECK();
     pp.grp = grp;
-    k_group_panel<<<(unsigned)(pp.ctas_per_unit * units), 256, panel_smem, st>>>(pp);
-    TB_LAUNCH_CHECK();
-    if (c1 >= d) break;
-    // Wk[:, c1:] -= Err U[c0:c1, c1:]  (- Arr P[c0:c1, c1:])
-    GemmP g = gemm_params();
-    g.A = p.dynErr;
-    g.a_m = seg;
-    g.a_k = 1;
-    g.a_batch = (long long)pp.rows_per_unit * seg;
-    g.B = U_in + (long long)c0 * d + c1;
-    g.b_k = d;
-    g.b_n = 1;
-    g.b_batch = (units > 1) ? dd : 0;
-    g.C = p.Wk + c1;
-    g.ldc = d;
-    g.c_batch = (long long)pp.rows_per_unit * d;
-    g.M = pp.rows_per_unit;
-    g.N = d - c1;
-    g.K = seg;
-    g.n_batch = units;
-    g.alpha = -1.0;
-    g.beta = 1.0;
-    TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
-    if (P) {
-      g.A = p.dynArr;
-      g.B = P + (long long)c0 * d + c1;
-      TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
-    }
+    TB_TRY(group_panel(pp, st));
   }
   return TB_OK;
 }

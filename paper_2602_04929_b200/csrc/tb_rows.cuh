@@ -68,6 +68,26 @@ tb_status sweep_prepare(const float* U, const float* P, int d, int units, const 
 // a.src: the weights (mapped); a.Err, a.Arr, blk0, blk1 and the like are set here
 tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st);
 
+// Dynamic-grid variant of the sweep (the grid of a column group is searched when the sweep arrives at the group, from the
+// group's current values).  Right-looking, one column group of up to 128 columns at a time on a contiguous working copy of
+// the step's rows: the search, then group_panel: Algorithm 2's column loop restricted to the group, and the rank-seg
+// update of every column right of it.
+struct GroupPanelP {
+  double* Wk;            // [M][d] working copy of the step's rows
+  const float* U;        // [n_hin][d][d]
+  const float* P;        // or nullptr
+  double* Err;           // [M][seg] normalised errors of this group
+  double* Arr;           // [M][seg] arrival values of this group (with P)
+  unsigned char* codes;  // [d_out][d]
+  const double* sD;      // [d_out][ng]
+  const int* z;          // [d_out][ng]
+  tb_stats* stats;
+  RowMap rm;
+  int M, d, seg, ng, maxq, grp;
+  int units, rows_per_unit;
+};
+tb_status group_panel(const GroupPanelP& p, cudaStream_t st);
+
 // Scale refinement of heads with few coordinates (d_head x groups) as a triangular solve (tb_cd_gram.cu).
 enum { CD_GRAM_MAX = 2048 };
 struct CdGram {

@@ -989,4 +989,230 @@ tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st) {
   return TB_OK;
 }
 
+// ---------------------------------------------------------------------------
+// One column group of the dynamic-grid sweep: 8 rows of a unit per CTA, the group's factor rows in shared memory.  The
+// chain is the sweep's (a thread per row, 16 columns at a time); after a piece all warps apply its errors to the group's
+// later columns by FP64 tensor steps, and while the next piece is walked they write the piece's outputs (not the warp
+// that shares the chain's scheduler).  Bound by the chain's latency.  1152 rows, group of 64: 8.9 us; a warp per row with
+// two divisions and a broadcast per column, as it was, 32.6.
+// ---------------------------------------------------------------------------
+template <bool WITH_P>
+struct PanelSmem {
+  alignas(16) double w[8][SW_LDW], Es[8][SW_LDW], As[WITH_P ? 8 : 1][SW_LDW];
+  alignas(16) double cU[8][16][16], cP[WITH_P ? 8 : 1][16][16];
+  alignas(16) double rd[128];
+  double gs[8][3];
+  float U[128][SW_LDB], P[WITH_P ? 128 : 1][SW_LDB];
+};
+
+template <bool WITH_P>
+__global__ void __launch_bounds__(256) k_group_panel(GroupPanelP p, int ctas_per_unit) {
+  extern __shared__ __align__(16) unsigned char gp_raw[];
+  PanelSmem<WITH_P>& sm = *reinterpret_cast<PanelSmem<WITH_P>*>(gp_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, fr = lane >> 2, fk = lane & 3;
+  const int seg = p.seg, d = p.d, c0 = p.grp * seg;
+  const int unit = blockIdx.x / ctas_per_unit, r_first = (blockIdx.x % ctas_per_unit) * 8;
+  const int rows = min(8, p.rows_per_unit - r_first), m0 = unit * p.rows_per_unit + r_first;
+  const long long uoff = ((p.units > 1) ? (long long)unit * d * d : 0) + (long long)c0 * (d + 1);
+  for (int i = tid; i < seg * seg / 4; i += 256) {
+    const int j = i / (seg / 4), c = 4 * (i % (seg / 4));
+    if (c + 3 >= j) {  // the strictly lower triangle is not read
+      *reinterpret_cast<float4*>(&sm.U[j][c]) = *reinterpret_cast<const float4*>(p.U + uoff + (long long)j * d + c);
+      if (WITH_P) *reinterpret_cast<float4*>(&sm.P[j][c]) = *reinterpret_cast<const float4*>(p.P + uoff + (long long)j * d + c);
+    }
+  }
+  for (int i = tid; i < 8 * seg; i += 256) {
+    const int r = i / seg, c = i % seg;
+    sm.w[r][c] = (r < rows) ? p.Wk[(long long)(m0 + r) * d + c0 + c] : 0.0;
+  }
+  if (tid < 8) {
+    double s = 1.0, z = 0.0;
+    if (tid < rows) {
+      const long long so = p.rm.row(m0 + tid) * p.ng + p.grp;
+      s = p.sD[so];
+      z = (double)p.z[so];
+    }
+    sm.gs[tid][0] = s;
+    sm.gs[tid][1] = 1.0 / s;
+    sm.gs[tid][2] = z;
+  }
+  __syncthreads();
+  if (tid < seg) sm.rd[tid] = 1.0 / (double)sm.U[tid][tid];
+  __syncthreads();
+  for (int i = tid; i < seg * 16; i += 256) {
+    const int j = i >> 4, c = i & 15, jl = j & 15, cc = (j & ~15) + c;
+    sm.cU[j >> 4][jl][c] = (c > jl) ? (double)sm.U[j][cc] * sm.rd[j] : 0.0;
+    if (WITH_P) sm.cP[WITH_P ? j >> 4 : 0][jl][c] = (c > jl) ? (double)sm.P[WITH_P ? j : 0][cc] : 0.0;
+  }
+  unsigned int n_near = 0, n_clamp = 0;
+  auto outputs = [&](int sb, int t, int nt) {  // codes, errors and counters of a piece
+    for (int i = t; i < 128; i += nt) {
+      const int r = i >> 4, cl = 16 * sb + (i & 15);
+      if (r < rows) {
+        const double z = sm.gs[r][2], maxq = (double)p.maxq;
+        const double v = sm.w[r][cl], x = v + z, xm = v + (z + 6755399441055744.0);  // the chain's own operations
+        const double xr = xm - 6755399441055744.0;
+        int unused = 0;
+        const double q = sw_quant<true>(xm, p.maxq, unused);
+        p.codes[p.rm.row(m0 + r) * d + c0 + cl] = (unsigned char)(int)q;
+        p.Err[(long long)(m0 + r) * seg + cl] = sm.Es[r][cl];
+        if (WITH_P) p.Arr[(long long)(m0 + r) * seg + cl] = sm.As[WITH_P ? r : 0][cl];
+        const double fl = floor(x);
+        const double a0 = fmin(fmax(fl, 0.0), maxq), a1 = fmin(fmax(fl + 1.0, 0.0), maxq);
+        if (fabs(x - (fl + 0.5)) < 1e-6 && a0 != a1) ++n_near;
+        if (xr != q) ++n_clamp;
+      }
+    }
+  };
+  for (int sb = 0; sb < seg / 16; ++sb) {
+    __syncthreads();
+    if (warp == 0) {
+      const int r = lane & 7;
+      const double s = sm.gs[r][0], rs = sm.gs[r][1], z = sm.gs[r][2];
+      double* wr = &sm.w[r][16 * sb];
+      double* er = &sm.Es[r][16 * sb];
+      double v[16];
+      auto load = [&]() {
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+          const double2 t = sw_ld2(wr + j);
+          v[j] = t.x * rs;
+          v[j + 1] = t.y * rs;
+        }
+      };
+      load();
+      const int off = sw_walk<WITH_P, false>(v, er, s, z, p.maxq, &sm.rd[16 * sb], sm.cU[sb], sm.cP[WITH_P ? sb : 0]);
+      if (__any_sync(0xffffffffu, off != 0)) {  // again, with the range test in the chain
+        load();
+        sw_walk<WITH_P, true>(v, er, s, z, p.maxq, &sm.rd[16 * sb], sm.cU[sb], sm.cP[WITH_P ? sb : 0]);
+      }
+      __syncwarp();  // (lanes of one row read its values before one of them overwrites them)
+#pragma unroll
+      for (int j = 0; j < 16; j += 2) {
+        sw_st2(wr + j, v[j], v[j + 1]);
+        if (WITH_P) sw_st2(&sm.As[WITH_P ? r : 0][16 * sb + j], v[j] * s, v[j + 1] * s);
+      }
+    } else if (sb > 0 && warp != 4) {
+      outputs(sb - 1, (warp - (warp > 4 ? 2 : 1)) * 32 + lane, 192);
+    }
+    __syncthreads();
+    for (int n = 2 * (sb + 1) + warp; n < seg / 8; n += 8) {
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        sw_mma(acc[q & 1], sm.Es[fr][16 * sb + 4 * q + fk], (double)sm.U[16 * sb + 4 * q + fk][8 * n + fr]);
+      if (WITH_P)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          sw_mma(acc[q & 1], sm.As[WITH_P ? fr : 0][16 * sb + 4 * q + fk],
+                 (double)sm.P[WITH_P ? 16 * sb + 4 * q + fk : 0][8 * n + fr]);
+      double2* wp = reinterpret_cast<double2*>(&sm.w[fr][8 * n + 2 * fk]);
+      const double2 o = *wp;
+      *wp = make_double2(o.x - (acc[0][0] + acc[1][0]), o.y - (acc[0][1] + acc[1][1]));
+    }
+  }
+  outputs(seg / 16 - 1, tid, 256);
+  if (p.stats) {
+    n_near = __reduce_add_sync(0xffffffffu, n_near);
+    n_clamp = __reduce_add_sync(0xffffffffu, n_clamp);
+    if (lane == 0) {
+      if (n_near) atomicAdd(&p.stats->near_tie_codes, (unsigned long long)n_near);
+      if (n_clamp) atomicAdd(&p.stats->clamped_codes, (unsigned long long)n_clamp);
+      if (m0 == 0 && warp == 0) atomicAdd(&p.stats->column_steps, (unsigned long long)seg);
+    }
+  }
+}
+
+// Wk[:, c1 ..] -= Err U[c0 .. c1, c1 ..] (- Arr P): 64 rows x 64 columns per CTA, the contraction (one group, or one group twice)
+// 32 rows at a time, the next ones fetched meanwhile.  8 warps of 32 x 16.  Bound by latency: 141 MFLOP a launch.
+// 1152 x 960 columns, group of 64: 11.5 us (tiles of 128 x 128 19.1).
+__global__ void __launch_bounds__(256, 2) k_group_update(GroupPanelP p) {
+  __shared__ double As[64][36];
+  __shared__ float Bs[32][72];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, fr = lane >> 2, fk = lane & 3;
+  const int d = p.d, seg = p.seg, k_first = p.grp * seg, c0 = k_first + seg + blockIdx.x * 64;
+  const int tiles = (p.rows_per_unit + 63) / 64, unit = blockIdx.y / tiles, r0 = (blockIdx.y % tiles) * 64;
+  const int rows = min(64, p.rows_per_unit - r0), m0 = unit * p.rows_per_unit + r0;
+  const long long uoff = (p.units > 1) ? (long long)unit * d * d : 0;
+  const int wr = (warp >> 2) * 32, wc = (warp & 3) * 16;
+  const int n_k = p.P ? 2 * seg : seg;
+  double acc[4][2][2];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) (&acc[0][0][0])[i] = 0.0;
+  double av[8];
+  float bv[8];
+  auto fetch = [&](int k0) {
+    const bool second = k0 >= seg;
+    const int kk = second ? k0 - seg : k0;
+    const double* E = second ? p.Arr : p.Err;
+    const float* F = (second ? p.P : p.U) + uoff;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int rr = warp + 8 * i, n = tid & 63, k = (tid >> 6) + 4 * i;
+      av[i] = (rr < rows) ? E[(long long)(m0 + rr) * seg + kk + lane] : 0.0;
+      bv[i] = (c0 + n < d) ? F[(long long)(k_first + kk + k) * d + c0 + n] : 0.0f;
+    }
+  };
+  fetch(0);
+  double2 old[4][2];  // the values to be updated, on their way while the product is formed
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int rr = wr + 8 * i + fr, n = c0 + wc + 8 * j + 2 * fk;
+      old[i][j] = (rr < rows && n < d) ? *reinterpret_cast<const double2*>(p.Wk + (long long)(m0 + rr) * d + n) : make_double2(0.0, 0.0);
+    }
+  for (int k0 = 0; k0 < n_k; k0 += 32) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      As[warp + 8 * i][lane] = av[i];
+      Bs[(tid >> 6) + 4 * i][tid & 63] = bv[i];
+    }
+    __syncthreads();
+    if (k0 + 32 < n_k) fetch(k0 + 32);
+#pragma unroll
+    for (int k4 = 0; k4 < 8; ++k4) {
+      double a[4], b[2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = As[wr + 8 * i + fr][4 * k4 + fk];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) b[j] = (double)Bs[4 * k4 + fk][wc + 8 * j + fr];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) sw_mma(acc[i][j], a[i], b[j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int rr = wr + 8 * i + fr, n = c0 + wc + 8 * j + 2 * fk;
+      if (rr < rows && n < d)
+        *reinterpret_cast<double2*>(p.Wk + (long long)(m0 + rr) * d + n) =
+            make_double2(old[i][j].x - acc[i][j][0], old[i][j].y - acc[i][j][1]);
+    }
+}
+
+tb_status group_panel(const GroupPanelP& p, cudaStream_t st) {
+  static bool conf[64] = {false}, conf_p[64] = {false};
+  const int ctas = (p.rows_per_unit + 7) / 8, tiles = (p.rows_per_unit + 63) / 64;
+  if ((long long)tiles * p.units > 65535) return TB_ERR_UNSUPPORTED;
+  if (p.P) {
+    TB_TRY(allow_smem(k_group_panel<true>, sizeof(PanelSmem<true>), conf_p));
+    k_group_panel<true><<<(unsigned)(ctas * p.units), 256, sizeof(PanelSmem<true>), st>>>(p, ctas);
+  } else {
+    TB_TRY(allow_smem(k_group_panel<false>, sizeof(PanelSmem<false>), conf));
+    k_group_panel<false><<<(unsigned)(ctas * p.units), 256, sizeof(PanelSmem<false>), st>>>(p, ctas);
+  }
+  TB_LAUNCH_CHECK();
+  const int right = p.d - (p.grp + 1) * p.seg;
+  if (right > 0) {
+    k_group_update<<<dim3((right + 63) / 64, tiles * p.units), 256, 0, st>>>(p);
+    TB_LAUNCH_CHECK();
+  }
+  return TB_OK;
+}
+
 }  // namespace tb
