@@ -111,13 +111,90 @@ __global__ void __launch_bounds__(256) k_damp_diagonal(float* __restrict__ H,
   }
 }
 
-// H_out[h] = combination of the per-block Grams, plus damp * mean(diag) on the diagonal.
-__global__ void __launch_bounds__(256) k_combine_hout(float* __restrict__ Hout,
-                                                      const double* __restrict__ blocks,
-                                                      int n_heads, int g_heads, int dh, double damp) {
-  __shared__ double part[256];
+// Grams of blocks of rows, C_b = A_b G_b^T (A: G Hsum in double, or G itself): a CTA takes 64 x 64 entries of one block and a
+// part of the contraction, 32 steps at a time, the next ones fetched meanwhile; 8 warps of 32 x 16, FP64 tensor steps.
+// The parts (hout_parts) are there because the blocks alone do not fill the SMs: 32 blocks of 128 x 128 over 4096 columns
+// took 0.70 ms in one tile each, under 0.25 ms here (0.12 at the FP64 pipe's rate).
+template <typename TA>
+__global__ void __launch_bounds__(256, 3) k_block_gram(const TA* __restrict__ A, const float* __restrict__ G, double* __restrict__ C,
+                                                       int dh, int d, int g_heads) {
+  __shared__ double As[64][36];
+  __shared__ float Bs[64][36];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, fr = lane >> 2, fk = lane & 3;
+  const int tiles = (dh + 63) / 64, block = blockIdx.x / (tiles * tiles), tile = blockIdx.x % (tiles * tiles);
+  const int m0 = (tile / tiles) * 64, n0 = (tile % tiles) * 64, part = blockIdx.y, parts = gridDim.y;
+  const int steps = (d + 31) / 32, k_lo = (int)((long long)steps * part / parts) * 32,
+            k_hi = min(d, (int)((long long)steps * (part + 1) / parts) * 32);
+  const TA* Ab = A + (long long)block * dh * d;
+  const float* Gb = G + (long long)block * dh * d;
+  const int wr = (warp >> 2) * 32, wc = (warp & 3) * 16;
+  double acc[4][2][2];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) (&acc[0][0][0])[i] = 0.0;
+  TA av[8];
+  float bv[8];
+  auto fetch = [&](int k0) {
+    const int k = k0 + lane;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = warp + 8 * i;
+      av[i] = (m0 + r < dh && k < k_hi) ? Ab[(long long)(m0 + r) * d + k] : (TA)0;
+      bv[i] = (n0 + r < dh && k < k_hi) ? Gb[(long long)(n0 + r) * d + k] : 0.0f;
+    }
+  };
+  fetch(k_lo);
+  for (int k0 = k_lo; k0 < k_hi; k0 += 32) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      As[warp + 8 * i][lane] = (double)av[i];
+      Bs[warp + 8 * i][lane] = bv[i];
+    }
+    __syncthreads();
+    if (k0 + 32 < k_hi) fetch(k0 + 32);
+#pragma unroll
+    for (int k4 = 0; k4 < 8; ++k4) {
+      double a[4], b[2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = As[wr + 8 * i + fr][4 * k4 + fk];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) b[j] = (double)Bs[wc + 8 * j + fr][4 * k4 + fk];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+                       : "+d"(acc[i][j][0]), "+d"(acc[i][j][1])
+                       : "d"(a[i]), "d"(b[j]));
+    }
+  }
+  double* Cb = C + ((long long)part * g_heads + block) * dh * dh;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int m = m0 + wr + 8 * i + fr, n = n0 + wc + 8 * j + 2 * fk + e;
+        if (m < dh && n < dh) Cb[(long long)m * dh + n] = acc[i][j][e];
+      }
+}
+
+// parts of the contraction: as many CTAs as the SMs hold (three each), at least 256 columns a part
+static int hout_parts(int g_heads, int d_head, int d) {
+  const long long tiles = (d_head + 63) / 64, ctas = tiles * tiles * g_heads;
+  long long s = 444 / ctas;
+  if (s > d / 256) s = d / 256;
+  return s < 1 ? 1 : s > 16 ? 16 : (int)s;
+}
+
+// H_out[h] = combination of the per-block Grams (each the sum of its parts), plus damp * mean(diag) on the diagonal.
+__global__ void __launch_bounds__(1024) k_combine_hout(float* __restrict__ Hout,
+                                                       const double* __restrict__ blocks,
+                                                       int n_heads, int g_heads, int dh, int parts, double damp) {
+  __shared__ double part[1024];
   const int h = blockIdx.x;
-  const long long bb = (long long)dh * dh;
+  const long long bb = (long long)dh * dh, pp = bb * g_heads;
   int b_first, b_count;
   if (g_heads >= n_heads) {
     b_count = g_heads / n_heads;
@@ -126,22 +203,29 @@ __global__ void __launch_bounds__(256) k_combine_hout(float* __restrict__ Hout,
     b_count = 1;
     b_first = h / (n_heads / g_heads);
   }
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < dh; i += 256) {
+  auto entry = [&](long long idx) {
     double v = 0.0;
-    for (int b = 0; b < b_count; ++b) v += blocks[(b_first + b) * bb + (long long)i * dh + i];
-    acc += v;
-  }
+    for (int b = 0; b < b_count; ++b) {
+      const double* t = blocks + (b_first + b) * bb + idx;
+      double s = 0.0;
+#pragma unroll 4
+      for (int q = 0; q < parts; ++q) s += t[q * pp];
+      v += s;
+    }
+    return v;
+  };
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < dh; i += 1024) acc += entry((long long)i * dh + i);
   part[threadIdx.x] = acc;
   __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
+  for (int s = 512; s > 0; s >>= 1) {
     if (threadIdx.x < s) part[threadIdx.x] += part[threadIdx.x + s];
     __syncthreads();
   }
   const double mean = part[0] / (double)dh;
-  for (long long idx = threadIdx.x; idx < bb; idx += 256) {
-    double v = 0.0;
-    for (int b = 0; b < b_count; ++b) v += blocks[(b_first + b) * bb + idx];
+  const long long lo = bb * blockIdx.y / gridDim.y, hi = bb * (blockIdx.y + 1) / gridDim.y;
+  for (long long idx = lo + threadIdx.x; idx < hi; idx += 1024) {
+    double v = entry(idx);
     if (idx / dh == idx % dh) v += damp * mean;
     Hout[h * bb + idx] = (float)v;
   }
@@ -251,7 +335,7 @@ extern "C" size_t tb_build_hout_workspace(int g_heads, int d_head, int d) {
   if (g_heads <= 0 || d_head <= 0 || d <= 0) return 0;
   Bump b(nullptr);
   b.take<double>((size_t)g_heads * d_head * d);       // G Hsum
-  b.take<double>((size_t)g_heads * d_head * d_head);  // per-block Grams
+  b.take<double>((size_t)g_heads * d_head * d_head * hout_parts(g_heads, d_head, d));  // per-block Grams
   if (hout_on_tensor(g_heads * d_head, d)) {
     b.take<__nv_bfloat16>((size_t)3 * g_heads * d_head * d);  // G^T in three bf16 pieces
     b.take<__nv_bfloat16>((size_t)3 * d * d);                 // Hsum in three bf16 pieces
@@ -270,15 +354,14 @@ extern "C" tb_status tb_build_hout(float* H_out, const float* G, const float* Hs
   cudaStream_t st = as_stream(stream);
   Bump b(ws);
   double* T = b.take<double>((size_t)g_heads * d_head * d);
-  double* blocks = b.take<double>((size_t)g_heads * d_head * d_head);
+  const int parts = hout_parts(g_heads, d_head, d);
+  double* blocks = b.take<double>((size_t)g_heads * d_head * d_head * parts);
   const int rows = g_heads * d_head;
-  GemmP q = gemm_params();
   if (Hsum && hout_on_tensor(rows, d)) {
     // T = G Hsum from exact bf16 splits of both operands (float-accurate products, double chunk sums)
     __nv_bfloat16* GT = b.take<__nv_bfloat16>((size_t)3 * rows * d);
     __nv_bfloat16* Hp = b.take<__nv_bfloat16>((size_t)3 * d * d);
     TB_TRY(gemm_split_tensor(T, d, G, Hsum, GT, Hp, rows, d, d, st));
-    q.A = T;
   } else if (Hsum) {
     GemmP g = gemm_params();  // T = G Hsum
     g.A = G;
@@ -293,29 +376,17 @@ extern "C" tb_status tb_build_hout(float* H_out, const float* G, const float* Hs
     g.N = d;
     g.K = d;
     TB_TRY((gemm_launch<float, float, double, double, false, true>(g, st)));
-    q.A = T;  // blocks_b = T_b G_b^T
   }
-  q.a_m = d;
-  q.a_k = 1;
-  q.a_batch = (long long)d_head * d;
-  q.B = G;  // B(k, n) = G_b[n][k]
-  q.b_k = 1;
-  q.b_n = d;
-  q.b_batch = (long long)d_head * d;
-  q.C = blocks;
-  q.ldc = d_head;
-  q.c_batch = (long long)d_head * d_head;
-  q.M = d_head;
-  q.N = d_head;
-  q.K = d;
-  q.n_batch = g_heads;
-  if (Hsum) {
-    TB_TRY((gemm_launch<double, float, double, double, false, false>(q, st)));
-  } else {
-    q.A = G;
-    TB_TRY((gemm_launch<float, float, double, double, false, false>(q, st)));
-  }
-  k_combine_hout<<<n_heads, 256, 0, st>>>(H_out, blocks, n_heads, g_heads, d_head, (double)damp);
+  const int tiles = (d_head + 63) / 64;
+  if ((long long)tiles * tiles * g_heads > 0x7fffffffll) return TB_ERR_UNSUPPORTED;
+  const dim3 grid((unsigned)(tiles * tiles * g_heads), parts);
+  if (Hsum)
+    k_block_gram<double><<<grid, 256, 0, st>>>(T, G, blocks, d_head, d, g_heads);
+  else
+    k_block_gram<float><<<grid, 256, 0, st>>>(G, G, blocks, d_head, d, g_heads);
+  TB_LAUNCH_CHECK();
+  const dim3 cgrid(n_heads, n_heads * 4 <= 592 ? 4 : 1);
+  k_combine_hout<<<cgrid, 1024, 0, st>>>(H_out, blocks, n_heads, g_heads, d_head, parts, (double)damp);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
