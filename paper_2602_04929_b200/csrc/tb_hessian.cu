@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) k_damp_diagonal(float* __restrict__ H,
 // Grams of blocks of rows, C_b = A_b G_b^T (A: G Hsum in double, or G itself): a CTA takes 64 x 64 entries of one block and a
 // part of the contraction, 32 steps at a time, the next ones fetched meanwhile; 8 warps of 32 x 16, FP64 tensor steps.
 // The parts (hout_parts) are there because the blocks alone do not fill the SMs: 32 blocks of 128 x 128 over 4096 columns
-// took 0.70 ms in one tile each, under 0.25 ms here (0.12 at the FP64 pipe's rate).
+// took 0.70 ms in one tile each, 0.18 ms here (0.12 at the FP64 pipe's rate).
 template <typename TA>
 __global__ void __launch_bounds__(256, 3) k_block_gram(const TA* __restrict__ A, const float* __restrict__ G, double* __restrict__ C,
                                                        int dh, int d, int g_heads) {

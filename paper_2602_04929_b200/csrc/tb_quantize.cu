@@ -21,6 +21,7 @@
 #include "tb_i8.cuh"
 #include "tb_profile.cuh"
 #include "tb_rows.cuh"
+#include "tb_tma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -711,14 +712,20 @@ __global__ void __launch_bounds__(CDH_THREADS, 1) k_cd_head(CdHeadP p) {
 // Column-parallel form of the same pass, for up to 32 groups and at most 1024
 // columns per CTA.  The quadratic forms A[g2][g] = Wbar_g2^T H_in[g2, g] Wbar_g
 // of a row depend on the integers only, so k_cd_amat forms them for every row
-// up front, in parallel.  In the walk, thread t owns columns 2t, 2t+1 of its
+// up front, in parallel, and with them the row's whole chain over its groups as one
+// triangular matrix: delta = -M num / hjj.  In the walk, thread t owns columns 2t, 2t+1 of its
 // CTA for the whole pass: the u_i of the current block of 16 rows stay in its
 // registers, the lazily corrected row of G is formed there, and one row costs
-// two block barriers, one cluster barrier and a 32-step chain run in registers
-// by warp 0 of every CTA.  What the next row needs (its row of G, Wbar, A and
-// H_out) is fetched while the current row is processed, and the next row's
-// slice of Yw is pulled into L2.
+// four block barriers, one cluster barrier and a product with M by warp 0 of every CTA.
+// What the next row needs (its row of G, Wbar, M and H_out) is fetched while the current row is
+// processed; its slice of Yw (float: up to 128 KB) is copied into shared memory meanwhile.
+// A row of 32 heads with 32 groups of 128 takes 8 us (18 k clocks: numerators and their exchange 5 k, the product with
+// M 1.5, u 2.7, its float -> double conversions most of it, the fold at a block's end 4.2), of which 2.5 are the HBM time
+// of Yw.  It took 11 when the chain ran group by group (2.7 k clocks), Yw came from L2 (6.7 k) and the fold read
+// H_out entry by entry (5.4 k).  4096 rows: 1.40 -> 1.02 ms, k_cd_chain 0.03.
 // ---------------------------------------------------------------------------
+enum { CDC_THREADS = 512, CDC_MAXG = 32, CDC_FOLD = 64 };
+
 template <typename TY>
 __global__ void __launch_bounds__(256) k_cd_amat(const void* __restrict__ Yw_, const float* __restrict__ Wb,
                                                  double* __restrict__ Amat, int d, int seg, int ng) {
@@ -740,7 +747,30 @@ __global__ void __launch_bounds__(256) k_cd_amat(const void* __restrict__ Yw_, c
     }
 }
 
-enum { CDC_THREADS = 512, CDC_MAXG = 32 };
+// In place, A[g2][g] -> M[g2][g], g2 <= g: with r_g = 1 / A[g][g] (0 for a skipped coordinate), the group-by-group rule
+// n_g -= sum_(g2 < g) A[g2][g] r_g2 n_g2 as a product, n = L num, and M[g2][g] = r_g L[g][g2].  A warp per row, a lane
+// per column of L in registers.  (At the end of k_cd_amat it would cost that kernel its occupancy: 844 us instead of 308.)
+__global__ void __launch_bounds__(128) k_cd_chain(double* __restrict__ Amat, long long rows, int ng) {
+  __shared__ double sA[4][CDC_MAXG][CDC_MAXG];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long row = (long long)blockIdx.x * 4 + warp;
+  if (row >= rows) return;
+  double* A = Amat + row * ng * ng;
+  double(*As)[CDC_MAXG] = sA[warp];
+  for (int g2 = 0; g2 < CDC_MAXG; ++g2) As[g2][lane] = (g2 < ng && lane < ng && g2 <= lane) ? A[g2 * ng + lane] : 0.0;
+  __syncwarp();
+  const double r_mine = (As[lane][lane] == 0.0) ? 0.0 : 1.0 / As[lane][lane];
+  double L[CDC_MAXG];
+#pragma unroll
+  for (int g = 0; g < CDC_MAXG; ++g) {
+    double v[4] = {(g == lane) ? 1.0 : 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int g2 = 0; g2 < g; ++g2) v[g2 & 3] = fma(-As[g2][g], L[g2], v[g2 & 3]);
+    L[g] = __shfl_sync(0xffffffffu, r_mine, g) * ((v[0] + v[1]) + (v[2] + v[3]));
+    if (lane < ng && g < ng) A[lane * ng + g] = L[g];
+  }
+}
+
 __device__ __forceinline__ double2 load_pair(const float* q) {
   const float2 v = *reinterpret_cast<const float2*>(q);
   return make_double2((double)v.x, (double)v.y);
@@ -752,11 +782,22 @@ struct CdColP {
   const void* Yw;      // [heads*dh][ng][d], element type TY of the kernel
   const float* Wb;     // [heads*dh][d]
   const float* Hout;   // [heads][dh][dh]
-  const double* Amat;  // [heads*dh][ng][ng], entries g2 <= g
+  const double* Mmat;  // [heads*dh][ng][ng], of k_cd_chain
   double* sD;          // [heads*dh][ng]
   int d, seg, ng, dh;
   int csize;           // CTAs per cluster (divides ng)
 };
+
+__device__ int g_cd_error = 0;
+int cd_error_read_clear() {
+  int v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_cd_error, sizeof(int)) != cudaSuccess) return -1;
+  if (v) {
+    int z = 0;
+    cudaMemcpyToSymbol(g_cd_error, &z, sizeof(int));
+  }
+  return v;
+}
 
 template <typename TY>
 __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
@@ -764,8 +805,12 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
   __shared__ double Am[2][CDC_MAXG * CDC_MAXG];
   __shared__ double num[2][CDC_MAXG];
   __shared__ double delta[CDC_MAXG];
-  __shared__ float hs[2][CDH_BLOCK];
-  __shared__ float hd[2];
+  __shared__ double hs[CDH_BLOCK][2 * CDH_BLOCK];  // the block's rows of H_out: columns of the block behind as many zeros
+  __shared__ __align__(16) double hf[CDC_FOLD][CDH_BLOCK];  // columns of H_out for the fold
+  __shared__ unsigned long long slab_bar;
+  __shared__ int abort_flag;
+  extern __shared__ __align__(128) unsigned char cdc_slab[];  // float: this CTA's columns of the row's Yw, [ng][c_cnt]
+  constexpr bool STAGED = sizeof(TY) == 4;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = (int)cluster.block_rank();
@@ -781,7 +826,22 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
   const TY* Yw = static_cast<const TY*>(p.Yw);
   const int a_cnt = ng * ng;
   const int half = seg / 2;  // partial sums per group
-  const size_t slab_lines = ((size_t)c_cnt * sizeof(TY) + 127) / 128;
+  const int slab_lines = (c_cnt * (int)sizeof(TY) + 127) / 128;
+  const uint32_t sbar = smem_u32(&slab_bar);
+  if (tid == 0) {
+    mbar_init(sbar, 1);
+    abort_flag = 0;
+    mbar_fence_init();
+  }
+  auto fetch_slab = [&](long long row) {  // one warp, a group per lane
+    if (lane == 0) mbar_expect_tx(sbar, (uint32_t)(ng * c_cnt) * 4u);
+    __syncwarp();
+    if (lane < ng)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       smem_u32(cdc_slab) + (uint32_t)(lane * c_cnt) * 4u),
+                   "l"(Yw + (row * ng + lane) * d + c_lo), "r"((uint32_t)c_cnt * 4u), "r"(sbar)
+                   : "memory");
+  };
 
   // what row 0 needs
   double2 gn = make_double2(0.0, 0.0);
@@ -791,14 +851,18 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
     gn = *reinterpret_cast<const double2*>(p.G + row0 * d + col);
     wn = *reinterpret_cast<const float2*>(p.Wb + row0 * d + col);
   }
-  if (tid < a_cnt) an0 = p.Amat[row0 * a_cnt + tid];
-  if (tid + CDC_THREADS < a_cnt) an1 = p.Amat[row0 * a_cnt + tid + CDC_THREADS];
+  if (tid < a_cnt) an0 = p.Mmat[row0 * a_cnt + tid];
+  if (tid + CDC_THREADS < a_cnt) an1 = p.Mmat[row0 * a_cnt + tid + CDC_THREADS];
   double sdn = (rank == 0 && tid < ng) ? p.sD[row0 * ng + tid] : 0.0;  // the row's scales, fetched one row ahead
-  // hs[.][k] multiplies ureg[k]; the vectors move down one slot per row, so slot k of row j
-  // holds u of row j - 16 + k (zero while that row lies before the block)
-  if (tid < CDH_BLOCK) hs[0][tid] = 0.0f;
-  if (tid == CDH_BLOCK) hd[0] = Ho[0];
+  // the vectors move down one slot per row, so slot k of row j holds u of row j - 16 + k (zero while that row lies
+  // before the block) and meets hs[j % 16][j % 16 + k]
+  auto fetch_h = [&](int blk) {
+    const int r = tid >> 5, c = (tid & 31) - CDH_BLOCK;
+    if (r < CDH_BLOCK) hs[r][tid & 31] = (c >= 0 && blk + r < dh && blk + c < dh) ? (double)Ho[(long long)(blk + r) * dh + blk + c] : 0.0;
+  };
+  fetch_h(0);
   __syncthreads();
+  if (STAGED && warp == CDC_THREADS / 32 - 1) fetch_slab(row0);
 
   double2 ureg[CDH_BLOCK];
 #pragma unroll
@@ -806,7 +870,7 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
 #pragma unroll 1
   for (int j = 0; j < dh; ++j) {
     const long long row = row0 + j;
-    const int buf = j & 1;
+    const int buf = j & 1, jl = j % CDH_BLOCK;
     double2 gv = gn;
     const float2 w = wn;
     const double sd_cur = sdn;
@@ -819,30 +883,25 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
         gn = *reinterpret_cast<const double2*>(p.G + rn * d + col);
         wn = *reinterpret_cast<const float2*>(p.Wb + rn * d + col);
       }
-      if (tid < a_cnt) an0 = p.Amat[rn * a_cnt + tid];
-      if (tid + CDC_THREADS < a_cnt) an1 = p.Amat[rn * a_cnt + tid + CDC_THREADS];
+      if (tid < a_cnt) an0 = p.Mmat[rn * a_cnt + tid];
+      if (tid + CDC_THREADS < a_cnt) an1 = p.Mmat[rn * a_cnt + tid + CDC_THREADS];
       if (rank == 0 && tid < ng) sdn = p.sD[rn * ng + tid];
-      const int blkn = ((j + 1) / CDH_BLOCK) * CDH_BLOCK;
-      if (tid < CDH_BLOCK) {
-        const int ci = j + 1 - CDH_BLOCK + tid;
-        hs[buf ^ 1][tid] = (ci >= blkn && ci <= j) ? Ho[(long long)(j + 1) * dh + ci] : 0.0f;
-      }
-      if (tid == CDH_BLOCK) hd[buf ^ 1] = Ho[(long long)(j + 1) * dh + j + 1];
-      for (size_t idx = tid; idx < slab_lines * ng; idx += CDC_THREADS) {
-        const size_t g2 = idx / slab_lines, l = idx % slab_lines;
-        const char* ptr = reinterpret_cast<const char*>(Yw + (rn * ng + (long long)g2) * d + c_lo) + l * 128;
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
-      }
+      if (!STAGED)
+        for (int idx = tid; idx < slab_lines * ng; idx += CDC_THREADS) {
+          const int g2 = idx / slab_lines, l = idx % slab_lines;
+          const char* ptr = reinterpret_cast<const char*>(Yw + (rn * ng + (long long)g2) * d + c_lo) + l * 128;
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
+        }
     }
     // ---- numerators of this CTA's groups: Wbar . (G + pending rank-1 terms of the block) ----
 #pragma unroll
     for (int i = 0; i < CDH_BLOCK; ++i) {
-      const double h = (double)hs[buf][i];
+      const double h = hs[jl][jl + i];
       gv.x = fma(h, ureg[i].x, gv.x);
       gv.y = fma(h, ureg[i].y, gv.y);
     }
     part[tid] = on ? fma((double)w.y, gv.y, (double)w.x * gv.x) : 0.0;
-    const double hjj = (double)hd[buf];
+    const double hjj = hs[jl][jl + CDH_BLOCK];
     __syncthreads();
     for (int gl = warp; gl < gpc; gl += CDC_THREADS / 32) {
       double v = 0.0;
@@ -852,42 +911,40 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
         for (int r = 0; r < p.csize; ++r) cluster.map_shared_rank(&num[0][0], r)[buf * CDC_MAXG + g_lo + gl] = v;
     }
     cluster.sync();
-    // ---- the scalar chain over the row's groups, lane g holding num[g] (every CTA runs it) ----
+    // ---- the row's groups: delta = -M num / hjj, lane g (every CTA) ----
     if (warp == 0) {
-      // delta_g2 = -num[g2] / (A[g2][g2] hjj); num[g] += hjj delta_g2 A[g2][g] for g > g2.  Only num is
-      // carried from step to step: the factor -A[g2][g] / A[g2][g2] of lane g is formed beside the
-      // chain, which is then one shuffle and one multiply-add per step.
       const bool in = lane < ng;
-      double nm = in ? num[buf][lane] : 0.0;
-      const double den = in ? Am[buf][lane * ng + lane] * hjj : 0.0;
-      const double rinv = (den == 0.0) ? 0.0 : 1.0 / den;   // 1 / (A[g][g] hjj)
-      const double ratio = -hjj * rinv;                     // -1 / A[g][g], or 0 for a skipped coordinate
-      double mine = 0.0;
-#pragma unroll 4
-      for (int g2 = 0; g2 < ng; ++g2) {
-        const double k = __shfl_sync(0xffffffffu, ratio, g2) * ((in && lane > g2) ? Am[buf][g2 * ng + lane] : 0.0);
-        const double n2 = __shfl_sync(0xffffffffu, nm, g2);
-        if (lane == g2) mine = -n2 * rinv;
-        nm = fma(n2, k, nm);
+      double a4[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int g2 = 0; g2 < CDC_MAXG; ++g2) {  // selects, not branches: those keep the loads of one step behind another's
+        const double t = fma(Am[buf][g2 * ng + lane], num[buf][g2], a4[g2 & 3]);
+        a4[g2 & 3] = (g2 <= lane) ? t : a4[g2 & 3];
       }
+      const double mine = (hjj == 0.0) ? 0.0 : -((a4[0] + a4[1]) + (a4[2] + a4[3])) / hjj;
       if (in) {
         delta[lane] = mine;
         if (rank == 0) p.sD[row * ng + lane] = sd_cur + mine;
       }
     }
     __syncthreads();
+    if (STAGED) mbar_wait(sbar, (uint32_t)buf, &abort_flag, &g_cd_error);
     // ---- u_j on this thread's columns ----
     double2 u = make_double2(0.0, 0.0);
     if (on) {
-      const TY* y = Yw + row * ng * d + col;
+      const TY* y = STAGED ? reinterpret_cast<const TY*>(cdc_slab) + c0 : Yw + row * ng * d + col;
+      const long long ld = STAGED ? c_cnt : d;
 #pragma unroll 8
       for (int g2 = 0; g2 < ng; ++g2) {
         const double dl = delta[g2];
-        const double2 yv = load_pair(y + (long long)g2 * d);
+        const double2 yv = load_pair(y + g2 * ld);
         u.x = fma(dl, yv.x, u.x);
         u.y = fma(dl, yv.y, u.y);
       }
       *reinterpret_cast<double2*>(p.Uacc + row * d + col) = u;
+    }
+    if (STAGED && j + 1 < dh) {
+      __syncthreads();  // the slice is read: the next row's takes its place
+      if (warp == CDC_THREADS / 32 - 1) fetch_slab(row + 1);
     }
 #pragma unroll
     for (int i = 0; i + 1 < CDH_BLOCK; ++i) ureg[i] = ureg[i + 1];
@@ -895,21 +952,38 @@ __global__ void __launch_bounds__(CDC_THREADS, 1) k_cd_head_cols(CdColP p) {
     // ---- end of a block: fold its vectors into the rows of G still to come ----
     if ((j + 1) % CDH_BLOCK == 0 && j + 1 < dh) {
       const int blk0 = j + 1 - CDH_BLOCK;
-      if (on) {
-#pragma unroll 2
-        for (int jj = j + 1; jj < dh; ++jj) {
-          const float* hr = Ho + (long long)jj * dh + blk0;
-          double2 g = *reinterpret_cast<const double2*>(p.G + (row0 + jj) * d + col);
+      for (int jb = j + 1; jb < dh; jb += CDC_FOLD) {
+        const int n = min((int)CDC_FOLD, dh - jb);
+        __syncthreads();
+        for (int i = tid; i < n * CDH_BLOCK; i += CDC_THREADS)
+          hf[i / CDH_BLOCK][i % CDH_BLOCK] = (double)Ho[(long long)(jb + i / CDH_BLOCK) * dh + blk0 + i % CDH_BLOCK];
+        __syncthreads();
+        if (on) {
+          for (int jj = 0; jj < n; jj += 4) {  // four rows of G on their way at a time
+            double2* gp = reinterpret_cast<double2*>(p.G + (row0 + jb + jj) * d + col);
+            double2 g[4];
 #pragma unroll
-          for (int i = 0; i < CDH_BLOCK; ++i) {
-            const double h = (double)__ldg(hr + i);
-            g.x = fma(h, ureg[i].x, g.x);
-            g.y = fma(h, ureg[i].y, g.y);
+            for (int q = 0; q < 4; ++q)
+              if (jj + q < n) g[q] = gp[(long long)q * d / 2];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (jj + q < n) {
+#pragma unroll
+                for (int i = 0; i < CDH_BLOCK; i += 2) {
+                  const double2 h = *reinterpret_cast<const double2*>(&hf[jj + q][i]);
+                  g[q].x = fma(h.x, ureg[i].x, g[q].x);
+                  g[q].y = fma(h.x, ureg[i].y, g[q].y);
+                  g[q].x = fma(h.y, ureg[i + 1].x, g[q].x);
+                  g[q].y = fma(h.y, ureg[i + 1].y, g[q].y);
+                }
+                gp[(long long)q * d / 2] = g[q];
+                if (jb + jj + q == j + 1) gn = g[q];
+              }
           }
-          *reinterpret_cast<double2*>(p.G + (row0 + jj) * d + col) = g;
-          if (jj == j + 1) gn = g;
         }
       }
+      fetch_h(j + 1);  // (the first barrier of the fold came after the block's last use)
+      __syncthreads();
 #pragma unroll
       for (int i = 0; i < CDH_BLOCK; ++i) ureg[i] = make_double2(0.0, 0.0);
     }
@@ -1568,7 +1642,7 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
         cp2.Yw = hp.Yw;
         cp2.Wb = hp.Wb;
         cp2.Hout = hp.Hout;
-        cp2.Amat = p.Amat;
+        cp2.Mmat = p.Amat;
         cp2.sD = hp.sD;
         cp2.d = d;
         cp2.seg = p.seg;
@@ -1580,6 +1654,8 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
             k_cd_amat<float><<<(unsigned)rows, 256, (size_t)d * sizeof(float), st>>>(p.Yw, hp.Wb, p.Amat, d, p.seg, p.ng);
           else
             k_cd_amat<double><<<(unsigned)rows, 256, (size_t)d * sizeof(float), st>>>(p.Yw, hp.Wb, p.Amat, d, p.seg, p.ng);
+          TB_LAUNCH_CHECK();
+          k_cd_chain<<<(unsigned)((rows + 3) / 4), 128, 0, st>>>(p.Amat, rows, p.ng);
           TB_LAUNCH_CHECK();
         }
         for (int it = 0; it < p.cd_iters; ++it) {
@@ -1607,7 +1683,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
           cudaLaunchConfig_t cfg = {};
           cfg.gridDim = dim3((unsigned)(heads_b * csize));
           cfg.blockDim = dim3(by_cols ? CDC_THREADS : CDH_THREADS);
-          cfg.dynamicSmemBytes = by_cols ? 0 : sm_head;
+          const size_t slab = p.yw_tensor ? (size_t)p.ng * c_cnt * sizeof(float) : 0;
+          static bool conf_cols[64] = {false};
+          if (by_cols && slab) TB_TRY(allow_smem(k_cd_head_cols<float>, (size_t)CDC_MAXG * 2 * CDC_THREADS * sizeof(float), conf_cols));
+          cfg.dynamicSmemBytes = by_cols ? slab : sm_head;
           cfg.stream = st;
           cudaLaunchAttribute attr[1];
           attr[0].id = cudaLaunchAttributeClusterDimension;

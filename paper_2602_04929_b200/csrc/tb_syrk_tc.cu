@@ -249,6 +249,7 @@ tb_status syrk_bf16_tensor(float* H, const __nv_bfloat16* X, long long n_tok, in
 // 0, or 1 once a bounded wait inside a tensor-core kernel has run out (sticky until read).
 namespace tb {
 int i8_error_read_clear();     // the products on the integer tensor cores (tb_i8.cu)
+int cd_error_read_clear();           // scale refinement (tb_quantize.cu)
 int grid_digits_error_read_clear();  // the grid search's products (tb_grid_digits.cu)
 int sweep_error_read_clear();  // the same word of the column-sweep kernel (tb_sweep.cu)
 int yw_error_read_clear();     // and of the tensor-core product of the scale refinement (tb_gemm_tc.cu)
@@ -291,10 +292,11 @@ extern "C" int tb_device_error_flag(void) {
   }
   const int e = tb::i8_error_read_clear();
   const int g = tb::grid_digits_error_read_clear();
+  const int c = tb::cd_error_read_clear();
   const int w = tb::sweep_error_read_clear();
   const int y = tb::yw_error_read_clear();
   const int x = tb::cross_error_read_clear();
   const int q = tb::pair_error_read_clear();
-  if (e < 0 || g < 0 || w < 0 || y < 0 || x < 0 || q < 0) return -1;
-  return (v || e || g || w || y || x || q) ? 1 : 0;
+  if (e < 0 || c < 0 || g < 0 || w < 0 || y < 0 || x < 0 || q < 0) return -1;
+  return (v || e || c || g || w || y || x || q) ? 1 : 0;
 }

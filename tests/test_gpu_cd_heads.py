@@ -28,3 +28,13 @@ def test_groups_of_32_columns_shared_hessian():
 def test_coordinates_per_head(d, heads, dh, gq, iters):
     prob = make_problem(72, d, heads, dh, 2048, hout="spd")
     compare(prob, run_gpu(prob, 3, gq, dh, CD | ADAPT, cd_iters=iters), 3, gq, dh, CD | ADAPT, cd_iters=iters, label=f"coords{dh}")
+
+
+# heads walked row by row with the row's columns staged in shared memory: 16 and 32 groups, rows that end inside a block of 16
+# and beyond a fold's 64, a cluster of one CTA and of several, a group of zeros (a coordinate that is skipped)
+@pytest.mark.parametrize("d,heads,dh,gq,iters", [(1024, 2, 21, 64, 1), (2048, 3, 150, 64, 2), (1152, 1, 97, 128, 1),
+                                                 (2048, 30, 16, 64, 1)])
+def test_rows_staged_in_shared_memory(d, heads, dh, gq, iters):
+    prob = make_problem(73, d, heads, dh, 2048, hout="spd")
+    prob["W"][3, :gq] = 0.0
+    compare(prob, run_gpu(prob, 3, gq, dh, CD | ADAPT, cd_iters=iters), 3, gq, dh, CD | ADAPT, cd_iters=iters, label=f"staged{dh}")
