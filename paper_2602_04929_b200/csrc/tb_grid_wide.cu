@@ -12,9 +12,8 @@
 //   k_grid_pick    adds the partial scores of a group in column order, takes the lowest
 // The work is FP64 tensor steps (half of d_group^2 per candidate row); what a step of few rows lacks is
 // CTAs, hence the column split, and tiles of 32 x 32 instead of 128 x 128 while the large ones would not
-// fill the SMs.  Against one CTA that walks all columns of its rows with the full product: the searches of
-// a 1664-wide layer with one scale per row (6656 rows) 99.9 ms before, 16.2 ms now (0.49 of the FP64
-// rate); 32 searches of 8 rows x 256 columns 3.44 ms before, 0.67 ms now.
+// fill the SMs (0.49 of the FP64 rate with large ones).  32 searches of 8 rows x 256 columns, against one CTA that walks
+// all columns of its rows with the full product: 3.44 ms before, 0.67 ms now.
 #include "tb_gemm.cuh"
 #include "tb_grid.cuh"
 #include "tb_rows.cuh"
@@ -35,6 +34,7 @@ struct GwSmem {  // CR candidate rows x CR columns
 
 __global__ void __launch_bounds__(256) k_row_range(GridP p, int m0, double2* range) {
   __shared__ double smn[8], smx[8];
+  pdl_wait();
   const int m = m0 + blockIdx.y, grp = blockIdx.x;
   const double* w = p.Wt + p.rm.row(m) * p.d + (long long)grp * p.seg;
   double mn = 0.0, mx = 0.0;
@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(256) k_row_range(GridP p, int m0, double2* ran
     mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
     mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
+  pdl_trigger();
   if ((threadIdx.x & 31) == 0) {
     smn[threadIdx.x >> 5] = mn;
     smx[threadIdx.x >> 5] = mx;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(CR == 128 ? 512 : 256, 1)
   const int n0 = ct * CR, k_end = min(seg, n0 + CR);
   const float* H = p.Hin + ((p.units > 1) ? (long long)(p.rm.row(m0 + unit * unit_rows) / p.rm.d_head) * d * d : 0);
 
+  pdl_wait();
   if (tid < CR) {
     const int r = tile * rt + tid / p.ncp, k = tid % p.ncp;
     const bool valid = r < unit_rows && k < p.n_cand;
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(CR == 128 ? 512 : 256, 1)
     }
     __syncthreads();
   }
+  pdl_trigger();
   // row dots of (E T) with E: quads by shuffle, warps through shared memory in a fixed order
 #pragma unroll
   for (int i = 0; i < NF; ++i) {
@@ -205,6 +208,8 @@ __global__ void __launch_bounds__(256) k_grid_pick(GridP p, int m0, long long li
                                                    const double* __restrict__ partial) {
   const long long line = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_trigger();
   if (line >= lines) return;
   double t = 0.0;
   if (lane < p.n_cand)
@@ -263,7 +268,7 @@ tb_status grid_wide(const GridP& p, double* scratch, size_t scratch_doubles, cud
     double2* range = reinterpret_cast<double2*>(scratch);
     double* partial = scratch + (size_t)2 * cnt * p.ng;
     const int units = cnt / rows;
-    k_row_range<<<dim3(p.ng, cnt), 256, 0, st>>>(p, u0, range);
+    TB_CUDA_CHECK(launch_pdl(k_row_range, dim3(p.ng, cnt), dim3(256), 0, st, p, u0, range));
     TB_LAUNCH_CHECK();
     // 128 x 128 tiles when they fill the SMs, else 32 x 32
     const int rt128 = 128 / p.ncp, rt32 = 32 / p.ncp;
@@ -274,12 +279,12 @@ tb_status grid_wide(const GridP& p, double* scratch, size_t scratch_doubles, cud
     if ((long long)units * tiles > 65535) return TB_ERR_UNSUPPORTED;
     const dim3 grid((unsigned)(p.ng * col_tiles), (unsigned)(units * tiles));
     if (small)
-      k_grid_score<32><<<grid, 256, sizeof(GwSmem<32>), st>>>(p, u0, rows, tiles, col_tiles, range, partial);
+      TB_CUDA_CHECK(launch_pdl(k_grid_score<32>, grid, dim3(256), sizeof(GwSmem<32>), st, p, u0, rows, tiles, col_tiles, range, partial));
     else
-      k_grid_score<128><<<grid, 512, sizeof(GwSmem<128>), st>>>(p, u0, rows, tiles, col_tiles, range, partial);
+      TB_CUDA_CHECK(launch_pdl(k_grid_score<128>, grid, dim3(512), sizeof(GwSmem<128>), st, p, u0, rows, tiles, col_tiles, range, partial));
     TB_LAUNCH_CHECK();
     const long long lines = (long long)cnt * p.ng;
-    k_grid_pick<<<(unsigned)((lines + 7) / 8), 256, 0, st>>>(p, u0, lines, col_tiles, range, partial);
+    TB_CUDA_CHECK(launch_pdl(k_grid_pick, dim3((unsigned)((lines + 7) / 8)), dim3(256), 0, st, p, u0, lines, col_tiles, range, partial));
     TB_LAUNCH_CHECK();
     u0 += cnt;
   }

@@ -2,14 +2,16 @@
 //
 // Per step i (a group of g = out_block rows of every head, M = n_heads * g
 // rows in all, heads being independent):
-//   grid     k_grid_tri       Algorithm 1, grid     candidate search per (row, column group)
+//   grid     k_grid_tri       Algorithm 1, grid     candidate search per (row, column group); tb_grid_wide.cu,
+//                                                   tb_grid_digits.cu
 //   sweep    k_sweep_rows     Algorithm 2 / Eq. 2   one launch, 8 to 32 rows per CTA for the whole sweep (tb_sweep.cu)
 //   update   k_compensate     W~[rem] -= T_i E      (Algorithm 1, update), E = W0 - Q_B (Proposition 3.1);
 //            with R first k_residual and a product: E -= W0 C (Proposition 3.2)
 // then, once: coordinate descent on the scales (Algorithm 3), Q = s (W_int - z),
 // and the loss of the proofs of Propositions 3.1 / 3.2.
 //
-// All of this runs in IEEE double on the CUDA cores.  The codes are integer
+// All of this runs in IEEE double, on the FP64 pipe or as exact digit products on the integer tensor cores
+// (tb_i8.cuh, tb_grid_digits.cu).  The codes are integer
 // decisions inside an error-feedback chain d_in steps long; in float the
 // accumulated rounding error of the chain (a few 1e-6 code units) exceeds the
 // 1e-6 band inside which a rounding decision may legitimately differ, and one
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(256) k_compensate(double* __restrict__ Wt, con
   const int nrem = dh - i0 - g;
   const int tid = threadIdx.x, ct = (tid & 63) * 2, rt = tid >> 6;  // rows rt + 4 k
   const double* Th = T + head * t_head;
+  pdl_wait();
   double acc[8][2];
 #pragma unroll
   for (int k = 0; k < 8; ++k) acc[k][0] = acc[k][1] = 0.0;
@@ -378,6 +381,7 @@ __global__ void __launch_bounds__(256) k_compensate(double* __restrict__ Wt, con
     }
     __syncthreads();
   }
+  pdl_trigger();
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int r = q0 + rt + 4 * k;
@@ -1499,9 +1503,9 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     const double* Ti = p.T + (long long)step * p.dh * p.g;
     const long long t_head = (long long)p.S * p.dh * p.g;
     if (with_r)
-      k_compensate<true><<<cgrid, 256, 0, st>>>(p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng);
+      TB_CUDA_CHECK(launch_pdl(k_compensate<true>, cgrid, dim3(256), 0, st, p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng));
     else
-      k_compensate<false><<<cgrid, 256, 0, st>>>(p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng);
+      TB_CUDA_CHECK(launch_pdl(k_compensate<false>, cgrid, dim3(256), 0, st, p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng));
     TB_LAUNCH_CHECK();
   }
 

@@ -204,9 +204,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   // What a block needs besides its values, by threads t of nt, in two parts with a barrier between: grids and 1 / U_jj,
   // then the scaled triangles (consecutive threads on consecutive columns: a thread per row would meet 32-way bank
   // conflicts, and the chain's own loads with them)
+  auto prepare_pivots = [&](int b, int t, int nt) {
+    for (int j = t; j < 128; j += nt) sm.rd[b & 1][j] = 1.0 / (double)U[(long long)(b * 128 + j) * (d + 1)];
+  };
   auto prepare_scales = [&](int b, int t, int nt) {
     const int pb = b & 1, c0 = b * 128;
-    for (int j = t; j < 128; j += nt) sm.rd[pb][j] = 1.0 / (double)U[(long long)(c0 + j) * (d + 1)];
     for (int i = t; i < R * 4; i += nt) {
       const int r = i >> 2, sb = i & 3;
       double s = 1.0, z = 0.0;
@@ -239,13 +241,16 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
     sm.abort_flag = 0;
     mbar_fence_init();
   }
+  // the first block: what depends on the factors alone, then, behind the kernel before, its values and grids
+  prepare_pivots(a.blk0, tid, SW_THREADS);
+  __syncthreads();
+  prepare_triangles(a.blk0, tid, SW_THREADS);
+  pdl_wait();
   for (int i = tid; i < R * 128; i += SW_THREADS) {  // the first block arrives unchanged
     const int r = i >> 7, c = i & 127;
     sm.w[a.blk0 & 1][r][c] = (r < rows_here) ? a.src[src_row(r) + a.blk0 * 128 + c] : 0.0;
   }
   prepare_scales(a.blk0, tid, SW_THREADS);
-  __syncthreads();
-  prepare_triangles(a.blk0, tid, SW_THREADS);
   __syncthreads();
   if (CLUSTER) cg::this_cluster().sync();  // every CTA of the cluster runs before anybody writes into it
   auto next_block = [&]() {  // block b + 1 has been handed over (by all CTAs of the cluster)
@@ -262,6 +267,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
     for (int b = a.blk0; b < a.blk1; ++b) {
       const int pb = b & 1;
       const bool more = b + 1 < a.blk1;
+      if (!more) pdl_trigger();
 #pragma unroll 1
       for (int sb = 0; sb < 8; ++sb) {
         const double* g = sm.gs[pb][r][sb >> 1];
@@ -511,6 +517,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
       next_block();
       break;
     }
+    prepare_pivots(b + 1, hw * 32 + lane, 32 * SW_HIST);
     prepare_scales(b + 1, hw * 32 + lane, 32 * SW_HIST);
     sw_sync<32 * SW_HIST>(SW_JOIN);
     prepare_triangles(b + 1, hw * 32 + lane, 32 * SW_HIST);
@@ -729,13 +736,15 @@ static tb_status sweep_launch(SweepP p, cudaStream_t st) {
   cfg.blockDim = dim3(SW_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)(CLUSTER ? p.cs : 1);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)(CLUSTER ? p.cs : 1);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = CLUSTER ? 1 : 0;
+  cfg.numAttrs = CLUSTER ? 2 : 1;
   TB_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, p, map_u, map_e, map_p, map_a));
   TB_LAUNCH_CHECK();
   return TB_OK;
@@ -779,6 +788,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restri
   const int d = a.d, K = c1 - k0;
   const long long uoff = (a.units > 1) ? (long long)unit * d * d : 0;
   const int m0 = unit * rows_per_unit + r0, rows = min(RT, rows_per_unit - r0);
+  pdl_wait();
   const int steps = K / 32, kw = warp * (K / 8);  // steps of four contraction rows per warp (a multiple of four)
   double acc[MF][NF][2];
 #pragma unroll
@@ -811,6 +821,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restri
 #pragma unroll
     for (int n = 0; n < NF; ++n)
       *reinterpret_cast<double2*>(rr_part + (warp * RT + 8 * m + fr) * CT + 8 * n + 2 * fk) = make_double2(acc[m][n][0], acc[m][n][1]);
+  pdl_trigger();
   __syncthreads();
   for (int i = threadIdx.x; i < RT * CT; i += 256) {
     const int r = i / CT, c = i % CT;
@@ -902,7 +913,7 @@ static tb_status rank_launch(const SweepArgs& a, double* work, int rows_per_unit
   auto kern = k_rank_rows<WITH_P, MF>;
   TB_TRY(allow_smem(kern, smem, configured));
   const dim3 grid((a.d - c1 + CT - 1) / CT, (rows_per_unit + 8 * MF - 1) / (8 * MF), a.units);
-  kern<<<grid, 256, smem, st>>>(a, work, rows_per_unit, k0, c1, err, arr);
+  TB_CUDA_CHECK(launch_pdl(kern, grid, dim3(256), smem, st, a, work, rows_per_unit, k0, c1, err, arr));
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
