@@ -773,39 +773,47 @@ tb_status sweep_columns(const SweepArgs& a, cudaStream_t st) {
 
 
 // ---------------------------------------------------------------------------
-// work[m][c] = src[m][c] - sum_k Err[m][k] U[k0 + k][c] (- Arr P) for the columns c >= c1 of few rows, K = c1 - k0 <= 512.
-// The eight warps of a CTA take an eighth of the contraction each, for 8 MF rows x 8 NF columns, straight from global
+// work[m][c] = src[m][c] - sum_k Err[m][k] U[k0 + k][c] (- Arr P) for the columns c >= c1 of few rows, K = c1 - k0 = 512.
+// The eight warps of a CTA take an eighth of the contraction each, for 8 MF rows x 32 columns, straight from global
 // memory (every entry of U is read once per row tile, in full sectors), and add up through shared memory in order.
-// Bound: reading U (HBM / L2) for 8 rows, the FP64 pipe from about 64 on.
+// Bound: reading U (HBM / L2) for 8 rows, the FP64 pipe from about 64 on.  Up to 16 rows the sweep before leaves most SMs
+// idle: the factors are copied into shared memory before the sweep has ended.
+// 8 rows x 4096 columns: 3.5 us from the sweep's end to this kernel's, 9.5 when the loads came after the wait.
 // ---------------------------------------------------------------------------
+template <bool WITH_P, int MF>
+struct RankTile {
+  static constexpr int RT = 8 * MF, CT = 32, LDF = 40;
+  static constexpr bool EARLY = MF <= 2;  // factors staged in shared memory ahead of the sweep's end
+  static constexpr size_t part = (size_t)8 * RT * CT * sizeof(double);
+  static constexpr size_t slab = (size_t)SWEEP_OUTER * LDF * sizeof(float);
+  static constexpr size_t smem = part + (EARLY ? slab * (WITH_P ? 2 : 1) : 0);
+};
+
 template <bool WITH_P, int MF>
 __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restrict__ work, int rows_per_unit, int k0, int c1,
                                                    const double* __restrict__ err, const double* __restrict__ arr) {
-  constexpr int NF = (MF == 4) ? 4 : 8, RT = 8 * MF, CT = 8 * NF;
-  extern __shared__ double rr_part[];  // [8][RT][CT]
+  using T = RankTile<WITH_P, MF>;
+  constexpr int NF = 4, RT = T::RT, CT = T::CT, STEPS = SWEEP_OUTER / 32;
+  extern __shared__ __align__(16) double rr_part[];  // [8][RT][CT], then the factors
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, fr = lane >> 2, fk = lane & 3;
   const int unit = blockIdx.z, r0 = blockIdx.y * RT, c0 = c1 + blockIdx.x * CT;
-  const int d = a.d, K = c1 - k0;
+  const int d = a.d;
   const long long uoff = (a.units > 1) ? (long long)unit * d * d : 0;
   const int m0 = unit * rows_per_unit + r0, rows = min(RT, rows_per_unit - r0);
-  pdl_wait();
-  const int steps = K / 32, kw = warp * (K / 8);  // steps of four contraction rows per warp (a multiple of four)
+  const int kw = warp * (SWEEP_OUTER / 8);  // STEPS steps of four contraction rows per warp
   double acc[MF][NF][2];
 #pragma unroll
   for (int i = 0; i < MF * NF * 2; ++i) (&acc[0][0][0])[i] = 0.0;
-  auto product = [&](const float* __restrict__ F, const double* __restrict__ E) {
-    const float* f = F + uoff + (long long)(k0 + kw + fk) * d + c0 + fr;
-    const double* e[MF];
-#pragma unroll
-    for (int m = 0; m < MF; ++m) e[m] = E + (long long)(m0 + min(8 * m + fr, rows - 1)) * a.err_ld + kw + fk;
-#pragma unroll 2
-    for (int q = 0; q < steps; ++q) {
+  // f: the entry of this lane's fragment in the first step, rows ldf apart
+  auto product = [&](const float* f, long long ldf, const double* __restrict__ E) {
+#pragma unroll(T::EARLY ? 8 : 2)
+    for (int q = 0; q < STEPS; ++q) {
       float b[NF];
       double av[MF];
 #pragma unroll
-      for (int n = 0; n < NF; ++n) b[n] = (c0 + 8 * n < d) ? __ldg(f + (long long)(4 * q) * d + 8 * n) : 0.0f;
+      for (int n = 0; n < NF; ++n) b[n] = f[4 * q * ldf + 8 * n];
 #pragma unroll
-      for (int m = 0; m < MF; ++m) av[m] = e[m][4 * q];
+      for (int m = 0; m < MF; ++m) av[m] = E[(long long)(m0 + min(8 * m + fr, rows - 1)) * a.err_ld + kw + fk + 4 * q];
 #pragma unroll
       for (int n = 0; n < NF; ++n) {
         const double bd = (double)b[n];
@@ -814,8 +822,30 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restri
       }
     }
   };
-  product(a.U, err);
-  if (WITH_P) product(a.P, arr);
+  if (T::EARLY) {
+    // asynchronous copies: loads into registers are scheduled behind the wait by the compiler.  Columns come in whole 32s.
+    float* slab = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(rr_part) + T::part);
+    auto stage = [&](const float* F, float* dst) {
+#pragma unroll 4
+      for (int i = threadIdx.x; i < SWEEP_OUTER * (CT / 4); i += 256) {
+        const int k = i / (CT / 4), c = 4 * (i % (CT / 4));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + k * T::LDF + c)),
+                     "l"(F + uoff + (long long)(k0 + k) * d + c0 + c)
+                     : "memory");
+      }
+    };
+    stage(a.U, slab);
+    if (WITH_P) stage(a.P, slab + SWEEP_OUTER * T::LDF);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    pdl_wait();
+    product(slab + (kw + fk) * T::LDF + fr, T::LDF, err);
+    if (WITH_P) product(slab + (SWEEP_OUTER + kw + fk) * T::LDF + fr, T::LDF, arr);
+  } else {
+    pdl_wait();
+    product(a.U + uoff + (long long)(k0 + kw + fk) * d + c0 + fr, d, err);
+    if (WITH_P) product(a.P + uoff + (long long)(k0 + kw + fk) * d + c0 + fr, d, arr);
+  }
 #pragma unroll
   for (int m = 0; m < MF; ++m)
 #pragma unroll
@@ -907,8 +937,8 @@ tb_status sweep_prepare(const float* U, const float* P, int d, int units, const 
 template <bool WITH_P, int MF>
 static tb_status rank_launch(const SweepArgs& a, double* work, int rows_per_unit, int k0, int c1, const double* err,
                              const double* arr, cudaStream_t st) {
-  constexpr int NF = (MF == 4) ? 4 : 8, CT = 8 * NF;
-  constexpr size_t smem = (size_t)8 * 8 * MF * CT * sizeof(double);
+  constexpr int CT = RankTile<WITH_P, MF>::CT;
+  constexpr size_t smem = RankTile<WITH_P, MF>::smem;
   static bool configured[64] = {false};
   auto kern = k_rank_rows<WITH_P, MF>;
   TB_TRY(allow_smem(kern, smem, configured));
