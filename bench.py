@@ -44,17 +44,17 @@ DEFAULT_WORKLOAD = "l2_70b_block"
 FP64_ALU_PEAK_TFLOPS = 148 * 64 * 2 * 1.965e9 / 1e12
 # FP32 FMA rate measured on this GPU by a register-resident FFMA loop (profiles/fp64_peak_microbench.md)
 FP32_FFMA_MEASURED_TFLOPS = 71.5
-FP64_KIND = "FP64 FMA / FP64 tensor pipe, 148 SM x 64 lanes x 2 x 1.965 GHz"
+# The large double-precision products of factor, sweep and grid search are exact int8 products of seven base-256 digits,
+# 28 per multiply-add at 8192 int8 multiply-adds a clock and SM: the higher of the two rates bounds those phases (TFLOP/s)
+DIGITS_PEAK_TFLOPS = 148 * 8192 * 2 * 1.965e9 / 28 / 1e12
+DIGITS_KIND = ("double products as 28 int8 products on the tensor cores, 148 SM x 8192 x 2 / 28 x 1.965 GHz; the FP64 pipe "
+               f"alone: {FP64_ALU_PEAK_TFLOPS:.1f}")
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under
 # profiles/ (bytes), keyed by (workload, kernel); absent where the kernel has changed since its capture
 # (the mean over the launches of that kernel in one layer; the Hessian kernel's figure holds for the
 # default 262 144 tokens only)
 NCU_TRAFFIC = {
-    ("l2_70b_block", "k_sweep_rows"): 759.0e6,     # 13 launches per layer, 9.9 GB in all
-    ("l2_70b_block", "k_grid_tri"): 314.1e6,       # 4 launches per layer
     ("l2_70b_block", "k_syrk_tc"): 55.2e9,         # 10 launches per layer (pair form, 66 pairs), 49.4 .. 58.7 GB read each
-    ("l2_7b_q", "k_sweep_rows"): 77.9e6,           # 4 launches per layer
-    ("l2_7b_q", "k_grid_tri"): 34.9e6,             # 4 launches per layer
     ("l2_7b_q", "k_syrk_tc"): 6.91e9,
 }
 NCU_TRAFFIC_TOKENS = 262144
@@ -468,15 +468,16 @@ def rooflines(cfg, n_tok, m, peaks):
     def alu(name, kernel, flops, ms):
         if ms:
             ach = flops / (ms * 1e-3) / 1e12
-            out[name] = {"kernel": kernel, "bound": "alu", "achieved": ach, "peak": FP64_ALU_PEAK_TFLOPS,
-                         "unit": "TFLOP/s", "frac": ach / FP64_ALU_PEAK_TFLOPS, "peak_kind": FP64_KIND,
+            out[name] = {"kernel": kernel, "bound": "alu", "achieved": ach, "peak": DIGITS_PEAK_TFLOPS,
+                         "unit": "TFLOP/s", "frac": ach / DIGITS_PEAK_TFLOPS, "peak_kind": DIGITS_KIND,
+                         "frac_of_fp64_pipe": ach / FP64_ALU_PEAK_TFLOPS,
                          "frac_of_measured_fp32_ffma": ach / FP32_FFMA_MEASURED_TFLOPS, "ms": ms,
                          "traffic": NCU_TRAFFIC.get((cfg.name, kernel))}
 
-    alu("sweep", "k_sweep_rows", sweep_flops(cfg), ph.get("sweep"))
+    alu("sweep", "k_sweep_rows + its updates (k_i8_gemm, k_rank_rows)", sweep_flops(cfg), ph.get("sweep"))
     seg_fl = sum(16.0 * p.d_out * p.d_in * ((cfg.quant_group or p.d_in) + 1) for p in cfg.projections)
-    alu("grid", "k_grid_tri", seg_fl, ph.get("grid"))
-    alu("factor", "k_chol_panel + FP64 GEMM engine", factor_flops(cfg), ph.get("factor"))
+    alu("grid", "k_gd_score, k_gd_codes, k_gd_h (k_grid_tri, k_grid_score: few rows)", seg_fl, ph.get("grid"))
+    alu("factor", "k_chol_panel, k_i8_gemm, gemm64_kernel", factor_flops(cfg), ph.get("factor"))
     loop_ms = ph.get("grid", 0.0) + ph.get("sweep", 0.0) + ph.get("compensation", 0.0)
     alu("loop", "grid + sweep + compensation", loop_flops(cfg), loop_ms)
     if ph.get("hessian"):
@@ -499,7 +500,7 @@ def config_entry(cfg, n_tok, m, peaks, oracle_info, steps):
         "prerequisites_ms": {k: ph.get(k, 0.0) for k in ("hessian", "cross", "hout", "factor", "prep")},
         "quantize_ms": {k: ph.get(k, 0.0) for k in ("setup", "grid", "sweep", "compensation", "cd", "output", "loss")},
         "loop_ms": loop_ms, "loop_out_channels_per_s": out_channels(cfg) / (loop_ms * 1e-3) if loop_ms else None,
-        "loop_frac_of_fp64_peak": roofs.get("loop", {}).get("frac"),
+        "loop_frac_of_fp64_peak": roofs.get("loop", {}).get("frac_of_fp64_pipe"),
         "loop_frac_of_measured_fp32_ffma": roofs.get("loop", {}).get("frac_of_measured_fp32_ffma"),
         "rooflines": roofs, "loss": m["loss"], "gpu_launches_per_step": m["launches"] / max(steps, 1),
     }

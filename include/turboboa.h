@@ -254,7 +254,8 @@ tb_status tb_prepare_correction(const float* R, const float* U_in, int n_batch, 
  *   loss   [n_heads] double or NULL: tr(dW H_in dW^T H_out) + 2 tr(H_out W R dW^T),
  *          dW = Q - W (the objective in the proofs of Propositions 3.1 / 3.2)
  *   stats  tb_stats (device) or NULL
- * The arithmetic of the loop is IEEE double precision: codes are integer
+ * The arithmetic of the loop is double precision (IEEE, or exact integer
+ * products of operands rounded to 54 bits): codes are integer
  * decisions taken inside an error-feedback chain d_in steps long, and they
  * only reproduce across implementations when the chain is carried in double. */
 size_t tb_quantize_layer_workspace(const tb_layer_desc* desc, int with_r, int with_loss);
