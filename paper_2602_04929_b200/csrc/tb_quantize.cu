@@ -68,8 +68,9 @@ __global__ void k_gather(const double* __restrict__ Wt, double* __restrict__ Wk,
 // With A = U_out^T lower triangular, T A_BB = A_remB is solved row by row,
 // last column first.  T is stored [head][step][d_head][g] (first rem rows used).
 // ---------------------------------------------------------------------------
-// The g factor rows of the step are staged in shared memory ([c][column from i0 on], when they fit), the solve of a
-// row keeps its T in the row's own storage.
+// The g factor rows of the step are staged in shared memory ([c][column from i0 on], when they fit); four threads
+// share a row, every fourth term of a dot product each.  Bound by the chain of g divisions and dot products: two steps of
+// 64 rows in 8 heads of 128 take 54 us (76 with a thread per row).
 __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restrict__ T, int dh,
                                 int g, int n_steps, int staged) {
   extern __shared__ __align__(16) float cm_u[];
@@ -83,26 +84,35 @@ __global__ void k_comp_matrices(const float* __restrict__ Uout, double* __restri
     for (int i = threadIdx.x; i < g * w; i += blockDim.x) cm_u[i] = Uo[(long long)(i0 + i / w) * dh + i0 + i % w];
     __syncthreads();
   }
-  for (int r = threadIdx.x; r < nrem; r += blockDim.x) {
-    double* Tr = Th + (long long)r * g;
-    // the row under construction: in shared memory where the factor rows are, [c][thread]
-    double* ct = staged ? reinterpret_cast<double*>(cm_u + (((size_t)g * dh + 3) & ~(size_t)3)) + threadIdx.x : Tr;
+  const int part = threadIdx.x & 3, slot = threadIdx.x >> 2;
+  for (int rb = 0; rb < nrem; rb += 128) {
+    const int r = rb + slot;
+    const bool on = r < nrem;
+    double* Tr = Th + (long long)(on ? r : 0) * g;
+    // the row under construction: in shared memory where the factor rows are, [c][row]
+    double* ct = staged ? reinterpret_cast<double*>(cm_u + (((size_t)g * dh + 3) & ~(size_t)3)) + slot : Tr;
     const int cs = staged ? 128 : 1;
     for (int c = g - 1; c >= 0; --c) {
       const float* urow = staged ? cm_u + c * w - i0 : Uo + (long long)(i0 + c) * dh;
-      double v0 = (double)urow[r0 + r], v1 = 0.0, v2 = 0.0, v3 = 0.0;
-      int c2 = c + 1;
-      for (; c2 + 3 < g; c2 += 4) {
-        v0 = fma(-ct[c2 * cs], (double)urow[i0 + c2], v0);
-        v1 = fma(-ct[(c2 + 1) * cs], (double)urow[i0 + c2 + 1], v1);
-        v2 = fma(-ct[(c2 + 2) * cs], (double)urow[i0 + c2 + 2], v2);
-        v3 = fma(-ct[(c2 + 3) * cs], (double)urow[i0 + c2 + 3], v3);
+      double v0 = 0.0, v1 = 0.0;
+      if (on) {
+        if (part == 0) v0 = (double)urow[r0 + r];
+        int c2 = c + 1 + part;
+        for (; c2 + 4 < g; c2 += 8) {
+          v0 = fma(-ct[c2 * cs], (double)urow[i0 + c2], v0);
+          v1 = fma(-ct[(c2 + 4) * cs], (double)urow[i0 + c2 + 4], v1);
+        }
+        if (c2 < g) v0 = fma(-ct[c2 * cs], (double)urow[i0 + c2], v0);
       }
-      for (; c2 < g; ++c2) v0 = fma(-ct[c2 * cs], (double)urow[i0 + c2], v0);
-      ct[c * cs] = ((v0 + v1) + (v2 + v3)) / (double)urow[i0 + c];
+      v0 += v1;
+      v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
+      v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
+      if (on && part == 0) ct[c * cs] = v0 / (double)urow[i0 + c];
+      __syncwarp();
     }
-    if (staged)
-      for (int c = 0; c < g; ++c) Tr[c] = ct[c * cs];
+    if (staged && on)
+      for (int c = part; c < g; c += 4) Tr[c] = ct[c * cs];
+    __syncwarp();
   }
 }
 
@@ -1405,7 +1415,7 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
       const bool staged = cm_smem <= 200 * 1024;
       static bool conf_cm[64] = {false};
       TB_TRY(allow_smem(k_comp_matrices, 200 * 1024, conf_cm));
-      k_comp_matrices<<<dim3(p.S, p.H), 128, staged ? cm_smem : 0, st>>>(U_out, p.T, p.dh, p.g, p.S, staged ? 1 : 0);
+      k_comp_matrices<<<dim3(p.S, p.H), 512, staged ? cm_smem : 0, st>>>(U_out, p.T, p.dh, p.g, p.S, staged ? 1 : 0);
       TB_LAUNCH_CHECK();
     }
     if (p.c_max) {  // C by columns, once for all steps
