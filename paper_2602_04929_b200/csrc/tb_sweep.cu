@@ -91,10 +91,11 @@ enum { SW_PUB = 1, SW_READY = 3, SW_JOIN = 5, SW_PIECE = 8 };  // two, two, one,
 // of the full value; otherwise `off` becomes nonzero there.
 template <bool CHECKED>
 __device__ __forceinline__ double sw_quant(double xm, int maxq, int& off) {
-  const int lo = __double2loint(xm), hw = __double2hiint(xm) - 0x43380000;
+  const int lo = __double2loint(xm), hi = __double2hiint(xm);
+  const int hw = (int)((unsigned)hi - 0x43380000u);  // modulo 2^32: a negative xm has a high word far below
   int n = __vimin_s32_relu(lo, maxq);
   if (CHECKED)
-    n = (hw == (lo >> 31)) ? n : ((hw >= 0) ? maxq : 0);
+    n = (hw == (lo >> 31)) ? n : ((hi >= 0x43380000) ? maxq : 0);  // (the sign of hw would be wrong for xm < 0)
   else
     off |= hw ^ (lo >> 31);
   return __hiloint2double(0x43380000, n) - 6755399441055744.0;

@@ -34,13 +34,26 @@ def test_one_hessian_per_head(n_hin):
     _case(prob, 4, 64, 20)
 
 
-def test_values_beyond_the_integer_range():
-    """A row whose later columns are 2^40 times its grid (all-zero first group, fixed grid of another group) saturates
-    like the oracle's clamp: the walk's range test has to see it."""
-    prob = make_problem(63, 256, 2, 16, 1024, hout="spd")
-    W = prob["W"]
-    W[3, :] *= 1e-9
-    W[3, 128:] *= 1e3
-    W[5, 0:32] = 0.0
-    W[5, 7] = 1e-12
-    _case(prob, 2, 32, 16, flags=0)
+# one big factor entry a column, so that the rounding error of the first column drives every later one to a chosen magnitude
+# in units of its grid, 2^31 and far beyond, in both directions; columns of the first piece of 16, of the first block of 128
+# and of the second
+@pytest.mark.parametrize("flags", [0, 4])
+def test_values_beyond_the_integer_range(flags):
+    """The walk's range test has to see them, and the code is the end of the grid that the value lies beyond."""
+    d, gq, bits = 256, 128, 4
+    prob = make_problem(63, d, 3, 16, 1024, hout=None)
+    rng = np.random.default_rng(5)
+    U = np.eye(d)
+    cols = np.r_[1:16, 20:128:3, 130:256:2] if flags == 0 else np.r_[1:16, 20:128:3]
+    # x = w / s + z - e U[0][c] / s: e is up to s / 2, so the magnitudes below reach both sides of 6.8e15 and 1.4e16
+    U[0, cols] = rng.choice([-1.0, 1.0], len(cols)) * 10.0 ** rng.uniform(8.0, 18.0, len(cols))
+    prob["Uin"] = U[None].astype(np.float32)
+    gpu = run_gpu(prob, bits, gq, 16, flags)
+    rep = compare(prob, gpu, bits, gq, 16, flags, label=f"beyond{flags}")
+    assert rep["code_mismatch"] == 0
+    W, u = prob["W"].astype(np.float64), prob["Uin"][0].astype(np.float64)
+    sc, z = np.repeat(gpu["scales"], gq, 1).astype(np.float64), np.repeat(gpu["zeros"], gq, 1)
+    e = W[:, 0] - sc[:, 0] * (gpu["codes"][:, 0].astype(np.float64) - z[:, 0])
+    x = (W - e[:, None] * u[0][None, :]) / sc + z
+    assert np.any(x[:, cols] > 2.0 ** 31) and np.any(x[:, cols] < -2.0 ** 31)
+    assert np.any((x[:, cols] > -1.35e16) & (x[:, cols] < -6.8e15))
