@@ -88,14 +88,15 @@ enum { SW_PUB = 1, SW_READY = 3, SW_JOIN = 5, SW_PIECE = 8 };  // two, two, one,
 // integer in its low word, where the clamp is one integer instruction.  The low word alone is the integer only below
 // 2^31 in magnitude; the high word tells (it is the constant's, or one less for a negative integer, exactly when the
 // low word's sign says the same).  CHECKED: beyond that range, infinities included, the code saturates like the clamp
-// of the full value; otherwise `off` becomes nonzero there.
+// of the full value, and is 0 for what is no number (a NaN's high word is above infinity's); otherwise `off` becomes
+// nonzero there.
 template <bool CHECKED>
 __device__ __forceinline__ double sw_quant(double xm, int maxq, int& off) {
   const int lo = __double2loint(xm), hi = __double2hiint(xm);
   const int hw = (int)((unsigned)hi - 0x43380000u);  // modulo 2^32: a negative xm has a high word far below
   int n = __vimin_s32_relu(lo, maxq);
   if (CHECKED)
-    n = (hw == (lo >> 31)) ? n : ((hi >= 0x43380000) ? maxq : 0);  // (the sign of hw would be wrong for xm < 0)
+    n = (hw == (lo >> 31)) ? n : (((unsigned)hw <= 0x7ff00000u - 0x43380000u) ? maxq : 0);  // up to infinity
   else
     off |= hw ^ (lo >> 31);
   return __hiloint2double(0x43380000, n) - 6755399441055744.0;

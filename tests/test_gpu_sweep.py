@@ -57,3 +57,17 @@ def test_values_beyond_the_integer_range(flags):
     x = (W - e[:, None] * u[0][None, :]) / sc + z
     assert np.any(x[:, cols] > 2.0 ** 31) and np.any(x[:, cols] < -2.0 ** 31)
     assert np.any((x[:, cols] > -1.35e16) & (x[:, cols] < -6.8e15))
+
+
+# few rows: rank-512 updates straight from the factor
+@pytest.mark.parametrize("heads,dh", [(2, 12)])
+def test_a_weight_that_is_no_number(heads, dh):
+    """Everything behind it in its row is no number either and takes code 0; no other row notices."""
+    prob = make_problem(64, 640, heads, dh, 1024, hout=None)
+    clean = run_gpu(prob, 3, 128, dh, 0, want_loss=False)
+    prob["W"][5, 40] = np.nan
+    gpu = run_gpu(prob, 3, 128, dh, 0, want_loss=False)
+    assert np.all(gpu["codes"][5, 40:] == 0)
+    others = np.arange(heads * dh) != 5
+    for k in ("codes", "scales", "zeros", "cand"):
+        assert np.array_equal(gpu[k][others], clean[k][others]), k
