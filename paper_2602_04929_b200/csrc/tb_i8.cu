@@ -44,6 +44,14 @@ __device__ __forceinline__ int i8_exponent(unsigned long long bits) {
   return e < -900 ? -900 : (e > 900 ? 900 : e);
 }
 __device__ __forceinline__ double i8_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+// A row with an entry that is no finite number has no digits: its largest magnitude (a bit pattern, a NaN's above
+// infinity's, both above every number's) is kept as it is, and the scale of its results is no number.
+__device__ __forceinline__ double i8_result_scale(unsigned long long bits) {
+  return (bits >> 52) >= 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : i8_pow2(i8_exponent(bits) - 54 + 24);
+}
+__device__ __forceinline__ unsigned long long i8_magnitude(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
 
 __device__ __forceinline__ bool i8_masked(int mask, int k, int row) {
   return (mask == 1 && k > row) || (mask == 2 && k < row) || (mask == 3 && k <= row);
@@ -53,7 +61,7 @@ template <typename T, bool KCONTIG>
 __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long* out, long long out_batch) {
   const T* X = static_cast<const T*>(s.X) + blockIdx.z * s.batch;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double m = 0.0;
+  unsigned long long m = 0;
   if (KCONTIG) {  // a warp per row, 512 contraction steps
     const int row = blockIdx.x * 8 + warp, k0 = blockIdx.y * 512;
     if (row >= s.rows) return;
@@ -62,13 +70,13 @@ __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long*
 #pragma unroll 4
     for (int k = k0 + lane; k < k_hi; k += 32)
       if (!i8_masked(s.mask, k, row)) {
-        double v = fabs((double)x[k]);
+        double v = (double)x[k];
         if (s.k_exp) v *= i8_pow2(s.k_sign * s.k_exp[k]);
-        m = fmax(m, v);
+        m = max(m, i8_magnitude(v));
       }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) atomicMax(out + blockIdx.z * out_batch + row, (unsigned long long)__double_as_longlong(m));
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) atomicMax(out + blockIdx.z * out_batch + row, m);
   } else {  // a lane per row, 8 warps x 16 contraction steps
     const int row = blockIdx.x * 32 + lane, k0 = blockIdx.y * 128 + warp * 16;
     if (row >= s.rows) return;
@@ -77,12 +85,12 @@ __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long*
     for (int i = 0; i < 16; ++i) {
       const int k = k0 + i;
       if (k < s.K && !i8_masked(s.mask, k, row)) {
-        double v = fabs((double)x[(long long)k * s.ld]);
+        double v = (double)x[(long long)k * s.ld];
         if (s.k_exp) v *= i8_pow2(s.k_sign * s.k_exp[k]);
-        m = fmax(m, v);
+        m = max(m, i8_magnitude(v));
       }
     }
-    if (m > 0.0) atomicMax(out + blockIdx.z * out_batch + row, (unsigned long long)__double_as_longlong(m));
+    if (m) atomicMax(out + blockIdx.z * out_batch + row, m);
   }
 }
 
@@ -401,9 +409,9 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
         o[j] = o[j + 1] = o[j + 2] = o[j + 3] = 0.0;
         if (p.add && in_m && n0 + j < p.N) i8_ld4(c + j, o[j], o[j + 1], o[j + 2], o[j + 3]);
       }
-      const int ea = (p.a_max && in_m) ? i8_exponent(p.a_max[b * p.a_max_batch + m]) : p.a_exp;
-      const int eb = (p.b_max && lane < 16 && n0 + lane < p.N) ? i8_exponent(p.b_max[b * p.b_max_batch + n0 + lane]) : p.b_exp;
-      double sa = i8_pow2(ea - 54 + 24);
+      double sa = (p.a_max && in_m) ? i8_result_scale(p.a_max[b * p.a_max_batch + m]) : i8_pow2(p.a_exp - 54 + 24);
+      const double sb_mine = (p.b_max && lane < 16 && n0 + lane < p.N) ? i8_result_scale(p.b_max[b * p.b_max_batch + n0 + lane])
+                                                                       : i8_pow2(p.b_exp - 54 + 24);
       if (p.negate) sa = -sa;
       if (!mbar_wait(accf_bar, tile_it & 1u, abort_flag, &g_i8_error)) break;
       __syncwarp();
@@ -426,7 +434,7 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
             lo = lo * 256 + (int)r[5][j];
             lo = lo * 256 + (int)r[6][j];
             const double v = fma((double)hi, 16777216.0, (double)lo);
-            const double sb = i8_pow2(__shfl_sync(0xffffffffu, eb, 8 * g + j) - 54 + 24);
+            const double sb = __shfl_sync(0xffffffffu, sb_mine, 8 * g + j);
             o[8 * g + j] = fma(v * sa, sb, o[8 * g + j]);
           }
         }

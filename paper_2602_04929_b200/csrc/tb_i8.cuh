@@ -12,6 +12,8 @@
 // 4.4e-17 and 7.6e-17.  The one thing a caller has to see to is that a small entry of a row that also has a
 // large one keeps fewer digits: operands whose rows (A) and columns (B) are of one size, as triangular
 // factors of an equilibrated matrix are, lose nothing.
+// A row of A or a column of B with an entry that is no finite number (and that no mask takes out) makes all of that
+// row or column of C no number.
 // 160 TFLOP/s of double-precision products is what the issue rate allows (37 on the FP64 pipe).
 #pragma once
 

@@ -59,8 +59,8 @@ def test_values_beyond_the_integer_range(flags):
     assert np.any((x[:, cols] > -1.35e16) & (x[:, cols] < -6.8e15))
 
 
-# few rows: rank-512 updates straight from the factor
-@pytest.mark.parametrize("heads,dh", [(2, 12)])
+# few rows (rank-512 updates straight from the factor) and many (digit products)
+@pytest.mark.parametrize("heads,dh", [(2, 12), (16, 128)])
 def test_a_weight_that_is_no_number(heads, dh):
     """Everything behind it in its row is no number either and takes code 0; no other row notices."""
     prob = make_problem(64, 640, heads, dh, 1024, hout=None)
