@@ -866,11 +866,12 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restri
   }
 }
 
+// rows along x, the one grid dimension that holds any number of them
 __global__ void k_sweep_gather(SweepArgs a, double* __restrict__ work, int c1) {
-  const int m = blockIdx.y;
+  const int m = blockIdx.x;
   const double2* src = reinterpret_cast<const double2*>(a.src + a.rm.row(m) * a.d);
   double2* dst = reinterpret_cast<double2*>(work + (long long)m * a.d);
-  for (int c = c1 / 2 + blockIdx.x * blockDim.x + threadIdx.x; c < a.d / 2; c += gridDim.x * blockDim.x) dst[c] = src[c];
+  for (int c = c1 / 2 + blockIdx.y * blockDim.x + threadIdx.x; c < a.d / 2; c += gridDim.y * blockDim.x) dst[c] = src[c];
 }
 
 // exps[k] = exponent of the diagonal entry U_kk
@@ -966,7 +967,7 @@ tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st) {
   a.Arr = A;
   a.err_ld = SWEEP_OUTER;
   if (s.use_i8) {
-    k_sweep_gather<<<dim3((d / 2 + 255) / 256, a.M), 256, 0, st>>>(a, s.work, SWEEP_OUTER);
+    k_sweep_gather<<<dim3(a.M, (d / 2 + 255) / 256), 256, 0, st>>>(a, s.work, SWEEP_OUTER);
     TB_LAUNCH_CHECK();
   }
   for (int b0 = 0; b0 < nblk; b0 += OB) {

@@ -71,3 +71,16 @@ def test_a_weight_that_is_no_number(heads, dh):
     others = np.arange(heads * dh) != 5
     for k in ("codes", "scales", "zeros", "cand"):
         assert np.array_equal(gpu[k][others], clean[k][others]), k
+
+
+def test_more_rows_than_a_grid_dimension_holds():
+    """66 000 rows in one step, and columns beyond the first 512: the last rows against the oracle."""
+    n, d = 66000, 640
+    prob = make_problem(65, d, 1, 48, 1024, hout=None)
+    reps = n // 48
+    big = dict(prob, W=np.tile(prob["W"], (reps, 1)), d_out=n, d_head=n)
+    gpu = run_gpu(big, 3, 128, n, ADAPT, want_loss=False)
+    rows = np.r_[0:48, 65520:65568, n - 48:n].reshape(3, 48)
+    for r in rows:
+        part = {k: (v[r] if k in ("codes", "scales", "zeros", "cand", "w_hat", "w_comp") else v) for k, v in gpu.items()}
+        compare(prob, part, 3, 128, 48, ADAPT, label=f"rows{r[0]}")
