@@ -162,16 +162,17 @@ __global__ void __launch_bounds__(512) k_cd_solve(const double* __restrict__ K, 
   }
 }
 
-// Dm_j += sum_g2 delta[j][g2] Yw[j][g2][:] and s += delta.  A CTA per row and 1024 columns.
+// Dm_j += sum_g2 delta[j][g2] Yw[j][g2][:] and s += delta.  A CTA per row (along x, which holds any
+// number of them) and 1024 columns.
 template <typename TY>
 __global__ void __launch_bounds__(256) k_cd_apply(double* __restrict__ Dm, const TY* __restrict__ Yw,
                                                   const double* __restrict__ delta, double* __restrict__ sD, int d, int ng) {
-  const long long row = blockIdx.y;
+  const long long row = blockIdx.x;
   const double* dr = delta + row * ng;  // [head][j ng + g] is [row][g]
-  if (blockIdx.x == 0)
+  if (blockIdx.y == 0)
     for (int g = threadIdx.x; g < ng; g += 256) sD[row * ng + g] += dr[g];
   const TY* y = Yw + row * ng * d;
-  for (int c = blockIdx.x * 1024 + threadIdx.x; c < min(d, (int)(blockIdx.x + 1) * 1024); c += 256) {
+  for (int c = blockIdx.y * 1024 + threadIdx.x; c < min(d, (int)(blockIdx.y + 1) * 1024); c += 256) {
     double v = Dm[row * d + c];
 #pragma unroll 8
     for (int g = 0; g < ng; ++g) v = fma(dr[g], (double)y[(long long)g * d + c], v);
@@ -212,7 +213,7 @@ tb_status cd_gram_pass(const CdGram& p, const double* G, double* Dm, double* sD,
   TB_TRY(allow_smem(k_cd_solve, CD_GRAM_MAX * sizeof(double), configured));
   k_cd_solve<<<p.heads, 512, (size_t)n * sizeof(double), st>>>(p.scratch, n0, delta, p.ng, p.dh);
   TB_LAUNCH_CHECK();
-  const dim3 grid((p.d + 1023) / 1024, (unsigned)rows);
+  const dim3 grid((unsigned)rows, (p.d + 1023) / 1024);
   if (p.yw_float)
     k_cd_apply<float><<<grid, 256, 0, st>>>(Dm, static_cast<const float*>(p.Yw), delta, sD, p.d, p.ng);
   else

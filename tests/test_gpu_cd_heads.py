@@ -38,3 +38,11 @@ def test_rows_staged_in_shared_memory(d, heads, dh, gq, iters):
     prob = make_problem(73, d, heads, dh, 2048, hout="spd")
     prob["W"][3, :gq] = 0.0
     compare(prob, run_gpu(prob, 3, gq, dh, CD | ADAPT, cd_iters=iters), 3, gq, dh, CD | ADAPT, cd_iters=iters, label=f"staged{dh}")
+
+
+def test_more_rows_than_a_grid_dimension_holds():
+    """66 560 rows with one scale each in one batch: heads at the beginning, past row 65 535 and at the end."""
+    prob = make_problem(74, 128, 520, 128, 512, hout="spd")
+    flags = CD | ADAPT
+    gpu = run_gpu(prob, 3, 0, 32, flags)
+    compare(prob, gpu, 3, 0, 32, flags, heads=[0, 511, 512, 519], label="rows66560")
