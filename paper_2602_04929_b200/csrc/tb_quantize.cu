@@ -1065,6 +1065,7 @@ struct Plan {
   bool adaptive, dynamic, cd, with_r, with_loss, has_hout;
   double *dynErr, *dynArr;  // [Mmax][seg] errors / arrival values of the current column group (dynamic grid)
   int Mmax;
+  size_t e_doubles;   // of E
   long long cd_rows;  // rows per coordinate-descent batch
   // workspace
   double *Wt, *Wk, *W0c, *E, *sD, *T, *Dq, *Dm, *Yw, *n0, *Amat, *G2;
@@ -1134,7 +1135,14 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
   const size_t dd = (size_t)p.d;
   p.Wt = b.take<double>((size_t)p.d_out * dd);
   p.Wk = b.take<double>((size_t)p.Mmax * dd);
-  p.E = b.take<double>((size_t)p.Mmax * dd);
+  // E is also the scratch of the search of wide groups, which needs a little more than d_in doubles a row with 17 and
+  // more candidates: a step's rows go through in one chunk
+  p.e_doubles = (size_t)p.Mmax * dd;
+  if (p.seg > 128) {
+    const size_t search = (size_t)p.Mmax * grid_wide_row_doubles(p.d, p.ng, p.ncp);
+    if (search > p.e_doubles) p.e_doubles = search;
+  }
+  p.E = b.take<double>(p.e_doubles);
   p.W0c = with_r ? b.take<double>((size_t)p.Mmax * dd) : nullptr;
   p.sweep = SweepScratch{};
   if (!p.dynamic) {
@@ -1246,7 +1254,7 @@ static tb_status run_grid(const Plan& p, const float* H_in, float* scales, int* 
   gp.grp0 = 0;
   if (p.grid_digits) return grid_digits(gp, p.gd, st);
   if (p.seg > 128)  // E is free until the sweep of a step
-    return grid_wide(gp, p.E, (size_t)p.Mmax * p.d, st);
+    return grid_wide(gp, p.E, p.e_doubles, st);
   static bool configured_tri[64] = {false};
   TB_TRY(allow_smem(k_grid_tri, GRID_TRI_SMEM, configured_tri));
   const long long ytiles = (long long)gp.units * gp.tiles_per_unit;

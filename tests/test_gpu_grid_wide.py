@@ -17,6 +17,8 @@ ADAPT = 1
     (384, 2, 32, 1, 192, 8, ADAPT, 1),  # a single candidate
     (512, 3, 64, 3, 256, 16, ADAPT, 5),  # one H_in per head
     (512, 3, 64, 3, 0, 4, 0, 16),       # one H_in per head, chunks inside a head
+    (384, 1, 4, 1, 0, 1, ADAPT, 20),    # steps of one row, more than 16 candidates
+    (256, 1, 6, 1, 0, 1, 0, 32),        # the fixed grid with scratch for one row
 ])
 def test_wide_groups(d, heads, dh, n_hin, gq, g, flags, n_cand):
     prob = make_problem(21, d, heads, dh, 1024, n_hin=n_hin)
