@@ -26,8 +26,8 @@
 //      look-ahead they run beside the later panels.  L^{-1} takes the place of L: a block of L
 //      is dead once its pair has been formed.
 //   5. U = J L^{-1} J D^-1, written as float with an explicit zero lower triangle.
-// From 1024 columns on the rank-256 updates and the doubling steps of 512 columns and more run on the
-// integer tensor cores (tb_i8.cuh).  The digits of L (one exponent for all, see the scaling) serve the
+// From 1024 columns on the rank-256 updates and the doubling steps of 512 to 16384 columns run on the
+// integer tensor cores (tb_i8.cuh); a step of 32768 contracts more than their sums hold and stays on the FP64 pipe.  The digits of L (one exponent for all, see the scaling) serve the
 // updates and the first product of a pair; the digits of a pair's inverse halves and of its first product
 // take the places of the digits of L that the pair has used up.
 #include "tb_common.cuh"
@@ -740,6 +740,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
     for (int sblk = G; sblk < dp; sblk <<= 1, ++level) {
       const int mblk = sblk / G;  // blocks per half of a pair at this level
       if (!last && (j + 1) % mblk) break;
+      const bool level_i8 = f.use_i8 && sblk <= I8_MAX_K_BLOCKS * I8_KB;
       const int half = j / mblk;  // which half of that size this block completes (the last one may be short)
       if (!(half & 1)) {
         if (last) continue;  // a first half without a second one: its inverse is complete
@@ -749,7 +750,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
         }
         const int o = half * sblk, m2 = (dp - o - sblk < sblk) ? dp - o - sblk : sblk;
         cudaStream_t s1 = side ? side->inv2[level & 7] : inv_st;
-        if (f.use_i8)
+        if (level_i8)
           TB_TRY(pair_first_i8(sblk, m2, o, high_tmp(sblk), s1));
         else
           TB_TRY(pair_first(sblk, m2, (long long)o * (dp + 1), pp, n_batch, high_tmp(sblk), (long long)f.tmp_per, s1));
@@ -758,7 +759,7 @@ tb_status tb::factor_run(const float* H, int n_batch, int d, float* U, float* Hi
       }
       if (side) TB_CUDA_CHECK(cudaStreamWaitEvent(side->inv, side->first_done[level & 7], 0));
       const int o = (half - 1) * sblk, m2 = (dp - o - sblk < sblk) ? dp - o - sblk : sblk;
-      if (f.use_i8)
+      if (level_i8)
         TB_TRY(pair_second_i8(sblk, m2, o, high_tmp(sblk), inv_st));
       else
         TB_TRY(pair_second(sblk, m2, (long long)o * (dp + 1), pp, n_batch, high_tmp(sblk), (long long)f.tmp_per, inv_st));

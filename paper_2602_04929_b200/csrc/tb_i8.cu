@@ -477,8 +477,8 @@ static tb_status i8_map(CUtensorMap* map, const I8Mat& m, unsigned box_blocks) {
 
 tb_status i8_gemm(const I8Gemm& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.n_batch <= 0) return TB_OK;
-  // vectors of four doubles on C; int32 sums of at most 7 K digit products of 2^14
-  if (g.N % 4 || g.ldc % 4 || g.c_batch % 4 || !aligned(g.C, 32) || !aligned(g.Cf, 16) || (g.Cf && g.beta != 0.0) || g.k_blocks > 512) return TB_ERR_INVALID_ARG;
+  // vectors of four doubles on C
+  if (g.N % 4 || g.ldc % 4 || g.c_batch % 4 || !aligned(g.C, 32) || !aligned(g.Cf, 16) || (g.Cf && g.beta != 0.0) || g.k_blocks > I8_MAX_K_BLOCKS) return TB_ERR_INVALID_ARG;
   CUtensorMap ma, mb;
   TB_TRY(i8_map(&ma, g.A, 2));
   TB_TRY(i8_map(&mb, g.B, 1));

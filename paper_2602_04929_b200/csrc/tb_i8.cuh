@@ -26,6 +26,8 @@ namespace tb {
 // That order is, box by box, the shared-memory image of both operands (K-major, no swizzle), and one TMA box
 // loads a block with all its digits.
 enum { I8_DIGITS = 7, I8_RB = 64, I8_KB = 32, I8_BLOCK = I8_DIGITS * I8_RB * I8_KB };
+// the longest contraction (16384 steps): the int32 sums hold 7 digit products of 2^14 a step
+enum { I8_MAX_K_BLOCKS = 512 };
 struct I8Mat {
   unsigned char* data;
   long long row_blocks;  // of the whole allocation (all matrices of a batch)

@@ -57,3 +57,39 @@ def test_factor_names_the_first_bad_pivot(what):
         H[d - 1 - r, d - 1 - 300] = H[d - 1 - 300, d - 1 - r] = bad
     _, info = _factor(H)
     assert info.tolist() == [r + 1]
+
+
+def test_factor_wider_than_a_digit_product_contracts():
+    """33 000 columns: a doubling step of 32 768, beyond the 16 384 steps that an int32 sum of digit products holds.
+    H = S (1 + V V^T) S, and U H U^T x = x for random x, in double; U is rounded to float (6e-8 an entry, each way) on a
+    matrix whose condition number is about 10, so the residual stays below 1e-6 or so; a block that is off by one part in a
+    thousand shows."""
+    import torch
+    import paper_2602_04929_b200 as tb
+    d, dev = 33000, "cuda:0"
+    g = torch.Generator(device=dev).manual_seed(3)
+    V = torch.randn(d, 8, generator=g, device=dev) * (3.0 / d ** 0.5)
+    s = torch.exp2(torch.randint(-8, 9, (d,), generator=g, device=dev).float())
+    H = V @ V.T
+    H = 0.5 * (H + H.T)
+    H.diagonal().add_(1.0)
+    H *= s[:, None]
+    H *= s[None, :]
+    U, info = tb.tb_factor(H)
+    torch.cuda.synchronize()
+    assert tb.tb_device_error_flag() == 0 and info.tolist() == [0]
+
+    def times(A, x, transposed=False):  # in double, 2048 rows of A at a time
+        y = torch.zeros_like(x)
+        for r in range(0, d, 2048):
+            a = A[r:r + 2048].double()
+            if transposed:
+                y += a.T @ x[r:r + 2048]
+            else:
+                y[r:r + 2048] = a @ x
+        return y
+
+    x = torch.randn(d, 4, generator=g, device=dev, dtype=torch.float64)
+    y = times(U, times(H, times(U, x, True)))
+    assert float((y - x).norm() / x.norm()) <= 1e-5
+    assert torch.count_nonzero(torch.tril(U[32000:], 31999)).item() == 0
