@@ -67,8 +67,7 @@ __global__ void __launch_bounds__(256) k_row_range(GridP p, int m0, double2* ran
 // CR = 128: 16 warps of 32 x 32; CR = 32: 8 warps, four of 16 x 16 times two halves of every chunk.
 template <int CR>
 __global__ void __launch_bounds__(CR == 128 ? 512 : 256, 1)
-    k_grid_score(GridP p, int m0, int unit_rows, int tiles_per_unit, int col_tiles, const double2* __restrict__ range,
-                 double* __restrict__ partial) {
+    k_grid_score(GridP p, int m0, int unit_rows, int tiles_per_unit, int col_tiles, const double2* range, double* partial) {
   extern __shared__ __align__(16) unsigned char gw_raw[];
   using Smem = GwSmem<CR>;
   constexpr int THREADS = (CR == 128) ? 512 : 256;
@@ -204,8 +203,7 @@ __global__ void __launch_bounds__(CR == 128 ? 512 : 256, 1)
 
 // one warp per (row, group), one lane per candidate; strict '<' and the lower k on ties
 __global__ void __launch_bounds__(256) k_grid_pick(GridP p, int m0, long long lines, int col_tiles,
-                                                   const double2* __restrict__ range,
-                                                   const double* __restrict__ partial) {
+                                                   const double2* range, const double* partial) {
   const long long line = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   pdl_wait();

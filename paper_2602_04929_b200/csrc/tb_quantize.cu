@@ -345,10 +345,9 @@ __global__ void k_residual(const double* __restrict__ Wt, const unsigned char* _
 // Bound: reading and writing W~ once.  As a residual launch and a product of the 128 x 128 engine it took, per step of
 // one row in 8 heads x 4096 columns, 24 us, of 32 rows in 32 heads 115 us; now 12 us and 80 us.
 template <bool HAVE_E>
-__global__ void __launch_bounds__(256) k_compensate(double* __restrict__ Wt, const unsigned char* __restrict__ codes,
-                                                    const double* __restrict__ sD, const int* __restrict__ z,
-                                                    const double* __restrict__ E, const double* __restrict__ T, int i0, int g,
-                                                    int dh, long long t_head, int d, int seg, int ng) {
+__global__ void __launch_bounds__(256) k_compensate(double* Wt, const unsigned char* codes, const double* sD, const int* z,
+                                                    const double* E, const double* T, int i0, int g, int dh,
+                                                    long long t_head, int d, int seg, int ng) {
   __shared__ double Es[32][128], Ts[32][33];
   const int head = blockIdx.y, c0 = blockIdx.x * 128, q0 = blockIdx.z * 32;  // first of 32 remaining rows
   const int nrem = dh - i0 - g;

@@ -792,8 +792,8 @@ struct RankTile {
 };
 
 template <bool WITH_P, int MF>
-__global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restrict__ work, int rows_per_unit, int k0, int c1,
-                                                   const double* __restrict__ err, const double* __restrict__ arr) {
+__global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, int rows_per_unit, int k0, int c1, const double* err,
+                                                   const double* arr) {
   using T = RankTile<WITH_P, MF>;
   constexpr int NF = 4, RT = T::RT, CT = T::CT, STEPS = SWEEP_OUTER / 32;
   extern __shared__ __align__(16) double rr_part[];  // [8][RT][CT], then the factors
@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* __restri
 #pragma unroll
   for (int i = 0; i < MF * NF * 2; ++i) (&acc[0][0][0])[i] = 0.0;
   // f: the entry of this lane's fragment in the first step, rows ldf apart
-  auto product = [&](const float* f, long long ldf, const double* __restrict__ E) {
+  auto product = [&](const float* f, long long ldf, const double* E) {
 #pragma unroll(T::EARLY ? 8 : 2)
     for (int q = 0; q < STEPS; ++q) {
       float b[NF];
