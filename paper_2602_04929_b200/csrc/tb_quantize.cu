@@ -367,10 +367,10 @@ __global__ void __launch_bounds__(256) k_compensate(double* Wt, const unsigned c
       } else {
         const long long row = (long long)head * dh + i0 + e0 + r, so = row * ng + (c0 + c) / seg;  // groups: multiples of 32
         v = *reinterpret_cast<const double2*>(Wt + row * d + c0 + c);
-        const uchar2 q = *reinterpret_cast<const uchar2*>(codes + row * d + c0 + c);
+        const unsigned char* q = codes + row * d + c0 + c;  // the caller's pointer: of any alignment
         const double s = sD[so], zz = (double)z[so];
-        v.x -= s * ((double)q.x - zz);
-        v.y -= s * ((double)q.y - zz);
+        v.x -= s * ((double)q[0] - zz);
+        v.y -= s * ((double)q[1] - zz);
       }
       *reinterpret_cast<double2*>(&Es[r][c]) = v;
     }

@@ -11,3 +11,21 @@ pytestmark = pytest.mark.gpu
 def test_compensation_matrices(dh, g):
     prob = make_problem(75, 128, 2, dh, 512, hout="spd")
     compare(prob, run_gpu(prob, 3, 64, g, 0), 3, 64, g, 0, label=f"comp{dh}")
+
+
+def test_codes_at_an_odd_address():
+    """The codes may lie anywhere: the joint compensation reads them back a byte at a time."""
+    import torch
+    import paper_2602_04929_b200 as tb
+    prob = make_problem(76, 256, 2, 24, 512, hout="spd")
+    dev = "cuda:0"
+    desc = tb.layer_desc(48, 256, 2, 24, 4, 64, 8)
+    args = [torch.from_numpy(prob[k]).to(dev) for k in ("W", "Hin", "Uin", "Hout", "Uout")]
+    ref = tb.tb_quantize_layer(desc, *args, want_loss=False)
+    out = tb.tb_quantize_layer(desc, *args, want_loss=False)
+    buf = torch.zeros(48 * 256 + 1, dtype=torch.uint8, device=dev)
+    out.codes = buf[1:].view(48, 256)
+    assert out.codes.data_ptr() % 2 == 1
+    tb.tb_quantize_layer(desc, *args, want_loss=False, out=out)
+    torch.cuda.synchronize()
+    assert torch.equal(out.codes, ref.codes) and torch.equal(out.w_hat, ref.w_hat)
