@@ -1079,6 +1079,7 @@ struct Plan {
   bool yw_tensor;
   bool dm_tensor;  // (Q - W) H_in through the split-bf16 tensor-core product as well
   bool loss_tensor;  // the loss's own dW H_in (no scale refinement) through it too
+  int piece_heads;   // with one H_in per head: heads per launch of the refinement's products
   int loss_heads;    // with one H_in per head: heads per launch of that product (their pieces of H_in fit 2 GiB)
   size_t ws_total;
 };
@@ -1198,8 +1199,11 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
     p.yw_tensor = tiles_ok && p.seg % 64 == 0;
     p.dm_tensor = tiles_ok && p.d % 32 == 0;
     if (p.yw_tensor) p.WbT = b.take<__nv_bfloat16>((size_t)rows * dd);
-    if (p.yw_tensor || p.dm_tensor)
-      p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (p.n_hin > 1 ? (size_t)(rows / p.dh) : 1));
+    // with one H_in per head: as many heads per launch as their pieces of H_in fit 4 GiB, like Yw (42 of 4096 columns)
+    p.piece_heads = (p.n_hin > 1) ? (int)(rows / p.dh) : 1;
+    const size_t head_pieces = (size_t)3 * dd * dd * sizeof(__nv_bfloat16);
+    if ((size_t)p.piece_heads * head_pieces > budget) p.piece_heads = (budget / head_pieces > 1) ? (int)(budget / head_pieces) : 1;
+    if (p.yw_tensor || p.dm_tensor) p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (size_t)p.piece_heads);
     const long long lines = rows;  // one set of statistics per row (the column-parallel pass keeps them all)
     if (has_hout && cd_gram_pays(p.dh, p.ng)) p.gram = b.take<double>(cd_gram_doubles((int)(rows / p.dh), p.dh, p.ng));
     p.n0 = b.take<double>((size_t)lines * p.ng);
@@ -1540,28 +1544,33 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     TB_LAUNCH_CHECK();
     for (long long r0 = 0; r0 < p.d_out; r0 += p.cd_rows) {
       const long long rows = (p.d_out - r0 < p.cd_rows) ? (p.d_out - r0) : p.cd_rows;
-      // Dm = (Q - W) H_in (+ W R); Yw = blockwise Wbar H_in.  With one H_in per head the batch is whole heads: one launch
-      // for all of them on the tensor cores, head by head on the FP64 engine.
-      const int hunits = (units > 1) ? (int)(rows / p.dh) : 1;
+      // Dm = (Q - W) H_in (+ W R); Yw = blockwise Wbar H_in.  With one H_in per head the batch is whole heads: on the tensor
+      // cores piece_heads of them in a launch, head by head on the FP64 engine.
       const long long rows_per_prod = (units > 1) ? p.dh : rows;
-      const float* Hb = H_in + ((units > 1) ? (r0 / p.dh) * dd : 0);
-      const bool split_h = r0 == 0 || with_r || units > 1;  // with R the pieces of R replace H_in's below
-      if (p.yw_tensor)  // also splits H_in into its bf16 pieces
-        TB_TRY(yw_tensor(reinterpret_cast<float*>(p.Yw), codes + r0 * d, zeros + r0 * p.ng, Hb, p.WbT, p.Hp, split_h, rows, d,
-                         p.seg, p.ng, hunits, st));
-      else if (p.dm_tensor && split_h)
-        TB_TRY(split3(Hb, p.Hp, dd * hunits, st));
-      if (p.dm_tensor) {
-        // the pieces of (Q - W), transposed, live in this batch's rows of the W~ buffer (free by now,
-        // and overwritten by G = H_out Dm only after the product)
-        __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + r0 * d);
-        TB_TRY(split3_transpose(p.Dq + r0 * d, DqT, rows, d, st));
-        TB_TRY(gemm_split_presplit(p.Dm + r0 * d, d, DqT, p.Hp, rows, d, d, false, st, hunits));
-        if (with_r) {
-          // Dm += W R through the same split-bf16 product; the pieces of R take the place of H_in's
-          TB_TRY(split3_transpose(W + r0 * d, DqT, rows, d, st));
-          TB_TRY(split3(R + ((units > 1) ? (r0 / p.dh) * dd : 0), p.Hp, dd * hunits, st));
-          TB_TRY(gemm_split_presplit(p.Dm + r0 * d, d, DqT, p.Hp, rows, d, d, true, st, hunits));
+      const long long rows_per_launch = (units > 1) ? (long long)p.piece_heads * p.dh : rows;
+      for (long long q0 = 0; q0 < rows && (p.yw_tensor || p.dm_tensor); q0 += rows_per_launch) {
+        const long long rr = r0 + q0, rl = (rows - q0 < rows_per_launch) ? rows - q0 : rows_per_launch;
+        const int hunits = (units > 1) ? (int)(rl / p.dh) : 1;
+        const long long head0 = (units > 1) ? (rr / p.dh) * dd : 0;
+        const float* Hb = H_in + head0;
+        const bool split_h = r0 == 0 || with_r || units > 1;  // with R the pieces of R replace H_in's below
+        if (p.yw_tensor)  // also splits H_in into its bf16 pieces
+          TB_TRY(yw_tensor(reinterpret_cast<float*>(p.Yw) + q0 * p.ng * d, codes + rr * d, zeros + rr * p.ng, Hb, p.WbT, p.Hp,
+                           split_h, rl, d, p.seg, p.ng, hunits, st));
+        else if (split_h)
+          TB_TRY(split3(Hb, p.Hp, dd * hunits, st));
+        if (p.dm_tensor) {
+          // the pieces of (Q - W), transposed, live in these rows of the W~ buffer (free by now,
+          // and overwritten by G = H_out Dm only after the product)
+          __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + rr * d);
+          TB_TRY(split3_transpose(p.Dq + rr * d, DqT, rl, d, st));
+          TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rl, d, d, false, st, hunits));
+          if (with_r) {
+            // Dm += W R through the same split-bf16 product; the pieces of R take the place of H_in's
+            TB_TRY(split3_transpose(W + rr * d, DqT, rl, d, st));
+            TB_TRY(split3(R + head0, p.Hp, dd * hunits, st));
+            TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rl, d, d, true, st, hunits));
+          }
         }
       }
       for (long long q0 = 0; q0 < rows && !(p.yw_tensor && p.dm_tensor); q0 += rows_per_prod) {

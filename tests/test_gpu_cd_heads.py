@@ -46,3 +46,38 @@ def test_more_rows_than_a_grid_dimension_holds():
     flags = CD | ADAPT
     gpu = run_gpu(prob, 3, 0, 32, flags)
     compare(prob, gpu, 3, 0, 32, flags, heads=[0, 511, 512, 519], label="rows66560")
+
+
+@pytest.mark.parametrize("with_r", [False, True])
+def test_heads_whose_pieces_go_through_in_two_launches(with_r):
+    """12 heads of 8192 columns, 10 to a launch: every head has the same H_in, so the result is that of the shared one (the
+    products per head are the same, only the launches differ)."""
+    import torch
+    import paper_2602_04929_b200 as tb
+    H, dh, d, dev = 12, 8, 8192, "cuda:0"
+    g = torch.Generator(device=dev).manual_seed(9)
+    V = torch.randn(d, 16, generator=g, device=dev) / 16
+    Hin = V @ V.T
+    Hin = 0.5 * (Hin + Hin.T)
+    Hin.diagonal().add_(1.0)
+    U, info = tb.tb_factor(Hin)
+    W = 0.02 * torch.randn(H * dh, d, generator=g, device=dev)
+    Ho = torch.eye(dh, device=dev) + 0.3
+    Hout = Ho.expand(H, dh, dh).contiguous()
+    Uout, _ = tb.tb_factor(Hout)
+    ops = [None] * 3
+    if with_r:
+        R = 0.05 * torch.randn(d, d, generator=g, device=dev) / d ** 0.5
+        ops = [R, *tb.tb_prepare_correction(R, U)]
+
+    def run(n_hin):
+        def per(t):
+            return None if t is None else t.expand(n_hin, d, d).contiguous()
+        desc = tb.layer_desc(H * dh, d, H, dh, 3, 128, 8, n_hin=n_hin, flags=CD | ADAPT)
+        out = tb.tb_quantize_layer(desc, W, per(Hin), per(U), Hout, Uout, *[per(t) for t in ops], want_loss=False)
+        torch.cuda.synchronize()
+        return out
+
+    one, many = run(1), run(H)
+    assert torch.equal(one.codes, many.codes) and torch.equal(one.zeros, many.zeros)
+    assert float((one.scales - many.scales).norm() / one.scales.norm()) <= 1e-6

@@ -55,6 +55,15 @@ def test_workspace_queries_and_growth():
     assert tb.tb_quantize_from_host_workspace(d, 2048, 1) > b
 
 
+def test_refinement_scratch_does_not_grow_with_the_heads_hessians():
+    """With one H_in per head their bf16 pieces (6 bytes an entry) go through at most 4 GiB at a time."""
+    def query(heads, d, n_hin, flags):
+        return tb.tb_quantize_layer_workspace(tb.layer_desc(heads * 128, d, heads, 128, 3, 0, 32, n_hin=n_hin, flags=flags), False, False)
+
+    for heads, d in ((64, 8192), (96, 12288), (32, 4096)):
+        assert query(heads, d, heads, 3) - query(heads, d, 1, 3) <= 4 << 30, (heads, d)
+
+
 def test_bad_descriptions_are_rejected_on_the_host():
     lib = tb.load()
     one = ctypes.c_void_p(256)  # never dereferenced: validation fails first
