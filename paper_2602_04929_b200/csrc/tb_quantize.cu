@@ -1147,7 +1147,7 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
   p.sweep = SweepScratch{};
   if (!p.dynamic) {
     const int units = (p.n_hin == 1) ? 1 : p.H;
-    sweep_scratch(b, p.Mmax, p.d, units, with_r, sweep_wants_i8(p.d, p.Mmax / units) && units == 1, &p.sweep);
+    sweep_scratch(b, p.Mmax, p.d, with_r, sweep_wants_i8(p.d, units, p.Mmax / units), &p.sweep);
     p.sweep.work = p.Wk;
   }
   p.Cdig = p.Wdig = I8Mat{nullptr, 0, 0};
@@ -1437,7 +1437,7 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
   }
   if (!p.dynamic) {
     PhaseScope ph(PH_SWEEP, st);
-    TB_TRY(sweep_prepare(U_in, P, d, (p.n_hin == 1) ? 1 : p.H, p.sweep, st));
+    TB_TRY(sweep_prepare(U_in, P, d, p.sweep, st));
   }
   if (p.grid_digits) {
     PhaseScope ph(PH_GRID, st);

@@ -56,15 +56,15 @@ enum { SWEEP_OUTER = 512, SWEEP_I8_WORK = 1200000 };
 struct SweepScratch {
   double *work;          // [M][d]
   double *err, *arr;     // [M][SWEEP_OUTER], arr with P only
-  bool use_i8;           // the updates on the integer tensor cores (sweep_wants_i8); then:
+  bool use_i8;           // the updates on the integer tensor cores (one shared U, sweep_wants_i8); then:
   I8Mat Udig, Pdig;      // digits of U and P by columns (prepared by sweep_prepare, one set for all steps)
   I8Mat Edig, Adig;      // digits of a block's errors and arrival values
   unsigned long long *u_max, *p_max, *e_max, *a_max;
   int* u_exp;            // exponents of U's diagonal
 };
-bool sweep_wants_i8(int d, int rows_per_unit);
-void sweep_scratch(Bump& b, int M, int d, int units, bool with_p, bool use_i8, SweepScratch* s);  // err .. u_exp
-tb_status sweep_prepare(const float* U, const float* P, int d, int units, const SweepScratch& s, cudaStream_t st);
+bool sweep_wants_i8(int d, int units, int rows_per_unit);
+void sweep_scratch(Bump& b, int M, int d, bool with_p, bool use_i8, SweepScratch* s);  // err .. u_exp
+tb_status sweep_prepare(const float* U, const float* P, int d, const SweepScratch& s, cudaStream_t st);
 // a.src: the weights (mapped); a.Err, a.Arr, blk0, blk1 and the like are set here
 tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st);
 

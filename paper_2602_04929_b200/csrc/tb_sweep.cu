@@ -878,19 +878,20 @@ __global__ void k_sweep_gather(SweepArgs a, double* __restrict__ work, int c1) {
 __global__ void k_sweep_exp(const float* __restrict__ U, int* __restrict__ exps, int d) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= d) return;
-  const float u = fabsf(U[(long long)blockIdx.y * d * d + (long long)k * (d + 1)]);
+  const float u = fabsf(U[(long long)k * (d + 1)]);
   int e = 0;
   if (u > 0.0f && u <= 3.4e38f) frexpf(u, &e);
-  exps[blockIdx.y * d + k] = e;
+  exps[k] = e;
 }
 
 // An update on digits costs three launches whatever its size, k_rank_rows the FP64 pipe's time for rows x width: about
-// equal at 300 rows of 4096 columns.  208 rows of 1664 with P: 11.0 ms of sweep with digits, 7.2 ms without.
-bool sweep_wants_i8(int d, int rows_per_unit) {
-  return d > SWEEP_OUTER && d <= 16384 && (long long)rows_per_unit * d >= SWEEP_I8_WORK;
+// equal at 300 rows of 4096 columns.  208 rows of 1664 with P: 11.0 ms of sweep with digits, 7.2 ms without.  With one
+// U per head the digits of all of them would have to be kept, for rows of one head each: not taken.
+bool sweep_wants_i8(int d, int units, int rows_per_unit) {
+  return units == 1 && d > SWEEP_OUTER && d <= I8_MAX_K_BLOCKS * I8_KB && (long long)rows_per_unit * d >= SWEEP_I8_WORK;
 }
 
-void sweep_scratch(Bump& b, int M, int d, int units, bool with_p, bool use_i8, SweepScratch* s) {
+void sweep_scratch(Bump& b, int M, int d, bool with_p, bool use_i8, SweepScratch* s) {
   *s = SweepScratch{};
   s->use_i8 = use_i8;
   if (d <= SWEEP_OUTER) return;
@@ -904,35 +905,32 @@ void sweep_scratch(Bump& b, int M, int d, int units, bool with_p, bool use_i8, S
     m.data = b.take<unsigned char>(i8_bytes(row_blocks, k_blocks));
     return m;
   };
-  const long long rb_unit = (M / units + I8_RB - 1) / I8_RB;
-  s->Udig = mat((long long)units * (d / I8_RB), d / I8_KB);
-  s->Edig = mat(units * rb_unit, SWEEP_OUTER / I8_KB);
-  s->u_max = b.take<unsigned long long>((size_t)units * d);
+  const long long row_blocks = (M + I8_RB - 1) / I8_RB;
+  s->Udig = mat(d / I8_RB, d / I8_KB);
+  s->Edig = mat(row_blocks, SWEEP_OUTER / I8_KB);
+  s->u_max = b.take<unsigned long long>((size_t)d);
   s->e_max = b.take<unsigned long long>((size_t)M);
-  s->u_exp = b.take<int>((size_t)units * d);
+  s->u_exp = b.take<int>((size_t)d);
   if (with_p) {
-    s->Pdig = mat((long long)units * (d / I8_RB), d / I8_KB);
-    s->Adig = mat(units * rb_unit, SWEEP_OUTER / I8_KB);
-    s->p_max = b.take<unsigned long long>((size_t)units * d);
+    s->Pdig = mat(d / I8_RB, d / I8_KB);
+    s->Adig = mat(row_blocks, SWEEP_OUTER / I8_KB);
+    s->p_max = b.take<unsigned long long>((size_t)d);
     s->a_max = b.take<unsigned long long>((size_t)M);
   }
 }
 
 // Rows of U scale as 1 / U_kk scales the errors: the exponents of the diagonal take that out of both operands.
-tb_status sweep_prepare(const float* U, const float* P, int d, int units, const SweepScratch& s, cudaStream_t st) {
+tb_status sweep_prepare(const float* U, const float* P, int d, const SweepScratch& s, cudaStream_t st) {
   if (!s.use_i8) return TB_OK;
-  const long long dd = (long long)d * d;
-  k_sweep_exp<<<dim3((d + 255) / 256, units), 256, 0, st>>>(U, s.u_exp, d);
+  k_sweep_exp<<<(d + 255) / 256, 256, 0, st>>>(U, s.u_exp, d);
   TB_LAUNCH_CHECK();
-  for (int u = 0; u < units; ++u) {  // (one exponent vector per matrix)
-    const I8Src us{U + u * dd, d, 0, d, d, 1, true, false, 1, s.u_exp + (long long)u * d, -1};
-    TB_TRY(i8_row_max(us, s.u_max + (long long)u * d, d, st));
-    TB_TRY(i8_slice(us, s.u_max + (long long)u * d, d, 0, s.Udig, (long long)u * (d / I8_RB), 0, 0, st));
-  }
+  const I8Src us{U, d, 0, d, d, 1, true, false, 1, s.u_exp, -1};
+  TB_TRY(i8_row_max(us, s.u_max, d, st));
+  TB_TRY(i8_slice(us, s.u_max, d, 0, s.Udig, 0, 0, 0, st));
   if (P) {
-    const I8Src ps{P, d, dd, d, d, units, true, false, 1, nullptr, 0};
+    const I8Src ps{P, d, 0, d, d, 1, true, false, 1, nullptr, 0};
     TB_TRY(i8_row_max(ps, s.p_max, d, st));
-    TB_TRY(i8_slice(ps, s.p_max, d, 0, s.Pdig, 0, d / I8_RB, 0, st));
+    TB_TRY(i8_slice(ps, s.p_max, d, 0, s.Pdig, 0, 0, 0, st));
   }
   return TB_OK;
 }
@@ -978,36 +976,28 @@ tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st) {
     TB_TRY(sweep_columns(a, st));
     if (c1 >= d) break;
     if (s.use_i8) {
-      const long long rb_unit = (rows_per_unit + I8_RB - 1) / I8_RB, batch = (long long)rows_per_unit * SWEEP_OUTER;
-      // one exponent vector per launch: with several units the scales of all but the first stay in their digits
-      const I8Src es{E, SWEEP_OUTER, batch, rows_per_unit, c1 - k0, a.units, false, true, 0, a.units == 1 ? s.u_exp + k0 : nullptr, 1};
-      TB_TRY(i8_row_max(es, s.e_max, rows_per_unit, st));
-      TB_TRY(i8_slice(es, s.e_max, rows_per_unit, 0, s.Edig, 0, rb_unit, 0, st));
+      const I8Src es{E, SWEEP_OUTER, 0, a.M, c1 - k0, 1, false, true, 0, s.u_exp + k0, 1};
+      TB_TRY(i8_row_max(es, s.e_max, a.M, st));
+      TB_TRY(i8_slice(es, s.e_max, a.M, 0, s.Edig, 0, 0, 0, st));
       I8Gemm g = i8_gemm_params();
       g.A = s.Edig;
       g.B = s.Udig;
-      g.a_rb_batch = rb_unit;
       g.b_rb = c1 / I8_RB;
-      g.b_rb_batch = d / I8_RB;
       g.b_kb = k0 / I8_KB;
       g.k_blocks = (c1 - k0) / I8_KB;
       g.a_max = s.e_max;
-      g.a_max_batch = rows_per_unit;
       g.b_max = s.u_max + c1;
-      g.b_max_batch = d;
       g.C = s.work + c1;
       g.ldc = d;
-      g.c_batch = (long long)rows_per_unit * d;
-      g.M = rows_per_unit;
+      g.M = a.M;
       g.N = d - c1;
-      g.n_batch = a.units;
       g.alpha = -1.0;
       g.beta = 1.0;
       TB_TRY(i8_gemm(g, st));
       if (a.P) {
-        const I8Src as{A, SWEEP_OUTER, batch, rows_per_unit, c1 - k0, a.units, false, true, 0, nullptr, 0};
-        TB_TRY(i8_row_max(as, s.a_max, rows_per_unit, st));
-        TB_TRY(i8_slice(as, s.a_max, rows_per_unit, 0, s.Adig, 0, rb_unit, 0, st));
+        const I8Src as{A, SWEEP_OUTER, 0, a.M, c1 - k0, 1, false, true, 0, nullptr, 0};
+        TB_TRY(i8_row_max(as, s.a_max, a.M, st));
+        TB_TRY(i8_slice(as, s.a_max, a.M, 0, s.Adig, 0, 0, 0, st));
         g.A = s.Adig;
         g.B = s.Pdig;
         g.a_max = s.a_max;

@@ -34,6 +34,12 @@ def test_one_hessian_per_head(n_hin):
     _case(prob, 4, 64, 20)
 
 
+def test_one_hessian_per_head_and_many_rows():
+    """As many rows of as many columns as take digit products with a shared factor: with one per head they do not."""
+    prob = make_problem(66, 640, 2, 1920, 1024, n_hin=2, hout=None)
+    _case(prob, 3, 128, 1920)
+
+
 # one big factor entry a column, so that the rounding error of the first column drives every later one to a chosen magnitude
 # in units of its grid, 2^31 and far beyond, in both directions; columns of the first piece of 16, of the first block of 128
 # and of the second
