@@ -50,7 +50,7 @@ __global__ void k_scale_exp(const float* __restrict__ H, int* __restrict__ exps,
   if (r < d) {
     const int i = d - 1 - r;
     const float h = H[((long long)b * d + i) * d + i];
-    if (h > 0.0f && h <= 3.4e38f) {
+    if (h > 0.0f && h < INFINITY) {
       int x;
       frexp((double)h, &x);  // h = f 2^x, f in [1/2, 1)
       e = x >> 1;            // floor(x / 2): f or 2 f remains
@@ -404,7 +404,7 @@ __global__ void k_diag_exp(const float* __restrict__ U, int* __restrict__ exps, 
   if (k >= d) return;
   const float u = fabsf(U[(long long)k * d + k]);
   int e = 0;
-  if (u > 0.0f && u <= 3.4e38f) frexpf(u, &e);
+  if (u > 0.0f && u < INFINITY) frexpf(u, &e);
   exps[k] = e;
 }
 

@@ -880,7 +880,7 @@ __global__ void k_sweep_exp(const float* __restrict__ U, int* __restrict__ exps,
   if (k >= d) return;
   const float u = fabsf(U[(long long)k * (d + 1)]);
   int e = 0;
-  if (u > 0.0f && u <= 3.4e38f) frexpf(u, &e);
+  if (u > 0.0f && u < INFINITY) frexpf(u, &e);
   exps[k] = e;
 }
 

@@ -59,6 +59,20 @@ def test_factor_names_the_first_bad_pivot(what):
     assert info.tolist() == [r + 1]
 
 
+def test_factor_of_the_largest_diagonal():
+    """Diagonal entries up to the largest float are pivots like any other, whatever stands beside them."""
+    d, top = 1024, np.float64(np.finfo(np.float32).max)
+    H = np.diag(np.full(d, top))
+    H[10, 700] = H[700, 10] = 0.5 * top
+    U, info = _factor(H.astype(np.float32))
+    assert info.tolist() == [0]
+    # the pair's block of H^-1 is 4/3 [[1, -1/2], [-1/2, 1]] / top = U^T U
+    want = np.diag(np.full(d, top ** -0.5))
+    want[10, 10] *= (4.0 / 3.0) ** 0.5
+    want[10, 700] = -0.5 * want[10, 10]
+    assert rel_fro(U, want) <= 6e-8
+
+
 def test_factor_wider_than_a_digit_product_contracts():
     """33 000 columns: a doubling step of 32 768, beyond the 16 384 steps that an int32 sum of digit products holds.
     H = S (1 + V V^T) S, and U H U^T x = x for random x, in double; U is rounded to float (6e-8 an entry, each way) on a
