@@ -34,6 +34,7 @@
 #include "tb_gemm.cuh"
 #include "tb_gemm64.cuh"
 #include "tb_i8.cuh"
+#include "tb_rcp.cuh"
 
 namespace tb {
 
@@ -108,8 +109,7 @@ __global__ void __launch_bounds__(256) k_reverse_out(double* __restrict__ Li, co
 //
 // The chain of 64 dependent pivots bounds a panel.  It runs in one warp, 16 columns at a time: lane (row, half) holds
 // 8 entries of its row of [remaining block | inverse so far] (what is eliminated on the left becomes the inverse of
-// the unit factor in the same registers), a step is a broadcast of the pivot row, a reciprocal (the hardware's
-// approximation and one third-order step) and one multiply-add per entry, about 100 clocks of dependent work.  Nothing
+// the unit factor in the same registers), a step is a broadcast of the pivot row, a reciprocal (tb_rcp.cuh) and one multiply-add per entry, about 100 clocks of dependent work.  Nothing
 // else runs on that warp's scheduler meanwhile (beside FP64 tensor steps a dependent multiply-add waits 137 clocks
 // instead of 9); the warps of the other three apply the previous panel's update to the panel rows.  Everything
 // between the blocks of 16 - solving the rows below, updating them - is FP64 tensor steps from shared memory, and so
@@ -130,13 +130,6 @@ __device__ __forceinline__ void pmma(double (&c)[2], double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
                : "+d"(c[0]), "+d"(c[1])
                : "d"(a), "d"(b));
-}
-// 1 / p: the hardware's approximation (2^-20) and one third-order step, r (1 + e + e^2) with e = 1 - p r
-__device__ __forceinline__ double panel_rcp(double p) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
-  const double e = fma(-p, r, 1.0);
-  return fma(r, fma(e, e, e), r);
 }
 
 // 16 x 16 block at (o, o) of D (lower triangle) -> inverse of its lower Cholesky factor at (o, o) of I, by one warp
