@@ -9,9 +9,9 @@
 //   k_cd_start   numerators before the pass, n0[g][i] = W_i,g . (H_out Dm)_i,g
 //   k_cd_solve   one CTA per head, 32 coordinates at a time: their chain in one warp, then the rest of the vector
 //   k_cd_apply   Dm_j += sum_g2 delta Yw[j][g2], and the scales
-// 256 rows x 256 columns, one scale per row: 1.53 ms a pass before, 0.07 ms now; 8 heads x 128 rows, 8 groups of 256
-// columns: 0.81 ms before, 0.51 ms now.  The solve costs 10 us per 32 coordinates at 1024 of them (reading K), so with
-// many groups a row the walk is the better one: 32 heads x 64 rows, 16 groups: 0.45 ms walking, 0.55 ms here.
+// The whole refinement, one pass, walking the rows and here: 8 heads x 128 rows x 1024 columns, one scale per row 0.64 and
+// 0.25 ms; 8 x 512 rows, 4 groups of 256 columns 3.90 and 1.90 ms.  The solve costs 10 us per 32 coordinates at 1024 of
+// them (reading K), and so with many groups a row the walk is the better one (cd_gram_pays).
 #include "tb_gemm.cuh"
 #include "tb_rows.cuh"
 
@@ -180,9 +180,14 @@ __global__ void __launch_bounds__(256) k_cd_apply(double* __restrict__ Dm, const
   }
 }
 
-bool cd_gram_pays(int dh, int ng) {
+// Measured, walk / triangular solve, one pass, in us.  Up to 4 groups the solve is ahead wherever it fits: 2048 coordinates
+// as 512 rows x 4 groups of 512 columns 3746 / 1031 (1 head), 4641 / 2697 (8), 7768 / 6927 (32).  With 8 groups reading the
+// heads' matrices decides, and it grows with their number: 128 x 8 groups of 256, 654 / 390 (1 head), 732 / 705 (8),
+// 1294 / 1597 (32); 64 x 8 groups of 128, 315 / 186, 343 / 224, 455 / 461; 256 x 8 groups of 128, 1520 / 1582 (8).  With 16
+// groups it is behind at 8 heads: 64 x 16, 451 / 627.
+bool cd_gram_pays(int heads, int dh, int ng) {
   const long long n = (long long)dh * ng;
-  return (ng <= 8 && n <= 1024) || (ng <= 4 && n <= CD_GRAM_MAX);
+  return (ng <= 4 && n <= CD_GRAM_MAX) || (ng <= 8 && n <= 1024 && heads * n <= 16384);
 }
 
 size_t cd_gram_doubles(int heads, int dh, int ng) {  // K, n0, delta

@@ -1205,7 +1205,7 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
     if ((size_t)p.piece_heads * head_pieces > budget) p.piece_heads = (budget / head_pieces > 1) ? (int)(budget / head_pieces) : 1;
     if (p.yw_tensor || p.dm_tensor) p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (size_t)p.piece_heads);
     const long long lines = rows;  // one set of statistics per row (the column-parallel pass keeps them all)
-    if (has_hout && cd_gram_pays(p.dh, p.ng)) p.gram = b.take<double>(cd_gram_doubles((int)(rows / p.dh), p.dh, p.ng));
+    if (has_hout && cd_gram_pays((int)(rows / p.dh), p.dh, p.ng)) p.gram = b.take<double>(cd_gram_doubles((int)(rows / p.dh), p.dh, p.ng));
     p.n0 = b.take<double>((size_t)lines * p.ng);
     p.Amat = b.take<double>((size_t)lines * p.ng * p.ng);
   }

@@ -98,7 +98,7 @@ struct CdGram {
   double* scratch;     // cd_gram_doubles
   int heads, d, seg, ng, dh;
 };
-bool cd_gram_pays(int dh, int ng);
+bool cd_gram_pays(int heads, int dh, int ng);  // heads of a batch
 size_t cd_gram_doubles(int heads, int dh, int ng);
 tb_status cd_gram_form(const CdGram& p, cudaStream_t st);
 tb_status cd_gram_pass(const CdGram& p, const double* G, double* Dm, double* sD, cudaStream_t st);

@@ -21,10 +21,11 @@ def test_groups_of_32_columns_shared_hessian():
     compare(prob, run_gpu(prob, 3, 32, 16, CD | ADAPT), 3, 32, 16, CD | ADAPT, label="gq32")
 
 
-# coordinates per head (rows x groups): 21, 256 (one group), 33 x 6, 128 x 8, 512 x 4 (the most), 64 x 16 and 128 x 24
-# (walked row by row)
+# coordinates per head (rows x groups): 21, 256 (one group), 33 x 6, 128 x 8, 512 x 4 (the most), 64 x 16, 128 x 24 and 17
+# heads of 128 x 8 (walked row by row)
 @pytest.mark.parametrize("d,heads,dh,gq,iters", [(384, 2, 21, 0, 1), (256, 1, 256, 0, 2), (384, 3, 33, 64, 1), (512, 2, 64, 32, 1),
-                                                 (1024, 1, 128, 128, 2), (512, 1, 512, 128, 1), (768, 1, 128, 32, 1)])
+                                                 (1024, 1, 128, 128, 2), (512, 1, 512, 128, 1), (768, 1, 128, 32, 1),
+                                                 (1024, 17, 128, 128, 1)])
 def test_coordinates_per_head(d, heads, dh, gq, iters):
     prob = make_problem(72, d, heads, dh, 2048, hout="spd")
     compare(prob, run_gpu(prob, 3, gq, dh, CD | ADAPT, cd_iters=iters), 3, gq, dh, CD | ADAPT, cd_iters=iters, label=f"coords{dh}")
