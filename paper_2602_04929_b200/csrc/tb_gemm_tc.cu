@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
 
-  // hunits > 1: every block of rows_per_hunit rows (a head; a multiple of 8) has its own H_in, whose
+  // hunits > 1: every block of rows_per_hunit rows (a head; a multiple of 128) has its own H_in, whose
   // pieces are stacked [piece][head][k]; the units then also run over the heads
   const int m_tiles = (rows_per_hunit + YT_BM - 1) / YT_BM, n_tilesN = (d + YT_BN - 1) / YT_BN;
   const int units_per_head = ng * n_tilesN;
@@ -222,7 +222,6 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(acce_bar(b));   // the accumulator may be overwritten
         const long long gr0 = (long long)hu * rows_per_hunit + (long long)mi * YT_BM + q * 32;
-        const long long r_end = (long long)(hu + 1) * rows_per_hunit;  // a head's last tile may be short
         const int gc0 = nj * YT_BN + hf * 64;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -233,7 +232,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
           if (gc < d) {
 #pragma unroll 8
             for (int r = 0; r < 32; ++r)
-              if (gr0 + r < r_end) Yw[((gr0 + r) * ng + g) * (long long)d + gc] = st[r * 33 + lane];
+              if (gr0 + r < rows) Yw[((gr0 + r) * ng + g) * (long long)d + gc] = st[r * 33 + lane];
           }
           __syncwarp();
         }
@@ -262,7 +261,7 @@ enum {
 
 __global__ void __launch_bounds__(YT_THREADS, 1)
     k_yw_tc_stream(float* __restrict__ Yw, const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-            int d, int seg, int ng, int n_tiles, int hunits, int rows_per_hunit) {
+            int rows, int d, int seg, int ng, int n_tiles) {
   extern __shared__ unsigned char ys_raw[];
   const uint32_t raw = smem_u32(ys_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -301,22 +300,21 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
 
   const int n_stages = seg / YS_BK;                       // stages per tile
-  const int m_tiles = (rows_per_hunit + YT_BM - 1) / YT_BM, n_tilesN = (d + YT_BN - 1) / YT_BN;
-  // tile t -> (head hu, group g, row tile of the head mi, column tile nj), column tiles innermost
-  auto tile_of = [&](int t, int& hu, int& g, int& mi, int& nj) {
+  const int m_tiles = (rows + YT_BM - 1) / YT_BM, n_tilesN = (d + YT_BN - 1) / YT_BN;
+  // tile t -> (group g, row tile mi, column tile nj), column tiles innermost
+  auto tile_of = [&](int t, int& g, int& mi, int& nj) {
     nj = t % n_tilesN;
     mi = (t / n_tilesN) % m_tiles;
-    g = (t / (n_tilesN * m_tiles)) % ng;
-    hu = t / (n_tilesN * m_tiles * ng);
+    g = t / (n_tilesN * m_tiles);
   };
 
   if (warp == 8) {
     if (lane == 0) {
       uint32_t it = 0;
       for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x) {
-        int hu, g, mi, nj;
-        tile_of(t, hu, g, mi, nj);
-        const int m0 = hu * rows_per_hunit + mi * YT_BM, n0 = nj * YT_BN, k00 = g * seg;
+        int g, mi, nj;
+        tile_of(t, g, mi, nj);
+        const int m0 = mi * YT_BM, n0 = nj * YT_BN, k00 = g * seg;
         for (int st = 0; st < n_stages; ++st, ++it) {
           const int s = it % YS_STAGES;
           const uint32_t ph = (it / YS_STAGES) & 1u;
@@ -330,7 +328,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
           for (int pc = 0; pc < 3; ++pc)
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-              tma_load_2d(sb + (pc * 2 + j) * YT_BOX, &map_b, n0 + 64 * j, (pc * hunits + hu) * d + k0, full_bar(s));
+              tma_load_2d(sb + (pc * 2 + j) * YT_BOX, &map_b, n0 + 64 * j, pc * d + k0, full_bar(s));
         }
       }
     }
@@ -374,8 +372,8 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
     const int row = q * 32 + lane;
     uint32_t tile_it = 0;
     for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x, ++tile_it) {
-      int hu, g, mi, nj;
-      tile_of(t, hu, g, mi, nj);
+      int g, mi, nj;
+      tile_of(t, g, mi, nj);
       const int b = tile_it & 1;
       if (!mbar_wait(accf_bar(b), (tile_it >> 1) & 1u, abort_flag, &g_yt_error)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -387,9 +385,9 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(acce_bar(b));   // the accumulator may be overwritten
-      const long long gr = (long long)hu * rows_per_hunit + mi * YT_BM + row;
+      const long long gr = (long long)mi * YT_BM + row;
       const int gc = nj * YT_BN + hf * 64;
-      if (mi * YT_BM + row < rows_per_hunit) {
+      if (gr < rows) {
         float* dst = Yw + (gr * ng + g) * (long long)d + gc;
 #pragma unroll
         for (int i = 0; i < 32; i += 4) {
@@ -417,7 +415,7 @@ tb_status yw_tensor(float* Yw, const unsigned char* codes, const int* zeros, con
                     __nv_bfloat16* Hp, bool split_h, long long rows, int d, int seg, int ng, int hunits,
                     cudaStream_t st) {
   const long long dd = (long long)d * d;
-  if (hunits > 1 && (rows % hunits || (rows / hunits) % 8)) return TB_ERR_UNSUPPORTED;  // a tile starts on 16 bytes
+  if (hunits > 1 && (seg > 128 || (rows / hunits) % YT_BM || rows % hunits)) return TB_ERR_UNSUPPORTED;
   if (split_h) {
     k_split3<<<148 * 8, 256, 0, st>>>(H_in, Hp, dd * hunits);
     TB_LAUNCH_CHECK();
@@ -429,10 +427,10 @@ tb_status yw_tensor(float* Yw, const unsigned char* codes, const int* zeros, con
                      64, 64, CU_TENSOR_MAP_SWIZZLE_128B));
   TB_TRY(make_map_2d(&map_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Hp, (unsigned long long)d,
                      (unsigned long long)3 * hunits * d, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B));
-  const int m_tiles = (int)((rows / hunits + YT_BM - 1) / YT_BM), n_tilesN = (d + YT_BN - 1) / YT_BN;  // of a head
+  const int m_tiles = (int)((rows + YT_BM - 1) / YT_BM), n_tilesN = (d + YT_BN - 1) / YT_BN;
   const bool resident = (seg <= 128);  // the group's slice of H_in fits next to the Wbar^T ring
   const long long n_tiles = resident ? (long long)n_tilesN * ng * hunits   // units: one (head, group, column tile) each
-                                     : (long long)m_tiles * n_tilesN * ng * hunits;
+                                     : (long long)m_tiles * n_tilesN * ng;
   if (n_tiles > 0x7fffffffll) return TB_ERR_UNSUPPORTED;
   int dev = 0, sms = 0;
   TB_CUDA_CHECK(cudaGetDevice(&dev));
@@ -452,8 +450,7 @@ tb_status yw_tensor(float* Yw, const unsigned char* codes, const int* zeros, con
     k_yw_tc<<<grid, YT_THREADS, YT_SMEM, st>>>(Yw, map_a, map_b, (int)rows, d, seg, ng, (int)n_tiles, hunits,
                                                (int)(rows / hunits));
   else
-    k_yw_tc_stream<<<grid, YT_THREADS, YS_SMEM, st>>>(Yw, map_a, map_b, d, seg, ng, (int)n_tiles, hunits,
-                                                      (int)(rows / hunits));
+    k_yw_tc_stream<<<grid, YT_THREADS, YS_SMEM, st>>>(Yw, map_a, map_b, (int)rows, d, seg, ng, (int)n_tiles);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
@@ -550,14 +547,14 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
 
   const int n_stages = (K + GS_BK - 1) / GS_BK;
-  const int n_tilesN = (N + GS_BN - 1) / GS_BN, m_tiles = (rows_per_hunit + GS_BM - 1) / GS_BM;  // row tiles of a head
+  const int n_tilesN = (N + GS_BN - 1) / GS_BN;
 
   if (warp == 8) {
     if (lane == 0) {
       uint32_t it = 0;
       for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x) {
-        const int mt = t / n_tilesN, hu = mt / m_tiles;  // the block of rows (head) whose B this tile multiplies
-        const int m0 = hu * rows_per_hunit + (mt % m_tiles) * GS_BM, n0 = (t % n_tilesN) * GS_BN;
+        const int m0 = (t / n_tilesN) * GS_BM, n0 = (t % n_tilesN) * GS_BN;
+        const int hu = (hunits > 1) ? m0 / rows_per_hunit : 0;  // the block of rows (head) whose B this tile multiplies
         for (int st = 0; st < n_stages; ++st, ++it) {
           const int s = it % GS_STAGES;
           const uint32_t ph = (it / GS_STAGES) & 1u;
@@ -619,9 +616,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
     const int row = q * 32 + lane;
     uint32_t chunk_it = 0;
     for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x) {
-      const int mt = t / n_tilesN, lm0 = (mt % m_tiles) * GS_BM;
-      const long long m0 = (long long)(mt / m_tiles) * rows_per_hunit + lm0;
-      const int n0 = (t % n_tilesN) * GS_BN;
+      const int m0 = (t / n_tilesN) * GS_BM, n0 = (t % n_tilesN) * GS_BN;
       double run[64];
 #pragma unroll
       for (int i = 0; i < 64; ++i) run[i] = 0.0;
@@ -645,8 +640,8 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
         if (lane == 0) mbar_arrive(acce_bar(b));
       }
       if (ok) {
-        const long long gm = m0 + row;
-        if (lm0 + row < rows_per_hunit && gm < M) {
+        const long long gm = (long long)m0 + row;
+        if (gm < M) {
           double* dst = C + gm * ldc + n0 + hf * 64;
 #pragma unroll
           for (int i = 0; i < 64; i += 2)
@@ -673,16 +668,16 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
 
 // C (+)= A B (double result) from operands already split: AT [3][K][M], Bp [3][K][N].
 // Requires M % 8 == 0, N % 8 == 0, K % 32 == 0.
-// hunits > 1: every block of M / hunits rows (a multiple of 8) multiplies its own B, Bp stacked [3][hunits][K][N].
+// hunits > 1: every block of M / hunits rows (a multiple of 128) multiplies its own B, Bp stacked [3][hunits][K][N].
 tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT, const __nv_bfloat16* Bp, long long M,
                               int N, int K, bool accumulate, cudaStream_t st, int hunits) {
-  if (hunits > 1 && (M % hunits || (M / hunits) % 8)) return TB_ERR_UNSUPPORTED;  // a tile starts on 16 bytes
+  if (hunits > 1 && (M % hunits || (M / hunits) % GS_BM)) return TB_ERR_UNSUPPORTED;
   CUtensorMap map_a, map_b;
   TB_TRY(make_map_2d(&map_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, AT, (unsigned long long)M, (unsigned long long)3 * K,
                      64, 32, CU_TENSOR_MAP_SWIZZLE_128B));
   TB_TRY(make_map_2d(&map_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Bp, (unsigned long long)N,
                      (unsigned long long)3 * hunits * K, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B));
-  const long long n_tiles = hunits * ((M / hunits + GS_BM - 1) / GS_BM) * (long long)((N + GS_BN - 1) / GS_BN);
+  const long long n_tiles = ((M + GS_BM - 1) / GS_BM) * (long long)((N + GS_BN - 1) / GS_BN);
   if (n_tiles > 0x7fffffffll) return TB_ERR_UNSUPPORTED;
   int dev = 0, sms = 0;
   TB_CUDA_CHECK(cudaGetDevice(&dev));

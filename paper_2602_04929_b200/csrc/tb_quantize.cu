@@ -1076,10 +1076,8 @@ struct Plan {
   unsigned long long *c_max, *w_max;
   float* Wb;
   __nv_bfloat16 *WbT, *Hp;  // tensor-core path of the blockwise product
-  bool yw_tensor;
-  bool dm_tensor;  // (Q - W) H_in through the split-bf16 tensor-core product as well
+  bool yw_tensor;    // and with it (Q - W) H_in through the split-bf16 product
   bool loss_tensor;  // the loss's own dW H_in (no scale refinement) through it too
-  int piece_heads;   // with one H_in per head: heads per launch of the refinement's products
   int loss_heads;    // with one H_in per head: heads per launch of that product (their pieces of H_in fit 2 GiB)
   size_t ws_total;
 };
@@ -1173,7 +1171,7 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
   p.Dq = p.Dm = p.Yw = p.n0 = p.Amat = p.G2 = p.gram = nullptr;
   p.Wb = nullptr;
   p.WbT = p.Hp = nullptr;
-  p.yw_tensor = p.dm_tensor = false;
+  p.yw_tensor = false;
   p.cd_rows = 0;
   if (p.cd || with_loss) {
     p.Dq = b.take<double>((size_t)p.d_out * dd);
@@ -1192,26 +1190,27 @@ static tb_status make_plan(const tb_layer_desc* D, bool has_hout, bool with_r, b
     if (!(has_hout || p.n_hin > 1) && rows > 128) rows = (rows / 128) * 128;
     p.cd_rows = rows;
     p.Yw = b.take<double>((size_t)rows * p.ng * dd);
-    // blockwise product on the tensor cores (float result): one shared H_in, groups that are whole TMA boxes
-    // With one H_in per head the heads of a batch go through the same launches, each against its own pieces of H_in.
-    const bool tiles_ok = (p.n_hin == 1 || (p.dh % 8 == 0 && rows % p.dh == 0)) && rows % 8 == 0 && p.d_out % 8 == 0 &&
-                          (p.dh % 8 == 0 || rows == p.d_out);
-    p.yw_tensor = tiles_ok && p.seg % 64 == 0;
-    p.dm_tensor = tiles_ok && p.d % 32 == 0;
-    if (p.yw_tensor) p.WbT = b.take<__nv_bfloat16>((size_t)rows * dd);
-    // with one H_in per head: as many heads per launch as their pieces of H_in fit 4 GiB, like Yw (42 of 4096 columns)
-    p.piece_heads = (p.n_hin > 1) ? (int)(rows / p.dh) : 1;
-    const size_t head_pieces = (size_t)3 * dd * dd * sizeof(__nv_bfloat16);
-    if ((size_t)p.piece_heads * head_pieces > budget) p.piece_heads = (budget / head_pieces > 1) ? (int)(budget / head_pieces) : 1;
-    if (p.yw_tensor || p.dm_tensor) p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (size_t)p.piece_heads);
+    // Products on the tensor cores, the blockwise one with a float result: one shared H_in, groups that are whole TMA boxes.
+    // With one H_in per head the heads of a batch go through the same launches, each against its own pieces of H_in
+    // (with these groups the batch of Yw holds at most 3 GiB of them): heads of whole 128-row tiles and groups of at most
+    // 128 columns.  Everything else is formed in double, its scales correctly rounded and its loss good to 1e-15; the split
+    // products leave 1e-6 of the loss and twice the scales' rounding error.
+    const bool per_head_ok = (p.n_hin > 1) && (p.dh % 128 == 0) && (p.seg <= 128) && (rows % p.dh == 0);
+    p.yw_tensor = (p.n_hin == 1 || per_head_ok) && (p.seg % 64 == 0) && (rows % 8 == 0) && (p.d_out % 8 == 0) &&
+                  (p.dh % 8 == 0 || rows == p.d_out);
+    if (p.yw_tensor) {
+      p.WbT = b.take<__nv_bfloat16>((size_t)rows * dd);
+      p.Hp = b.take<__nv_bfloat16>((size_t)3 * dd * dd * (p.n_hin > 1 ? (size_t)(rows / p.dh) : 1));
+    }
     const long long lines = rows;  // one set of statistics per row (the column-parallel pass keeps them all)
     if (has_hout && cd_gram_pays((int)(rows / p.dh), p.dh, p.ng)) p.gram = b.take<double>(cd_gram_doubles((int)(rows / p.dh), p.dh, p.ng));
     p.n0 = b.take<double>((size_t)lines * p.ng);
     p.Amat = b.take<double>((size_t)lines * p.ng * p.ng);
   }
   // without the scale refinement the loss forms dW H_in itself: the same split-bf16 product
-  // (with one H_in per head the heads of a batch share the launch, each against its own pieces)
-  p.loss_tensor = with_loss && !p.cd && (p.n_hin == 1 || p.dh % 8 == 0) && (p.d % 32 == 0) && (p.d_out % 8 == 0);
+  // (with one H_in per head the heads of a batch share the launch, each against its own pieces: that
+  // needs heads of whole 128-row tiles)
+  p.loss_tensor = with_loss && !p.cd && (p.n_hin == 1 || p.dh % 128 == 0) && (p.d % 32 == 0) && (p.d_out % 8 == 0);
   p.loss_heads = 1;
   if (p.loss_tensor && p.n_hin > 1) {
     const size_t per_head = (size_t)3 * dd * dd * sizeof(__nv_bfloat16);
@@ -1544,77 +1543,74 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     TB_LAUNCH_CHECK();
     for (long long r0 = 0; r0 < p.d_out; r0 += p.cd_rows) {
       const long long rows = (p.d_out - r0 < p.cd_rows) ? (p.d_out - r0) : p.cd_rows;
-      // Dm = (Q - W) H_in (+ W R); Yw = blockwise Wbar H_in.  With one H_in per head the batch is whole heads: on the tensor
-      // cores piece_heads of them in a launch, head by head on the FP64 engine.
-      const long long rows_per_prod = (units > 1) ? p.dh : rows;
-      const long long rows_per_launch = (units > 1) ? (long long)p.piece_heads * p.dh : rows;
-      for (long long q0 = 0; q0 < rows && (p.yw_tensor || p.dm_tensor); q0 += rows_per_launch) {
-        const long long rr = r0 + q0, rl = (rows - q0 < rows_per_launch) ? rows - q0 : rows_per_launch;
-        const int hunits = (units > 1) ? (int)(rl / p.dh) : 1;
-        const long long head0 = (units > 1) ? (rr / p.dh) * dd : 0;
-        const float* Hb = H_in + head0;
-        const bool split_h = r0 == 0 || with_r || units > 1;  // with R the pieces of R replace H_in's below
-        if (p.yw_tensor)  // also splits H_in into its bf16 pieces
-          TB_TRY(yw_tensor(reinterpret_cast<float*>(p.Yw) + q0 * p.ng * d, codes + rr * d, zeros + rr * p.ng, Hb, p.WbT, p.Hp,
-                           split_h, rl, d, p.seg, p.ng, hunits, st));
-        else if (split_h)
-          TB_TRY(split3(Hb, p.Hp, dd * hunits, st));
-        if (p.dm_tensor) {
-          // the pieces of (Q - W), transposed, live in these rows of the W~ buffer (free by now,
-          // and overwritten by G = H_out Dm only after the product)
-          __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + rr * d);
-          TB_TRY(split3_transpose(p.Dq + rr * d, DqT, rl, d, st));
-          TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rl, d, d, false, st, hunits));
-          if (with_r) {
-            // Dm += W R through the same split-bf16 product; the pieces of R take the place of H_in's
-            TB_TRY(split3_transpose(W + rr * d, DqT, rl, d, st));
-            TB_TRY(split3(R + head0, p.Hp, dd * hunits, st));
-            TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rl, d, d, true, st, hunits));
-          }
+      // Dm = (Q - W) H_in (+ W R); Yw = blockwise Wbar H_in.  With one H_in per head the batch is whole heads, which share
+      // the launches.
+      const int hunits = (units > 1) ? (int)(rows / p.dh) : 1;
+      const long long head0 = (units > 1) ? (r0 / p.dh) * dd : 0;
+      const float* Hb = H_in + head0;
+      if (p.yw_tensor) {
+        // also splits H_in into its bf16 pieces (with R the pieces of R replace them below)
+        TB_TRY(yw_tensor(reinterpret_cast<float*>(p.Yw), codes + r0 * d, zeros + r0 * p.ng, Hb, p.WbT, p.Hp,
+                         r0 == 0 || with_r || units > 1, rows, d, p.seg, p.ng, hunits, st));
+        // the pieces of (Q - W), transposed, live in this batch's rows of the W~ buffer (free by now,
+        // and overwritten by G = H_out Dm only after the product)
+        __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + r0 * d);
+        TB_TRY(split3_transpose(p.Dq + r0 * d, DqT, rows, d, st));
+        TB_TRY(gemm_split_presplit(p.Dm + r0 * d, d, DqT, p.Hp, rows, d, d, false, st, hunits));
+        if (with_r) {
+          // Dm += W R through the same split-bf16 product; the pieces of R take the place of H_in's
+          TB_TRY(split3_transpose(W + r0 * d, DqT, rows, d, st));
+          TB_TRY(split3(R + head0, p.Hp, dd * hunits, st));
+          TB_TRY(gemm_split_presplit(p.Dm + r0 * d, d, DqT, p.Hp, rows, d, d, true, st, hunits));
         }
-      }
-      for (long long q0 = 0; q0 < rows && !(p.yw_tensor && p.dm_tensor); q0 += rows_per_prod) {
-        const long long rr = r0 + q0;
-        const float* Hh = H_in + ((units > 1) ? (rr / p.dh) * dd : 0);
-        if (!p.dm_tensor) {
-          GemmP g = gemm_params();
-          g.A = p.Dq + rr * d;
-          g.a_m = d;
-          g.a_k = 1;
-          g.B = Hh;
-          g.b_k = d;
-          g.b_n = 1;
-          g.C = p.Dm + rr * d;
-          g.ldc = d;
-          g.M = (int)rows_per_prod;
-          g.N = d;
-          g.K = d;
-          TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
-          if (with_r) {
-            GemmP h = g;
-            h.A = W + rr * d;
-            h.B = R + ((units > 1) ? (rr / p.dh) * dd : 0);
-            h.beta = 1.0;
-            TB_TRY((gemm_launch<float, float, double, double, false, true>(h, st)));
-          }
+      } else {
+        const long long per = rows / hunits;  // rows against one H_in
+        GemmP g = gemm_params();
+        g.A = p.Dq + r0 * d;
+        g.a_m = d;
+        g.a_k = 1;
+        g.a_batch = per * d;
+        g.B = Hb;
+        g.b_k = d;
+        g.b_n = 1;
+        g.b_batch = dd;
+        g.C = p.Dm + r0 * d;
+        g.ldc = d;
+        g.c_batch = per * d;
+        g.M = (int)per;
+        g.N = d;
+        g.K = d;
+        g.n_batch = hunits;
+        TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
+        if (with_r) {
+          GemmP h = g;
+          h.A = W + r0 * d;
+          h.B = R + head0;
+          h.beta = 1.0;
+          TB_TRY((gemm_launch<float, float, double, double, false, true>(h, st)));
         }
-        if (!p.yw_tensor) {
+        // Yw: a launch for each group with all heads, or for each head with all groups, whichever are fewer.  Refinement of 8
+        // heads of 128 rows x 2048 columns, groups of 256: 4.00 ms head by head, 1.34 together; 32 heads x 4096, one group:
+        // 46.9 and 10.4.
+        const bool by_group = p.ng < hunits;
+        const long long head_y = per * p.ng * d;
+        for (int i = 0; i < (by_group ? p.ng : hunits); ++i) {
           GemmP y = gemm_params();
-          y.A = p.Wb + rr * d;
+          y.A = p.Wb + r0 * d + (by_group ? (long long)i * p.seg : i * per * d);
           y.a_m = d;
           y.a_k = 1;
-          y.a_batch = p.seg;
-          y.B = Hh;
+          y.a_batch = by_group ? per * d : p.seg;
+          y.B = Hb + (by_group ? (long long)i * p.seg * d : i * dd);
           y.b_k = d;
           y.b_n = 1;
-          y.b_batch = (long long)p.seg * d;
-          y.C = p.Yw + q0 * p.ng * d;
+          y.b_batch = by_group ? dd : (long long)p.seg * d;
+          y.C = p.Yw + (by_group ? (long long)i * d : i * head_y);
           y.ldc = (long long)p.ng * d;
-          y.c_batch = d;
-          y.M = (int)rows_per_prod;
+          y.c_batch = by_group ? head_y : d;
+          y.M = (int)per;
           y.N = d;
           y.K = p.seg;
-          y.n_batch = p.ng;
+          y.n_batch = by_group ? hunits : p.ng;
           TB_TRY((gemm_launch<float, float, double, double, false, true>(y, st)));
         }
       }
@@ -1852,7 +1848,7 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     } else if (!dm_is_current) {
       TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
     }
-    if (with_r && (p.loss_tensor || (dm_is_current && p.dm_tensor)) && units == 1) {
+    if (with_r && (p.loss_tensor || (dm_is_current && p.yw_tensor)) && units == 1) {
       __nv_bfloat16* WT = reinterpret_cast<__nv_bfloat16*>(p.Wt);  // W~ is no longer needed
       TB_TRY(split3_transpose(W, WT, p.d_out, d, st));
       TB_TRY(split3(R, p.Hp, dd, st));
