@@ -46,9 +46,7 @@ __global__ void __launch_bounds__(256) k_cd_gram(const TY* __restrict__ Yw, cons
       const double av = As[8 * warp + fr][4 * q + fk];
 #pragma unroll
       for (int t = 0; t < 8; ++t)
-        asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                     : "+d"(acc[t][0]), "+d"(acc[t][1])
-                     : "d"(av), "d"(Bs[8 * t + fr][4 * q + fk]));
+        dmma(acc[t], av, Bs[8 * t + fr][4 * q + fk]);
     }
     __syncthreads();
   }

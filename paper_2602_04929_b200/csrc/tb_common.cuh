@@ -79,6 +79,15 @@ inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t 
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+// One FP64 tensor step: c (8 x 8, two entries of a lane) += a (8 x 4) b (4 x 8); lane: row / column lane / 4, k lane % 4, entries
+// of c at columns 2 (lane % 4), + 1.
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+               : "+d"(c[0]), "+d"(c[1])
+               : "d"(a), "d"(b));
+}
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }  // -1022 .. 1023
+
 inline cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
 template <typename TO, typename TI>

@@ -60,7 +60,6 @@ __global__ void k_scale_exp(const float* __restrict__ H, int* __restrict__ exps,
   exps[(long long)b * dp + r] = e;
   bad[(long long)b * dp + r] = 0;
 }
-__device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
 // A (dp x dp) <- J D^-1 H D^-1 J in the leading d x d block, identity elsewhere (lower triangle and the
 // diagonal blocks only: nothing else is read).  A CTA: 8 rows x 256 columns.
@@ -76,7 +75,7 @@ __global__ void __launch_bounds__(256) k_reverse_in(const float* __restrict__ H,
   for (int k = 0; k < 8; ++k) {
     const int i = i0 + k;
     double v = (i == j) ? 1.0 : 0.0;
-    if (i < d && j < d) v = (double)Hb[(long long)(d - 1 - i) * d + (d - 1 - j)] * pow2i(-(eb[i] + ej));
+    if (i < d && j < d) v = (double)Hb[(long long)(d - 1 - i) * d + (d - 1 - j)] * pow2d(-(eb[i] + ej));
     Ab[(long long)i * dp + j] = v;
   }
 }
@@ -89,7 +88,7 @@ __global__ void __launch_bounds__(256) k_reverse_out(double* __restrict__ Li, co
   double* Lb = Li + (long long)blockIdx.z * dp * dp;
   float* Ub = U + (long long)blockIdx.z * d * d;
   const int c = d - 1 - j;
-  const double sc = pow2i(-exps[(long long)blockIdx.z * dp + c]);
+  const double sc = pow2d(-exps[(long long)blockIdx.z * dp + c]);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int i = blockIdx.y * 8 + k;
@@ -125,11 +124,6 @@ static constexpr size_t PANEL_SMEM = (size_t)(5 * 64 + 32) * PLD * sizeof(double
 __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem_dst)), "l"(gsrc)
                : "memory");
-}
-__device__ __forceinline__ void pmma(double (&c)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-               : "+d"(c[0]), "+d"(c[1])
-               : "d"(a), "d"(b));
 }
 
 // 16 x 16 block at (o, o) of D (lower triangle) -> inverse of its lower Cholesky factor at (o, o) of I, by one warp
@@ -228,7 +222,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
     for (int q = 0; q < 16; ++q)
 #pragma unroll
       for (int i = 0; i < 5; ++i)
-        if (i < nt) pmma(acc[i], sPd[(8 * fm[i] + fr) * PLD + 4 * q + fk], sPd[(8 * fn[i] + fr) * PLD + 4 * q + fk]);
+        if (i < nt) dmma(acc[i], sPd[(8 * fm[i] + fr) * PLD + 4 * q + fk], sPd[(8 * fn[i] + fr) * PLD + 4 * q + fk]);
 #pragma unroll
     for (int i = 0; i < 5; ++i)
       if (i < nt) {
@@ -244,7 +238,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
     double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll 4
     for (int q = 0; q < 16; ++q)
-      pmma(acc[q & 1], sPr[(8 * m + fr) * PLD + 4 * q + fk], sPd[(8 * n + fr) * PLD + 4 * q + fk]);
+      dmma(acc[q & 1], sPr[(8 * m + fr) * PLD + 4 * q + fk], sPd[(8 * n + fr) * PLD + 4 * q + fk]);
     double2* d = reinterpret_cast<double2*>(sR + (8 * m + fr) * PLD + 8 * n + 2 * fk);
     const double2 v = *d;
     *d = make_double2(v.x - (acc[0][0] + acc[1][0]), v.y - (acc[0][1] + acc[1][1]));
@@ -257,8 +251,8 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
       const int m = i / nfs, n = i % nfs;
       double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
       for (int q = 2 * n; q < s / 4; q += 2) {  // A^{-1}(k, n) = 0 for k < n
-        pmma(acc[0], sD[(o + s + 8 * m + fr) * PLD + o + 4 * q + fk], sI[(o + 4 * q + fk) * PLD + o + 8 * n + fr]);
-        pmma(acc[1], sD[(o + s + 8 * m + fr) * PLD + o + 4 * q + 4 + fk], sI[(o + 4 * q + 4 + fk) * PLD + o + 8 * n + fr]);
+        dmma(acc[0], sD[(o + s + 8 * m + fr) * PLD + o + 4 * q + fk], sI[(o + 4 * q + fk) * PLD + o + 8 * n + fr]);
+        dmma(acc[1], sD[(o + s + 8 * m + fr) * PLD + o + 4 * q + 4 + fk], sI[(o + 4 * q + 4 + fk) * PLD + o + 8 * n + fr]);
       }
       *reinterpret_cast<double2*>(sT + (8 * m + fr) * PLD + tc + 8 * n + 2 * fk) =
           make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
@@ -270,8 +264,8 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
       const int m = nfs - 1 - i / nfs, n = i % nfs;
       double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
       for (int q = 0; q < 2 * (m + 1); q += 2) {  // B^{-1}(m, k) = 0 for k > m
-        pmma(acc[0], sI[(o + s + 8 * m + fr) * PLD + o + s + 4 * q + fk], sT[(4 * q + fk) * PLD + tc + 8 * n + fr]);
-        pmma(acc[1], sI[(o + s + 8 * m + fr) * PLD + o + s + 4 * q + 4 + fk], sT[(4 * q + 4 + fk) * PLD + tc + 8 * n + fr]);
+        dmma(acc[0], sI[(o + s + 8 * m + fr) * PLD + o + s + 4 * q + fk], sT[(4 * q + fk) * PLD + tc + 8 * n + fr]);
+        dmma(acc[1], sI[(o + s + 8 * m + fr) * PLD + o + s + 4 * q + 4 + fk], sT[(4 * q + 4 + fk) * PLD + tc + 8 * n + fr]);
       }
       *reinterpret_cast<double2*>(sI + (o + s + 8 * m + fr) * PLD + o + 8 * n + 2 * fk) =
           make_double2(-(acc[0][0] + acc[1][0]), -(acc[0][1] + acc[1][1]));
@@ -308,7 +302,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int n = 0; n < 2; ++n) pmma(acc[n], a[q], sI[(o + 8 * n + fr) * PLD + o + 4 * q + fk]);
+        for (int n = 0; n < 2; ++n) dmma(acc[n], a[q], sI[(o + 8 * n + fr) * PLD + o + 4 * q + fk]);
       __syncwarp();
 #pragma unroll
       for (int n = 0; n < 2; ++n)
@@ -322,7 +316,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
       double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        pmma(acc[q & 1], sD[(r + fr) * PLD + o + 4 * q + fk], sD[(c + fr) * PLD + o + 4 * q + fk]);
+        dmma(acc[q & 1], sD[(r + fr) * PLD + o + 4 * q + fk], sD[(c + fr) * PLD + o + 4 * q + fk]);
       double2* d = reinterpret_cast<double2*>(sD + (r + fr) * PLD + c + 2 * fk);
       const double2 v = *d;
       *d = make_double2(v.x - (acc[0][0] + acc[1][0]), v.y - (acc[0][1] + acc[1][1]));
@@ -361,7 +355,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(double* __restrict
     for (int n = 0; n < 8; ++n) {
       double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
-      for (int q = 0; q < 2 * (n + 1); ++q) pmma(acc[q & 1], a[q], sI[(8 * n + fr) * PLD + 4 * q + fk]);
+      for (int q = 0; q < 2 * (n + 1); ++q) dmma(acc[q & 1], a[q], sI[(8 * n + fr) * PLD + 4 * q + fk]);
       *reinterpret_cast<double2*>(out + 8 * n) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
     }
   }
@@ -389,16 +383,6 @@ __global__ void k_mask_strict_upper(const double* __restrict__ src, double* __re
     const int i = (int)(idx / d), j = (int)(idx % d);
     dst[idx] = (j > i) ? src[idx] : 0.0;
   }
-}
-
-// exps[k] = exponent of the diagonal entry U_kk: the scale of row k of U^T, column k of H^{-1/2}
-__global__ void k_diag_exp(const float* __restrict__ U, int* __restrict__ exps, int d) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= d) return;
-  const float u = fabsf(U[(long long)k * d + k]);
-  int e = 0;
-  if (u > 0.0f && u < INFINITY) frexpf(u, &e);
-  exps[k] = e;
 }
 
 enum { INV_BLOCK = 512 };  // the inverse is completed block by block of this many columns (see factor_run)
@@ -997,8 +981,7 @@ extern "C" tb_status tb_prepare_correction(const float* R, const float* U_in, in
     const float* Rb = R + i * dd;
     const float* Ub = U_in + i * dd;
     if (digits) {
-      k_diag_exp<<<(d + 255) / 256, 256, 0, st>>>(Ub, w.exps, d);
-      TB_LAUNCH_CHECK();
+      TB_TRY(i8_diag_exp(Ub, w.exps, d, st));
       const I8Src r{Rb, d, 0, d, d, 1, true, true, 0, w.exps, 1};
       const I8Src ut{Ub, d, 0, d, d, 1, true, true, 2, w.exps, -1};  // row n of the operand: U[n][k], zero for k < n
       TB_TRY(i8_row_max(r, w.ma, d, st));

@@ -155,9 +155,7 @@ __device__ __forceinline__ void gemm_chunk(GemmAcc<double>& acc, const double* a
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                     : "+d"(acc.v[i][j][0]), "+d"(acc.v[i][j][1])
-                     : "d"(a[i]), "d"(b[j]));
+        dmma(acc.v[i][j], a[i], b[j]);
   }
 }
 

@@ -141,9 +141,7 @@ __global__ void __launch_bounds__(G64_THREADS, 2) gemm64_kernel(GemmP p) {
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                       : "+d"(acc[i][j][0]), "+d"(acc[i][j][1])
-                       : "d"(a[i]), "d"(b[j]));
+          dmma(acc[i][j], a[i], b[j]);
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");

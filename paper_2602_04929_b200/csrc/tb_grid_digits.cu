@@ -72,7 +72,6 @@ __host__ __device__ inline long long gd_block(const GdGeom& g, int ct, int pr, i
   return (long long)GD_PAIRS * ct * (ct + 1) / 2 + (long long)pr * (ct + 1) + c;
 }
 __device__ __forceinline__ int gd_exponent(unsigned int bits) { return (int)(bits >> 23) - 126; }  // |x| < 2^E
-__device__ __forceinline__ double gd_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
 __global__ void __launch_bounds__(256) k_gd_hmax(const float* __restrict__ H, int d, int seg, unsigned int* hmax) {
   const float* Hg = H + (long long)blockIdx.z * d * d + (long long)blockIdx.y * seg * (d + 1);
@@ -96,7 +95,7 @@ __global__ void __launch_bounds__(256) k_gd_slice(const float* __restrict__ H, G
   const int n0 = ct * 128, k0 = c * 128, nt = min(128, g.seg - n0), kn = min(128, g.seg - k0);
   const int n = threadIdx.x & 127;
   if (n >= nt) return;
-  const double scale = gd_pow2(46 - gd_exponent(hmax[gi]));
+  const double scale = pow2d(46 - gd_exponent(hmax[gi]));
   const long long blk_bytes = 2ll * g.kc * g.kc;
   unsigned char* base = dst + gi * g.blocks * blk_bytes;
   for (int kb = threadIdx.x >> 7; kb < kn / 16; kb += 2) {
@@ -215,9 +214,7 @@ __global__ void __launch_bounds__(256, NT == 128 ? 2 : 3) k_gd_h(GdP q) {
       for (int i = 0; i < MF; ++i)
 #pragma unroll
         for (int j = 0; j < NF; ++j)
-          asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                       : "+d"(acc[i][j][0]), "+d"(acc[i][j][1])
-                       : "d"(a[i]), "d"(b[j]));
+          dmma(acc[i][j], a[i], b[j]);
     }
   }
 #pragma unroll
@@ -375,23 +372,6 @@ __global__ void __launch_bounds__(256) k_gd_codes(GdP q) {
   }
 }
 
-__device__ __forceinline__ uint64_t gd_desc(uint32_t addr, uint32_t k_step) {
-  // K-major, no swizzle: core matrices of 8 rows x 16 bytes, 128 bytes apart along the rows, k_step along K
-  uint64_t d = 0;
-  d |= (uint64_t)((addr >> 4) & 0x3FFF);
-  d |= (uint64_t)((k_step >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)(128 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-__device__ __forceinline__ void gd_mma(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 __device__ __forceinline__ void gd_bulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
                "r"(bytes), "r"(bar)
@@ -536,8 +516,8 @@ __global__ void __launch_bounds__(GD_THREADS, 1) k_gd_score(GdP q, int n_work) {
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int k = 0; k < kn / 32; ++k)
-              gd_mma(tmem + 256 * buf, gd_desc(base + s * GD_A_BYTES + k * 4096, 2048),
-                     gd_desc(b_base + sb * GD_B_BYTES + k * 64 * nt, 32 * nt), idesc, (c > 0 || k > 0) ? 1u : 0u);
+              umma_i8(tmem + 256 * buf, smem_desc_k(base + s * GD_A_BYTES + k * 4096, 2048),
+                     smem_desc_k(b_base + sb * GD_B_BYTES + k * 64 * nt, 32 * nt), idesc, (c > 0 || k > 0) ? 1u : 0u);
             if (WIDE || pr == GD_PAIRS - 1) {
               umma_commit(a_empty(s));
               ++ai;
@@ -670,7 +650,7 @@ __global__ void __launch_bounds__(256) k_gd_pick(GdP q, long long lines) {
       P += q.part[(line * g.cts + c) * q.ncp + cand];
       L += q.lin[(line * g.cts + c) * q.ncp + cand];
     }
-  const double J = s * fma(s * gd_pow2(gd_exponent(hb) - 46), P, -L);
+  const double J = s * fma(s * pow2d(gd_exponent(hb) - 46), P, -L);
   const double seg = (double)g.seg;
   const double SW = 2.0 * range.z + seg * s * (q.eight ? 192.5 : 0.5);
   const double delta = (double)__uint_as_float(hb) * SW * SW * (0x1p-45 + (6.0 * seg + 64.0) * 0x1p-53);

@@ -165,9 +165,7 @@ __global__ void __launch_bounds__(CR == 128 ? 512 : 256, 1)
       for (int i = 0; i < NF; ++i)
 #pragma unroll
         for (int j = 0; j < NF; ++j)
-          asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                       : "+d"(acc[i][j][0]), "+d"(acc[i][j][1])
-                       : "d"(a[i]), "d"(b[j]));
+          dmma(acc[i][j], a[i], b[j]);
     }
     __syncthreads();
   }

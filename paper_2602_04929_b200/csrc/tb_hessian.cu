@@ -163,9 +163,7 @@ __global__ void __launch_bounds__(256, 3) k_block_gram(const TA* __restrict__ A,
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j)
-          asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                       : "+d"(acc[i][j][0]), "+d"(acc[i][j][1])
-                       : "d"(a[i]), "d"(b[j]));
+          dmma(acc[i][j], a[i], b[j]);
     }
   }
   double* Cb = C + ((long long)part * g_heads + block) * dh * dh;

@@ -43,11 +43,10 @@ __device__ __forceinline__ int i8_exponent(unsigned long long bits) {
   const int e = (int)(bits >> 52) - 1022;
   return e < -900 ? -900 : (e > 900 ? 900 : e);
 }
-__device__ __forceinline__ double i8_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 // A row with an entry that is no finite number has no digits: its largest magnitude (a bit pattern, a NaN's above
 // infinity's, both above every number's) is kept as it is, and the scale of its results is no number.
 __device__ __forceinline__ double i8_result_scale(unsigned long long bits) {
-  return (bits >> 52) >= 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : i8_pow2(i8_exponent(bits) - 54 + 24);
+  return (bits >> 52) >= 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : pow2d(i8_exponent(bits) - 54 + 24);
 }
 __device__ __forceinline__ unsigned long long i8_magnitude(double v) {
   return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
@@ -71,7 +70,7 @@ __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long*
     for (int k = k0 + lane; k < k_hi; k += 32)
       if (!i8_masked(s.mask, k, row)) {
         double v = (double)x[k];
-        if (s.k_exp) v *= i8_pow2(s.k_sign * s.k_exp[k]);
+        if (s.k_exp) v *= pow2d(s.k_sign * s.k_exp[k]);
         m = max(m, i8_magnitude(v));
       }
 #pragma unroll
@@ -86,7 +85,7 @@ __global__ void __launch_bounds__(256) k_i8_row_max(I8Src s, unsigned long long*
       const int k = k0 + i;
       if (k < s.K && !i8_masked(s.mask, k, row)) {
         double v = (double)x[(long long)k * s.ld];
-        if (s.k_exp) v *= i8_pow2(s.k_sign * s.k_exp[k]);
+        if (s.k_exp) v *= pow2d(s.k_sign * s.k_exp[k]);
         m = max(m, i8_magnitude(v));
       }
     }
@@ -132,7 +131,7 @@ __global__ void __launch_bounds__(128) k_i8_slice(I8Src s, const unsigned long l
   }
   int e = fixed_exp;
   if (max_bits) e = row < s.rows ? i8_exponent(max_bits[blockIdx.z * max_batch + row]) : 0;
-  const double scale = i8_pow2(54 - e), limit = i8_pow2(fixed_exp);
+  const double scale = pow2d(54 - e), limit = pow2d(fixed_exp);
   unsigned int w[I8_DIGITS][4];
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
@@ -142,7 +141,7 @@ __global__ void __launch_bounds__(128) k_i8_slice(I8Src s, const unsigned long l
       const int k = k0 + 4 * g + i;
       double v = (double)x[4 * g + i];
       if (i8_masked(s.mask, k, row)) v = 0.0;
-      if (s.k_exp && k < s.K) v *= i8_pow2(s.k_sign * s.k_exp[k]);
+      if (s.k_exp && k < s.K) v *= pow2d(s.k_sign * s.k_exp[k]);
       if (bad && !(fabs(v) < limit)) bad[blockIdx.z * max_batch + row] = 1;
       // |v scale| <= 2^54: adding 128 to every digit makes the bytes of the sum the digits plus 128
       const unsigned long long y = (unsigned long long)__double2ll_rn(v * scale) + 0x0080808080808080ull;
@@ -171,6 +170,20 @@ __global__ void __launch_bounds__(128) k_i8_slice(I8Src s, const unsigned long l
 #pragma unroll
   for (int n = 0; n < I8_DIGITS; ++n)
     *reinterpret_cast<uint4*>(blk + n * 1024) = make_uint4(w[n][0], w[n][1], w[n][2], w[n][3]);
+}
+
+__global__ void k_i8_diag_exp(const float* __restrict__ U, int* __restrict__ exps, int d) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= d) return;
+  const float u = fabsf(U[(long long)k * (d + 1)]);
+  int e = 0;
+  if (u > 0.0f && u < INFINITY) frexpf(u, &e);
+  exps[k] = e;
+}
+tb_status i8_diag_exp(const float* U, int* exps, int d, cudaStream_t st) {
+  k_i8_diag_exp<<<(d + 255) / 256, 256, 0, st>>>(U, exps, d);
+  TB_LAUNCH_CHECK();
+  return TB_OK;
 }
 
 tb_status i8_row_max(const I8Src& s, unsigned long long* max_bits, long long max_batch, cudaStream_t st) {
@@ -219,25 +232,8 @@ tb_status i8_slice(const I8Src& s, const unsigned long long* max_bits, long long
 
 // ------------------------------------------------------------------------------------------ the product
 
-__device__ __forceinline__ uint64_t i8_desc(uint32_t addr, uint32_t k_step) {
-  // K-major, no swizzle: core matrices of 8 rows x 16 bytes, 128 bytes apart along the rows, k_step along K
-  uint64_t d = 0;
-  d |= (uint64_t)((addr >> 4) & 0x3FFF);
-  d |= (uint64_t)((k_step >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)(128 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
 __device__ __forceinline__ uint32_t i8_idesc(uint32_t n) {  // D = s32, A = B = s8, M = 128
   return (2u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
-}
-__device__ __forceinline__ void i8_mma(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-      : "memory");
 }
 __device__ __forceinline__ void i8_tma(uint32_t dst, const CUtensorMap* map, int rb, int kb, uint32_t bar) {
   asm volatile(
@@ -377,11 +373,11 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
 #pragma unroll
           for (int i = 0; i < I8_DIGITS; ++i) {
             const int n = I8_BN * (I8_DIGITS - i);
-            const uint64_t a = i8_desc(sa + i * 2048, I8_A_BYTES / 2);
+            const uint64_t a = smem_desc_k(sa + i * 2048, I8_A_BYTES / 2);
             const uint32_t acc = (k > kb || i > 0) ? 1u : 0u;
-            i8_mma(tmem + I8_BN * i, a, i8_desc(sb, I8_B_BYTES / 2), i8_idesc(n > 256 ? 256 : n), acc);
+            umma_i8(tmem + I8_BN * i, a, smem_desc_k(sb, I8_B_BYTES / 2), i8_idesc(n > 256 ? 256 : n), acc);
             if (n > 256)
-              i8_mma(tmem + I8_BN * i + 256, a, i8_desc(sb + 4 * 1024, I8_B_BYTES / 2), i8_idesc(n - 256), acc);
+              umma_i8(tmem + I8_BN * i + 256, a, smem_desc_k(sb + 4 * 1024, I8_B_BYTES / 2), i8_idesc(n - 256), acc);
           }
           umma_commit(empty_bar(s));
         }
@@ -409,9 +405,9 @@ __global__ void __launch_bounds__(I8_THREADS, 1) k_i8_gemm(const I8K p, const __
         o[j] = o[j + 1] = o[j + 2] = o[j + 3] = 0.0;
         if (p.add && in_m && n0 + j < p.N) i8_ld4(c + j, o[j], o[j + 1], o[j + 2], o[j + 3]);
       }
-      double sa = (p.a_max && in_m) ? i8_result_scale(p.a_max[b * p.a_max_batch + m]) : i8_pow2(p.a_exp - 54 + 24);
+      double sa = (p.a_max && in_m) ? i8_result_scale(p.a_max[b * p.a_max_batch + m]) : pow2d(p.a_exp - 54 + 24);
       const double sb_mine = (p.b_max && lane < 16 && n0 + lane < p.N) ? i8_result_scale(p.b_max[b * p.b_max_batch + n0 + lane])
-                                                                       : i8_pow2(p.b_exp - 54 + 24);
+                                                                       : pow2d(p.b_exp - 54 + 24);
       if (p.negate) sa = -sa;
       if (!mbar_wait(accf_bar, tile_it & 1u, abort_flag, &g_i8_error)) break;
       __syncwarp();

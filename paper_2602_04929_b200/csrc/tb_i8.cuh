@@ -51,6 +51,8 @@ struct I8Src {
   const int* k_exp;  // or nullptr
   int k_sign;
 };
+// exps[k] = exponent of the diagonal entry U_kk of an upper factor: the scale of row k of U, column k of H^{-1/2}
+tb_status i8_diag_exp(const float* U, int* exps, int d, cudaStream_t st);
 tb_status i8_row_max(const I8Src& s, unsigned long long* max_bits, long long max_batch, cudaStream_t st);
 tb_status i8_slice(const I8Src& s, const unsigned long long* max_bits, long long max_batch, int fixed_exp,
                    const I8Mat& dst, long long rb0, long long rb_batch, int kb0, cudaStream_t st, int* bad = nullptr);

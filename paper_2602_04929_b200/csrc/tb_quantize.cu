@@ -264,9 +264,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_grid_tri(GridP p) {
       const double b = (double)bp[k4 * 4 * GT_LDB + 8 * fr[j]];
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                     : "+d"(acc[i][j][0]), "+d"(acc[i][j][1])
-                     : "d"(a[i]), "d"(b));
+        dmma(acc[i][j], a[i], b);
     }
   }
 

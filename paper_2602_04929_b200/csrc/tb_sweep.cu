@@ -69,11 +69,6 @@ struct SweepSmem {
 
 __device__ int g_sweep_error = 0;
 
-__device__ __forceinline__ void sw_mma(double (&c)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-               : "+d"(c[0]), "+d"(c[1])
-               : "d"(a), "d"(b));
-}
 template <int N>
 __device__ __forceinline__ void sw_sync(int id) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(N) : "memory");
@@ -409,11 +404,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
               const int m = fm0 + MS * mm;
               double acc[2][2] = {{old[mm].x, old[mm].y}, {0.0, 0.0}};
 #pragma unroll
-              for (int q = 0; q < 4; ++q) sw_mma(acc[q & 1], sm.Es[8 * m + fr][16 * sb + 4 * q + fk], nu[q]);
+              for (int q = 0; q < 4; ++q) dmma(acc[q & 1], sm.Es[8 * m + fr][16 * sb + 4 * q + fk], nu[q]);
               if (WITH_P)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                  sw_mma(acc[q & 1], sm.As[WITH_P ? 8 * m + fr : 0][16 * sb + 4 * q + fk], np[WITH_P ? q : 0]);
+                  dmma(acc[q & 1], sm.As[WITH_P ? 8 * m + fr : 0][16 * sb + 4 * q + fk], np[WITH_P ? q : 0]);
               *reinterpret_cast<double2*>(&sm.w[pb][8 * m + fr][8 * nn + 2 * fk]) =
                   make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
             }
@@ -430,11 +425,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
                 double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                  sw_mma(acc[q & 1], sm.Es[8 * m + fr][16 * sb + 4 * q + fk], (double)u[i][q]);
+                  dmma(acc[q & 1], sm.Es[8 * m + fr][16 * sb + 4 * q + fk], (double)u[i][q]);
                 if (WITH_P)
 #pragma unroll
                   for (int q = 0; q < 4; ++q)
-                    sw_mma(acc[q & 1], sm.As[WITH_P ? 8 * m + fr : 0][16 * sb + 4 * q + fk], (double)pp[WITH_P ? i : 0][q]);
+                    dmma(acc[q & 1], sm.As[WITH_P ? 8 * m + fr : 0][16 * sb + 4 * q + fk], (double)pp[WITH_P ? i : 0][q]);
                 double2* wp = reinterpret_cast<double2*>(&sm.w[pb][8 * m + fr][8 * n + 2 * fk]);
                 const double2 v = *wp;
                 *wp = make_double2(v.x - (acc[0][0] + acc[1][0]), v.y - (acc[0][1] + acc[1][1]));
@@ -577,8 +572,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
         if (q0 + 8 < n_steps) fetch(q0 + 8);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          sw_mma(acc[0][0][i & 3], an[i], bn[i]);
-          if (WITH_P) sw_mma(acc[0][0][(i + 2) & 3], rn[i], pn[i]);
+          dmma(acc[0][0][i & 3], an[i], bn[i]);
+          if (WITH_P) dmma(acc[0][0][(i + 2) & 3], rn[i], pn[i]);
         }
       }
       // the block being walked, piece by piece: 4 / kgroups steps of this warp each
@@ -608,8 +603,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
         for (int i = 0; i < 4; ++i)
           if (i < own) {
             const int k = 16 * sb + 4 * (kg + kgroups * i) + fk;
-            sw_mma(acc[0][0][i], sm.Es[fr][k], (double)uc[i]);
-            if (WITH_P) sw_mma(acc[0][0][(i + 2) & 3], sm.As[WITH_P ? fr : 0][k], (double)pc[i]);
+            dmma(acc[0][0][i], sm.Es[fr][k], (double)uc[i]);
+            if (WITH_P) dmma(acc[0][0][(i + 2) & 3], sm.As[WITH_P ? fr : 0][k], (double)pc[i]);
           }
       }
     } else {
@@ -643,8 +638,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
 #pragma unroll
               for (int m = 0; m < MF; ++m) {
                 const double av = ap[8 * m * a_ld + 4 * q];
-                sw_mma(acc[m][0][i % NA], av, b0);
-                sw_mma(acc[m][FW - 1][i % NA], av, b1);
+                dmma(acc[m][0][i % NA], av, b0);
+                dmma(acc[m][FW - 1][i % NA], av, b1);
               }
             }
           }
@@ -820,7 +815,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, in
       for (int n = 0; n < NF; ++n) {
         const double bd = (double)b[n];
 #pragma unroll
-        for (int m = 0; m < MF; ++m) sw_mma(acc[m][n], av[m], bd);
+        for (int m = 0; m < MF; ++m) dmma(acc[m][n], av[m], bd);
       }
     }
   };
@@ -874,16 +869,6 @@ __global__ void k_sweep_gather(SweepArgs a, double* __restrict__ work, int c1) {
   for (int c = c1 / 2 + blockIdx.y * blockDim.x + threadIdx.x; c < a.d / 2; c += gridDim.y * blockDim.x) dst[c] = src[c];
 }
 
-// exps[k] = exponent of the diagonal entry U_kk
-__global__ void k_sweep_exp(const float* __restrict__ U, int* __restrict__ exps, int d) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= d) return;
-  const float u = fabsf(U[(long long)k * (d + 1)]);
-  int e = 0;
-  if (u > 0.0f && u < INFINITY) frexpf(u, &e);
-  exps[k] = e;
-}
-
 // An update on digits costs three launches whatever its size, k_rank_rows the FP64 pipe's time for rows x width: about
 // equal at 300 rows of 4096 columns.  208 rows of 1664 with P: 11.0 ms of sweep with digits, 7.2 ms without.  With one
 // U per head the digits of all of them would have to be kept, for rows of one head each: not taken.
@@ -922,8 +907,7 @@ void sweep_scratch(Bump& b, int M, int d, bool with_p, bool use_i8, SweepScratch
 // Rows of U scale as 1 / U_kk scales the errors: the exponents of the diagonal take that out of both operands.
 tb_status sweep_prepare(const float* U, const float* P, int d, const SweepScratch& s, cudaStream_t st) {
   if (!s.use_i8) return TB_OK;
-  k_sweep_exp<<<(d + 255) / 256, 256, 0, st>>>(U, s.u_exp, d);
-  TB_LAUNCH_CHECK();
+  TB_TRY(i8_diag_exp(U, s.u_exp, d, st));
   const I8Src us{U, d, 0, d, d, 1, true, false, 1, s.u_exp, -1};
   TB_TRY(i8_row_max(us, s.u_max, d, st));
   TB_TRY(i8_slice(us, s.u_max, d, 0, s.Udig, 0, 0, 0, st));
@@ -1134,11 +1118,11 @@ __global__ void __launch_bounds__(256) k_group_panel(GroupPanelP p, int ctas_per
       double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        sw_mma(acc[q & 1], sm.Es[fr][16 * sb + 4 * q + fk], (double)sm.U[16 * sb + 4 * q + fk][8 * n + fr]);
+        dmma(acc[q & 1], sm.Es[fr][16 * sb + 4 * q + fk], (double)sm.U[16 * sb + 4 * q + fk][8 * n + fr]);
       if (WITH_P)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          sw_mma(acc[q & 1], sm.As[WITH_P ? fr : 0][16 * sb + 4 * q + fk],
+          dmma(acc[q & 1], sm.As[WITH_P ? fr : 0][16 * sb + 4 * q + fk],
                  (double)sm.P[WITH_P ? 16 * sb + 4 * q + fk : 0][8 * n + fr]);
       double2* wp = reinterpret_cast<double2*>(&sm.w[fr][8 * n + 2 * fk]);
       const double2 o = *wp;
@@ -1215,7 +1199,7 @@ __global__ void __launch_bounds__(256, 2) k_group_update(GroupPanelP p) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) sw_mma(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < 2; ++j) dmma(acc[i][j], a[i], b[j]);
     }
   }
 #pragma unroll

@@ -56,12 +56,13 @@ def test_workspace_queries_and_growth():
 
 
 def test_refinement_scratch_does_not_grow_with_the_heads_hessians():
-    """With one H_in per head their bf16 pieces (6 bytes an entry) go through at most 4 GiB at a time."""
-    def query(heads, d, n_hin, flags):
-        return tb.tb_quantize_layer_workspace(tb.layer_desc(heads * 128, d, heads, 128, 3, 0, 32, n_hin=n_hin, flags=flags), False, False)
+    """With one H_in per head the bf16 pieces of them (6 bytes an entry) are those of a batch's heads, at most 4 GiB."""
+    def query(heads, d, n_hin, group):
+        return tb.tb_quantize_layer_workspace(tb.layer_desc(heads * 128, d, heads, 128, 3, group, 32, n_hin=n_hin, flags=3), False, False)
 
     for heads, d in ((64, 8192), (96, 12288), (32, 4096)):
-        assert query(heads, d, heads, 3) - query(heads, d, 1, 3) <= 4 << 30, (heads, d)
+        for group in (0, 128):
+            assert query(heads, d, heads, group) - query(heads, d, 1, group) <= 4 << 30, (heads, d, group)
 
 
 def test_bad_descriptions_are_rejected_on_the_host():
