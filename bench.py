@@ -42,15 +42,18 @@ FLAGS_ADAPT, FLAGS_CD = 1, 2
 DEFAULT_WORKLOAD = "l2_70b_block"
 # FP64 FMA peak of the CUDA cores: 148 SMs x 64 FP64 lanes x 2 flop x 1.965 GHz (TFLOP/s)
 FP64_ALU_PEAK_TFLOPS = 148 * 64 * 2 * 1.965e9 / 1e12
-# FP32 FMA rate measured on this GPU by a register-resident FFMA loop (profiles/fp64_peak_microbench.md)
+# FP32 FMA rate measured on this GPU by a register-resident FFMA loop
 FP32_FFMA_MEASURED_TFLOPS = 71.5
-# The large double-precision products of factor, sweep and grid search are exact int8 products of seven base-256 digits,
-# 28 per multiply-add at 8192 int8 multiply-adds a clock and SM: the higher of the two rates bounds those phases (TFLOP/s)
+# The large double-precision products of factor and sweep are exact int8 products of seven base-256 digits, 28 per
+# multiply-add at 8192 int8 multiply-adds a clock and SM: the higher of the two rates bounds those phases (TFLOP/s)
 DIGITS_PEAK_TFLOPS = 148 * 8192 * 2 * 1.965e9 / 28 / 1e12
 DIGITS_KIND = ("double products as 28 int8 products on the tensor cores, 148 SM x 8192 x 2 / 28 x 1.965 GHz; the FP64 pipe "
                f"alone: {FP64_ALU_PEAK_TFLOPS:.1f}")
-# dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised under
-# profiles/ (bytes), keyed by (workload, kernel); absent where the kernel has changed since its capture
+# The grid search of many rows scores 16 candidates a row with six int8 products per multiply-add (integer codes against six
+# digits) and one FP64 product per row, an eighth of the multiply-adds counted: the slower of the two bounds it
+GRID_PEAK_TFLOPS = min(148 * 8192 * 2 * 1.965e9 / 6 / 1e12, 8 * FP64_ALU_PEAK_TFLOPS)
+GRID_KIND = "one FP64 product per row for 16 candidates, 8 x the FP64 pipe; six int8 products per candidate's multiply-add: 794"
+# dram__bytes_read.sum + dram__bytes_write.sum per launch from ncu captures (bytes), keyed by (workload, kernel); absent where the kernel has changed since its capture
 # (the mean over the launches of that kernel in one layer; the Hessian kernel's figure holds for the
 # default 262 144 tokens only)
 NCU_TRAFFIC = {
@@ -465,21 +468,23 @@ def rooflines(cfg, n_tok, m, peaks):
     bf16_kind = ("measured cuBLAS bf16, sustained (MEASURED_PEAKS.json)" if peaks else "fallback 1.59 PFLOP/s")
     out = {}
 
-    def alu(name, kernel, flops, ms):
+    def alu(name, kernel, flops, ms, peak=DIGITS_PEAK_TFLOPS, kind=DIGITS_KIND):
         if ms:
             ach = flops / (ms * 1e-3) / 1e12
-            out[name] = {"kernel": kernel, "bound": "alu", "achieved": ach, "peak": DIGITS_PEAK_TFLOPS,
-                         "unit": "TFLOP/s", "frac": ach / DIGITS_PEAK_TFLOPS, "peak_kind": DIGITS_KIND,
+            out[name] = {"kernel": kernel, "bound": "alu", "achieved": ach, "peak": peak,
+                         "unit": "TFLOP/s", "frac": ach / peak, "peak_kind": kind,
                          "frac_of_fp64_pipe": ach / FP64_ALU_PEAK_TFLOPS,
                          "frac_of_measured_fp32_ffma": ach / FP32_FFMA_MEASURED_TFLOPS, "ms": ms,
                          "traffic": NCU_TRAFFIC.get((cfg.name, kernel))}
 
     alu("sweep", "k_sweep_rows + its updates (k_i8_gemm, k_rank_rows)", sweep_flops(cfg), ph.get("sweep"))
     seg_fl = sum(16.0 * p.d_out * p.d_in * ((cfg.quant_group or p.d_in) + 1) for p in cfg.projections)
-    alu("grid", "k_gd_score, k_gd_codes, k_gd_h (k_grid_tri, k_grid_score: few rows)", seg_fl, ph.get("grid"))
+    alu("grid", "k_gd_score, k_gd_codes, k_gd_h (k_grid_tri, k_grid_score: few rows)", seg_fl, ph.get("grid"), GRID_PEAK_TFLOPS, GRID_KIND)
     alu("factor", "k_chol_panel, k_i8_gemm, gemm64_kernel", factor_flops(cfg), ph.get("factor"))
     loop_ms = ph.get("grid", 0.0) + ph.get("sweep", 0.0) + ph.get("compensation", 0.0)
-    alu("loop", "grid + sweep + compensation", loop_flops(cfg), loop_ms)
+    loop_fl = loop_flops(cfg)
+    loop_peak = loop_fl / (seg_fl / GRID_PEAK_TFLOPS + (loop_fl - seg_fl) / DIGITS_PEAK_TFLOPS)
+    alu("loop", "grid + sweep + compensation", loop_fl, loop_ms, loop_peak, "grid and the rest, each at its own peak")
     if ph.get("hessian"):
         ach = hessian_flops(cfg, n_tok) / (ph["hessian"] * 1e-3) / 1e12
         out["hessian"] = {"kernel": "k_syrk_tc / k_syrk_tc_pair from 6144 columns on (+ mirror, finalize)", "bound": "tensor", "achieved": ach, "peak": bf16_peak,

@@ -8,7 +8,7 @@
 // one of many.  One warp walks it, ONE THREAD PER ROW, 16 columns in registers, in units of the row's scale:
 //   x = v + z;  q = clamp(round(x));  v' = v_next - x U' + q U',   U' = U[j][j+1] / U[j][j],
 // so that only add (rounds), integer clamp, add (back to double) and multiply-add lie between two columns: 33 clocks
-// measured, 55 with the other multiply-adds of a 16-column piece (a warp per row with the column's error broadcast
+// measured, 58 with the other multiply-adds of a 16-column piece (56 to 60 over 8 to 4096 rows; 93 with P; a warp per row with the column's error broadcast
 // by shuffles, as it was, takes 88 and 150).  Whether a value lies outside the 31 bits that the integer clamp
 // sees is only looked at after a piece; such a piece is walked again with the test in the chain.
 // That warp has its scheduler for itself: beside FP64 tensor steps of the same scheduler a dependent multiply-add
@@ -98,7 +98,7 @@ __device__ __forceinline__ double sw_quant(double xm, int maxq, int& off) {
 }
 
 // Shared-memory accesses that the compiler leaves in their order: by itself it moves all of a piece's factor loads to
-// its beginning and spills them (78 clocks a column instead of 57).
+// its beginning and spills them (78 clocks a column instead of 58).
 __device__ __forceinline__ double2 sw_ld2(const double* p) {
   double2 v;
   asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(smem_u32(p)) : "memory");

@@ -3,7 +3,7 @@ of Propositions 3.1 / 3.2) as a function of the out-block N (the paper's Table 2
 number of coordinate-descent passes (App. F.4, Table 9), on the synthetic 4096-wide and 8192-wide
 q_proj shapes.  Every point is the GPU's loss over all heads, with the oracle's value for one sampled
 head beside the GPU's for that head (1e-4 relative, codes bit-exact: the full parity bar).  Printed as
-PROXY lines; `profiles/accuracy_proxy.md` is made from them."""
+PROXY lines."""
 import json
 
 import numpy as np

@@ -14,7 +14,7 @@ def _case(prob, bits, gq, g, flags=ADAPT):
     return compare(prob, run_gpu(prob, bits, gq, g, flags), bits, gq, g, flags, label=f"sweep g{g}")
 
 
-# rows of a step: 5 (cluster of 8), 150 (4 CTAs), 300 (4), 590 (2), 900 (8 rows a CTA), 1300 (16), 2500 (32)
+# rows of a step: 5 (cluster of 8), 150 (4 CTAs), 300 and 590 (2), 900 (8 rows a CTA), 1300 (16), 2500 (32)
 @pytest.mark.parametrize("heads,dh", [(1, 5), (6, 25), (12, 25), (10, 59), (18, 50), (13, 100), (25, 100)])
 @pytest.mark.parametrize("with_r", [False, True])
 def test_rows_per_cta(heads, dh, with_r):
