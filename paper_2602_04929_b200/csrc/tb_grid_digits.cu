@@ -18,8 +18,8 @@
 //   k_gd_score             n T n: 128 candidate rows x a column tile x two digits at a time
 //   k_gd_pick, k_gd_rescore, k_gd_repick
 // 4096 rows x 4096 columns, groups of 128, 16 candidates: 1.93 ms directly (0.48 of the FP64 pipe's rate), 0.84 ms
-// here: k_gd_score 0.30 (integer multiply-adds of the epilogue and TMEM reads, each 0.37 of their rate, tensor pipe
-// 0.29), k_gd_codes 0.25 (instructions, 0.6 of the issue slots), k_gd_h 0.22 (0.54 of the FP64 rate), k_gd_pick 0.03.
+// here: k_gd_score 0.30 (the tensor pipe 0.32 busy, reading its results 0.36, integer instructions of the epilogue 0.33),
+// k_gd_codes 0.25 (0.61 of the issue slots), k_gd_h 0.22 (FP64 tensor steps 0.56 busy), k_gd_pick 0.04.
 // Groups of 64: 2.44 -> 1.08 ms; of 32: 3.76 -> 1.88; 208 rows x one group of 1664: 0.63 -> 0.22 ms a step.
 #include "tb_grid.cuh"
 #include "tb_gemm.cuh"
