@@ -179,13 +179,15 @@ __global__ void __launch_bounds__(256) k_cd_apply(double* __restrict__ Dm, const
 }
 
 // Measured, walk / triangular solve, one pass, in us.  Up to 4 groups the solve is ahead wherever it fits: 2048 coordinates
-// as 512 rows x 4 groups of 512 columns 3746 / 1031 (1 head), 4641 / 2697 (8), 7768 / 6927 (32).  With 8 groups reading the
-// heads' matrices decides, and it grows with their number: 128 x 8 groups of 256, 654 / 390 (1 head), 732 / 705 (8),
-// 1294 / 1597 (32); 64 x 8 groups of 128, 315 / 186, 343 / 224, 455 / 461; 256 x 8 groups of 128, 1520 / 1582 (8).  With 16
-// groups it is behind at 8 heads: 64 x 16, 451 / 627.
+// as 512 rows x 4 groups of 512 columns 3746 / 1031 (1 head), 4641 / 2697 (8), 7768 / 6927 (32); with 64 heads of 256 rows x 4
+// groups of 256 2632 / 2268, with 128 they meet.  5 to 7 groups do not divide over the walk's cluster of 4 or 8 CTAs: 128 rows x
+// 5 groups of 256 1489 / 342 (8 heads), 1959 / 814 (32), 3096 / 2323 (128).  8 groups do, and reading the heads' matrices
+// decides, which grows with their number: 128 rows x 8 groups of 128, 642 / 400 (4 heads), 672 / 530 (8), 1260 / 729 (16),
+// 920 / 1043 (32), 1326 / 1656 (64); 64 rows, 586 / 291 (16), 455 / 459 (32), 644 / 732 (64).  With 16 groups it is behind at 8
+// heads: 64 rows, 451 / 627.
 bool cd_gram_pays(int heads, int dh, int ng) {
   const long long n = (long long)dh * ng;
-  return (ng <= 4 && n <= CD_GRAM_MAX) || (ng <= 8 && n <= 1024 && heads * n <= 16384);
+  return (ng <= 4 && n <= CD_GRAM_MAX) || (ng <= 8 && n <= 1024 && (ng < 8 || heads * n <= 16384));
 }
 
 size_t cd_gram_doubles(int heads, int dh, int ng) {  // K, n0, delta
