@@ -835,6 +835,9 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, in
     if (WITH_P) stage(a.P, slab + SWEEP_OUTER * T::LDF);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    // The next sweep of few rows is a handful of CTAs; they prepare their first block from the factors meanwhile (1024 rows of
+    // 4096 columns, 8 rows a step: 42.88 -> 42.38 ms).
+    pdl_trigger();
     pdl_wait();
     product(slab + (kw + fk) * T::LDF + fr, T::LDF, err);
     if (WITH_P) product(slab + (SWEEP_OUTER + kw + fk) * T::LDF + fr, T::LDF, arr);
@@ -848,7 +851,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, in
 #pragma unroll
     for (int n = 0; n < NF; ++n)
       *reinterpret_cast<double2*>(rr_part + (warp * RT + 8 * m + fr) * CT + 8 * n + 2 * fk) = make_double2(acc[m][n][0], acc[m][n][1]);
-  pdl_trigger();
+  if (!T::EARLY) pdl_trigger();
   __syncthreads();
   for (int i = threadIdx.x; i < RT * CT; i += 256) {
     const int r = i / CT, c = i % CT;
