@@ -64,22 +64,20 @@ __global__ void __launch_bounds__(256) k_row_range(GridP p, int m0, double2* ran
 }
 
 // Candidate rows: row m of the chunk and candidate k at m * ncp + k; tiles never cross units (rows of one H_in).
-// 16 warps; CR = 128: of 32 x 32; CR = 32: four of 16 x 16 times four quarters of every chunk, and what a chunk reads is
-// fetched a chunk ahead, the first one's factors before the wait: a step of few rows waits for nothing
-// else (8 rows x 256 columns 7.0 -> 6.4 us from launch to launch; 8 warps that load as they go).
+// CR = 128: 16 warps of 32 x 32; CR = 32: 8 warps, four of 16 x 16 times two halves of every chunk.
 template <int CR>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(CR == 128 ? 512 : 256, 1)
     k_grid_score(GridP p, int m0, int unit_rows, int tiles_per_unit, int col_tiles, const double2* range, double* partial) {
   extern __shared__ __align__(16) unsigned char gw_raw[];
   using Smem = GwSmem<CR>;
-  constexpr int THREADS = 512;
+  constexpr int THREADS = (CR == 128) ? 512 : 256;
   constexpr int NF = (CR == 128) ? 4 : 2;   // 8 x 8 fragments per warp and direction
-  constexpr int KSPLIT = (CR == 128) ? 1 : 4;
+  constexpr int KSPLIT = (CR == 128) ? 1 : 2;
   constexpr int WPR = (CR == 128) ? 4 : 2;  // warps along a direction
   Smem& sm = *reinterpret_cast<Smem*>(gw_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int fr = lane >> 2, fk = lane & 3;
-  const int kh = (KSPLIT == 4) ? warp >> 2 : 0;
+  const int kh = (KSPLIT == 2) ? warp >> 2 : 0;
   const int wr = (warp % (WPR * WPR)) / WPR, wc = warp % WPR;
   // the last column tiles have the longest contraction: they start first
   const int grp = blockIdx.x / col_tiles, ct = col_tiles - 1 - blockIdx.x % col_tiles;
@@ -90,6 +88,22 @@ __global__ void __launch_bounds__(512, 1)
   const int n0 = ct * CR, k_end = min(seg, n0 + CR);
   const float* H = p.Hin + ((p.units > 1) ? (long long)(p.rm.row(m0 + unit * unit_rows) / p.rm.d_head) * d * d : 0);
 
+  pdl_wait();
+  if (tid < CR) {
+    const int r = tile * rt + tid / p.ncp, k = tid % p.ncp;
+    const bool valid = r < unit_rows && k < p.n_cand;
+    double s = 1.0, z = 0.0;
+    long long src = -1;
+    if (valid) {
+      const int m = unit * unit_rows + r;
+      gw_candidate(range[(long long)m * p.ng + grp], k, p.maxq, &s, &z);
+      src = p.rm.row(m0 + m) * d + seg0;
+    }
+    sm.s[tid] = s;
+    sm.rs[tid] = 1.0 / s;
+    sm.z[tid] = z;
+    sm.src[tid] = src;
+  }
   // T chunk: rows k0 .. +63, columns n0 .. +CR-1 of the upper triangle (diagonal halved)
   constexpr int TPT = GW_KC * CR / 4 / THREADS;  // float4 per thread
   float4 tv[TPT];
@@ -116,52 +130,13 @@ __global__ void __launch_bounds__(512, 1)
       *reinterpret_cast<float4*>(&sm.T[buf][kk][c4]) = make_float4(v[0], v[1], v[2], v[3]);
     }
   };
-  fetch_t(0);
-  pdl_wait();
-  if (tid < CR) {
-    const int r = tile * rt + tid / p.ncp, k = tid % p.ncp;
-    const bool valid = r < unit_rows && k < p.n_cand;
-    double s = 1.0, z = 0.0;
-    long long src = -1;
-    if (valid) {
-      const int m = unit * unit_rows + r;
-      gw_candidate(range[(long long)m * p.ng + grp], k, p.maxq, &s, &z);
-      src = p.rm.row(m0 + m) * d + seg0;
-    }
-    sm.s[tid] = s;
-    sm.rs[tid] = 1.0 / s;
-    sm.z[tid] = z;
-    sm.src[tid] = src;
-  }
   // E chunk: thread = (candidate row, every THREADS / CR -th k)
   constexpr int EPT = GW_KC * CR / THREADS, ESTEP = THREADS / CR;
   const int e_cr = tid % CR, e_k = tid / CR;
+  fetch_t(0);
   __syncthreads();
   const double es = sm.s[e_cr], ers = sm.rs[e_cr], ez = sm.z[e_cr];
   const long long e_src = sm.src[e_cr];
-  constexpr bool AHEAD = CR == 32;
-  double wv[AHEAD ? EPT : 1];
-  auto fetch_w = [&](int k0) {
-#pragma unroll
-    for (int i = 0; i < (AHEAD ? EPT : 0); ++i) {
-      const int kk = e_k + i * ESTEP;
-      wv[AHEAD ? i : 0] = (e_src >= 0 && k0 + kk < k_end) ? p.Wt[e_src + k0 + kk] : 0.0;
-    }
-  };
-  fetch_w(0);
-  double dv[AHEAD ? NF : 1][NF][2];  // the values of the row dots
-  if (AHEAD)
-#pragma unroll
-    for (int i = 0; i < (AHEAD ? NF : 0); ++i) {
-      const long long src = sm.src[wr * NF * 8 + i * 8 + fr];
-#pragma unroll
-      for (int j = 0; j < NF; ++j) {
-        const int n = n0 + wc * NF * 8 + j * 8 + 2 * fk;  // groups are multiples of 32 columns
-        const double2 w = (src >= 0 && n < seg) ? *reinterpret_cast<const double2*>(p.Wt + src + n) : make_double2(0.0, 0.0);
-        dv[AHEAD ? i : 0][j][0] = w.x;
-        dv[AHEAD ? i : 0][j][1] = w.y;
-      }
-    }
   double acc[NF][NF][2];
 #pragma unroll
   for (int i = 0; i < NF * NF * 2; ++i) (&acc[0][0][0])[i] = 0.0;
@@ -172,14 +147,11 @@ __global__ void __launch_bounds__(512, 1)
     for (int i = 0; i < EPT; ++i) {
       const int kk = e_k + i * ESTEP;
       double e = 0.0;
-      if (e_src >= 0 && k0 + kk < k_end) e = gw_error(AHEAD ? wv[AHEAD ? i : 0] : p.Wt[e_src + k0 + kk], es, ers, ez, p.maxq);
+      if (e_src >= 0 && k0 + kk < k_end) e = gw_error(p.Wt[e_src + k0 + kk], es, ers, ez, p.maxq);
       sm.E[kk][e_cr] = e;
     }
     __syncthreads();
-    if (k0 + GW_KC < k_end) {
-      fetch_t(k0 + GW_KC);
-      fetch_w(k0 + GW_KC);
-    }
+    if (k0 + GW_KC < k_end) fetch_t(k0 + GW_KC);
     const double* ap = &sm.E[fk][wr * NF * 8 + fr];
     const float* bp = &sm.T[buf][fk][wc * NF * 8 + fr];
 #pragma unroll 4
@@ -210,7 +182,7 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int n = n0 + wc * NF * 8 + j * 8 + 2 * fk + e;
-          if (n < seg) v = fma(acc[i][j][e], gw_error(AHEAD ? dv[AHEAD ? i : 0][j][e] : p.Wt[src + n], sm.s[cr], sm.rs[cr], sm.z[cr], p.maxq), v);
+          if (n < seg) v = fma(acc[i][j][e], gw_error(p.Wt[src + n], sm.s[cr], sm.rs[cr], sm.z[cr], p.maxq), v);
         }
     }
     v += __shfl_xor_sync(0xffffffffu, v, 1);
@@ -303,7 +275,7 @@ tb_status grid_wide(const GridP& p, double* scratch, size_t scratch_doubles, cud
     if ((long long)units * tiles > 65535) return TB_ERR_UNSUPPORTED;
     const dim3 grid((unsigned)(p.ng * col_tiles), (unsigned)(units * tiles));
     if (small)
-      TB_CUDA_CHECK(launch_pdl(k_grid_score<32>, grid, dim3(512), sizeof(GwSmem<32>), st, p, u0, rows, tiles, col_tiles, range, partial));
+      TB_CUDA_CHECK(launch_pdl(k_grid_score<32>, grid, dim3(256), sizeof(GwSmem<32>), st, p, u0, rows, tiles, col_tiles, range, partial));
     else
       TB_CUDA_CHECK(launch_pdl(k_grid_score<128>, grid, dim3(512), sizeof(GwSmem<128>), st, p, u0, rows, tiles, col_tiles, range, partial));
     TB_LAUNCH_CHECK();
