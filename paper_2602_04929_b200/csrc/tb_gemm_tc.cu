@@ -51,22 +51,6 @@ __global__ void k_split3(const float* __restrict__ H, __nv_bfloat16* __restrict_
   }
 }
 
-// The same of the upper triangle that a symmetric H folds into: twice the entries right of the diagonal, the diagonal, and
-// zeros left of it (matrices of d x d one after the other; doubling is exact)
-__global__ void k_split3_folded(const float* __restrict__ H, __nv_bfloat16* __restrict__ out, int d, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int col = (int)(i % d), row = (int)((i / d) % d);
-    float x = 0.0f;
-    if (col >= row) x = (col > row) ? 2.0f * H[i] : H[i];
-    const __nv_bfloat16 p1 = __float2bfloat16_rn(x);
-    const float r1 = x - __bfloat162float(p1);
-    const __nv_bfloat16 p2 = __float2bfloat16_rn(r1);
-    out[i] = p1;
-    out[n + i] = p2;
-    out[2 * n + i] = __float2bfloat16_rn(r1 - __bfloat162float(p2));
-  }
-}
-
 // WbT[k][r] = code[r][k] - z[r][group(k)] as bf16 (exact), tiled transpose
 __global__ void k_wbar_transpose(const unsigned char* __restrict__ codes, const int* __restrict__ z,
                                  __nv_bfloat16* __restrict__ WbT, long long rows, int d, int seg, int ng) {
@@ -524,7 +508,7 @@ __global__ void k_split3_transpose(const TA* __restrict__ A, __nv_bfloat16* __re
 __global__ void __launch_bounds__(YT_THREADS, 1)
     k_gsplit_tc(double* C, long long ldc, const __grid_constant__ CUtensorMap map_a,
                 const __grid_constant__ CUtensorMap map_b, int M, int N, int K, int n_tiles, const double* add, int hunits,
-                int rows_per_hunit, int upper) {
+                int rows_per_hunit) {
   extern __shared__ unsigned char gs_raw[];
   const uint32_t raw = smem_u32(gs_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -553,7 +537,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
     mbar_fence_init();
   }
   if (warp == 8) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(256u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -562,17 +546,14 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
 
-  const int n_tilesN = (N + GS_BN - 1) / GS_BN, n_tilesM = n_tiles / n_tilesN;
-  // upper: the last column tiles, with the longest contraction, come first
-  auto m_of = [&](int t) { return (upper ? t % n_tilesM : t / n_tilesN) * GS_BM; };
-  auto n_of = [&](int t) { return (upper ? n_tilesN - 1 - t / n_tilesM : t % n_tilesN) * GS_BN; };
-  auto stages_of = [&](int t) { return (min(K, upper ? n_of(t) + GS_BN : K) + GS_BK - 1) / GS_BK; };
+  const int n_stages = (K + GS_BK - 1) / GS_BK;
+  const int n_tilesN = (N + GS_BN - 1) / GS_BN;
 
   if (warp == 8) {
     if (lane == 0) {
       uint32_t it = 0;
       for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x) {
-        const int m0 = m_of(t), n0 = n_of(t), n_stages = stages_of(t);
+        const int m0 = (t / n_tilesN) * GS_BM, n0 = (t % n_tilesN) * GS_BN;
         const int hu = (hunits > 1) ? m0 / rows_per_hunit : 0;  // the block of rows (head) whose B this tile multiplies
         for (int st = 0; st < n_stages; ++st, ++it) {
           const int s = it % GS_STAGES;
@@ -596,7 +577,6 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
       const uint32_t idesc = idesc_bf16_mn(GS_BM, GS_BN);
       uint32_t it = 0, chunk_it = 0;
       for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x) {
-        const int n_stages = stages_of(t);
         for (int st = 0; st < n_stages; ++st, ++it) {
           const int in_chunk = st % GS_CHUNK;
           const int b = chunk_it & 1;
@@ -609,7 +589,8 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
           if (!mbar_wait(full_bar(s), ph, abort_flag, &g_yt_error)) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t sa = base + s * GS_STAGE_BYTES, sb = sa + GS_A_BYTES;
-          const uint32_t tmem_d = tmem_base + (uint32_t)b * 2 * GS_BN;
+          const uint32_t tmem_d = tmem_base + (uint32_t)b * GS_BN;
+          bool first = (in_chunk == 0);
 #pragma unroll
           for (int kk = 0; kk < GS_BK / 16; ++kk) {
             // piece pairs (a, b): 1*1, 1*2, 2*1, 1*3, 3*1, 2*2
@@ -618,8 +599,8 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
             for (int i = 0; i < 6; ++i) {
               const uint64_t adesc = smem_desc_mn_sw128(sa + pa[i] * 2 * GS_BOX + kk * 2048, GS_BOX);
               const uint64_t bdesc = smem_desc_mn_sw128(sb + pb[i] * 2 * GS_BOX + kk * 2048, GS_BOX);
-              umma_bf16(tmem_d + (upper && i > 0 ? GS_BN : 0), adesc, bdesc, idesc,
-                        (in_chunk == 0 && kk == 0 && i < 1 + upper) ? 0u : 1u);
+              umma_bf16(tmem_d, adesc, bdesc, idesc, first ? 0u : 1u);
+              first = false;
             }
           }
           umma_commit(empty_bar(s));
@@ -635,7 +616,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
     const int row = q * 32 + lane;
     uint32_t chunk_it = 0;
     for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x) {
-      const int m0 = m_of(t), n0 = n_of(t), n_stages = stages_of(t);
+      const int m0 = (t / n_tilesN) * GS_BM, n0 = (t % n_tilesN) * GS_BN;
       double run[64];
 #pragma unroll
       for (int i = 0; i < 64; ++i) run[i] = 0.0;
@@ -645,22 +626,14 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
         ok = mbar_wait(accf_bar(b), (chunk_it >> 1) & 1u, abort_flag, &g_yt_error);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 2 * GS_BN + hf * 64);
+        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * GS_BN + hf * 64);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          uint32_t r[16];
-          tmem_ld_32x16(taddr + c * 16, r);
-          if (upper) {
-            uint32_t u[16];
-            tmem_ld_32x16(taddr + GS_BN + c * 16, u);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int c = 0; c < 2; ++c) {
+          uint32_t r[32];
+          tmem_ld_32x32(taddr + c * 32, r);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(u[i]));
-          } else {
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          }
-#pragma unroll
-          for (int i = 0; i < 16; ++i) run[c * 16 + i] += (double)__uint_as_float(r[i]);
+          for (int i = 0; i < 32; ++i) run[c * 32 + i] += (double)__uint_as_float(r[i]);
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -689,20 +662,15 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 8) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(256u) : "memory");
   }
 }
 
 // C = A B (+ add, laid out like C; may be C) (double result) from operands already split: AT [3][K][M], Bp [3][K][N].
 // Requires M % 8 == 0, N % 8 == 0, K % 32 == 0.
-// upper: B is upper triangular (K = N), half the contraction.  The tensor core truncates at every accumulation, always
-// towards zero, and what cancels in a product with a symmetric matrix does not in one with its folded triangle: there the
-// products of two leading pieces have an accumulator of their own (8 accumulations a chunk instead of 48), the five small
-// kinds another, and the epilogue adds the two.  Relative error of a loss against the sum in double, 512 to 8192 columns:
-// 5.7e-7 to 8.7e-7 with the whole matrix, 1.3e-6 to 4.1e-6 with the triangle in one accumulator, 1.5e-7 to 5.5e-7 in two.
 // hunits > 1: every block of M / hunits rows (a multiple of 128) multiplies its own B, Bp stacked [3][hunits][K][N].
 tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT, const __nv_bfloat16* Bp, long long M,
-                              int N, int K, const double* add, cudaStream_t st, int hunits, bool upper) {
+                              int N, int K, const double* add, cudaStream_t st, int hunits) {
   if (hunits > 1 && (M % hunits || (M / hunits) % GS_BM)) return TB_ERR_UNSUPPORTED;
   CUtensorMap map_a, map_b;
   TB_TRY(make_map_2d(&map_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, AT, (unsigned long long)M, (unsigned long long)3 * K,
@@ -724,8 +692,8 @@ tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT,
   // asking L2 at once, and less power, for the same time or less)
   const int rounds_of_tiles = (int)((n_tiles + sms - 1) / (sms > 0 ? sms : 1));
   const int grid = (int)((n_tiles + rounds_of_tiles - 1) / (rounds_of_tiles > 0 ? rounds_of_tiles : 1));
-  k_gsplit_tc<<<grid, YT_THREADS, GS_SMEM, st>>>(C, ldc, map_a, map_b, (int)M, N, K, (int)n_tiles, add, hunits,
-                                                 (int)(M / hunits), upper ? 1 : 0);
+  k_gsplit_tc<<<grid, YT_THREADS, GS_SMEM, st>>>(C, ldc, map_a, map_b, (int)M, N, K, (int)n_tiles, add,
+                                                 hunits, (int)(M / hunits));
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
@@ -733,12 +701,6 @@ tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT,
 // Bp[p][i] = piece p of B[i]
 tb_status split3(const float* B, __nv_bfloat16* Bp, long long n, cudaStream_t st) {
   k_split3<<<148 * 8, 256, 0, st>>>(B, Bp, n);
-  TB_LAUNCH_CHECK();
-  return TB_OK;
-}
-
-tb_status split3_folded(const float* H, __nv_bfloat16* Hp, int d, int n_mat, cudaStream_t st) {
-  k_split3_folded<<<148 * 8, 256, 0, st>>>(H, Hp, d, (long long)d * d * n_mat);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
@@ -760,7 +722,7 @@ tb_status gemm_split_tensor(double* C, long long ldc, const float* A, const floa
                             __nv_bfloat16* Bp, long long M, int N, int K, cudaStream_t st) {
   TB_TRY(split3(B, Bp, (long long)K * N, st));
   TB_TRY(split3_transpose(A, AT, M, K, st, 1.0f));
-  return gemm_split_presplit(C, ldc, AT, Bp, M, N, K, nullptr, st, 1, false);
+  return gemm_split_presplit(C, ldc, AT, Bp, M, N, K, nullptr, st, 1);
 }
 
 int yw_error_read_clear() {

@@ -32,12 +32,11 @@ namespace tb {
 tb_status yw_tensor(float* Yw, const unsigned char* codes, const int* zeros, const float* H_in, __nv_bfloat16* WbT,
                     __nv_bfloat16* Hp, bool split_h, long long rows, int d, int seg, int ng, int hunits,
                     cudaStream_t st);
-// C (+)= A B in double from operands split into three bf16 pieces each (tb_gemm_tc.cu)
+// C = A B (+ add) in double from operands split into three bf16 pieces each (tb_gemm_tc.cu)
 tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT, const __nv_bfloat16* Bp, long long M,
-                              int N, int K, const double* add, cudaStream_t st, int hunits = 1, bool upper = false);
+                              int N, int K, const double* add, cudaStream_t st, int hunits = 1);
 tb_status split3_transpose(const double* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st, double scale = 1.0);
 tb_status split3_transpose(const float* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st, float scale = 1.0f);
-tb_status split3_folded(const float* H, __nv_bfloat16* Hp, int d, int n_mat, cudaStream_t st);
 tb_status split3(const float* B, __nv_bfloat16* Bp, long long n, cudaStream_t st);
 }
 
@@ -1841,14 +1840,16 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     // Z = dW H_in (+ 2 W R).  After the scale refinement without R the buffer Dm already holds
     // dW H_in for the final scales (it was kept current through the pass), so the product is skipped.
     // With R the pass keeps Dm = dW H_in + W R, so only one more W R is missing.
-    // The loss is symmetric in the two dW, and H_in and H_out are symmetric, so a product of its own takes the upper triangle
-    // that H_in folds into instead of H_in: half the contraction.  4096 rows and columns 0.69 -> 0.42 ms.
+    // A product of its own takes all of H_in, not the triangle that it folds into (the loss is symmetric in the two dW): half
+    // the contraction (4096 rows and columns 0.69 -> 0.42 ms), but what cancels inside dW H_in then cancels after the tensor
+    // core's truncating float sums.  Relative error of the loss, 1024 to 2048 columns with a common factor of ten times the usual
+    // strength: 0.5e-6 to 1.5e-6 with all of H_in, 2.4e-6 to 3.6e-6 with the triangle; 8 bits, damping 1e-4: up to 4.4e-6, 17e-6.
     const bool dm_is_current = p.cd;
     if (!dm_is_current && p.loss_tensor && units == 1) {
       __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt);  // W~ is no longer needed
       TB_TRY(split3_transpose(p.Dq, DqT, p.d_out, d, st));
-      TB_TRY(split3_folded(H_in, p.Hp, d, 1, st));
-      TB_TRY(gemm_split_presplit(p.Dm, d, DqT, p.Hp, p.d_out, d, d, nullptr, st, 1, true));
+      TB_TRY(split3(H_in, p.Hp, dd, st));
+      TB_TRY(gemm_split_presplit(p.Dm, d, DqT, p.Hp, p.d_out, d, d, nullptr, st));
     } else if (!dm_is_current && p.loss_tensor) {
       // one H_in per head: a batch of heads per launch, every head against its own pieces
       for (int h0 = 0; h0 < p.H; h0 += p.loss_heads) {
@@ -1856,8 +1857,8 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
         const long long rr = (long long)h0 * p.dh, rows = (long long)nb * p.dh;
         __nv_bfloat16* DqT = reinterpret_cast<__nv_bfloat16*>(p.Wt + rr * d);  // W~ is no longer needed
         TB_TRY(split3_transpose(p.Dq + rr * d, DqT, rows, d, st));
-        TB_TRY(split3_folded(H_in + (long long)h0 * dd, p.Hp, d, nb, st));
-        TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rows, d, d, nullptr, st, nb, true));
+        TB_TRY(split3(H_in + (long long)h0 * dd, p.Hp, dd * nb, st));
+        TB_TRY(gemm_split_presplit(p.Dm + rr * d, d, DqT, p.Hp, rows, d, d, nullptr, st, nb));
       }
     } else if (!dm_is_current) {
       TB_TRY((gemm_launch<double, float, double, double, false, true>(g, st)));
