@@ -476,16 +476,16 @@ enum {
   GS_SMEM = GS_STAGES * GS_STAGE_BYTES + 1024 + 256
 };
 
-// AT[p][k][m] = piece p of scale A[m][k] (scale a power of two); a double input keeps its leading 24 bits
+// AT[p][k][m] = piece p of A[m][k]; a double input keeps its leading 24 bits
 template <typename TA>
-__global__ void k_split3_transpose(const TA* __restrict__ A, __nv_bfloat16* __restrict__ AT, long long M, int K, TA scale) {
+__global__ void k_split3_transpose(const TA* __restrict__ A, __nv_bfloat16* __restrict__ AT, long long M, int K) {
   __shared__ TA tile[32][33];
   const long long m0 = (long long)blockIdx.y * 32;
   const int k0 = blockIdx.x * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const long long m = m0 + i;
     const int k = k0 + threadIdx.x;
-    tile[i][threadIdx.x] = (m < M && k < K) ? scale * A[m * K + k] : (TA)0;
+    tile[i][threadIdx.x] = (m < M && k < K) ? A[m * K + k] : (TA)0;
   }
   __syncthreads();
   const long long plane = (long long)K * M;
@@ -508,7 +508,7 @@ __global__ void k_split3_transpose(const TA* __restrict__ A, __nv_bfloat16* __re
 __global__ void __launch_bounds__(YT_THREADS, 1)
     k_gsplit_tc(double* C, long long ldc, const __grid_constant__ CUtensorMap map_a,
                 const __grid_constant__ CUtensorMap map_b, int M, int N, int K, int n_tiles, const double* add, int hunits,
-                int rows_per_hunit) {
+                int rows_per_hunit, double alpha) {
   extern __shared__ unsigned char gs_raw[];
   const uint32_t raw = smem_u32(gs_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
 #pragma unroll
           for (int i = 0; i < 64; i += 2)
             if (n0 + hf * 64 + i + 1 < N) {
-              double2 v = make_double2(run[i], run[i + 1]);
+              double2 v = make_double2(alpha * run[i], alpha * run[i + 1]);
               if (add) {
                 const double2 old = *reinterpret_cast<const double2*>(add + at + i);
                 v.x += old.x;
@@ -666,11 +666,11 @@ __global__ void __launch_bounds__(YT_THREADS, 1)
   }
 }
 
-// C = A B (+ add, laid out like C; may be C) (double result) from operands already split: AT [3][K][M], Bp [3][K][N].
+// C = alpha A B (+ add, laid out like C; may be C) (double result) from operands already split: AT [3][K][M], Bp [3][K][N].
 // Requires M % 8 == 0, N % 8 == 0, K % 32 == 0.
 // hunits > 1: every block of M / hunits rows (a multiple of 128) multiplies its own B, Bp stacked [3][hunits][K][N].
 tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT, const __nv_bfloat16* Bp, long long M,
-                              int N, int K, const double* add, cudaStream_t st, int hunits) {
+                              int N, int K, const double* add, cudaStream_t st, int hunits, double alpha) {
   if (hunits > 1 && (M % hunits || (M / hunits) % GS_BM)) return TB_ERR_UNSUPPORTED;
   CUtensorMap map_a, map_b;
   TB_TRY(make_map_2d(&map_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, AT, (unsigned long long)M, (unsigned long long)3 * K,
@@ -693,7 +693,7 @@ tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT,
   const int rounds_of_tiles = (int)((n_tiles + sms - 1) / (sms > 0 ? sms : 1));
   const int grid = (int)((n_tiles + rounds_of_tiles - 1) / (rounds_of_tiles > 0 ? rounds_of_tiles : 1));
   k_gsplit_tc<<<grid, YT_THREADS, GS_SMEM, st>>>(C, ldc, map_a, map_b, (int)M, N, K, (int)n_tiles, add,
-                                                 hunits, (int)(M / hunits));
+                                                 hunits, (int)(M / hunits), alpha);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
@@ -705,14 +705,14 @@ tb_status split3(const float* B, __nv_bfloat16* Bp, long long n, cudaStream_t st
   return TB_OK;
 }
 
-tb_status split3_transpose(const float* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st, float scale) {
-  k_split3_transpose<float><<<dim3((K + 31) / 32, (unsigned)((M + 31) / 32)), dim3(32, 8), 0, st>>>(A, AT, M, K, scale);
+tb_status split3_transpose(const float* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st) {
+  k_split3_transpose<float><<<dim3((K + 31) / 32, (unsigned)((M + 31) / 32)), dim3(32, 8), 0, st>>>(A, AT, M, K);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
 
-tb_status split3_transpose(const double* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st, double scale) {
-  k_split3_transpose<double><<<dim3((K + 31) / 32, (unsigned)((M + 31) / 32)), dim3(32, 8), 0, st>>>(A, AT, M, K, scale);
+tb_status split3_transpose(const double* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st) {
+  k_split3_transpose<double><<<dim3((K + 31) / 32, (unsigned)((M + 31) / 32)), dim3(32, 8), 0, st>>>(A, AT, M, K);
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
@@ -721,8 +721,8 @@ tb_status split3_transpose(const double* A, __nv_bfloat16* AT, long long M, int 
 tb_status gemm_split_tensor(double* C, long long ldc, const float* A, const float* B, __nv_bfloat16* AT,
                             __nv_bfloat16* Bp, long long M, int N, int K, cudaStream_t st) {
   TB_TRY(split3(B, Bp, (long long)K * N, st));
-  TB_TRY(split3_transpose(A, AT, M, K, st, 1.0f));
-  return gemm_split_presplit(C, ldc, AT, Bp, M, N, K, nullptr, st, 1);
+  TB_TRY(split3_transpose(A, AT, M, K, st));
+  return gemm_split_presplit(C, ldc, AT, Bp, M, N, K, nullptr, st, 1, 1.0);
 }
 
 int yw_error_read_clear() {

@@ -32,11 +32,11 @@ namespace tb {
 tb_status yw_tensor(float* Yw, const unsigned char* codes, const int* zeros, const float* H_in, __nv_bfloat16* WbT,
                     __nv_bfloat16* Hp, bool split_h, long long rows, int d, int seg, int ng, int hunits,
                     cudaStream_t st);
-// C = A B (+ add) in double from operands split into three bf16 pieces each (tb_gemm_tc.cu)
+// C = alpha A B (+ add) in double from operands split into three bf16 pieces each (tb_gemm_tc.cu)
 tb_status gemm_split_presplit(double* C, long long ldc, const __nv_bfloat16* AT, const __nv_bfloat16* Bp, long long M,
-                              int N, int K, const double* add, cudaStream_t st, int hunits = 1);
-tb_status split3_transpose(const double* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st, double scale = 1.0);
-tb_status split3_transpose(const float* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st, float scale = 1.0f);
+                              int N, int K, const double* add, cudaStream_t st, int hunits = 1, double alpha = 1.0);
+tb_status split3_transpose(const double* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st);
+tb_status split3_transpose(const float* A, __nv_bfloat16* AT, long long M, int K, cudaStream_t st);
 tb_status split3(const float* B, __nv_bfloat16* Bp, long long n, cudaStream_t st);
 }
 
@@ -1868,9 +1868,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
       TB_LAUNCH_CHECK();
     } else if (with_r && p.loss_tensor && units == 1) {
       __nv_bfloat16* WT = reinterpret_cast<__nv_bfloat16*>(p.Wt);  // W~ is no longer needed
-      TB_TRY(split3_transpose(W, WT, p.d_out, d, st, 2.0f));       // 2 W
+      TB_TRY(split3_transpose(W, WT, p.d_out, d, st));
       TB_TRY(split3(R, p.Hp, dd, st));
-      TB_TRY(gemm_split_presplit(p.Dm, d, WT, p.Hp, p.d_out, d, d, p.Dm, st));
+      // doubled in the double result: 2 W would not hold entries above half the float range
+      TB_TRY(gemm_split_presplit(p.Dm, d, WT, p.Hp, p.d_out, d, d, p.Dm, st, 1, 2.0));
     } else if (with_r) {
       GemmP h = g;
       h.A = W;

@@ -142,3 +142,22 @@ def test_loss_after_refinement(d, heads, d_head, gq, hout):
     out = _quantized(p, heads, 4, gq, 3)
     terms = _loss_terms(p, out, heads, gq)
     assert ((out.loss - sum(terms)).abs() <= TRUNCATION * sum(abs(t) for t in terms)).all(), (out.loss, terms)
+
+
+# Weights in the upper half of the float range: every step scales by powers of two (the sweep takes ratios of entries of U), so
+# codes and loss are those of ordinary weights (up to pieces of small entries below the smallest bf16)
+@pytest.mark.parametrize("hout", [False, True])
+@pytest.mark.parametrize("flags", [1, 3])
+@pytest.mark.parametrize("with_r", [False, True])
+def test_loss_of_weights_near_the_float_range(hout, flags, with_r):
+    p = _correlated(256, 1, 128, 1, hout, with_r, 1e-2)
+    a = _quantized(p, 1, 4, 128, flags)
+    w, h = 127 - int(torch.floor(torch.log2(p["W"].abs().max()))), -24
+    q = dict(p, W=(p["W"].double() * 2.0 ** w).float(), H=p["H"] * 2.0 ** h)
+    if with_r:
+        q["R"] = p["R"] * 2.0 ** h
+    assert 2.0 ** 127 <= float(q["W"].abs().max()) < 2.0 ** 128
+    b = _quantized(q, 1, 4, 128, flags)
+    assert torch.equal(a.codes, b.codes)
+    want = a.loss * 2.0 ** (2 * w + h)
+    assert ((b.loss - want).abs() <= TRUNCATION * want.abs()).all(), (b.loss, want)
