@@ -59,8 +59,9 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 // one's CTAs start while the last of the one before still run (programmatic dependent launch).  Every kernel launched this
 // way calls pdl_wait() before it touches anything that an earlier kernel writes or reads back (it returns when the kernel
 // before has completed, which waited in turn), and pdl_trigger() shortly before its end: earlier, the next kernel's CTAs
-// would hold places that another stream's kernels could use.  (Where the next kernel is a handful of CTAs, earlier: it
-// may then start before the kernel before this one has ended, and has to wait for all it did not find at the call's start.)  None of their parameters is `const __restrict__`, and __ldg is
+// would hold places that another stream's kernels could use.  (k_rank_rows calls it earlier where the
+// next kernel's CTAs leave half of the SMs free: that one may then start before the kernel before this one has ended, and has
+// to wait for all it did not find at the call's start.)  None of their parameters is `const __restrict__`, and __ldg is
 // for what the whole call leaves alone (U, P): both promise that the data does not change while the kernel lives, which
 // here begins before the kernel that writes it has ended, and free the compiler to load it ahead of the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -759,25 +759,38 @@ static tb_status sweep_launch(SweepP p, cudaStream_t st) {
   return TB_OK;
 }
 
-tb_status sweep_columns(const SweepArgs& a, cudaStream_t st) {
+// How a launch over nblk blocks of 128 columns is split: rows a CTA, CTAs a cluster, CTAs in all.
+struct SweepShape {
+  int rows, cs;
+  long long ctas;
+};
+static SweepShape sweep_shape(int rows_per_unit, int units, bool with_p, int nblk) {
   const long long sms = 148;
+  const long long groups = (long long)((rows_per_unit + 7) / 8) * units;  // of 8 rows
+  // few rows: a cluster per group of 8 rows shares the contraction
+  if (nblk > 1 && groups * 2 <= sms) {
+    const int cs = (groups * 8 <= sms) ? 8 : (groups * 4 <= sms) ? 4 : 2;
+    return {8, cs, groups * cs};
+  }
+  // more rows per CTA as soon as 8 would take another round of CTAs: the chain's time does not depend on them
+  // (with both factors the registers of 16 rows spill)
+  if (with_p || groups <= sms) return {8, 1, groups};
+  const long long g16 = (long long)((rows_per_unit + 15) / 16) * units;
+  if (g16 <= sms) return {16, 1, g16};
+  return {32, 1, (long long)((rows_per_unit + 31) / 32) * units};
+}
+
+tb_status sweep_columns(const SweepArgs& a, cudaStream_t st) {
   SweepP p;
   p.a = a;
   p.rows_per_unit = a.M / a.units;
   p.ctas_per_unit = 0;
-  p.cs = 1;
-  const long long groups = (long long)((p.rows_per_unit + 7) / 8) * a.units;  // of 8 rows
-  const int nblk = a.blk1 - a.blk0;
-  // few rows: a cluster per group of 8 rows shares the contraction
-  if (nblk > 1 && groups * 2 <= sms) {
-    p.cs = (groups * 8 <= sms) ? 8 : (groups * 4 <= sms) ? 4 : 2;
-    return a.P ? sweep_launch<true, 8, true>(p, st) : sweep_launch<false, 8, true>(p, st);
-  }
-  // more rows per CTA as soon as 8 would take another round of CTAs: the chain's time does not depend on them
-  const long long g16 = (long long)((p.rows_per_unit + 15) / 16) * a.units;
-  if (a.P) return sweep_launch<true, 8, false>(p, st);  // the registers of 16 rows with both factors spill
-  if (groups <= sms) return sweep_launch<false, 8, false>(p, st);
-  return g16 <= sms ? sweep_launch<false, 16, false>(p, st) : sweep_launch<false, 32, false>(p, st);
+  const SweepShape s = sweep_shape(p.rows_per_unit, a.units, a.P != nullptr, a.blk1 - a.blk0);
+  p.cs = s.cs;
+  if (s.cs > 1) return a.P ? sweep_launch<true, 8, true>(p, st) : sweep_launch<false, 8, true>(p, st);
+  if (a.P) return sweep_launch<true, 8, false>(p, st);
+  if (s.rows == 8) return sweep_launch<false, 8, false>(p, st);
+  return s.rows == 16 ? sweep_launch<false, 16, false>(p, st) : sweep_launch<false, 32, false>(p, st);
 }
 
 
@@ -788,6 +801,8 @@ tb_status sweep_columns(const SweepArgs& a, cudaStream_t st) {
 // Bound: reading U (HBM / L2) for 8 rows, the FP64 pipe from about 64 on.  Up to 16 rows the sweep before leaves most SMs
 // idle: the factors are copied into shared memory before the sweep has ended.
 // 8 rows x 4096 columns: 3.5 us from the sweep's end to this kernel's, 9.5 when the loads came after the wait.
+// ahead: the sweep that follows is launched before this kernel's own wait and prepares its first block from the factors
+// meanwhile (RANK_AHEAD_CTAS).
 // ---------------------------------------------------------------------------
 template <bool WITH_P, int MF>
 struct RankTile {
@@ -800,7 +815,7 @@ struct RankTile {
 
 template <bool WITH_P, int MF>
 __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, int rows_per_unit, int k0, int c1, const double* err,
-                                                   const double* arr) {
+                                                   const double* arr, int ahead) {
   using T = RankTile<WITH_P, MF>;
   constexpr int NF = 4, RT = T::RT, CT = T::CT, STEPS = SWEEP_OUTER / 32;
   extern __shared__ __align__(16) double rr_part[];  // [8][RT][CT], then the factors
@@ -847,9 +862,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, in
     if (WITH_P) stage(a.P, slab + SWEEP_OUTER * T::LDF);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    // The next sweep of few rows is a handful of CTAs; they prepare their first block from the factors meanwhile (1024 rows of
-    // 4096 columns, 8 rows a step: 42.88 -> 42.38 ms).
-    pdl_trigger();
+    if (ahead) pdl_trigger();
     pdl_wait();
     product(slab + (kw + fk) * T::LDF + fr, T::LDF, err);
     if (WITH_P) product(slab + (SWEEP_OUTER + kw + fk) * T::LDF + fr, T::LDF, arr);
@@ -863,7 +876,7 @@ __global__ void __launch_bounds__(256) k_rank_rows(SweepArgs a, double* work, in
 #pragma unroll
     for (int n = 0; n < NF; ++n)
       *reinterpret_cast<double2*>(rr_part + (warp * RT + 8 * m + fr) * CT + 8 * n + 2 * fk) = make_double2(acc[m][n][0], acc[m][n][1]);
-  if (!T::EARLY) pdl_trigger();
+  if (!ahead) pdl_trigger();
   __syncthreads();
   for (int i = threadIdx.x; i < RT * CT; i += 256) {
     const int r = i / CT, c = i % CT;
@@ -934,16 +947,24 @@ tb_status sweep_prepare(const float* U, const float* P, int d, const SweepScratc
   return TB_OK;
 }
 
+// CTAs, of a whole SM each, of a sweep that the update before it launches ahead of its own wait: at most half of the SMs, so
+// that another stream's kernels find room while they wait.  Rows a step in 2048 or 4096 columns, without -> with: a sweep of 8
+// CTAs 41.00 -> 40.56 ms, 16 CTAs 2.811 -> 2.788, 32 CTAs 2.931 -> 2.901, 64 CTAs 3.404 -> 3.366, 128 CTAs 3.116 -> 3.108 (the
+// runs of one side differ by as much).
+constexpr int RANK_AHEAD_CTAS = 74;
+
 template <bool WITH_P, int MF>
 static tb_status rank_launch(const SweepArgs& a, double* work, int rows_per_unit, int k0, int c1, const double* err,
-                             const double* arr, cudaStream_t st) {
+                             const double* arr, int next_blocks, cudaStream_t st) {
   constexpr int CT = RankTile<WITH_P, MF>::CT;
   constexpr size_t smem = RankTile<WITH_P, MF>::smem;
   static bool configured[64] = {false};
   auto kern = k_rank_rows<WITH_P, MF>;
   TB_TRY(allow_smem(kern, smem, configured));
   const dim3 grid((a.d - c1 + CT - 1) / CT, (rows_per_unit + 8 * MF - 1) / (8 * MF), a.units);
-  TB_CUDA_CHECK(launch_pdl(kern, grid, dim3(256), smem, st, a, work, rows_per_unit, k0, c1, err, arr));
+  const int ahead =
+      RankTile<WITH_P, MF>::EARLY && sweep_shape(rows_per_unit, a.units, WITH_P, next_blocks).ctas <= RANK_AHEAD_CTAS;
+  TB_CUDA_CHECK(launch_pdl(kern, grid, dim3(256), smem, st, a, work, rows_per_unit, k0, c1, err, arr, ahead));
   TB_LAUNCH_CHECK();
   return TB_OK;
 }
@@ -1005,15 +1026,15 @@ tb_status sweep_step(SweepArgs a, const SweepScratch& s, cudaStream_t st) {
       }
     } else {
       // rows per tile: 8, 16 or 32, as few tiles as cover the unit's rows
-      const int mf = rows_per_unit <= 8 ? 1 : rows_per_unit <= 16 ? 2 : 4;
+      const int mf = rows_per_unit <= 8 ? 1 : rows_per_unit <= 16 ? 2 : 4, nb = nblk - b1 < OB ? nblk - b1 : OB;
       if (a.P) {
-        if (mf == 1) TB_TRY((rank_launch<true, 1>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
-        if (mf == 2) TB_TRY((rank_launch<true, 2>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
-        if (mf == 4) TB_TRY((rank_launch<true, 4>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+        if (mf == 1) TB_TRY((rank_launch<true, 1>(a, s.work, rows_per_unit, k0, c1, E, A, nb, st)));
+        if (mf == 2) TB_TRY((rank_launch<true, 2>(a, s.work, rows_per_unit, k0, c1, E, A, nb, st)));
+        if (mf == 4) TB_TRY((rank_launch<true, 4>(a, s.work, rows_per_unit, k0, c1, E, A, nb, st)));
       } else {
-        if (mf == 1) TB_TRY((rank_launch<false, 1>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
-        if (mf == 2) TB_TRY((rank_launch<false, 2>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
-        if (mf == 4) TB_TRY((rank_launch<false, 4>(a, s.work, rows_per_unit, k0, c1, E, A, st)));
+        if (mf == 1) TB_TRY((rank_launch<false, 1>(a, s.work, rows_per_unit, k0, c1, E, A, nb, st)));
+        if (mf == 2) TB_TRY((rank_launch<false, 2>(a, s.work, rows_per_unit, k0, c1, E, A, nb, st)));
+        if (mf == 4) TB_TRY((rank_launch<false, 4>(a, s.work, rows_per_unit, k0, c1, E, A, nb, st)));
       }
     }
     a.src = s.work;

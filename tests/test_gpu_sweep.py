@@ -34,6 +34,14 @@ def test_one_hessian_per_head(n_hin):
     _case(prob, 4, 64, 20)
 
 
+# the sweep after an update of few rows: 48 CTAs, launched ahead of the update's own wait, and 96, which are not
+@pytest.mark.parametrize("n_hin", [3, 12])
+@pytest.mark.parametrize("with_r", [False, True])
+def test_one_hessian_per_head_beyond_512_columns(n_hin, with_r):
+    prob = make_problem(67, 768, n_hin, 32, 1024, n_hin=n_hin, with_r=with_r, hout="spd")
+    _case(prob, 3, 128, 16)
+
+
 def test_one_hessian_per_head_and_many_rows():
     """As many rows of as many columns as take digit products with a shared factor: with one per head they do not."""
     prob = make_problem(66, 640, 2, 1920, 1024, n_hin=2, hout=None)
