@@ -341,10 +341,12 @@ __global__ void k_residual(const double* __restrict__ Wt, const unsigned char* _
 // rows x 128 columns of one head; thread: 8 rows x 2 columns, the group's rows 32 at a time from shared memory.  E is the
 // group's residual W~ - s (code - z), formed where it is needed, or (HAVE_E, propagated error) a matrix.
 // Bound: reading and writing W~ once.  As a residual launch and a product of the 128 x 128 engine it took, per step of
-// one row in 8 heads x 4096 columns, 24 us, of 32 rows in 32 heads 115 us; now 12 us and 80 us.
-// In short steps it is the loads that follow one another: the matrices come ahead of the wait for the sweep, the rows to be
-// updated beside the residual (256 rows of 256 columns in 32 steps, whole chain 1.70 -> 1.66 ms).
-template <bool HAVE_E>
+// one row in 8 heads x 4096 columns, 24 us, of 32 rows in 32 heads 115 us; now 13 us and 82 us.
+// AHEAD: in short launches it is the loads that follow one another, so the matrices come ahead of the wait for the sweep and
+// the rows to be updated beside the residual (256 rows of 256 columns in 32 steps, whole chain 1.70 -> 1.66 ms).  Held through
+// the product, those rows take 128 registers instead of 74 (64 with HAVE_E), two CTAs an SM instead of three (four): where
+// several waves of CTAs hide one another's loads anyway it loses (comp_ahead()).
+template <bool HAVE_E, bool AHEAD>
 __global__ void __launch_bounds__(256) k_compensate(double* Wt, const unsigned char* codes, const double* sD, const int* z,
                                                     const double* E, const double* T, int i0, int g, int dh,
                                                     long long t_head, int d, int seg, int ng) {
@@ -359,13 +361,16 @@ __global__ void __launch_bounds__(256) k_compensate(double* Wt, const unsigned c
       Ts[c][r] = (q0 + r < nrem) ? Th[(long long)(q0 + r) * g + e0 + c] : 0.0;
     }
   };
-  matrices(0, min(32, g));  // from the call's beginning: ahead of the wait
+  if (AHEAD) matrices(0, min(32, g));  // from the call's beginning: ahead of the wait
   pdl_wait();
+  auto to_update = [&](int r) { return reinterpret_cast<double2*>(Wt + ((long long)head * dh + i0 + g + r) * d + c0 + ct); };
   double2 old[8];  // the rows to be updated, on their way while the product is formed
+  if (AHEAD) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int r = q0 + rt + 4 * k;
-    old[k] = (r < nrem) ? *reinterpret_cast<const double2*>(Wt + ((long long)head * dh + i0 + g + r) * d + c0 + ct) : make_double2(0.0, 0.0);
+    for (int k = 0; k < 8; ++k) {
+      const int r = q0 + rt + 4 * k;
+      old[k] = (r < nrem) ? *to_update(r) : make_double2(0.0, 0.0);
+    }
   }
   double acc[8][2];
 #pragma unroll
@@ -387,7 +392,7 @@ __global__ void __launch_bounds__(256) k_compensate(double* Wt, const unsigned c
       }
       *reinterpret_cast<double2*>(&Es[r][c]) = v;
     }
-    if (e0 > 0) matrices(e0, ge);
+    if (!AHEAD || e0 > 0) matrices(e0, ge);
     __syncthreads();
     for (int i = 0; i < ge; ++i) {
       const double2 e = *reinterpret_cast<const double2*>(&Es[i][ct]);
@@ -404,11 +409,17 @@ __global__ void __launch_bounds__(256) k_compensate(double* Wt, const unsigned c
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int r = q0 + rt + 4 * k;
-    if (r < nrem)
-      *reinterpret_cast<double2*>(Wt + ((long long)head * dh + i0 + g + r) * d + c0 + ct) =
-          make_double2(old[k].x - acc[k][0], old[k].y - acc[k][1]);
+    if (r >= nrem) continue;
+    const double2 v = AHEAD ? old[k] : *to_update(r);
+    *to_update(r) = make_double2(v.x - acc[k][0], v.y - acc[k][1]);
   }
 }
+
+// Which form of k_compensate: ahead without R for steps of up to 8 rows (4096 columns, 64 heads: 94 -> 88 us) and as long as CTAs
+// times rows stay below 48 K (4096 columns, 16 heads: 16 rows 35.6 -> 33.1 us, 32 rows 47.8 -> 44.2, 64 rows 73.5 against 75.0 with
+// it; 8192 columns, 64 heads, 64 rows 490 against 536); with R for what the SMs hold at once in that form (4096 columns, 4 heads, 64
+// rows 18.7 -> 17.0; 16 heads 46.4 against 61.9, 8192 columns and 64 heads 317 against 494).
+static bool comp_ahead(long long ctas, int g, bool with_r) { return with_r ? ctas <= 2 * 148 : g <= 8 || ctas * g <= 48 * 1024; }
 
 // ---------------------------------------------------------------------------
 // Coordinate descent on the scales (Proposition 3.3 / Algorithm 3), with the
@@ -1533,10 +1544,10 @@ extern "C" tb_status tb_quantize_layer(const tb_layer_desc* desc, const float* W
     const dim3 cgrid(d / 128, p.H, (nrem + 31) / 32);
     const double* Ti = p.T + (long long)step * p.dh * p.g;
     const long long t_head = (long long)p.S * p.dh * p.g;
-    if (with_r)
-      TB_CUDA_CHECK(launch_pdl(k_compensate<true>, cgrid, dim3(256), 0, st, p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng));
-    else
-      TB_CUDA_CHECK(launch_pdl(k_compensate<false>, cgrid, dim3(256), 0, st, p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng));
+    const bool ahead = comp_ahead((long long)cgrid.x * cgrid.y * cgrid.z, p.g, with_r);
+    auto* kern = with_r ? (ahead ? k_compensate<true, true> : k_compensate<true, false>)
+                        : (ahead ? k_compensate<false, true> : k_compensate<false, false>);
+    TB_CUDA_CHECK(launch_pdl(kern, cgrid, dim3(256), 0, st, p.Wt, codes, p.sD, zeros, p.E, Ti, i0, p.g, p.dh, t_head, d, p.seg, p.ng));
     TB_LAUNCH_CHECK();
   }
 

@@ -13,6 +13,15 @@ def test_compensation_matrices(dh, g):
     compare(prob, run_gpu(prob, 3, 64, g, 0), 3, 64, g, 0, label=f"comp{dh}")
 
 
+# launches of few CTAs, which fetch the rows to be updated ahead, and of many, which do not: steps that take the group in one
+# pass of 32 rows and in two, remaining rows that are no whole tile
+@pytest.mark.parametrize("d,heads,dh,g,with_r", [(256, 3, 90, 45, False), (1152, 64, 96, 48, False), (1152, 64, 69, 23, False),
+                                                 (256, 3, 90, 45, True), (640, 40, 90, 45, True), (640, 40, 81, 9, True)])
+def test_compensation_of_few_and_many_rows(d, heads, dh, g, with_r):
+    prob = make_problem(77, d, heads, dh, 1024, with_r=with_r, hout="spd")
+    compare(prob, run_gpu(prob, 3, 128, g, 0), 3, 128, g, 0, heads=[0, heads // 2, heads - 1], label=f"comp{heads}")
+
+
 def test_codes_at_an_odd_address():
     """The codes may lie anywhere: the joint compensation reads them back a byte at a time."""
     import torch
